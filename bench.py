@@ -240,6 +240,18 @@ def time_router(mr, torch, bufs, k, gate_mode, steps, warmup, stream):
     return ev0.elapsed_time(ev1) * 1e-3
 
 
+def kernel_of(mr, plan, bufs, k, gate_mode, stream):
+    """Which kernels serve a shape: the chain launches three per call, the others are one kernel each."""
+    X, R1, R2, idx, gate, counts = bufs[0]
+    l0 = mr.launches()
+    mr.more_route(X, R1, R2, k, gate_mode, idx, gate, counts, stream)
+    if plan.path != 2:
+        return "generic_route_tokens"
+    if mr.launches() - l0 > 1:
+        return "project_kernel + sweep_kernel + finish"
+    return "route_tcgen05_kernel" if plan.paired else "route_lowrank_kernel"
+
+
 def make_bufs(torch, case, copies):
     def dev(a):
         return torch.from_numpy(a.view(np.int16)).cuda().view(torch.bfloat16)
@@ -488,8 +500,7 @@ def main():
     cnt = counters.get(f"{name}/mode{gate_mode}", {})
     plan = mr.more_route_plan_ex(case.T, case.h, case.r, case.M, k, gate_mode)
     roof = roofline(case.T, case.h, case.r, case.M, k, secs / args.steps, peaks, cnt.get("dram_bytes"))
-    roof["kernel"] = ("generic_route_tokens" if plan.path != 2 else
-                      ("route_tcgen05_kernel" if plan.paired else "route_lowrank_kernel"))
+    roof["kernel"] = kernel_of(mr, plan, bufs, k, gate_mode, stream)
     roof.update(diagnostic_bounds(case.T, case.M, gate_mode, cnt.get("warp_instr_per_chunk"), clocks.get("sm_mhz")))
     roof["traffic_source"] = cnt.get("source")
     line = dict(metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
@@ -560,7 +571,7 @@ def main():
                                                     bound=r["bound"], roofline_frac=r["frac"], msplit=oplan.msplit,
                                                     ctas=oplan.ctas, block_tokens=oplan.block_tokens,
                                                     expert_ranges=oplan.expert_ranges,
-                                                    kernel="route_tcgen05_kernel" if oplan.paired else "route_lowrank_kernel",
+                                                    kernel=kernel_of(mr, oplan, obufs, ocase.k, gm, stream),
                                                     host_us_per_call=host_us_per_call(mr, torch, obufs, ocase.k, gm, stream, 100),
                                                     **diagnostic_bounds(ocase.T, ocase.M, gm, ocnt.get("warp_instr_per_chunk"),
                                                                         clocks.get("sm_mhz")))

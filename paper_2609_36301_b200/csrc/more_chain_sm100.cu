@@ -1,0 +1,1393 @@
+// The low-rank router (Algorithm 1 with the gates of Section 2 / Eq. app_softmax and the per-expert counts) for few tokens
+// and for long sweeps, as three kernels chained with programmatic dependent launches:
+//
+//   project_kernel   z = X R1, narrowed to a bf16 pair [hi | lo] per token, to scratch (T x 128 or 256 bytes).
+//   sweep_kernel     y = z R2 tile by tile on the tensor cores, reduced on chip to a short list of candidates per token
+//                    (and the online (max, sum) pair of Eq. app_online); the T x M logits never reach memory.
+//   finish_*_kernel  the candidates of all of a token's expert ranges -> sorted top-k, gates, histogram.
+//
+// Why three.  The projection is bound by reading X, the sweep by the tensor cores and by looking at every logit; with z
+// in scratch the sweep can be cut anywhere along tokens x experts (every CTA gets the same number of steps, whatever T
+// and M are), a token block whose experts are shared by many CTAs is projected once instead of once per CTA, and shared
+// and tensor memory belong to the sweep alone.  z costs 2 x T x 256 bytes of L2 traffic, 1/8 of X at h = 2048.
+#include "more_topk.cuh"
+#include "sm100_common.cuh"
+
+#include <cuda_bf16.h>
+
+#include <type_traits>
+
+namespace more {
+
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kRows = 128;                         // tokens per block: the rows of one accumulator
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// ============================================================================================== projection
+// One cluster of `cs` CTAs per 128-token block; CTA `rank` contracts an even share of the h / 64 k-tiles.  With cs > 1
+// the partial sums are exchanged through distributed shared memory: every CTA collects 128 / cs rows from all, adds them
+// in rank order (so the result does not depend on timing) and narrows them.
+constexpr int kPThreads = 192;                     // warp 0 TMA, warp 1 MMA, warps 2..5 one token per thread
+constexpr int kPStages = 4;
+constexpr int kPStageBytes = kRows * 128 + 64 * 128;      // X tile 128 x 64, R1 tile 64 x 64 (columns >= r zero-filled)
+constexpr int kPExchange = kRows * 64 * 4;         // [rank][row share][64] fp32
+constexpr int kPCtl = 1024;
+
+struct ProjectParams {
+    int T, h, cs, n, zc;                           // n: columns of z computed (16, 32, 48, 64); zc: bf16 per row of z
+    uint32_t* z;                                   // [blocks * 128][zc / 2]
+    int32_t* counts;                               // cleared here: [M] (null for the later chunks of one call)
+    int M;
+    int* status;
+};
+
+__device__ __forceinline__ void narrow2(float a, float b, uint32_t& hi, uint32_t& lo)
+{
+    const __nv_bfloat16 h0 = __float2bfloat16_rn(a), h1 = __float2bfloat16_rn(b);
+    const __nv_bfloat16 l0 = __float2bfloat16_rn(a - __bfloat162float(h0)), l1 = __float2bfloat16_rn(b - __bfloat162float(h1));
+    hi = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+    lo = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+}
+
+__global__ void __launch_bounds__(kPThreads)
+project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_r1, const ProjectParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t ring = (raw + 1023u) & ~1023u;
+    uint8_t* ring_ptr = smem_raw + (ring - raw);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(ring_ptr + kPStages * kPStageBytes);
+    constexpr int B_FULL = 0, B_EMPTY = kPStages, B_DONE = 2 * kPStages, B_COUNT = B_DONE + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    float* exch = reinterpret_cast<float*>(ring_ptr + kPStages * kPStageBytes + kPCtl);
+    const uint32_t bar0 = smem_u32(bars);
+    auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cs = p.cs, rank = blockIdx.x % cs, blk = blockIdx.x / cs;
+    const int nkt = (p.h + 63) / 64;
+    const int kt_lo = nkt * rank / cs, kt_hi = nkt * (rank + 1) / cs;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(smem_u32(tmem_slot)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (cs > 1) cluster_sync();                    // every CTA of the cluster is running before anyone writes into it
+    pdl_wait();                                    // the set-up above overlaps the end of what ran before
+    // The sweep may be placed next to this kernel from here on: this CTA's tensor memory is allocated, so the sweep's
+    // own allocation can only wait for it, never take it away.
+    pdl_launch_dependents();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            bool ok = true;
+            for (int kt = kt_lo, i = 0; kt < kt_hi && ok; ++kt, ++i) {
+                const int s = i % kPStages;
+                if (i >= kPStages) ok = mbar_wait(bar(B_EMPTY + s), ((i / kPStages) - 1) & 1, abort_flag, p.status);
+                if (!ok) break;
+                const uint32_t dst = ring + s * kPStageBytes;
+                mbar_expect_tx(bar(B_FULL + s), kPStageBytes);
+                tma_load_2d(dst, &map_x, bar(B_FULL + s), kt * 64, blk * kRows);
+                tma_load_2d(dst + kRows * 128, &map_r1, bar(B_FULL + s), 0, kt * 64);
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        bool ok = true;
+        const uint32_t idesc = umma_idesc(p.n);
+        const uint64_t xd = umma_desc_sw128(ring, 16, 1024), rd = umma_desc_sw128(ring + kRows * 128, 8192, 1024);
+        const uint32_t x_lo0 = (uint32_t)xd, x_hi = (uint32_t)(xd >> 32), r_lo0 = (uint32_t)rd, r_hi = (uint32_t)(rd >> 32);
+        for (int kt = kt_lo, i = 0; kt < kt_hi && ok; ++kt, ++i) {
+            const int s = i % kPStages;
+            ok = __all_sync(kFull, mbar_wait(bar(B_FULL + s), (i / kPStages) & 1, abort_flag, p.status));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t x_lo = x_lo0 + s * (kPStageBytes >> 4), r_lo = r_lo0 + s * (kPStageBytes >> 4);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)         // A: +32 B per K = 16; B: 16 K-rows of 128 B
+                tc_mma_bf16_ss_elect(tmem_base, x_lo + kk * 2, x_hi, r_lo + kk * (2048 >> 4), r_hi, idesc, (i | kk) != 0);
+            tc_commit_elect(bar(B_EMPTY + s));
+        }
+        if (ok) tc_commit_elect(bar(B_DONE));
+        __syncwarp();
+    } else {
+        const int et = threadIdx.x - 64;           // 0..127
+        if (p.counts)
+            for (int e = blockIdx.x * kRows + et; e < p.M; e += gridDim.x * kRows) p.counts[e] = 0;
+        const int row = (warp & 3) * 32 + lane;    // the tensor-memory lane this thread may read
+        const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        const bool ok = __all_sync(kFull, mbar_wait(bar(B_DONE), 0, abort_flag, p.status));
+        tc_fence_after();
+        if (cs == 1) {
+            if (ok) {
+                uint4* zr = reinterpret_cast<uint4*>(p.z + (size_t)(blk * kRows + row) * (p.zc / 2));
+                const int lo_off = p.zc / 16;      // 16-byte chunks of the hi half
+                for (int c = 0; c < p.zc / 32; ++c) {
+                    float v[16];
+                    if (c * 16 < p.n) {
+                        tmem_ld16(t_lane + c * 16, v);
+                        tmem_ld_wait16(v);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) v[e] = 0.f;
+                    }
+                    uint32_t hi[8], lo[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) narrow2(v[2 * e], v[2 * e + 1], hi[e], lo[e]);
+                    zr[2 * c] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                    zr[2 * c + 1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
+                    zr[lo_off + 2 * c] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                    zr[lo_off + 2 * c + 1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+                }
+            }
+        } else if (ok) {
+            const int share = kRows / cs, dst = row / share;
+            const uint32_t a = smem_u32(exch) + (uint32_t)((rank * share + row % share) * 64) * 4u;
+            uint32_t remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(a), "r"(dst));
+            for (int c = 0; c * 16 < p.n; ++c) {
+                float v[16];
+                tmem_ld16(t_lane + c * 16, v);
+                tmem_ld_wait16(v);
+#pragma unroll
+                for (int e = 0; e < 16; e += 4)
+                    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};"
+                                 ::"r"(remote + (c * 16 + e) * 4), "f"(v[e]), "f"(v[e + 1]), "f"(v[e + 2]), "f"(v[e + 3]) : "memory");
+            }
+        }
+    }
+    tc_fence_before();
+    if (cs > 1) {
+        cluster_sync();
+        if (warp >= 2) {
+            const int share = kRows / cs, q4 = p.zc / 8;         // float4s of one row of z
+            for (int i = threadIdx.x - 64; i < share * q4; i += kRows) {
+                const int rr = i / q4, c4 = i % q4;
+                float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c4 * 4 < p.n) {
+                    for (int q = 0; q < cs; ++q) {
+                        const float4 v = *reinterpret_cast<const float4*>(exch + (q * share + rr) * 64 + c4 * 4);
+                        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+                    }
+                }
+                uint2 hi, lo;
+                narrow2(s.x, s.y, hi.x, lo.x);
+                narrow2(s.z, s.w, hi.y, lo.y);
+                uint2* zr = reinterpret_cast<uint2*>(p.z + (size_t)(blk * kRows + rank * share + rr) * (p.zc / 2));
+                zr[c4] = hi;
+                zr[q4 + c4] = lo;
+            }
+        }
+    }
+    __syncthreads();
+    if (*abort_flag && threadIdx.x == 0)
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);         // copies still in flight land before the memory is released
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem_base) : "memory");
+    }
+}
+
+// ================================================================================================== sweep
+// Two CTAs per SM, 18 warps each: warp 0 TMA, warp 1 MMA, warps 2..17 selection.  The work is a line of blocks x steps
+// units (unit = 128 tokens x 128 experts) cut into equal contiguous parts, one per CTA; what a CTA has of one token block
+// is a segment.  Per unit 2 r / 16 MMAs (hi then lo) of 128 x 128 x 16 fill one of two accumulators; four warps per
+// tensor-memory lane quarter look at 32 columns each, so a token is swept by four threads.  (What bounds the sweep is
+// the selection's instructions and their latencies: 32 selecting warps per SM at 56 registers hide these about twice
+// as well as 16 at 96, with any arrangement of the accumulators that was tried.)
+//
+// Selection.  A thread keeps the maxima of NB disjoint sets of its columns ("buckets": runs of 8 or 4 columns, by their
+// position in the units) and a threshold.  The k-th largest of a token's 4 NB bucket maxima is reached by
+// at least k of its logits, so nothing strictly below it can be selected; its expected rank is ~11 for k = 8 of 16
+// buckets, ~22 for k = 16 of 32.  Every group of four whose maximum beats the threshold is appended, values and first
+// column, to the thread's list in global scratch (which stays in L2): two predicated stores and an add, and nothing
+// waits for them.  A sweep starts with a threshold: the bucket maxima of its first eighth (of its first two units, if
+// that is no more) are formed before anything is selected; this costs an eighth more MMAs, and saves the appends of the
+// start, when nearly everything beats what has been seen.  After 1/8 of the sweep, and whenever half as much again is done, the buckets are published
+// in shared memory, one of the four warps of a lane quarter computes new thresholds from them, and the others pick these
+// up when they see them (all values are monotone lower bounds, so no synchronisation is needed).  At the end of a
+// segment a thread goes once through its list and keeps what beats the final threshold (~11 logits per token).
+constexpr int kSThreads = 576;
+constexpr int kEpi = 512;
+constexpr int W = 128;                             // experts of a unit
+constexpr int kCols = W / 4;                       // columns of a thread
+constexpr int kMaxStages = 8;
+constexpr int kListCap = 64;                       // entries of a thread's list
+constexpr uint32_t kEntry = kEpi * 32;             // bytes between its entries (32 bytes each: four logits, the first one's column)
+
+// Units whose bucket maxima are formed ahead of a segment of `steps` units; up to two stay in the accumulators.
+__host__ __device__ __forceinline__ int lead_of(int steps) { return steps >= 24 ? steps / 8 : (steps < 2 ? steps : 2); }
+
+struct SweepParams {
+    int T, M, k;
+    int nsteps, ks, rk, wide;                      // steps per token block; K-steps per half; rows of an R2 box; r > 32
+    long long total;                               // units
+    int maxseg, cap;                               // candidate lists per token block in scratch, entries per list and token
+    int nst, st_bytes, zbufs, z_bytes;
+    int off_r2, off_pub, off_ctl;
+    uint8_t* list;                                 // [CTA][kListCap][512] x 32 bytes
+    uint2* ent;                                    // [block][seg][128][cap] (logit bits, expert id)
+    int* cnt;                                      // [block][seg][128]
+    float2* mz;                                    // [block][seg][128] (max in log2 units, sum); LSE only
+    int* status;
+};
+
+// CTA that owns unit u when `total` units are cut into g parts, part c = [total c / g, total (c + 1) / g)
+__host__ __device__ __forceinline__ int owner_of(long long u, long long total, int g) { return (int)(((u + 1) * g - 1) / total); }
+
+// 16 consecutive fp32 columns of this thread's tensor-memory lane, complete on return.  (Load and wait in one statement:
+// with the destination registers tied to a separate wait the compiler copies them.)
+__device__ __forceinline__ void tmem_get16(uint32_t taddr, float (&v)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+                 : "r"(taddr)
+                 : "memory");
+}
+// One arrival for a warp whose lanes have all completed their tensor-memory loads (the wait for these is warp-wide).
+__device__ __forceinline__ void arrive_lane0(uint32_t bar, int lane)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"(lane) : "memory");
+}
+// Wait that lets the caller go on after a time-out (what it computes then is not used): the code that follows keeps its
+// warp-uniform control flow and its barriers.
+__device__ __forceinline__ void wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status)
+{
+    (void)mbar_wait(bar, parity, abort_flag, status);
+}
+
+// descending compare-exchange, and sorting networks over registers
+__device__ __forceinline__ void cx(float& a, float& b)
+{
+    const float h = fmaxf(a, b);
+    b = fminf(a, b);
+    a = h;
+}
+__device__ __forceinline__ void sort8(float (&s)[8])
+{
+    cx(s[0], s[1]); cx(s[2], s[3]); cx(s[4], s[5]); cx(s[6], s[7]);
+    cx(s[0], s[2]); cx(s[1], s[3]); cx(s[4], s[6]); cx(s[5], s[7]);
+    cx(s[1], s[2]); cx(s[5], s[6]);
+    cx(s[0], s[4]); cx(s[1], s[5]); cx(s[2], s[6]); cx(s[3], s[7]);
+    cx(s[2], s[4]); cx(s[3], s[5]);
+    cx(s[1], s[2]); cx(s[3], s[4]); cx(s[5], s[6]);
+}
+template <int N>
+__device__ __forceinline__ void bitonic_down(float (&s)[N])
+{
+#pragma unroll
+    for (int d = N / 2; d > 0; d >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if ((i & d) == 0) cx(s[i], s[i + d]);
+}
+// Append the groups of four (maxima t, values v, first column col + 4 i) that beat thr to a list that ends at `end`.  The
+// four tests come first: only the adds to the list's end depend on each other.  `one` is 1, unknown to the compiler: a
+// predicated 64-bit multiply-add is one instruction, a predicated 64-bit add is four.
+__device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t, const float* v, int col, uint32_t one)
+{
+#define MORE_APPEND(P, COL, A, B, C, D)                                                                     \
+    "@" P " st.global.v4.f32 [%0], {" A ", " B ", " C ", " D "};\n\t@" P " st.global.b32 [%0+16], " COL ";\n\t" \
+    "@" P " mad.wide.u32 %0, %24, %22, %0;\n\t"
+    asm volatile(
+        "{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 c1, c2, c3;\n\t"
+        "setp.gt.f32 p0, %2, %1;\n\tsetp.gt.f32 p1, %3, %1;\n\tsetp.gt.f32 p2, %4, %1;\n\tsetp.gt.f32 p3, %5, %1;\n\t"
+        "add.u32 c1, %23, 4;\n\tadd.u32 c2, %23, 8;\n\tadd.u32 c3, %23, 12;\n\t"
+        MORE_APPEND("p0", "%23", "%6", "%7", "%8", "%9") MORE_APPEND("p1", "c1", "%10", "%11", "%12", "%13")
+        MORE_APPEND("p2", "c2", "%14", "%15", "%16", "%17") MORE_APPEND("p3", "c3", "%18", "%19", "%20", "%21") "}"
+        : "+l"(end)
+        : "f"(thr), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]),
+          "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]),
+          "f"(v[15]), "n"(kEntry), "r"(col), "r"(one)
+        : "memory");
+#undef MORE_APPEND
+}
+// strictly below x, by a hair: a logit equal to x still beats it
+__device__ __forceinline__ float just_below(float x) { return fmaf(-fabsf(x), 2.4e-7f, x) - 1e-37f; }
+
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate)
+{
+    if (accumulate)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, 0, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                     ::"r"(d), "l"(a), "l"(b), "r"(idesc) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, 0, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                     ::"r"(d), "l"(a), "l"(b), "r"(idesc) : "memory");
+}
+
+__device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory"); }
+
+template <int KCAP, bool LSE>
+__global__ void __launch_bounds__(kSThreads, 2)
+sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_r2, const SweepParams p)
+{
+    constexpr int NB = KCAP <= 8 ? 4 : 8;          // buckets of a thread
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* base_ptr = smem_raw + (base - raw);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base_ptr + p.off_ctl);
+    constexpr int B_ZF = 0, B_ZE = 2, B_RF = 4, B_RE = B_RF + kMaxStages, B_AF = B_RE + kMaxStages, B_AE = B_AF + 2,
+                  B_COUNT = B_AE + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const uint32_t bar0 = smem_u32(bars);
+    auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+
+    const int warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (the compiler sees a uniform value)
+    const int g = (int)gridDim.x;
+    const long long lo = p.total * blockIdx.x / g, hi = p.total * (blockIdx.x + 1) / g;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < B_AE; ++i) mbar_init(bar(i), 1);
+        mbar_init(bar(B_AE), kEpi / 32);
+        mbar_init(bar(B_AE + 1), kEpi / 32);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(256)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        // ===================================================================================== TMA producer
+        if (lane == 0) {
+            bool ok = true;
+            int st = 0, ph = 0;
+            const uint32_t r2 = base + p.off_r2;
+            auto load_r2 = [&](int step) {
+                ok = mbar_wait(bar(B_RE + st), ph ^ 1, abort_flag, p.status);
+                if (!ok) return;
+                mbar_expect_tx(bar(B_RF + st), p.st_bytes);
+#pragma unroll
+                for (int j = 0; j < W / 64; ++j)
+                    tma_load_2d(r2 + st * p.st_bytes + j * p.rk * 128, &map_r2, bar(B_RF + st), step * W + j * 64, 0);
+                if (++st == p.nst) { st = 0; ph ^= 1; }
+            };
+            int blk = (int)(lo / p.nsteps), s0 = (int)(lo - (long long)blk * p.nsteps), seg = 0;
+            for (int left = (int)(hi - lo); left > 0 && ok; ++blk, ++seg, s0 = 0) {
+                const int steps = min(left, p.nsteps - s0);
+                left -= steps;
+                const int lead = lead_of(steps), total = steps + (lead > 2 ? lead : 0);
+                auto step_of = [&](int v) { return s0 + (v >= lead && lead > 2 ? v - lead : v); };
+                int v = 0;
+                if (seg == 0) {
+                    // R2 comes from the caller, not from the projection: the first stages are requested before waiting for it
+                    for (; v < total && v < p.nst && ok; ++v) load_r2(step_of(v));
+                    pdl_wait();
+                }
+                const int zb = seg % p.zbufs;
+                if (seg >= p.zbufs) ok = ok && mbar_wait(bar(B_ZE + zb), ((seg / p.zbufs) - 1) & 1, abort_flag, p.status);
+                if (!ok) break;
+                mbar_expect_tx(bar(B_ZF + zb), p.z_bytes);
+                tma_load_2d(base + zb * p.z_bytes, &map_z, bar(B_ZF + zb), 0, blk * kRows);
+                if (p.wide) tma_load_2d(base + zb * p.z_bytes + kRows * 128, &map_z, bar(B_ZF + zb), 64, blk * kRows);
+                for (; v < total && ok; ++v) load_r2(step_of(v));
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ======================================================================================= MMA issuer
+        // One elected lane runs the whole loop, unrolled over the K-steps: with eight or nine other warps on its scheduler
+        // every instruction here counts several times, and one unit's MMAs compute for 150 to 584 clocks only.
+        constexpr uint32_t idesc = umma_idesc(W);
+        auto run = [&](auto ksteps) {
+            constexpr int KS = decltype(ksteps)::value;
+            const uint64_t zd = umma_desc_sw128(base, 16, 1024), bd = umma_desc_sw128(base + p.off_r2, KS * 2048, 1024);
+            const uint32_t lo_off = KS > 2 ? (kRows * 128) >> 4 : 4;     // from the hi half of z to the lo half, in 16 bytes
+            int st = 0, ph = 0, seg = 0;
+            uint32_t n = 0;
+            int s0 = (int)(lo % p.nsteps);
+            for (int left = (int)(hi - lo); left > 0; ++seg, s0 = 0) {
+                const int steps = min(left, p.nsteps - s0);
+                left -= steps;
+                const int lead = lead_of(steps), total = steps + (lead > 2 ? lead : 0);
+                const int zb = p.zbufs == 2 ? seg & 1 : 0, zuse = p.zbufs == 2 ? seg >> 1 : seg;
+                wait_or_abort(bar(B_ZF + zb), zuse & 1, abort_flag, p.status);
+                const uint64_t z = zd + zb * (p.z_bytes >> 4);
+                for (int v = 0; v < total; ++v, ++n) {
+                    const int buf = n & 1;
+                    // (both are mostly complete: two tests, one branch)
+                    if (!(mbar_try_wait(bar(B_RF + st), ph) & mbar_try_wait(bar(B_AE + buf), ((n >> 1) & 1) ^ 1))) {
+                        wait_or_abort(bar(B_RF + st), ph, abort_flag, p.status);
+                        wait_or_abort(bar(B_AE + buf), ((n >> 1) & 1) ^ 1, abort_flag, p.status);
+                    }
+                    tc_fence_after();
+                    const uint64_t b = bd + st * (p.st_bytes >> 4);
+                    const uint32_t d = tmem_base + buf * W;
+                    // hi, then lo, into one accumulator: z K-major (+32 bytes per K-step), R2 MN-major (+16 rows of 128 bytes)
+#pragma unroll
+                    for (int j = 0; j < KS; ++j) mma_ss(d, z + 2 * j, b + 128 * j, idesc, j != 0);
+#pragma unroll
+                    for (int j = 0; j < KS; ++j) mma_ss(d, z + lo_off + 2 * j, b + 128 * j, idesc, true);
+                    tc_commit(bar(B_AF + buf));
+                    tc_commit(bar(B_RE + st));
+                    if (++st == p.nst) { st = 0; ph ^= 1; }
+                }
+                tc_commit(bar(B_ZE + zb));
+            }
+        };
+        if (elect_one()) {
+            if (p.ks == 4) run(std::integral_constant<int, 4>{});
+            else if (p.ks == 3) run(std::integral_constant<int, 3>{});
+            else if (p.ks == 2) run(std::integral_constant<int, 2>{});
+            else run(std::integral_constant<int, 1>{});
+        }
+        __syncwarp();
+    } else {
+        // ======================================================================================== selection
+        const int q = warp & 3;                              // tensor-memory lane quarter
+        const int sub = (warp - 2) >> 2;                     // column quarter
+        const int row = q * 32 + lane;                       // token of the block
+        const int M = p.M, nsteps = p.nsteps;
+        const uint32_t t_col = tmem_base + ((uint32_t)(q * 32) << 16) + sub * kCols;
+        // the thread's list; a unit adds at most 8 entries between two looks at its length
+        const uint64_t first = reinterpret_cast<uint64_t>(p.list) + (uint64_t)blockIdx.x * (kListCap * kEntry) + (threadIdx.x - 64) * 32;
+        const uint64_t warn = first + (kListCap - kCols / 4) * kEntry;
+        // shared memory: published buckets [sub][128][NB], thresholds [128], counters [128], (m, Z) [sub - 1][128]
+        const uint32_t pub0 = base + p.off_pub + row * (NB * 4);
+        const uint32_t s_thr = base + p.off_pub + 4 * kRows * NB * 4 + row * 4;
+        const uint32_t s_cnt = s_thr + kRows * 4;
+        const uint32_t s_mz = base + p.off_pub + 4 * kRows * NB * 4 + kRows * 8 + row * 8;
+        uint32_t n = 0, one;
+        asm volatile("mov.u32 %0, 1;" : "=r"(one));
+        float b[NB];
+        float thr, m2, zsum;
+        uint64_t ptr;                                        // where the next entry goes
+
+        auto ent4 = [&](uint64_t o) { return *reinterpret_cast<const float4*>(o); };
+        auto ent_col = [&](uint64_t o) { return *reinterpret_cast<const int*>(o + 16); };
+        auto put = [&](uint64_t o, float4 e, int c) {
+            *reinterpret_cast<float4*>(o) = e;
+            *reinterpret_cast<int*>(o + 16) = c;
+        };
+        auto publish = [&]() {
+#pragma unroll
+            for (int i = 0; i < NB; i += 4)
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(pub0 + sub * (kRows * NB * 4) + i * 4), "f"(b[i]), "f"(b[i + 1]), "f"(b[i + 2]), "f"(b[i + 3]) : "memory");
+        };
+        // threshold of the token from the published buckets of its four threads
+        auto compute_thr = [&]() {
+            auto fetch4 = [&](uint32_t at, float* x) {
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(at) : "memory");
+            };
+            float kth;
+            if constexpr (KCAP <= 8) {
+                float a[8], y[8];
+                fetch4(pub0, a);
+                fetch4(pub0 + kRows * 16, a + 4);
+                fetch4(pub0 + kRows * 32, y);
+                fetch4(pub0 + kRows * 48, y + 4);
+                sort8(a);
+                sort8(y);
+                // the eight best of two sorted lists: entry against mirrored entry, then a bitonic sort
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] = fmaxf(a[i], y[7 - i]);
+                if (p.k == 8) {
+                    kth = fminf(fminf(fminf(a[0], a[1]), fminf(a[2], a[3])), fminf(fminf(a[4], a[5]), fminf(a[6], a[7])));
+                } else {
+                    bitonic_down(a);
+                    kth = a[0];
+#pragma unroll
+                    for (int i = 1; i < 8; ++i) kth = (i < p.k) ? a[i] : kth;
+                }
+            } else {
+                float a[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) a[i] = -INFINITY;
+                float least = INFINITY;
+#pragma unroll 1
+                for (int o = 0; o < 4; ++o) {
+                    float x[8];
+                    fetch4(pub0 + o * (kRows * 32), x);
+                    fetch4(pub0 + o * (kRows * 32) + 16, x + 4);
+                    sort8(x);
+                    least = fminf(least, x[7]);
+                    // the 16 best of two sorted lists
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) a[8 + i] = fmaxf(a[8 + i], x[7 - i]);
+                    bitonic_down(a);
+                }
+                kth = a[0];
+#pragma unroll
+                for (int i = 1; i < 16; ++i) kth = (i < p.k) ? a[i] : kth;
+                if (p.k > 16) kth = least;                   // all 32 buckets reach the smallest of them
+            }
+            return just_below(kth);
+        };
+        // k-th largest logit of this thread's own list and how many equal to it are wanted (all of them in a short list)
+        auto own_kth = [&](int& equal) {
+            float cur = INFINITY;
+            int need = p.k;
+            for (;;) {
+                float m = -INFINITY;
+                int c = 0;
+                for (uint64_t o = first; o < ptr; o += kEntry) {
+                    const float4 e = ent4(o);
+                    const float x[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (x[j] < cur) {
+                            if (x[j] > m) { m = x[j]; c = 1; }
+                            else if (x[j] == m) ++c;
+                        }
+                }
+                if (c >= need || c == 0) { equal = need; return m; }
+                need -= c;
+                cur = m;
+            }
+        };
+        // make room in the lists of a warp: drop what has fallen below the threshold, first raising it by what the thread
+        // knows itself; a list that stays long is cut to its k best (later equals then lose to those: larger ids)
+        auto compact = [&]() {
+            if (p.k <= NB) {
+                float mine = b[0];
+#pragma unroll
+                for (int i = 1; i < NB; ++i) mine = fminf(mine, b[i]);
+                thr = fmaxf(thr, just_below(mine));
+            }
+            auto keep = [&](float low, int equal) {
+                uint64_t wr = first;
+                for (uint64_t rd = first; rd < ptr; rd += kEntry) {
+                    const float4 e = ent4(rd);
+                    const float m = fmaxf(max3(e.x, e.y, e.z), e.w);
+                    const bool take = m > low || (m == low && equal > 0);
+                    if (equal > 0) equal -= (e.x == low) + (e.y == low) + (e.z == low) + (e.w == low);
+                    if (take) {
+                        put(wr, e, ent_col(rd));
+                        wr += kEntry;
+                    }
+                }
+                ptr = wr;
+            };
+            keep(just_below(thr), 0);
+            if (ptr > warn) {
+                int equal;
+                const float kth = own_kth(equal);
+                keep(kth, equal);
+                thr = fmaxf(thr, kth);
+            }
+            __syncwarp();
+        };
+        // candidates of the list that beat `low` (or are among the first `equal` that equal it) -> scratch
+        auto emit = [&](uint2* dst, float low, int equal) {
+            for (uint64_t o = first; o < ptr; o += 4 * kEntry) {
+                float4 e[4];
+                int c[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {                // (independent loads: one round trip for four entries)
+                    e[i] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                    c[i] = 0;
+                    if (o + i * kEntry < ptr) { e[i] = ent4(o + i * kEntry); c[i] = ent_col(o + i * kEntry); }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (!(fmaxf(max3(e[i].x, e[i].y, e[i].z), e[i].w) >= low)) continue;
+                    const float x[4] = {e[i].x, e[i].y, e[i].z, e[i].w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const bool eq = x[j] == low && equal > 0;
+                        if (x[j] > low || eq) {
+                            equal -= eq ? 1 : 0;
+                            int at;
+                            asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(at) : "r"(s_cnt) : "memory");
+                            if (at < p.cap) dst[at] = make_uint2(__float_as_uint(x[j]), (uint32_t)(c[i] + j));
+                        }
+                    }
+                }
+            }
+        };
+        auto lds = [&](uint32_t a) { float v; asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory"); return v; };
+        auto sts = [&](uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); };
+
+        // (units of this CTA as a block, a step in it and a count: 32-bit loop state)
+        int blk = (int)(lo / nsteps), s0 = (int)(lo - (long long)blk * nsteps);
+        for (int left = (int)(hi - lo); left > 0; ++blk, s0 = 0) {
+            const int steps = min(left, nsteps - s0);
+            left -= steps;
+            const int live = min(kRows, p.T - blk * kRows);
+            const bool warp_live = q * 32 < live;
+            const bool row_live = row < live;
+#pragma unroll
+            for (int i = 0; i < NB; ++i) b[i] = -INFINITY;
+            thr = row_live ? -INFINITY : INFINITY;
+            m2 = -INFINITY;
+            zsum = 0.f;
+            ptr = first;
+            const int lead = lead_of(steps), again = lead > 2 ? lead : 0;      // units ahead, and how many of them come again
+            int next = lead, turn = 0;
+            // maxima of 16 columns' groups of four; what lies beyond M is nothing (M is a multiple of 8)
+            auto group_max = [&](auto masked, const float (&v)[16], int col, float (&t)[4]) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    t[i] = fmaxf(max3(v[4 * i], v[4 * i + 1], v[4 * i + 2]), v[4 * i + 3]);
+                    if (decltype(masked)::value && col + 4 * i >= M) t[i] = -INFINITY;
+                }
+            };
+            // buckets of 16 columns at h in a unit: a bucket per 8 columns, or per 4
+            auto bucket = [&](int h, const float (&t)[4]) {
+                if constexpr (NB == 4) {
+                    b[h / 8] = max3(b[h / 8], t[0], t[1]);
+                    b[h / 8 + 1] = max3(b[h / 8 + 1], t[2], t[3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) b[h / 4 + i] = fmaxf(b[h / 4 + i], t[i]);
+                }
+            };
+            // ---- the buckets of the first units, for a threshold to start with
+#pragma unroll 1
+            for (int s = 0; s < lead; ++s) {
+                const uint32_t at = n + s;
+                const int buf = at & 1;
+                const int col0 = (s0 + s) * W + sub * kCols;
+                wait_or_abort(bar(B_AF + buf), (at >> 1) & 1, abort_flag, p.status);
+                if (warp_live) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int h = 0; h < kCols; h += 16) {
+                        float v[16], t[4];
+                        tmem_get16(t_col + buf * W + h, v);
+                        group_max(std::true_type{}, v, col0 + h, t);
+                        bucket(h, t);
+                    }
+                }
+                if (again) {
+                    tc_fence_before();
+                    arrive_lane0(bar(B_AE + buf), lane);
+                }
+            }
+            n += again;
+            if (warp_live) {
+                // (published by all four threads of a token before anyone reads: nothing of an earlier block is seen)
+                publish();
+                quarter_sync(q);
+                const float t0 = compute_thr();
+                sts(s_thr, t0);                              // (by all four, or a fast one could still read an earlier block's)
+                thr = fmaxf(thr, t0);
+            }
+            // One unit.  (One that reaches beyond M is an instantiation of its own, so that the others carry no masking.)
+            auto unit = [&](auto masked, int s) {
+                constexpr bool kMasked = decltype(masked)::value;
+                const int buf = n & 1;
+                const int col0 = (s0 + s) * W + sub * kCols;
+                const uint32_t t_acc = t_col + buf * W;
+                wait_or_abort(bar(B_AF + buf), (n >> 1) & 1, abort_flag, p.status);
+                tc_fence_after();
+#pragma unroll
+                for (int h = 0; h < kCols; h += 16) {
+                    const int col = col0 + h;
+                    float v[16], t[4];
+                    tmem_get16(t_acc + h, v);
+                    if (h + 16 == kCols) {
+                        tc_fence_before();
+                        arrive_lane0(bar(B_AE + buf), lane);         // everything is in registers: hand the accumulator back
+                    }
+                    group_max(masked, v, col, t);
+                    const float m = fmaxf(max3(t[0], t[1], t[2]), t[3]);
+                    if (LSE) {
+                        const float c2 = m * kLog2e;
+                        if (c2 > m2) { zsum *= ex2f(m2 - c2); m2 = c2; }
+                        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll
+                        for (int i = 0; i < 16; i += 8) {
+                            if (kMasked && col + i >= M) break;
+#pragma unroll
+                            for (int j = 0; j < 8; j += 4) {
+                                a0 += ex2f(fmaf(v[i + j], kLog2e, -m2));
+                                a1 += ex2f(fmaf(v[i + j + 1], kLog2e, -m2));
+                                a2 += ex2f(fmaf(v[i + j + 2], kLog2e, -m2));
+                                a3 += ex2f(fmaf(v[i + j + 3], kLog2e, -m2));
+                            }
+                        }
+                        zsum += (a0 + a1) + (a2 + a3);
+                    }
+                    if (__any_sync(kFull, m > thr)) {
+                        // (a bucket matters only once it beats the threshold, so it need not be kept up elsewhere)
+                        bucket(h, t);
+                        append4(ptr, thr, t, v, col, one);
+                    }
+                }
+                if (__any_sync(kFull, ptr > warn)) compact();
+                ++n;
+            };
+            if (!warp_live) {
+                for (int s = 0; s < steps; ++s, ++n) {
+                    wait_or_abort(bar(B_AF + (n & 1)), (n >> 1) & 1, abort_flag, p.status);
+                    arrive_lane0(bar(B_AE + (n & 1)), lane);
+                }
+            } else {
+                const int whole = min(steps, M / W - s0);            // units that do not reach beyond M
+                for (int s = 0; s < whole;) {
+                    const int stop = min(whole, next);               // a run of units, up to the next refresh of the threshold
+#pragma unroll 1
+                    for (; s < stop; ++s) {
+                        unit(std::false_type{}, s);
+                        thr = fmaxf(thr, lds(s_thr));
+                    }
+                    if (s == next) {
+                        publish();
+                        if (sub == (turn & 3)) sts(s_thr, compute_thr());
+                        ++turn;
+                        next += (next + 1) / 2;
+                    }
+                }
+                if (whole < steps) unit(std::true_type{}, steps - 1);
+            }
+            // ---- end of the segment: what still beats the threshold goes to scratch
+            if (warp_live) {
+                publish();
+                if (sub == 0) asm volatile("st.shared.u32 [%0], 0;" ::"r"(s_cnt) : "memory");
+                if (LSE && sub > 0)
+                    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(s_mz + (sub - 1) * (kRows * 8)), "f"(m2), "f"(zsum) : "memory");
+                quarter_sync(q);
+                thr = fmaxf(thr, compute_thr());
+                const int seg = (int)blockIdx.x - owner_of((long long)blk * nsteps, p.total, g);
+                const size_t slot = (size_t)blk * p.maxseg + seg;
+                uint2* dst = p.ent + (slot * kRows + row) * p.cap;
+                if (row_live) emit(dst, just_below(thr), 0);
+                quarter_sync(q);
+                int total = __float_as_int(lds(s_cnt));
+                if (__any_sync(kFull, total > p.cap)) {              // (the same in all four warps)
+                    // more than the scratch holds: the threads of such a token pass on their own k best each
+                    quarter_sync(q);
+                    if (sub == 0 && total > p.cap) sts(s_cnt, 0.f);
+                    quarter_sync(q);
+                    if (row_live && total > p.cap) {
+                        int equal;
+                        const float low = own_kth(equal);
+                        emit(dst, low, equal);
+                    }
+                    quarter_sync(q);
+                    total = __float_as_int(lds(s_cnt));
+                }
+                if (sub == 0 && row_live) {
+                    p.cnt[slot * kRows + row] = total;
+                    if (LSE) {
+                        float m = m2, z = zsum;
+#pragma unroll
+                        for (int o = 0; o < 3; ++o) {
+                            float om, oz;
+                            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(om), "=f"(oz) : "r"(s_mz + o * (kRows * 8)) : "memory");
+                            if (om > -INFINITY) {
+                                const float nm = fmaxf(m, om);
+                                z = z * ex2f(m - nm) + oz * ex2f(om - nm);
+                                m = nm;
+                            }
+                        }
+                        p.mz[slot * kRows + row] = make_float2(m, z);
+                    }
+                }
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    pdl_launch_dependents();
+    if (*abort_flag && threadIdx.x == 0)
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);         // copies still in flight land before the memory is released
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(256) : "memory");
+    }
+}
+
+// ================================================================================================= finish
+struct FinishParams {
+    int T, M, k, gate_mode;
+    int nsteps, g, share, maxseg, cap;
+    long long total;
+    const uint2* ent;
+    const int* cnt;
+    const float2* mz;
+    int32_t* out_idx;
+    float* out_gate;
+    int32_t* out_counts;
+    float* out_topval;
+    float* out_lse;
+};
+
+__device__ __forceinline__ void join_mz(float& m, float& z, float om, float oz)
+{
+    if (om > -INFINITY) {
+        const float nm = fmaxf(m, om);
+        z = z * ex2f(m - nm) + oz * ex2f(om - nm);
+        m = nm;
+    }
+}
+// segments of token block blk
+__device__ __forceinline__ int segments_of(const FinishParams& p, int blk)
+{
+    if (p.share > 0) return p.share;
+    const long long u0 = (long long)blk * p.nsteps;
+    return owner_of(u0 + p.nsteps - 1, p.total, p.g) - owner_of(u0, p.total, p.g) + 1;
+}
+__device__ __forceinline__ Cand load_cand(const uint2* at)
+{
+    const uint2 e = *at;
+    return Cand{__uint_as_float(e.x), (int)e.y};
+}
+// entry `rank` of a token's result; gate = 2^(v log2e - ref2) inv
+__device__ __forceinline__ void put_entry(const FinishParams& p, int tok, int rank, Cand c, float ref2, float inv)
+{
+    const int64_t o = (int64_t)tok * p.k + rank;
+    p.out_idx[o] = c.id;
+    p.out_gate[o] = ex2f(c.v * kLog2e - ref2) * inv;
+    if (p.out_topval) p.out_topval[o] = c.v;
+    if ((unsigned)c.id < (unsigned)p.M) atomicAdd(p.out_counts + c.id, 1);        // (non-finite inputs can leave a place unfilled)
+}
+
+// One or two segments per token (three where a part begins and ends inside a block): eight threads per token, which hold
+// its candidates (k and a few more per segment) in registers and rank them by counting: every logit against every other,
+// handed round by shuffles.  Bound by its instructions, so: logits alone are compared, and only if the ranks' sum shows
+// that two were equal are the ids; and a warp does as many rounds as its longest token needs.
+// (One thread per token that inserts into a sorted list took 27 us for 65536 tokens: one or two warps per scheduler, each
+// a chain of dependent instructions.)
+constexpr int kFewSegs = 3;
+constexpr int kFewRounds = 8;
+template <int R, class Fetch>
+__device__ __forceinline__ void rank_few(const FinishParams& p, int tok, bool live, int n, int j, float m2, float z, Fetch fetch)
+{
+    const int k = p.k;
+    Cand c[R];
+    int rank[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        c[r] = j + 8 * r < n ? fetch(j + 8 * r) : no_cand();
+        rank[r] = 0;
+    }
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float o = __shfl_sync(kFull, c[q].v, e, 8);
+#pragma unroll
+            for (int r = 0; r < R; ++r) rank[r] += o > c[r].v ? 1 : 0;
+        }
+    int sum = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) sum += j + 8 * r < n ? rank[r] : 0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o, 8);
+    if (__any_sync(kFull, sum != n * (n - 1) / 2)) {                  // some token has equal logits
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll 1
+            for (int e = 0; e < 8; ++e) {
+                const float o = __shfl_sync(kFull, c[q].v, e, 8);
+                const int id = __shfl_sync(kFull, c[q].id, e, 8);
+#pragma unroll
+                for (int r = 0; r < R; ++r) rank[r] += (o == c[r].v && id < c[r].id) ? 1 : 0;
+            }
+    }
+    float inv, ref2;
+    if (p.gate_mode == MORE_GATE_TOPK_SOFTMAX) {
+        float v0 = c[0].v;
+#pragma unroll
+        for (int r = 1; r < R; ++r) v0 = fmaxf(v0, c[r].v);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v0 = fmaxf(v0, __shfl_xor_sync(kFull, v0, o, 8));
+        float s = 0.f;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (j + 8 * r < n && rank[r] < k) s += ex2f((c[r].v - v0) * kLog2e);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o, 8);
+        inv = 1.f / s;
+        ref2 = v0 * kLog2e;
+    } else {
+        inv = 1.f / z;
+        ref2 = m2;
+    }
+    if (live) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (j + 8 * r < n && rank[r] < k) put_entry(p, tok, rank[r], c[r], ref2, inv);
+        for (int q = n + j; q < k; q += 8) put_entry(p, tok, q, no_cand(), ref2, inv);
+    }
+}
+
+__global__ void __launch_bounds__(256) finish_few_kernel(const FinishParams p)
+{
+    __shared__ int s_nseg;
+    const int lane = threadIdx.x & 31, j = lane & 7;
+    const int want = (blockIdx.x * 256 + threadIdx.x) >> 3;
+    const bool live = want < p.T;
+    const int tok = live ? want : p.T - 1;                    // (whole warps stay together; what is past the end writes nothing)
+    const int blk = tok / kRows, row = tok % kRows;           // (a CTA's 32 tokens lie in one block)
+    if (threadIdx.x == 0) s_nseg = segments_of(p, (blockIdx.x * 32) / kRows);
+    __syncthreads();
+    const int nseg = s_nseg;
+    pdl_wait();
+    int ends[kFewSegs];                                       // candidates in segments 0 .. s
+    float m2 = -INFINITY, z = 0.f;
+    {
+        int sum = 0;
+#pragma unroll
+        for (int s = 0; s < kFewSegs; ++s) {
+            if (s < nseg) {
+                const size_t slot = ((size_t)blk * p.maxseg + s) * kRows + row;
+                sum += p.cnt[slot];
+                if (p.mz) {
+                    const float2 o = p.mz[slot];
+                    join_mz(m2, z, o.x, o.y);
+                }
+            }
+            ends[s] = sum;
+        }
+    }
+    const int n = ends[kFewSegs - 1];
+    auto fetch = [&](int f) {                                 // candidate f of the token
+        int s = 0, before = 0;
+#pragma unroll
+        for (int q = 0; q + 1 < kFewSegs; ++q)
+            if (f >= ends[q]) { s = q + 1; before = ends[q]; }
+        return load_cand(p.ent + (((size_t)blk * p.maxseg + s) * kRows + row) * p.cap + (f - before));
+    };
+    const int rounds = (__reduce_max_sync(kFull, n) + 7) >> 3;
+    if (rounds <= 1) rank_few<1>(p, tok, live, n, j, m2, z, fetch);
+    else if (rounds == 2) rank_few<2>(p, tok, live, n, j, m2, z, fetch);
+    else if (rounds == 3) rank_few<3>(p, tok, live, n, j, m2, z, fetch);
+    else if (rounds == 4) rank_few<4>(p, tok, live, n, j, m2, z, fetch);
+    else if (rounds <= kFewRounds) rank_few<kFewRounds>(p, tok, live, n, j, m2, z, fetch);
+    else {
+        // more candidates than registers (many equal logits): k rounds of a maximum, twice, as the gates need their sum first
+        const bool topk = p.gate_mode == MORE_GATE_TOPK_SOFTMAX;
+        float sum = 0.f, v0 = 0.f;
+        for (int pass = topk ? 0 : 1; pass < 2; ++pass) {
+            Cand last{INFINITY, -1};
+            for (int r = 0; r < p.k; ++r) {
+                Cand top = no_cand();
+                for (int f = j; f < n; f += 8) {
+                    const Cand x = fetch(f);
+                    if (ahead(last, x) && ahead(x, top)) top = x;
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    const Cand x{__shfl_xor_sync(kFull, top.v, o, 8), __shfl_xor_sync(kFull, top.id, o, 8)};
+                    if (ahead(x, top)) top = x;
+                }
+                last = top;
+                if (pass == 0) {
+                    if (r == 0) v0 = top.v;
+                    sum += ex2f((top.v - v0) * kLog2e);
+                } else if (j == 0 && live) {
+                    put_entry(p, tok, r, top, topk ? v0 * kLog2e : m2, topk ? 1.f / sum : 1.f / z);
+                }
+            }
+        }
+    }
+    if (j == 0 && live && p.out_lse) p.out_lse[tok] = (m2 + log2f(z)) * kLn2;
+}
+
+// The result of one token from its k best, one per lane; called by a whole warp.
+__device__ __forceinline__ void put_token(const FinishParams& p, int tok, Cand c, float m2, float z, int lane)
+{
+    float inv, ref2;
+    if (p.gate_mode == MORE_GATE_TOPK_SOFTMAX) {
+        const float v0 = __shfl_sync(kFull, c.v, 0);
+        float s = lane < p.k ? ex2f((c.v - v0) * kLog2e) : 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        inv = 1.f / s;
+        ref2 = v0 * kLog2e;
+    } else {
+        inv = 1.f / z;
+        ref2 = m2;
+    }
+    if (lane < p.k) put_entry(p, tok, lane, c, ref2, inv);
+    if (lane == 0 && p.out_lse) p.out_lse[tok] = (m2 + log2f(z)) * kLn2;
+}
+
+// Up to kWarpSegs segments per token, or long lists: a warp per token.
+constexpr int kWarpSegs = 64;
+__global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
+{
+    __shared__ Cand buf[8][64];
+    __shared__ int counts[8][kWarpSegs];
+    __shared__ int s_nseg;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tok = blockIdx.x * 8 + warp;
+    if (threadIdx.x == 0) s_nseg = segments_of(p, (blockIdx.x * 8) / kRows);
+    __syncthreads();
+    const int nseg = s_nseg;
+    pdl_wait();
+    if (tok >= p.T) return;
+    const int blk = tok / kRows, row = tok % kRows;
+    const size_t slot0 = (size_t)blk * p.maxseg * kRows + row;
+    float m2 = -INFINITY, z = 0.f;
+    int most = 0;
+    for (int s = lane; s < nseg; s += 32) {
+        const int c = p.cnt[slot0 + (size_t)s * kRows];
+        counts[warp][s] = c;
+        most = max(most, c);
+        if (p.mz) {
+            const float2 o = p.mz[slot0 + (size_t)s * kRows];
+            join_mz(m2, z, o.x, o.y);
+        }
+    }
+    if (p.mz) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float om = __shfl_xor_sync(kFull, m2, o), oz = __shfl_xor_sync(kFull, z, o);
+            join_mz(m2, z, om, oz);
+        }
+    }
+    most = max(__reduce_max_sync(kFull, most), 1);
+    __syncwarp();
+    const uint32_t inv = most > 1 ? (uint32_t)(((1ull << 32) - 1) / (uint32_t)most) + 1u : 0u;      // f / most by multiplication
+    auto get = [&](int f) {
+        const int s = inv ? (int)__umulhi((uint32_t)f, inv) : f, i = f - s * most;
+        return i < counts[warp][s] ? load_cand(p.ent + (slot0 + (size_t)s * kRows) * p.cap + i) : no_cand();
+    };
+    const Cand c = warp_topk<4>(nseg * most, p.k, get, buf[warp], lane);
+    put_token(p, tok, c, m2, z, lane);
+}
+
+// More segments than that (a few tokens, whose experts are spread over the whole GPU): a CTA per token.  As above, with
+// 512 threads' maxima joined to 64 of which the k-th largest bounds the k-th best.
+constexpr int kManyThreads = 512;
+constexpr int kManySegs = 640;
+__global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishParams p)
+{
+    constexpr int kWarps = kManyThreads / 32, kKeep = 512;
+    __shared__ int counts[kManySegs];
+    __shared__ float maxima[64];
+    __shared__ float2 smz[kWarps];
+    __shared__ Cand keep[kKeep];
+    __shared__ Cand buf[64];
+    __shared__ int s_count, s_nseg;
+    __shared__ float s_thr;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tok = blockIdx.x;
+    const int blk = tok / kRows, row = tok % kRows;
+    if (threadIdx.x == 0) { s_nseg = segments_of(p, blk); s_count = 0; }
+    __syncthreads();
+    const int nseg = s_nseg;
+    const size_t slot0 = (size_t)blk * p.maxseg * kRows + row;
+    pdl_wait();
+    float m2 = -INFINITY, z = 0.f;
+    for (int s = threadIdx.x; s < nseg; s += kManyThreads) {
+        counts[s] = p.cnt[slot0 + (size_t)s * kRows];
+        if (p.mz) {
+            const float2 o = p.mz[slot0 + (size_t)s * kRows];
+            join_mz(m2, z, o.x, o.y);
+        }
+    }
+    if (p.mz) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float om = __shfl_xor_sync(kFull, m2, o), oz = __shfl_xor_sync(kFull, z, o);
+            join_mz(m2, z, om, oz);
+        }
+        if (lane == 0) smz[warp] = make_float2(m2, z);
+    }
+    __syncthreads();
+    // half a warp per segment, the next segment's entries requested before the current ones are used
+    const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
+    auto visit = [&](auto f) {
+        for (int s = half; s < nseg; s += kManyThreads / 16) {
+            const int c = counts[s];
+            const uint2* e = p.ent + (slot0 + (size_t)s * kRows) * p.cap;
+            for (int i = hl; i < c; i += 16) f(load_cand(e + i));
+        }
+    };
+    float m = -INFINITY;
+    visit([&](Cand x) { m = fmaxf(m, x.v); });
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));          // eight threads' maximum: 64 of them
+    if ((lane & 7) == 0) maxima[warp * 4 + (lane >> 3)] = m;
+    __syncthreads();
+    if (warp == 0) {
+        // k-th largest of the 64: two sorted halves; entry against mirrored entry gives the 32 largest
+        const float a = warp_sort_down(maxima[lane], lane), b = warp_sort_down(maxima[lane + 32], lane);
+        const float top = warp_sort_down(fmaxf(a, __shfl_sync(kFull, b, 31 - lane)), lane);
+        if (lane == p.k - 1) s_thr = top;
+    }
+    __syncthreads();
+    const float thr = s_thr;
+    visit([&](Cand x) {
+        if (x.v >= thr) {
+            const int at = atomicAdd(&s_count, 1);
+            if (at < kKeep) keep[at] = x;
+        }
+    });
+    __syncthreads();
+    if (warp == 0) {
+        const int n = s_count;
+        Cand c;
+        if (n <= kKeep) {
+            c = warp_topk<4>(n, p.k, [&](int f) { return keep[f]; }, buf, lane);
+        } else {
+            // more near the top than the buffer holds (many equal logits): over all of them
+            const int most = p.cap;
+            c = warp_topk<1>(nseg * most, p.k, [&](int f) {
+                const int s = f / most, i = f - s * most;
+                return i < counts[s] ? load_cand(p.ent + (slot0 + (size_t)s * kRows) * p.cap + i) : no_cand();
+            }, buf, lane);
+        }
+        m2 = smz[0].x;
+        z = smz[0].y;
+        if (p.mz)
+            for (int w = 1; w < kWarps; ++w) join_mz(m2, z, smz[w].x, smz[w].y);
+        put_token(p, tok, c, m2, z, lane);
+    }
+}
+
+// ================================================================================================ host side
+constexpr int kSweepSmem = (228 * 1024 - 2 * 1024) / 2;     // two CTAs per SM
+
+// Raise a kernel's dynamic shared-memory limit once per device; guarded by the API mutex.
+template <class K>
+bool allow_smem(K kern, int bytes, unsigned long long* done, bool wide_cluster = false)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (*done >> (dev & 63) & 1ull) return true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    if (wide_cluster && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+    *done |= 1ull << (dev & 63);
+    return true;
+}
+
+using SweepFn = void (*)(const CUtensorMap, const CUtensorMap, const SweepParams);
+
+template <int KCAP, bool LSE>
+SweepFn sweep_ready()
+{
+    static unsigned long long done = 0;
+    SweepFn f = sweep_kernel<KCAP, LSE>;
+    return allow_smem(f, kSweepSmem, &done) ? f : nullptr;
+}
+
+SweepFn sweep_fn(int k, bool lse)
+{
+    if (k <= 8) return lse ? sweep_ready<8, true>() : sweep_ready<8, false>();
+    return lse ? sweep_ready<32, true>() : sweep_ready<32, false>();
+}
+
+template <class... Args>
+cudaError_t launch(void (*kern)(Args...), int grid, int block, int smem, cudaStream_t st, bool dependent, int cluster, Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (dependent) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = (unsigned)cluster;
+        at[n].val.clusterDim.y = at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = (unsigned)n;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+constexpr int kChunkTokens = 131072;               // tokens per pass: bounds the scratch, whatever T is
+
+struct Layout {
+    size_t z, list, ent, cnt, mz, total;
+};
+
+Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
+{
+    Layout L{};
+    const size_t tokens = (size_t)(a.T < kChunkTokens ? a.T : kChunkTokens);
+    const size_t blocks = (tokens + kRows - 1) / kRows;
+    size_t off = 0;
+    L.z = off; off += align_up(blocks * kRows * (a.r <= 32 ? 128 : 256), 1024);
+    L.list = off; off += (size_t)p.parts * kListCap * kEntry;
+    L.ent = off; off += align_up(blocks * p.maxseg * (size_t)(4 * a.k) * kRows * 8, 1024);
+    L.cnt = off; off += align_up(blocks * p.maxseg * kRows * 4, 1024);
+    L.mz = off;
+    if (lse) off += align_up(blocks * p.maxseg * kRows * 8, 1024);
+    L.total = off;
+    return L;
+}
+
+}  // namespace
+
+// Launch plan.  The unit of work is 128 tokens x 128 experts.  Two CTAs per SM get contiguous parts of the line of units,
+// either equal ones wherever these begin (stretches of several token blocks are then cut into segments), or an equal share
+// of one block each.  The second leaves some SMs idle but every CTA with one segment; what a segment costs on its own (its
+// first MMAs, the threshold to start with, the pass through the lists at its end) is worth about four units.  A forced
+// split of s CTAs per token block is the second with that s.
+void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
+{
+    const long long blocks = ((T < kChunkTokens ? T : kChunkTokens) + kRows - 1) / kRows;
+    const long long nsteps = (M + W - 1) / W, total = blocks * nsteps, slots = 2 * sm_count;
+    const double kSegment = 4.0;
+    long long g = total < slots ? total : slots, share = 0;
+    if (msplit > 0) {
+        const int most = M / 256 > 1 ? M / 256 : 1;
+        share = msplit < most ? msplit : most;
+    } else if (blocks <= slots) {
+        const long long s = slots / blocks < nsteps ? slots / blocks : nsteps;
+        const double whole = (double)((nsteps + s - 1) / s) + kSegment;
+        const double cut = (double)total / g + kSegment * (double)((total / g) / nsteps + 2);
+        if (blocks == 1 || whole <= cut) share = s;
+    }
+    if (share > 0) {
+        g = blocks * share;
+        p->maxseg = (int)share;
+    } else {
+        p->maxseg = (int)(g / blocks) + 2;
+    }
+    p->parts = (int)g;
+    // reported: CTAs; where a token block is split, the two CTAs of an SM count as one
+    p->ctas = (int)(blocks < sm_count && g > sm_count && msplit <= 0 ? sm_count : g);
+    p->msplit = msplit > 0 ? (int)share : (int)(p->ctas / blocks > 1 ? p->ctas / blocks : 1);
+    p->share = (int)share;
+    p->chain = true;
+    p->block_tokens = kRows;
+    p->tg = 1;
+    p->es = 4;
+}
+
+size_t chain_scratch_bytes(const RouteArgs& a, const Plan& p)
+{
+    return layout_of(a, p, a.gate_mode == MORE_GATE_FULL_SOFTMAX || a.out_lse != nullptr).total;
+}
+
+int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scratch)
+{
+    const bool lse = a.gate_mode == MORE_GATE_FULL_SOFTMAX || a.out_lse != nullptr;
+    const Layout L = layout_of(a, plan, lse);
+    char* base = static_cast<char*>(scratch);
+    const int n16 = (a.r + 15) / 16 * 16, zc = a.r <= 32 ? 64 : 128;
+
+    SweepParams sp{};
+    const int nsteps = (a.M + W - 1) / W;
+    sp.M = a.M; sp.k = a.k; sp.nsteps = nsteps; sp.ks = n16 / 16; sp.rk = n16; sp.wide = a.r > 32;
+    sp.maxseg = plan.maxseg; sp.cap = 4 * a.k;
+    sp.st_bytes = W * n16 * 2;
+    sp.z_bytes = kRows * zc * 2;
+    const int nb = a.k <= 8 ? 4 : 8;
+    const int pub = 4 * kRows * nb * 4 + kRows * 8 + 3 * kRows * 8, ctl = 512;
+    const int room = kSweepSmem - 1024 - pub - ctl;
+    sp.zbufs = zc == 64 ? 2 : 1;
+    sp.nst = (room - sp.zbufs * sp.z_bytes) / sp.st_bytes;
+    if (sp.nst > kMaxStages) sp.nst = kMaxStages;
+    if (sp.nst < 2) return MORE_ERR_SHAPE;
+    sp.off_r2 = sp.zbufs * sp.z_bytes;
+    sp.off_pub = sp.off_r2 + sp.nst * sp.st_bytes;
+    sp.off_ctl = sp.off_pub + pub;
+    const int smem = sp.off_ctl + ctl + 1024;
+    sp.list = reinterpret_cast<uint8_t*>(base + L.list);
+    sp.ent = reinterpret_cast<uint2*>(base + L.ent);
+    sp.cnt = reinterpret_cast<int*>(base + L.cnt);
+    sp.mz = lse ? reinterpret_cast<float2*>(base + L.mz) : nullptr;
+    sp.status = ctx.status;
+
+    SweepFn sweep = sweep_fn(a.k, lse);
+    static unsigned long long project_done = 0;
+    const int psmem_max = kPStages * kPStageBytes + kPCtl + kPExchange + 1024;
+    if (!sweep || !allow_smem(project_kernel, psmem_max, &project_done)) return MORE_ERR_CUDA;
+
+    const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
+    CUtensorMap mr1, mr2;
+    int rc = get_tensor_map(a.R1, a.h, a.r, 64, 64, &mr1);
+    if (rc == MORE_OK) rc = get_tensor_map(a.R2, a.r, a.M, n16, 64, &mr2);
+    if (rc != MORE_OK) return rc;
+    for (int t0 = 0; t0 < a.T; t0 += kChunkTokens) {
+        const int T = a.T - t0 < kChunkTokens ? a.T - t0 : kChunkTokens;
+        const int blocks = (T + kRows - 1) / kRows;
+        CUtensorMap mx, mz;
+        rc = get_tensor_map(a.X + (size_t)t0 * a.h, T, a.h, kRows, 64, &mx);
+        if (rc == MORE_OK) rc = get_tensor_map(base + L.z, blocks * kRows, zc, kRows, 64, &mz);
+        if (rc != MORE_OK) return rc;
+
+        ProjectParams pp{};
+        pp.T = T; pp.h = a.h; pp.n = n16; pp.zc = zc;
+        pp.z = reinterpret_cast<uint32_t*>(base + L.z);
+        pp.counts = t0 == 0 ? a.out_counts : nullptr;
+        pp.M = a.M;
+        pp.status = ctx.status;
+        pp.cs = 1;
+        const int nkt = (a.h + 63) / 64;
+        while (pp.cs < 8 && 2 * pp.cs * blocks <= sms && nkt >= 4 * pp.cs) pp.cs *= 2;
+        const int psmem = psmem_max - (pp.cs == 1 ? kPExchange : 0);
+        if (launch(project_kernel, blocks * pp.cs, kPThreads, psmem, a.stream, true, pp.cs, mx, mr1, pp) != cudaSuccess)
+            return MORE_ERR_CUDA;
+
+        sp.T = T;
+        sp.total = (long long)blocks * nsteps;
+        int g = plan.parts;
+        if (a.T > kChunkTokens) {                            // (the last chunk of a long call may be shorter)
+            if (plan.share > 0) {
+                g = blocks * plan.share;
+            } else {
+                const long long most = (long long)(plan.maxseg - 1) * blocks - 1;      // floor(g / blocks) + 2 <= maxseg
+                if (g > sp.total) g = (int)sp.total;
+                if (g > most) g = (int)(most > 1 ? most : 1);
+            }
+        }
+        if (launch(sweep, g, kSThreads, smem, a.stream, true, 1, mz, mr2, sp) != cudaSuccess) return MORE_ERR_CUDA;
+
+        FinishParams fp{};
+        fp.T = T; fp.M = a.M; fp.k = a.k; fp.gate_mode = a.gate_mode;
+        fp.nsteps = nsteps; fp.g = g; fp.share = plan.share; fp.maxseg = plan.maxseg; fp.cap = sp.cap; fp.total = sp.total;
+        fp.ent = sp.ent; fp.cnt = sp.cnt; fp.mz = sp.mz;
+        const size_t ro = (size_t)t0 * a.k;
+        fp.out_idx = a.out_idx + ro; fp.out_gate = a.out_gate + ro; fp.out_counts = a.out_counts;
+        fp.out_topval = a.out_topval ? a.out_topval + ro : nullptr;
+        fp.out_lse = a.out_lse ? a.out_lse + t0 : nullptr;
+        cudaError_t e;
+        // (a list of k <= 16 holds ~1.4 k: with more than two of them, or longer ones, the threshold of the warp's selection
+        // saves more than its 32 lanes per token cost)
+        if (a.k <= 16 && plan.maxseg <= (plan.share > 0 ? 2 : kFewSegs))
+            e = launch(finish_few_kernel, (T + 31) / 32, 256, 0, a.stream, true, 1, fp);
+        else if (plan.maxseg <= kWarpSegs)
+            e = launch(finish_warp_kernel, (T + 7) / 8, 256, 0, a.stream, true, 1, fp);
+        else
+            e = launch(finish_many_kernel, T, kManyThreads, 0, a.stream, true, 1, fp);
+        if (e != cudaSuccess) return MORE_ERR_CUDA;
+        count_launch(3);
+    }
+    return MORE_OK;
+}
+
+}  // namespace more

@@ -54,6 +54,10 @@ struct Plan {
     int es = 1;   // ... and expert ranges swept side by side inside a CTA (tg * es <= 4)
     bool filter = false;   // low-rank router: approximate sweep + exact rescoring of the survivors
     bool paired = false;   // low-rank router: the kernel with 256-token CTAs, two per SM, instead of one CTA per SM
+    bool chain = false;    // low-rank router: projection, sweep and finish as three kernels
+    int parts = 1;         // ... CTAs of its sweep,
+    int share = 0;         // ... how many of them share one token block each, or 0 where their parts begin anywhere,
+    int maxseg = 1;        // ... and the most that can share one
 };
 
 bool tcgen05_shape_ok(int T, int h, int r, int M, int k);
@@ -63,7 +67,11 @@ int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, b
 bool lowrank_smem_plan(int rpad, int tg, int es, bool filter, int* nst1, int* st1_bytes, int* nst2, int* st2_bytes,
                        int* r2_off);
 
+// Launch plan of the three-kernel chain; fills everything but the path and rpad.
+void plan_chain(int T, int M, int msplit, int sm_count, Plan* p);
+
 // Scratch bytes each path needs for a problem.
+size_t chain_scratch_bytes(const RouteArgs& a, const Plan& p);
 size_t generic_scratch_bytes(const RouteArgs& a);
 size_t lowrank_scratch_bytes(const RouteArgs& a, const Plan& p);
 size_t full_scratch_bytes(const RouteArgs& a, const Plan& p);
@@ -71,7 +79,8 @@ size_t paired_scratch_bytes(const RouteArgs& a, const Plan& p);
 
 // Launchers: enqueue on a.stream, return MORE_OK / MORE_ERR_*.  `scratch` is at least *_scratch_bytes().
 int launch_generic(const RouteArgs& a, DeviceCtx& ctx, void* scratch);
-// Both tensor-core launchers clear out_counts on the stream themselves, after every host-side step that can fail.
+int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
+// All tensor-core launchers clear out_counts on the stream themselves, after every host-side step that can fail.
 int launch_lowrank(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
 int launch_full(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
 int launch_paired(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);

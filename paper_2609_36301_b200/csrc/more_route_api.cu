@@ -159,7 +159,8 @@ int route_device_locked(const RouteArgs& a, int path, int msplit)
     const size_t need = plan.path != MORE_PATH_TCGEN05
                             ? generic_scratch_bytes(a)
                             : (a.full ? full_scratch_bytes(a, plan)
-                                      : (plan.paired ? paired_scratch_bytes(a, plan) : lowrank_scratch_bytes(a, plan)));
+                                      : (plan.chain ? chain_scratch_bytes(a, plan)
+                                                    : (plan.paired ? paired_scratch_bytes(a, plan) : lowrank_scratch_bytes(a, plan))));
     rc = ensure_scratch(ctx, need, a.stream);
     if (rc != MORE_OK) return rc;
     if (a.T == 0 || plan.path != MORE_PATH_TCGEN05) {
@@ -169,6 +170,7 @@ int route_device_locked(const RouteArgs& a, int path, int msplit)
         return launch_generic(a, *ctx, ctx->scratch);
     }
     if (a.full) return launch_full(a, *ctx, plan, ctx->scratch);
+    if (plan.chain) return launch_chain(a, *ctx, plan, ctx->scratch);
     return plan.paired ? launch_paired(a, *ctx, plan, ctx->scratch) : launch_lowrank(a, *ctx, plan, ctx->scratch);
 }
 
@@ -183,6 +185,21 @@ int route_device(const RouteArgs& a, int path, int msplit)
 void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 namespace {
+
+// Whether the low-rank router runs as the chain projection -> sweep -> finish rather than as one of the two kernels that
+// do it all.  Measured on B200 over T = 1 ... 64 k, M = 256 ... 64 k, r = 16, 32, 64, k = 8 and 16, both gates (174
+// points).  The chain wins where one kernel repeats the projection or leaves SMs idle (few tokens: 1.1 to 1.9 times
+// faster) and on long sweeps (M = 64 k: 1.1 to 1.4); what it pays for every segment of a sweep, and its third launch,
+// lose on many tokens with few experts (T = 64 k, M = 1 k: half as fast).
+bool chain_wins(int T, int M, int k, int sm_count)
+{
+    const int per_sm = (T + sm_count - 1) / sm_count;
+    if (M < 512) return false;
+    if (per_sm <= 28) return true;
+    if (k > 8) return M >= 32768;
+    if (per_sm <= 60) return M >= 3072;
+    return M >= (per_sm > 250 ? 32768 : 16384);
+}
 
 // Launch plan of the paired low-rank kernel (256-token CTAs, two per SM).
 void plan_paired(int T, int h, int M, int msplit, int sm_count, Plan* p)
@@ -341,7 +358,12 @@ int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, b
     if (full) {
         plan_dense(T, h, M, msplit, sm_count, &p);
     } else {
-        // Two kernels serve the low-rank router.  Measured on B200 over T = 2 k ... 64 k tokens, M = 1 k ... 64 k
+        if (chain_wins(T, M, k, sm_count)) {
+            plan_chain(T, M, msplit, sm_count, &p);
+            *out = p;
+            return MORE_OK;
+        }
+        // Two kernels serve the rest.  Measured on B200 over T = 2 k ... 64 k tokens, M = 1 k ... 64 k
         // experts, r = 16, 32, 64 and both gates: the grouped kernel (one CTA per SM, up to four token groups / expert
         // ranges side by side) wins while an SM has fewer than ~120 tokens; between that and ~260 tokens per SM it
         // wins for up to ~8 k experts, and with the softmax sweep (whose epilogue is bound by its own instructions

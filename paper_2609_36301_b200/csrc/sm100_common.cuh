@@ -25,10 +25,6 @@ static_assert(kStagesP1 * kP1StageBytes <= kRingBytes, "phase-1 ring does not fi
 constexpr int kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers, flags*/;
 constexpr int kTmemCols = 256;                     // tensor-memory columns per CTA (two CTAs share the 512 of an SM)
 constexpr long long kWaitBudgetCycles = 4000000000LL;   // ~2 s
-#ifndef MORE_SUSPEND_NS
-#define MORE_SUSPEND_NS 20000
-#endif
-constexpr uint32_t kSuspendHintNs = MORE_SUSPEND_NS;             // a waiting thread may be parked this long per try
 
 // ------------------------------------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -50,10 +46,10 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"   // may suspend up to the hinted time
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"   // may suspend for a time of the hardware's choice
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
+        : "r"(bar), "r"(parity)
         : "memory");
     return ok;
 }
@@ -72,7 +68,8 @@ __device__ __forceinline__ uint32_t mbar_try_wait_now(uint32_t bar, uint32_t par
     return ok;
 }
 
-// Bounded wait.  Returns false if the CTA is aborting (this wait or another one ran out of budget).
+// Bounded wait.  Returns false if the CTA is aborting (this wait or another one ran out of budget).  The first test stands
+// apart from the loop: a completed phase then costs ~65 clocks instead of ~130.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           long long budget = kWaitBudgetCycles)
 {

@@ -1,0 +1,84 @@
+"""The chain projection -> sweep -> finish of the low-rank router, at the edges of its tiles: token blocks of 128, units of
+128 experts, K-steps of 16 ranks, the three finishing kernels (few, up to 64 and more segments per token), lists that
+overflow, equal logits, and a call that is cut into chunks of tokens."""
+import numpy as np
+import pytest
+
+from paper_2609_36301_b200 import binding as mr
+from paper_2609_36301_b200 import inputs
+
+from helpers import check_counts, check_rows, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _route_and_check(case, rows=None, launches=3):
+    import torch
+    X, R1, R2 = to_device(case)
+    before = mr.launches()
+    res = mr.route(X, R1, R2, case.k, case.gate_mode, want_topval=True, want_lse=case.gate_mode == 1)
+    assert mr.launches() - before == launches, "this shape is not served by the chain"
+    torch.cuda.synchronize()
+    assert mr.more_route_status() == 0
+    sel = slice(None) if rows is None else torch.from_numpy(rows).cuda()
+    st = check_rows(case, rows, res.idx[sel].cpu().numpy(), res.gate[sel].cpu().numpy(), res.topval[sel].cpu().numpy(),
+                    None if res.lse is None else res.lse[sel].cpu().numpy(), gate_mode=case.gate_mode, k=case.k)
+    counts = res.counts.cpu().numpy()
+    if rows is None:
+        check_counts(res.idx.cpu().numpy(), counts, case.M, st["ref"].counts, bool(st["differs_mask"].any()))
+    else:
+        check_counts(res.idx.cpu().numpy(), counts, case.M)
+    return st
+
+
+@pytest.mark.parametrize("gate_mode", [0, 1])
+@pytest.mark.parametrize("T,h,r,M,k", [
+    (1, 8, 8, 512, 1),            # one token, one k-tile, four whole units
+    (127, 72, 16, 520, 8),        # the last token row empty, a unit with eight live experts
+    (129, 128, 24, 640, 9),       # a second block with one token, lists longer than 8
+    (300, 200, 40, 1016, 16),     # three K-steps, the last unit short of eight experts
+    (1000, 512, 48, 4104, 17),    # k beyond 16: the smallest of all buckets is the threshold
+    (2000, 96, 56, 2000, 32),     # the longest lists
+    (4100, 64, 64, 768, 4),       # more token blocks than three per part: parts that begin inside a block
+    (8500, 64, 32, 3072, 8),      # one or two segments per token: the finishing kernel with eight threads per token
+    (40, 256, 64, 65536, 8),      # hundreds of segments per token: a CTA per token finishes
+])
+def test_edges(T, h, r, M, k, gate_mode):
+    _route_and_check(inputs.gaussian_case(T, h, r, M, k, gate_mode, seed=T + M))
+
+
+@pytest.mark.parametrize("k", [1, 8, 16, 32])
+@pytest.mark.parametrize("descending", [False, True])
+def test_logits_that_rise_or_fall_with_the_expert_id(k, descending):
+    """Every expert beats the threshold so far (the lists overflow again and again), or none does after the first."""
+    case = inputs.gaussian_case(200, 64, 8, 4096, k, 0, seed=13)
+    R1f = np.zeros((64, 8), dtype=np.float32)
+    R1f[0, 0] = 1.0
+    Xf = inputs.bf16_bits_to_f32(case.X)
+    Xf[:, 0] = np.abs(Xf[:, 0]) + 0.5
+    ramp = np.arange(4096, dtype=np.float32) / 512.0
+    R2f = np.zeros((8, 4096), dtype=np.float32)
+    R2f[0] = -ramp if descending else ramp
+    case.X, case.R1, case.R2 = inputs.to_bf16_bits(Xf), inputs.to_bf16_bits(R1f), inputs.to_bf16_bits(R2f)
+    _route_and_check(case)
+
+
+@pytest.mark.parametrize("T,M", [(64, 2048), (3000, 1024), (8500, 3072)])
+def test_all_logits_equal(T, M):
+    """Nothing beats anything: the first k experts are selected."""
+    import torch
+    case = inputs.gaussian_case(T, 64, 16, M, 8, 0, seed=3)
+    case.R2[:] = case.R2[:, :1]
+    X, R1, R2 = to_device(case)
+    res = mr.route(X, R1, R2, 8, 0)
+    torch.cuda.synchronize()
+    assert mr.more_route_status() == 0
+    assert bool((res.idx == torch.arange(8, device="cuda", dtype=torch.int32)).all())
+    assert int(res.counts[:8].sum()) == 8 * T and int(res.counts[8:].sum()) == 0
+
+
+def test_more_tokens_than_one_chunk():
+    T = 131072 + 130
+    case = inputs.gaussian_case(T, 64, 8, 32768, 4, 0, seed=9)
+    rows = np.concatenate([np.arange(64), np.arange(131072 - 64, T)])
+    _route_and_check(case, rows, launches=6)
