@@ -1,4 +1,5 @@
-"""Thin ctypes binding of ``libmore_route.so``: argument marshalling only.
+"""Thin binding of ``libmore_route.so``: argument marshalling only, through ctypes, and for the calls that enqueue work on
+device tensors through a small extension module (``csrc/more_binding.cpp``): a decode-sized call is ~20 us of GPU time.
 
 Every step of the router runs in the library's CUDA kernels; torch is used for device memory and streams.
 There is no CPU fallback: if the shared library is missing the import of a routing call raises.
@@ -78,6 +79,29 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_fast_module = None
+
+
+def _fast():
+    """Load (once) the extension module and point it at the loaded library's functions; raises if it has not been built."""
+    global _fast_module
+    if _fast_module is None:
+        L = lib()
+        if not os.path.exists(_build.BINDING_PATH):
+            raise FileNotFoundError(f"{_build.BINDING_PATH} is missing: build it with `python -m paper_2609_36301_b200.build`")
+        import importlib.machinery
+        import importlib.util
+
+        import torch  # noqa: F401  (its libraries first)
+        loader = importlib.machinery.ExtensionFileLoader("_more_binding", _build.BINDING_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_more_binding", loader))
+        loader.exec_module(module)
+        module.bind(*[ctypes.cast(f, ctypes.c_void_p).value for f in
+                      (L.more_route_ex, L.more_route_psum, L.more_dispatch, L.more_route_full, L.more_merge_shards)])
+        _fast_module = module
+    return _fast_module
+
+
 def strerror(code: int) -> str:
     return lib().more_strerror(code).decode()
 
@@ -131,10 +155,8 @@ def _stream(stream):
 def more_route(X, R1, R2, k, gate_mode, out_idx, out_gate, out_counts, stream=None):
     """``more_route`` of the C interface on torch CUDA tensors (bf16 ``X [T,h]``, ``R1 [h,r]``, ``R2 [r,M]``; int32
     ``out_idx [T,k]``, fp32 ``out_gate [T,k]``, int32 ``out_counts [M]``).  Asynchronous on ``stream``."""
-    T, h = X.shape
-    r, M = R2.shape
-    rc = lib().more_route(_ptr(X), _ptr(R1), _ptr(R2), T, h, r, M, k, gate_mode,
-                          _ptr(out_idx), _ptr(out_gate), _ptr(out_counts), _stream(stream))
+    rc = (_fast_module or _fast()).route_ex(X, R1, R2, k, gate_mode, out_idx, out_gate, out_counts, None, None, PATH_AUTO, 0,
+                                            stream)
     if rc != 0:
         raise MoreRouteError(rc, "more_route")
 
@@ -142,11 +164,8 @@ def more_route(X, R1, R2, k, gate_mode, out_idx, out_gate, out_counts, stream=No
 def more_route_ex(X, R1, R2, k, gate_mode, out_idx, out_gate, out_counts, out_topval=None, out_lse=None,
                   path=PATH_AUTO, msplit=0, stream=None):
     """``more_route_ex`` of the C interface (optional selected logits / log-sum-exp outputs, forced path and split)."""
-    T, h = X.shape
-    r, M = R2.shape
-    rc = lib().more_route_ex(_ptr(X), _ptr(R1), _ptr(R2), T, h, r, M, k, gate_mode,
-                             _ptr(out_idx), _ptr(out_gate), _ptr(out_counts), _ptr(out_topval), _ptr(out_lse),
-                             path, msplit, _stream(stream))
+    rc = (_fast_module or _fast()).route_ex(X, R1, R2, k, gate_mode, out_idx, out_gate, out_counts, out_topval, out_lse, path,
+                                            msplit, stream)
     if rc != 0:
         raise MoreRouteError(rc, "more_route_ex")
 
@@ -183,9 +202,7 @@ def more_route_noalloc_capacity() -> int:
 def more_route_psum(X, R1, R2, lse, out_psum, path=PATH_AUTO, stream=None):
     """``more_route_psum`` of the C interface: ``out_psum [M]`` (fp32, overwritten) = column sums of the softmax over
     all experts, given every token's ``lse [T]`` from :func:`more_route_ex` on the same inputs (Algorithm 2)."""
-    T, h = X.shape
-    r, M = R2.shape
-    rc = lib().more_route_psum(_ptr(X), _ptr(R1), _ptr(R2), T, h, r, M, _ptr(lse), _ptr(out_psum), path, _stream(stream))
+    rc = (_fast_module or _fast()).psum(X, R1, R2, lse, out_psum, path, stream)
     if rc != 0:
         raise MoreRouteError(rc, "more_route_psum")
 
@@ -194,9 +211,7 @@ def more_dispatch(idx, counts, out_offsets, out_sorted_pairs, stream=None):
     """``more_dispatch`` of the C interface: from ``idx [T,k]`` and ``counts [M]`` (int32, as written by
     :func:`more_route`) fill ``out_offsets [M+1]`` (exclusive prefix sum of the counts) and ``out_sorted_pairs [T*k]``
     (flat positions ``token*k + slot`` grouped by expert; order inside an expert's run unspecified)."""
-    T, k = idx.shape
-    M = counts.shape[0]
-    rc = lib().more_dispatch(_ptr(idx), _ptr(counts), T, k, M, _ptr(out_offsets), _ptr(out_sorted_pairs), _stream(stream))
+    rc = (_fast_module or _fast()).dispatch(idx, counts, out_offsets, out_sorted_pairs, stream)
     if rc != 0:
         raise MoreRouteError(rc, "more_dispatch")
 
@@ -204,10 +219,7 @@ def more_dispatch(idx, counts, out_offsets, out_sorted_pairs, stream=None):
 def more_route_full(X, W, k, gate_mode, out_idx, out_gate, out_counts, out_topval=None, out_lse=None, msplit=0,
                     stream=None):
     """``more_route_full`` of the C interface: the fused standard router, logits ``X [T,h] @ W [h,M]`` (bf16, device)."""
-    T, h = X.shape
-    M = W.shape[1]
-    rc = lib().more_route_full(_ptr(X), _ptr(W), T, h, M, k, gate_mode, _ptr(out_idx), _ptr(out_gate), _ptr(out_counts),
-                               _ptr(out_topval), _ptr(out_lse), msplit, _stream(stream))
+    rc = (_fast_module or _fast()).full(X, W, k, gate_mode, out_idx, out_gate, out_counts, out_topval, out_lse, msplit, stream)
     if rc != 0:
         raise MoreRouteError(rc, "more_route_full")
 
@@ -216,15 +228,8 @@ def more_merge_shards(idx, topval, lse, shard_base, M, gate_mode, out_idx, out_g
                       out_lse=None, stream=None):
     """``more_merge_shards`` of the C interface: ``idx``/``topval`` ``[S,T,k]`` (device), ``lse`` ``[S,T]`` or None,
     ``shard_base`` a host sequence of S ints or None; fills ``out_idx``/``out_gate`` ``[T,k]`` and ``out_counts [M]``."""
-    S, T, k = idx.shape
-    base = None
-    if shard_base is not None:
-        base = (ctypes.c_int32 * S)(*[int(b) for b in shard_base])
-    rc = lib().more_merge_shards(_ptr(idx), _ptr(topval), _ptr(lse) if lse is not None else None,
-                                 ctypes.cast(base, ctypes.c_void_p) if base is not None else None,
-                                 S, T, k, M, gate_mode, _ptr(out_idx), _ptr(out_gate),
-                                 _ptr(out_topval) if out_topval is not None else None,
-                                 _ptr(out_lse) if out_lse is not None else None, _ptr(out_counts), _stream(stream))
+    rc = (_fast_module or _fast()).merge(idx, topval, lse, shard_base, M, gate_mode, out_idx, out_gate, out_counts, out_topval,
+                                         out_lse, stream)
     if rc != 0:
         raise MoreRouteError(rc, "more_merge_shards")
 
@@ -255,15 +260,9 @@ class RouteResult:
 
 def route(X, R1, R2, k, gate_mode=GATE_TOPK_SOFTMAX, want_topval=False, want_lse=False, path=PATH_AUTO, msplit=0,
           stream=None) -> RouteResult:
-    """Convenience wrapper: allocate the outputs with torch and call :func:`more_route_ex`."""
-    import torch
-    T = X.shape[0]
-    M = R2.shape[1]
-    dev = X.device
-    idx = torch.empty((T, k), dtype=torch.int32, device=dev)
-    gate = torch.empty((T, k), dtype=torch.float32, device=dev)
-    counts = torch.empty((M,), dtype=torch.int32, device=dev)
-    topval = torch.empty((T, k), dtype=torch.float32, device=dev) if want_topval else None
-    lse = torch.empty((T,), dtype=torch.float32, device=dev) if want_lse else None
-    more_route_ex(X, R1, R2, k, gate_mode, idx, gate, counts, topval, lse, path, msplit, stream)
+    """Convenience wrapper: allocate the outputs with torch and do what :func:`more_route_ex` does."""
+    rc, idx, gate, counts, topval, lse = (_fast_module or _fast()).route(X, R1, R2, k, gate_mode, want_topval, want_lse, path,
+                                                                         msplit, stream)
+    if rc != 0:
+        raise MoreRouteError(rc, "more_route_ex")
     return RouteResult(idx, gate, counts, topval, lse)

@@ -1,4 +1,5 @@
-"""Build ``libmore_route.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Build ``libmore_route.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU), and ``_more_binding.so``, the
+extension module that binding.py calls it through, with g++ against torch's headers."""
 from __future__ import annotations
 
 import os
@@ -14,10 +15,33 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-shared", "-Xcompiler", "-fPIC"]
 
 
+BINDING_PATH = os.path.join(_HERE, "_more_binding.so")
+BINDING_SOURCE = os.path.join(_CSRC, "more_binding.cpp")
+
+
 def _newest_source_mtime() -> float:
-    paths = [os.path.join(_CSRC, f) for f in os.listdir(_CSRC)]
+    paths = [os.path.join(_CSRC, f) for f in os.listdir(_CSRC) if not f.endswith(".cpp")]
     paths.append(os.path.join(os.path.dirname(_HERE), "include", "more_route.h"))
     return max(os.path.getmtime(p) for p in paths)
+
+
+def build_binding(force: bool = False) -> str:
+    """Compile the extension module if it is missing or older than its sources; return its path."""
+    header = os.path.join(os.path.dirname(_HERE), "include", "more_route.h")
+    newest = max(os.path.getmtime(BINDING_SOURCE), os.path.getmtime(header))
+    if not force and os.path.exists(BINDING_PATH) and os.path.getmtime(BINDING_PATH) >= newest:
+        return BINDING_PATH
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    includes = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                sysconfig.get_paths()["include"], os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + i for i in includes] + \
+          ["-o", BINDING_PATH, BINDING_SOURCE, "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+           "-Wl,-rpath," + os.path.join(root, "lib")]
+    subprocess.run(cmd, check=True)
+    return BINDING_PATH
 
 
 def build(force: bool = False, verbose: bool = False, out: str | None = None, defines: tuple = ()) -> str:
@@ -48,3 +72,4 @@ if __name__ == "__main__":
         print(build(force=True, out=sys.argv[1], defines=tuple(sys.argv[2:])))
     else:
         print(build(force=True, verbose=True))
+        print(build_binding(force=True))
