@@ -11,7 +11,11 @@
 // sum with no cross-lane traffic -- and finishes with one atomic add into psum.  (In the router the lanes are tokens,
 // because there the reduction runs along the expert axis.)
 //
-// Warp roles, shared-memory ring, barriers and the bounded waits are those of the router kernel.
+// Warp roles, shared-memory ring, barriers and the bounded waits are those of the router kernel, but for 16 epilogue warps:
+// four per lane quarter, two per 128-token half, which take 64 token columns each.  Bound by the exponentials: 12 of 16 go
+// through the special-function unit (16 results per clock and SM), four through the FMA pipe, and with 32 epilogue warps
+// per SM the latencies around them are hidden (16 warps, which could each hold twice the registers: 53 % of the issue
+// slots used).
 #include "sm100_common.cuh"
 
 #include <math.h>
@@ -19,6 +23,43 @@
 namespace more {
 
 namespace {
+
+constexpr int kPsumEpi = 512;
+constexpr int kPsumThreads = 64 + kPsumEpi;
+
+// two fp32 operations in one instruction
+__device__ __forceinline__ uint64_t pack2(float a, float b)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void unpack2(uint64_t d, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// 16 consecutive fp32 columns of this thread's tensor-memory lane, complete on return.  (Load and wait in one statement:
+// with the destination registers tied to a separate wait the compiler copies them.)
+__device__ __forceinline__ void tmem_get16(uint32_t taddr, float (&v)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+          "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
 
 struct PsumParams {
     int T, h, r, M, msplit, tiles_total;
@@ -28,7 +69,7 @@ struct PsumParams {
 };
 
 template <int RPAD>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kPsumThreads, 2)
 psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_r1,
                     const __grid_constant__ CUtensorMap map_r2, const PsumParams p)
 {
@@ -68,7 +109,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         mbar_init(bar(B_ZACC), 1);
         mbar_init(bar(B_ZOP), kEpilogueThreads);
         for (int i = 0; i < 8; ++i) { mbar_init(bar(B_FULL2 + i), 1); mbar_init(bar(B_EMPTY2 + i), 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(bar(B_ACCF + i), 1); mbar_init(bar(B_ACCE + i), kEpilogueThreads / 2); }
+        for (int i = 0; i < 2; ++i) { mbar_init(bar(B_ACCF + i), 1); mbar_init(bar(B_ACCE + i), kPsumEpi / 32 / 2); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -170,23 +211,23 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     } else {
         // ========================================================================================= epilogue
         const int q = warp & 3;                              // TMEM lane group: token rows (phase 1), experts (phase 2)
-        const int half = (warp - 2) >> 2;                    // which 128-token half
+        const int half = ((warp - 2) >> 2) & 1;              // which 128-token half
+        const int part = (warp - 2) >> 3;                    // which 64 of its columns
         const int row_in_half = q * 32 + lane;
         const int row_in_blk = half * 128 + row_in_half;
         const int64_t row = (int64_t)tok0 + row_in_blk;
         const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16) + half * 128;
         bool ok = mbar_wait(bar(B_ZACC), 0, abort_flag, p.status);
-        if (ok) {
+        if (ok && part == 0) {
             tc_fence_after();
-            // (the phase-1 ring is free now) log2-scaled log-sum-exp of my token; +inf for rows past T, whose
+            // (the phase-1 ring is free now) minus the log2-scaled log-sum-exp of my token; -inf for rows past T, whose
             // zero-filled logits then contribute exp(-inf) = 0
-            lse2[row_in_blk] = (row < p.T) ? p.lse[row] * kLog2e : INFINITY;
+            lse2[row_in_blk] = (row < p.T) ? -p.lse[row] * kLog2e : -INFINITY;
             uint8_t* zrow = ring_ptr + half * kZopOne + row_in_half * 128;
 #pragma unroll
             for (int c = 0; c < RPAD / 16; ++c) {
                 float z[16];
-                tmem_ld16(t_lane + c * 16, z);
-                tmem_ld_wait16(z);
+                tmem_get16(t_lane + c * 16, z);
                 uint32_t hi[8], lo[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
@@ -211,42 +252,41 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             mbar_arrive(bar(B_ZOP));
         }
         // all 256 lse2 entries must be visible before anyone reads them in the sweep
-        asm volatile("bar.sync 1, 256;" ::: "memory");
+        asm volatile("bar.sync 1, 512;" ::: "memory");
 
         ok = __all_sync(0xffffffffu, ok);
-        const float4* lse4 = reinterpret_cast<const float4*>(lse2 + half * 128);
+        const ulonglong2* lse4 = reinterpret_cast<const ulonglong2*>(lse2 + half * 128 + part * 64);
+        const uint64_t scale = pack2(kLog2e, kLog2e);
         for (int it = 0; it < ntiles && ok; ++it) {
             const int expert = (tile_lo + it) * kTileExperts + q * 32 + lane;     // my lane's expert in this tile
             ok = __all_sync(0xffffffffu, mbar_wait(bar(B_ACCF + half), it & 1, abort_flag, p.status));
             if (!ok) break;
             tc_fence_after();
-            float va[16], vb[16];
-            float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, acc3 = 0.f;
-            auto add16 = [&](const float (&v)[16], int c16) {        // token columns c16*16 .. +15 of my half
+            uint64_t acc01 = 0, acc23 = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float v[16];
+                tmem_get16(t_lane + part * 64 + c * 16, v);
+                if (c == 3) {                                    // all columns are in registers: hand the accumulator back
+                    tc_fence_before();
+                    warp_arrive(bar(B_ACCE + half), lane);
+                }
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
-                    const float4 l = lse4[c16 * 4 + g];              // same address in every lane: a broadcast
-                    acc0 += ex2f(fmaf(v[4 * g], kLog2e, -l.x));
-                    acc1 += ex2f(fmaf(v[4 * g + 1], kLog2e, -l.y));
-                    acc2 += ex2f(fmaf(v[4 * g + 2], kLog2e, -l.z));
+                    const ulonglong2 l = lse4[c * 4 + g];        // same address in every lane: a broadcast
+                    float x0, x1, x2, x3;
+                    unpack2(fma2(pack2(v[4 * g], v[4 * g + 1]), scale, l.x), x0, x1);
+                    unpack2(fma2(pack2(v[4 * g + 2], v[4 * g + 3]), scale, l.y), x2, x3);
                     // (one exponential in four on the FMA pipe: the special-function unit's 16 results per clock per SM
-                    // are this loop's narrowest resource; more than one in four costs more issue slots than it frees)
-                    acc3 += ex2_poly(fmaf(v[4 * g + 3], kLog2e, -l.w));
+                    // are this loop's narrowest resource)
+                    acc01 = add2(acc01, pack2(ex2f(x0), ex2f(x1)));
+                    acc23 = add2(acc23, pack2(ex2f(x2), ex2_poly(x3)));
                 }
-            };
-            tmem_ld16(t_lane, va);
-#pragma unroll
-            for (int c = 0; c < 8; c += 2) {
-                tmem_ld_wait16(va);
-                tmem_ld16(t_lane + (c + 1) * 16, vb);
-                add16(va, c);
-                tmem_ld_wait16(vb);
-                if (c + 2 < 8) tmem_ld16(t_lane + (c + 2) * 16, va);
-                add16(vb, c + 1);
             }
-            tc_fence_before();
-            mbar_arrive(bar(B_ACCE + half));
-            if (expert < p.M) atomicAdd(p.psum + expert, (acc0 + acc1) + (acc2 + acc3));
+            float a0, a1, a2, a3;
+            unpack2(acc01, a0, a1);
+            unpack2(acc23, a2, a3);
+            if (expert < p.M) atomicAdd(p.psum + expert, (a0 + a1) + (a2 + a3));
         }
     }
 
@@ -275,7 +315,7 @@ int launch_psum_rpad(const CUtensorMap& mx, const CUtensorMap& m1, const CUtenso
             return MORE_ERR_CUDA;
         configured |= 1ull << (dev & 63);
     }
-    kern<<<ctas, kThreads, kSmemBytes, st>>>(mx, m1, m2, pp);
+    kern<<<ctas, kPsumThreads, kSmemBytes, st>>>(mx, m1, m2, pp);
     count_launch(1);
     return cudaGetLastError() == cudaSuccess ? MORE_OK : MORE_ERR_CUDA;
 }
