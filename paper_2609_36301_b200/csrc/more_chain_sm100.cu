@@ -1078,15 +1078,17 @@ __global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
     put_token(p, tok, c, m2, z, lane);
 }
 
-// More segments than that (a few tokens, whose experts are spread over the whole GPU): a CTA per token.  As above, with
-// 512 threads' maxima joined to 64 of which the k-th largest bounds the k-th best.
+// More segments than that (a few tokens, whose experts are spread over the whole GPU): a CTA per token, 16 threads per
+// segment.  A chain of latencies, so what can be is requested at once: the counts of all of a thread's segments, then all
+// their entries, which stay in registers; 512 threads' maxima are joined to 64, of which the k-th largest bounds the k-th
+// best entry; what reaches it is ranked by counting.
 constexpr int kManyThreads = 512;
-constexpr int kManySegs = 640;
+constexpr int kManyPer = 10;                       // segments per half warp
+constexpr int kManySegs = kManyPer * (kManyThreads / 16);
 __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishParams p)
 {
     constexpr int kWarps = kManyThreads / 32, kKeep = 512;
-    __shared__ int counts[kManySegs];
-    __shared__ float maxima[64];
+    __shared__ __align__(16) float maxima[64];
     __shared__ float2 smz[kWarps];
     __shared__ Cand keep[kKeep];
     __shared__ Cand buf[64];
@@ -1095,18 +1097,44 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tok = blockIdx.x;
     const int blk = tok / kRows, row = tok % kRows;
     if (threadIdx.x == 0) { s_nseg = segments_of(p, blk); s_count = 0; }
+    if (threadIdx.x < 64) buf[threadIdx.x] = no_cand();
     __syncthreads();
     const int nseg = s_nseg;
     const size_t slot0 = (size_t)blk * p.maxseg * kRows + row;
+    const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
+    auto entries = [&](int u) { return p.ent + (slot0 + (size_t)(half + u * (kManyThreads / 16)) * kRows) * p.cap; };
     pdl_wait();
+    int c[kManyPer];
+#pragma unroll
+    for (int u = 0; u < kManyPer; ++u) {
+        const int s = half + u * (kManyThreads / 16);
+        c[u] = s < nseg ? p.cnt[slot0 + (size_t)s * kRows] : 0;
+    }
     float m2 = -INFINITY, z = 0.f;
-    for (int s = threadIdx.x; s < nseg; s += kManyThreads) {
-        counts[s] = p.cnt[slot0 + (size_t)s * kRows];
-        if (p.mz) {
+    if (p.mz) {
+        for (int s = threadIdx.x; s < nseg; s += kManyThreads) {
             const float2 o = p.mz[slot0 + (size_t)s * kRows];
             join_mz(m2, z, o.x, o.y);
         }
     }
+    Cand x[kManyPer], y[kManyPer];
+    float m = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < kManyPer; ++u) {
+        x[u] = hl < c[u] ? load_cand(entries(u) + hl) : no_cand();
+        y[u] = hl + 16 < c[u] ? load_cand(entries(u) + hl + 16) : no_cand();
+    }
+    auto longer = [&](auto f) {                               // entries beyond the 32 that are in registers
+#pragma unroll
+        for (int u = 0; u < kManyPer; ++u)
+            for (int i = hl + 32; i < c[u]; i += 16) f(load_cand(entries(u) + i));
+    };
+#pragma unroll
+    for (int u = 0; u < kManyPer; ++u) m = max3(m, x[u].v, y[u].v);
+    longer([&](Cand e) { m = fmaxf(m, e.v); });
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));          // eight threads' maximum: 64 of them
+    if ((lane & 7) == 0) maxima[warp * 4 + (lane >> 3)] = m;
     if (p.mz) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -1116,54 +1144,62 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
         if (lane == 0) smz[warp] = make_float2(m2, z);
     }
     __syncthreads();
-    // half a warp per segment, the next segment's entries requested before the current ones are used
-    const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
-    auto visit = [&](auto f) {
-        for (int s = half; s < nseg; s += kManyThreads / 16) {
-            const int c = counts[s];
-            const uint2* e = p.ent + (slot0 + (size_t)s * kRows) * p.cap;
-            for (int i = hl; i < c; i += 16) f(load_cand(e + i));
-        }
-    };
-    float m = -INFINITY;
-    visit([&](Cand x) { m = fmaxf(m, x.v); });
+    if (threadIdx.x < 64) {
+        const int me = threadIdx.x;
+        const float mine = maxima[me];
+        int rank = 0;
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));          // eight threads' maximum: 64 of them
-    if ((lane & 7) == 0) maxima[warp * 4 + (lane >> 3)] = m;
-    __syncthreads();
-    if (warp == 0) {
-        // k-th largest of the 64: two sorted halves; entry against mirrored entry gives the 32 largest
-        const float a = warp_sort_down(maxima[lane], lane), b = warp_sort_down(maxima[lane + 32], lane);
-        const float top = warp_sort_down(fmaxf(a, __shfl_sync(kFull, b, 31 - lane)), lane);
-        if (lane == p.k - 1) s_thr = top;
+        for (int j = 0; j < 64; j += 4) {
+            const float4 o = *reinterpret_cast<const float4*>(maxima + j);
+            rank += (o.x > mine) + (o.y > mine) + (o.z > mine) + (o.w > mine);
+            rank += ((o.x == mine) & (j < me)) + ((o.y == mine) & (j + 1 < me)) + ((o.z == mine) & (j + 2 < me)) + ((o.w == mine) & (j + 3 < me));
+        }
+        if (rank == p.k - 1) s_thr = mine;
     }
     __syncthreads();
     const float thr = s_thr;
-    visit([&](Cand x) {
-        if (x.v >= thr) {
+    auto collect = [&](Cand e) {
+        if (e.v >= thr && e.v > -INFINITY) {
             const int at = atomicAdd(&s_count, 1);
-            if (at < kKeep) keep[at] = x;
+            if (at < kKeep) keep[at] = e;
         }
-    });
+    };
+#pragma unroll
+    for (int u = 0; u < kManyPer; ++u) {
+        collect(x[u]);
+        collect(y[u]);
+    }
+    longer(collect);
     __syncthreads();
+    const int n = s_count;
+    if (n <= kKeep) {
+        for (int i = threadIdx.x; i < n; i += kManyThreads) {
+            const Cand e = keep[i];
+            int rank = 0;
+            for (int j = 0; j < n; ++j) {
+                const Cand o = keep[j];
+                rank += (o.v > e.v) | ((o.v == e.v) & (o.id < e.id));
+            }
+            if (rank < p.k) buf[rank] = e;
+        }
+        __syncthreads();
+    }
     if (warp == 0) {
-        const int n = s_count;
-        Cand c;
-        if (n <= kKeep) {
-            c = warp_topk<4>(n, p.k, [&](int f) { return keep[f]; }, buf, lane);
-        } else {
+        Cand best = lane < p.k ? buf[lane] : no_cand();
+        if (n > kKeep) {
             // more near the top than the buffer holds (many equal logits): over all of them
             const int most = p.cap;
-            c = warp_topk<1>(nseg * most, p.k, [&](int f) {
+            best = warp_topk<1>(nseg * most, p.k, [&](int f) {
                 const int s = f / most, i = f - s * most;
-                return i < counts[s] ? load_cand(p.ent + (slot0 + (size_t)s * kRows) * p.cap + i) : no_cand();
+                const size_t slot = slot0 + (size_t)s * kRows;
+                return i < p.cnt[slot] ? load_cand(p.ent + slot * p.cap + i) : no_cand();
             }, buf, lane);
         }
         m2 = smz[0].x;
         z = smz[0].y;
         if (p.mz)
             for (int w = 1; w < kWarps; ++w) join_mz(m2, z, smz[w].x, smz[w].y);
-        put_token(p, tok, c, m2, z, lane);
+        put_token(p, tok, best, m2, z, lane);
     }
 }
 
@@ -1258,7 +1294,8 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
 void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
 {
     const long long blocks = ((T < kChunkTokens ? T : kChunkTokens) + kRows - 1) / kRows;
-    const long long nsteps = (M + W - 1) / W, total = blocks * nsteps, slots = 2 * sm_count;
+    const long long nsteps = (M + W - 1) / W, total = blocks * nsteps;
+    const long long slots = 2 * sm_count < kManySegs - 2 ? 2 * sm_count : kManySegs - 2;
     const double kSegment = 4.0;
     long long g = total < slots ? total : slots, share = 0;
     if (msplit > 0) {

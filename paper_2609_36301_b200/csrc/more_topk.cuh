@@ -73,8 +73,9 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
     __syncwarp();
     Cand best = no_cand();
     if (count <= 64) {
+        // Ranks by the logits alone, and by the ids as well only if the ranks' sum shows that two logits were equal.
         Cand mine[2];
-        int rank[2];
+        int rank[2], sum = 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int pos = lane + 32 * h;
@@ -82,12 +83,20 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
             if (32 * h < count) {
                 mine[h] = pos < count ? buf[pos] : no_cand();
                 int q = 0;
-#pragma unroll 4
-                for (int j = 0; j < count; ++j) {
-                    const Cand o = buf[j];
-                    q += (o.v > mine[h].v || (o.v == mine[h].v && (o.id < mine[h].id || (o.id == mine[h].id && j < pos)))) ? 1 : 0;
-                }
-                if (pos < count) rank[h] = q;
+#pragma unroll 8
+                for (int j = 0; j < count; ++j) q += buf[j].v > mine[h].v ? 1 : 0;
+                if (pos < count) { rank[h] = q; sum += q; }
+            }
+        }
+        if (__reduce_add_sync(kAll, sum) != count * (count - 1) / 2) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int pos = lane + 32 * h;
+                if (pos < count)
+                    for (int j = 0; j < count; ++j) {
+                        const Cand o = buf[j];
+                        rank[h] += (o.v == mine[h].v && (o.id < mine[h].id || (o.id == mine[h].id && j < pos))) ? 1 : 0;
+                    }
             }
         }
         __syncwarp();
