@@ -77,6 +77,7 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const int cs = p.cs, rank = blockIdx.x % cs, blk = blockIdx.x / cs;
     const int nkt = (p.h + 63) / 64;
     const int kt_lo = nkt * rank / cs, kt_hi = nkt * (rank + 1) / cs;
+    const int live = min(kRows, p.T - blk * kRows);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < B_COUNT; ++i) mbar_init(bar(i), 1);
@@ -159,7 +160,7 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     zr[lo_off + 2 * c + 1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
                 }
             }
-        } else if (ok) {
+        } else if (ok && row - lane < live) {      // (rows past the last token are not exchanged: nothing reads them)
             const int share = kRows / cs, dst = row / share;
             const uint32_t a = smem_u32(exch) + (uint32_t)((rank * share + row % share) * 64) * 4u;
             uint32_t remote;
@@ -168,10 +169,12 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 float v[16];
                 tmem_ld16(t_lane + c * 16, v);
                 tmem_ld_wait16(v);
+                if (row < live) {
 #pragma unroll
-                for (int e = 0; e < 16; e += 4)
-                    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};"
-                                 ::"r"(remote + (c * 16 + e) * 4), "f"(v[e]), "f"(v[e + 1]), "f"(v[e + 2]), "f"(v[e + 3]) : "memory");
+                    for (int e = 0; e < 16; e += 4)
+                        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};"
+                                     ::"r"(remote + (c * 16 + e) * 4), "f"(v[e]), "f"(v[e + 1]), "f"(v[e + 2]), "f"(v[e + 3]) : "memory");
+                }
             }
         }
     }
@@ -179,14 +182,19 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if (cs > 1) {
         cluster_sync();
         if (warp >= 2) {
-            const int share = kRows / cs, q4 = p.zc / 8;         // float4s of one row of z
-            for (int i = threadIdx.x - 64; i < share * q4; i += kRows) {
-                const int rr = i / q4, c4 = i % q4;
+            const int share = kRows / cs, q4_bits = p.zc == 64 ? 3 : 4, q4 = 1 << q4_bits;        // float4s of one row of z
+            const int mine = min(share, live - rank * share);
+            for (int i = threadIdx.x - 64; i < mine * q4; i += kRows) {
+                const int rr = i >> q4_bits, c4 = i & (q4 - 1);
                 float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (c4 * 4 < p.n) {
-                    for (int q = 0; q < cs; ++q) {
-                        const float4 v = *reinterpret_cast<const float4*>(exch + (q * share + rr) * 64 + c4 * 4);
-                        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+                    const float* e = exch + rr * 64 + c4 * 4;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if (q < cs) {
+                            const float4 v = *reinterpret_cast<const float4*>(e + q * share * 64);
+                            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+                        }
                     }
                 }
                 uint2 hi, lo;
@@ -604,18 +612,18 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         };
         // candidates of the list that beat `low` (or are among the first `equal` that equal it) -> scratch
         auto emit = [&](uint2* dst, float low, int equal) {
-            for (uint64_t o = first; o < ptr; o += 4 * kEntry) {
-                float4 e[4];
-                int c[4];
+            constexpr int U = 4;                             // (independent loads: one round trip for four entries)
+            for (uint64_t o = first; o < ptr; o += U * kEntry) {
+                float4 e[U];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {                // (independent loads: one round trip for four entries)
+                for (int i = 0; i < U; ++i) {
                     e[i] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                    c[i] = 0;
-                    if (o + i * kEntry < ptr) { e[i] = ent4(o + i * kEntry); c[i] = ent_col(o + i * kEntry); }
+                    if (o + i * kEntry < ptr) e[i] = ent4(o + i * kEntry);
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (!(fmaxf(max3(e[i].x, e[i].y, e[i].z), e[i].w) >= low)) continue;
+                for (int i = 0; i < U; ++i) {
+                    if (!(fmaxf(max3(e[i].x, e[i].y, e[i].z), e[i].w) >= low) || o + i * kEntry >= ptr) continue;
+                    const int c = ent_col(o + i * kEntry);
                     const float x[4] = {e[i].x, e[i].y, e[i].z, e[i].w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -624,7 +632,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                             equal -= eq ? 1 : 0;
                             int at;
                             asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(at) : "r"(s_cnt) : "memory");
-                            if (at < p.cap) dst[at] = make_uint2(__float_as_uint(x[j]), (uint32_t)(c[i] + j));
+                            if (at < p.cap) dst[at] = make_uint2(__float_as_uint(x[j]), (uint32_t)(c + j));
                         }
                     }
                 }
@@ -1079,9 +1087,10 @@ __global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
 }
 
 // More segments than that (a few tokens, whose experts are spread over the whole GPU): a CTA per token, 16 threads per
-// segment.  A chain of latencies, so what can be is requested at once: the counts of all of a thread's segments, then all
-// their entries, which stay in registers; 512 threads' maxima are joined to 64, of which the k-th largest bounds the k-th
-// best entry; what reaches it is ranked by counting.
+// segment.  A chain of latencies, so what can be is requested at once: the counts of all of a thread's segments, then their
+// entries; 512 threads' maxima are joined to 64, of which the k-th largest bounds the k-th best entry; what reaches it is
+// ranked by counting.  Code that runs once is fetched from L2 as it runs, so it is kept short (entries held in registers and
+// 20 unrolled tests took 2.5 us where reading them again takes 1).
 constexpr int kManyThreads = 512;
 constexpr int kManyPer = 10;                       // segments per half warp
 constexpr int kManySegs = kManyPer * (kManyThreads / 16);
@@ -1102,14 +1111,14 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     const int nseg = s_nseg;
     const size_t slot0 = (size_t)blk * p.maxseg * kRows + row;
     const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
-    auto entries = [&](int u) { return p.ent + (slot0 + (size_t)(half + u * (kManyThreads / 16)) * kRows) * p.cap; };
+    const int* const my_cnt = p.cnt + slot0 + (size_t)half * kRows;
+    const uint2* const my_ent = p.ent + (slot0 + (size_t)half * kRows) * p.cap + hl;
+    const size_t next_ent = (size_t)(kManyThreads / 16) * kRows * p.cap;
     pdl_wait();
     int c[kManyPer];
 #pragma unroll
-    for (int u = 0; u < kManyPer; ++u) {
-        const int s = half + u * (kManyThreads / 16);
-        c[u] = s < nseg ? p.cnt[slot0 + (size_t)s * kRows] : 0;
-    }
+    for (int u = 0; u < kManyPer; ++u)
+        c[u] = half + u * (kManyThreads / 16) < nseg ? my_cnt[u * (kManyThreads / 16) * kRows] : 0;
     float m2 = -INFINITY, z = 0.f;
     if (p.mz) {
         for (int s = threadIdx.x; s < nseg; s += kManyThreads) {
@@ -1117,21 +1126,22 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
             join_mz(m2, z, o.x, o.y);
         }
     }
-    Cand x[kManyPer], y[kManyPer];
     float m = -INFINITY;
+    {
+        float x[kManyPer], y[kManyPer];
+        const uint2* e = my_ent;
 #pragma unroll
-    for (int u = 0; u < kManyPer; ++u) {
-        x[u] = hl < c[u] ? load_cand(entries(u) + hl) : no_cand();
-        y[u] = hl + 16 < c[u] ? load_cand(entries(u) + hl + 16) : no_cand();
+        for (int u = 0; u < kManyPer; ++u, e += next_ent) {
+            x[u] = hl < c[u] ? __uint_as_float(e->x) : -INFINITY;
+            y[u] = hl + 16 < c[u] ? __uint_as_float(e[16].x) : -INFINITY;
+        }
+        e = my_ent;
+#pragma unroll
+        for (int u = 0; u < kManyPer; ++u, e += next_ent) {
+            m = max3(m, x[u], y[u]);
+            for (int i = hl + 32; i < c[u]; i += 16) m = fmaxf(m, __uint_as_float(e[i - hl].x));
+        }
     }
-    auto longer = [&](auto f) {                               // entries beyond the 32 that are in registers
-#pragma unroll
-        for (int u = 0; u < kManyPer; ++u)
-            for (int i = hl + 32; i < c[u]; i += 16) f(load_cand(entries(u) + i));
-    };
-#pragma unroll
-    for (int u = 0; u < kManyPer; ++u) m = max3(m, x[u].v, y[u].v);
-    longer([&](Cand e) { m = fmaxf(m, e.v); });
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));          // eight threads' maximum: 64 of them
     if ((lane & 7) == 0) maxima[warp * 4 + (lane >> 3)] = m;
@@ -1158,18 +1168,21 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     }
     __syncthreads();
     const float thr = s_thr;
-    auto collect = [&](Cand e) {
-        if (e.v >= thr && e.v > -INFINITY) {
-            const int at = atomicAdd(&s_count, 1);
-            if (at < kKeep) keep[at] = e;
+    if (m >= thr && m > -INFINITY) {                          // (few threads: their entries are read again, from L1)
+        const uint2* e = my_ent;
+#pragma unroll 1
+        for (int s = half; s < nseg; s += kManyThreads / 16, e += next_ent) {
+            const int count = p.cnt[slot0 + (size_t)s * kRows];
+#pragma unroll 1
+            for (int i = hl; i < count; i += 16) {
+                const Cand x = load_cand(e + (i - hl));
+                if (x.v >= thr && x.v > -INFINITY) {
+                    const int at = atomicAdd(&s_count, 1);
+                    if (at < kKeep) keep[at] = x;
+                }
+            }
         }
-    };
-#pragma unroll
-    for (int u = 0; u < kManyPer; ++u) {
-        collect(x[u]);
-        collect(y[u]);
     }
-    longer(collect);
     __syncthreads();
     const int n = s_count;
     if (n <= kKeep) {
