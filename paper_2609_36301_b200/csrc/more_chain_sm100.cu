@@ -243,8 +243,18 @@ constexpr int kMaxStages = 8;
 constexpr int kListCap = 64;                       // entries of a thread's list
 constexpr uint32_t kEntry = kEpi * 32;             // bytes between its entries (32 bytes each: four logits, the first one's column)
 
-// Units whose bucket maxima are formed ahead of a segment of `steps` units; up to two stay in the accumulators.
-__host__ __device__ __forceinline__ int lead_of(int steps) { return steps >= 24 ? steps / 8 : (steps < 2 ? steps : 2); }
+// Units whose bucket maxima are formed ahead of a segment of `steps` units.  All of a short one: its threshold is then the
+// final one before the first candidate is kept, and a thread keeps one or two groups instead of the ten that a rising
+// threshold lets through; what is saved is not the appending but the reading back at the end, a chain of trips to L2.
+// T = 3000, M = 16384: 49.9 -> 41.7 us; T = 1024, M = 65536, k = 16: 164 -> 77 us; T = 64, M = 131072, k = 16: 40.7 -> 34.3.
+// An eighth of a long one, where computing everything twice costs more.  The line is at 32 units for k <= 8 (at 41 units 84 us
+// against 81) and at 64 for longer lists, which keep three times the candidates (T = 17000, M = 16384, k = 16, 57 units:
+// 187 -> 143 us; at 111 units 437 -> 456).  For thousands of units 1/4, 1/6 and 1/8 are within 3 % of one another.  Up to
+// two units stay in the two accumulators, more are computed again.
+__host__ __device__ __forceinline__ int lead_of(int steps, bool longer)
+{
+    return steps <= (longer ? 64 : 32) ? steps : steps / 8;
+}
 
 struct SweepParams {
     int T, M, k;
@@ -408,7 +418,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             for (int left = (int)(hi - lo); left > 0 && ok; ++blk, ++seg, s0 = 0) {
                 const int steps = min(left, p.nsteps - s0);
                 left -= steps;
-                const int lead = lead_of(steps), total = steps + (lead > 2 ? lead : 0);
+                const int lead = lead_of(steps, KCAP > 8), total = steps + (lead > 2 ? lead : 0);
                 auto step_of = [&](int v) { return s0 + (v >= lead && lead > 2 ? v - lead : v); };
                 int v = 0;
                 if (seg == 0) {
@@ -441,7 +451,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             for (int left = (int)(hi - lo); left > 0; ++seg, s0 = 0) {
                 const int steps = min(left, p.nsteps - s0);
                 left -= steps;
-                const int lead = lead_of(steps), total = steps + (lead > 2 ? lead : 0);
+                const int lead = lead_of(steps, KCAP > 8), total = steps + (lead > 2 ? lead : 0);
                 const int zb = p.zbufs == 2 ? seg & 1 : 0, zuse = p.zbufs == 2 ? seg >> 1 : seg;
                 wait_or_abort(bar(B_ZF + zb), zuse & 1, abort_flag, p.status);
                 const uint64_t z = zd + zb * (p.z_bytes >> 4);
@@ -501,7 +511,13 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             *reinterpret_cast<float4*>(o) = e;
             *reinterpret_cast<int*>(o + 16) = c;
         };
+        // (sorted: which bucket a set of columns is in does not matter, only that the sets are disjoint)
         auto publish = [&]() {
+            if constexpr (NB == 4) {
+                cx(b[0], b[1]); cx(b[2], b[3]); cx(b[0], b[2]); cx(b[1], b[3]); cx(b[1], b[2]);
+            } else {
+                sort8(b);
+            }
 #pragma unroll
             for (int i = 0; i < NB; i += 4)
                 asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
@@ -512,47 +528,32 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             auto fetch4 = [&](uint32_t at, float* x) {
                 asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(at) : "memory");
             };
-            float kth;
-            if constexpr (KCAP <= 8) {
-                float a[8], y[8];
-                fetch4(pub0, a);
-                fetch4(pub0 + kRows * 16, a + 4);
-                fetch4(pub0 + kRows * 32, y);
-                fetch4(pub0 + kRows * 48, y + 4);
-                sort8(a);
-                sort8(y);
-                // the eight best of two sorted lists: entry against mirrored entry, then a bitonic sort
+            // 2 NB values at `at` and behind it, in descending order
+            auto fetch_pair = [&](uint32_t at, float (&x)[2 * NB]) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] = fmaxf(a[i], y[7 - i]);
-                if (p.k == 8) {
-                    kth = fminf(fminf(fminf(a[0], a[1]), fminf(a[2], a[3])), fminf(fminf(a[4], a[5]), fminf(a[6], a[7])));
-                } else {
-                    bitonic_down(a);
-                    kth = a[0];
+                for (int i = 0; i < NB; i += 4) fetch4(at + i * 4, x + i);
+                float y[NB];
 #pragma unroll
-                    for (int i = 1; i < 8; ++i) kth = (i < p.k) ? a[i] : kth;
-                }
+                for (int i = 0; i < NB; i += 4) fetch4(at + kRows * NB * 4 + i * 4, y + i);
+#pragma unroll
+                for (int i = 0; i < NB; ++i) x[NB + i] = y[NB - 1 - i];
+                bitonic_down(x);
+            };
+            // the 2 NB best of two sorted lists: entry against mirrored entry
+            float a[2 * NB], y[2 * NB];
+            fetch_pair(pub0, a);
+            fetch_pair(pub0 + 2 * kRows * NB * 4, y);
+#pragma unroll
+            for (int i = 0; i < 2 * NB; ++i) a[i] = fmaxf(a[i], y[2 * NB - 1 - i]);
+            float kth = a[0];
+            if (p.k == 2 * NB) {
+#pragma unroll
+                for (int i = 1; i < 2 * NB; ++i) kth = fminf(kth, a[i]);
             } else {
-                float a[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) a[i] = -INFINITY;
-                float least = INFINITY;
-#pragma unroll 1
-                for (int o = 0; o < 4; ++o) {
-                    float x[8];
-                    fetch4(pub0 + o * (kRows * 32), x);
-                    fetch4(pub0 + o * (kRows * 32) + 16, x + 4);
-                    sort8(x);
-                    least = fminf(least, x[7]);
-                    // the 16 best of two sorted lists
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) a[8 + i] = fmaxf(a[8 + i], x[7 - i]);
-                    bitonic_down(a);
-                }
+                bitonic_down(a);
                 kth = a[0];
 #pragma unroll
-                for (int i = 1; i < 16; ++i) kth = (i < p.k) ? a[i] : kth;
-                if (p.k > 16) kth = least;                   // all 32 buckets reach the smallest of them
+                for (int i = 1; i < 2 * NB; ++i) kth = (i < p.k) ? a[i] : kth;
             }
             return just_below(kth);
         };
@@ -655,8 +656,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             m2 = -INFINITY;
             zsum = 0.f;
             ptr = first;
-            const int lead = lead_of(steps), again = lead > 2 ? lead : 0;      // units ahead, and how many of them come again
-            int next = lead, turn = 0;
+            const int lead = lead_of(steps, KCAP > 8), again = lead > 2 ? lead : 0;      // units ahead, and how many of them come again
+            int next = lead + (lead + 1) / 2, turn = 0;
             // maxima of 16 columns' groups of four; what lies beyond M is nothing (M is a multiple of 8)
             auto group_max = [&](auto masked, const float (&v)[16], int col, float (&t)[4]) {
 #pragma unroll
@@ -705,6 +706,10 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 const float t0 = compute_thr();
                 sts(s_thr, t0);                              // (by all four, or a fast one could still read an earlier block's)
                 thr = fmaxf(thr, t0);
+                if (again) {                                 // (those units come again, and must not be in two buckets)
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) b[i] = -INFINITY;
+                }
             }
             // One unit.  (One that reaches beyond M is an instantiation of its own, so that the others carry no masking.)
             auto unit = [&](auto masked, int s) {
@@ -776,12 +781,13 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             }
             // ---- end of the segment: what still beats the threshold goes to scratch
             if (warp_live) {
-                publish();
+                const bool final = lead == steps;                    // (the threshold is that of all units already)
+                if (!final) publish();
                 if (sub == 0) asm volatile("st.shared.u32 [%0], 0;" ::"r"(s_cnt) : "memory");
                 if (LSE && sub > 0)
                     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(s_mz + (sub - 1) * (kRows * 8)), "f"(m2), "f"(zsum) : "memory");
                 quarter_sync(q);
-                thr = fmaxf(thr, compute_thr());
+                if (!final) thr = fmaxf(thr, compute_thr());
                 const int seg = (int)blockIdx.x - owner_of((long long)blk * nsteps, p.total, g);
                 const size_t slot = (size_t)blk * p.maxseg + seg;
                 uint2* dst = p.ent + (slot * kRows + row) * p.cap;
@@ -1245,7 +1251,7 @@ SweepFn sweep_ready()
 SweepFn sweep_fn(int k, bool lse)
 {
     if (k <= 8) return lse ? sweep_ready<8, true>() : sweep_ready<8, false>();
-    return lse ? sweep_ready<32, true>() : sweep_ready<32, false>();
+    return lse ? sweep_ready<16, true>() : sweep_ready<16, false>();
 }
 
 template <class... Args>
@@ -1426,9 +1432,10 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
         fp.out_topval = a.out_topval ? a.out_topval + ro : nullptr;
         fp.out_lse = a.out_lse ? a.out_lse + t0 : nullptr;
         cudaError_t e;
-        // (a list of k <= 16 holds ~1.4 k: with more than two of them, or longer ones, the threshold of the warp's selection
-        // saves more than its 32 lanes per token cost)
-        if (a.k <= 16 && plan.maxseg <= (plan.share > 0 ? 2 : kFewSegs))
+        // Eight threads per token rank up to two short lists by counting everything against everything; where there is
+        // more, the threshold of a warp's selection saves more than its 32 lanes per token cost (k = 16: T = 17000,
+        // M = 8192 121 -> 88 us, T = 32768, M = 4096 174 -> 114; k = 8 with two lists each, T = 17000, M = 4096 54 -> 51).
+        if (a.k <= 8 && plan.maxseg <= (plan.share > 0 ? 1 : kFewSegs))
             e = launch(finish_few_kernel, (T + 31) / 32, 256, 0, a.stream, true, 1, fp);
         else if (plan.maxseg <= kWarpSegs)
             e = launch(finish_warp_kernel, (T + 7) / 8, 256, 0, a.stream, true, 1, fp);

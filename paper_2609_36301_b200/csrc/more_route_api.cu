@@ -194,7 +194,7 @@ namespace {
 bool chain_wins(int T, int M, int k, int sm_count)
 {
     const int per_sm = (T + sm_count - 1) / sm_count;
-    if (M < 512) return false;
+    if (k > 16 || M < 128) return false;
     if (per_sm <= 28) return true;
     if (k > 8) return M >= 32768;
     if (per_sm <= 60) return M >= 3072;

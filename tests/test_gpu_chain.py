@@ -82,3 +82,10 @@ def test_more_tokens_than_one_chunk():
     case = inputs.gaussian_case(T, 64, 8, 32768, 4, 0, seed=9)
     rows = np.concatenate([np.arange(64), np.arange(131072 - 64, T)])
     _route_and_check(case, rows, launches=6)
+
+
+@pytest.mark.parametrize("k,gate_mode", [(8, 1), (12, 0)])
+def test_long_segments(k, gate_mode):
+    """More than 32 units per segment: the leading units are computed twice, the threshold rises on the way."""
+    case = inputs.gaussian_case(4800, 64, 16, 36008, k, gate_mode, seed=17)
+    _route_and_check(case, np.concatenate([np.arange(40), np.arange(2400, 2440), np.arange(4760, 4800)]))
