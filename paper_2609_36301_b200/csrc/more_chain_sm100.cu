@@ -1308,14 +1308,14 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
 // Launch plan.  The unit of work is 128 tokens x 128 experts.  Two CTAs per SM get contiguous parts of the line of units,
 // either equal ones wherever these begin (stretches of several token blocks are then cut into segments), or an equal share
 // of one block each.  The second leaves some SMs idle but every CTA with one segment; what a segment costs on its own (its
-// first MMAs, the threshold to start with, the pass through the lists at its end) is worth about four units.  A forced
+// first MMAs, the threshold to start with, the pass through the lists at its end) is worth about eight units.  A forced
 // split of s CTAs per token block is the second with that s.
 void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
 {
     const long long blocks = ((T < kChunkTokens ? T : kChunkTokens) + kRows - 1) / kRows;
     const long long nsteps = (M + W - 1) / W, total = blocks * nsteps;
     const long long slots = 2 * sm_count < kManySegs - 2 ? 2 * sm_count : kManySegs - 2;
-    const double kSegment = 4.0;
+    const double kSegment = 8.0;
     long long g = total < slots ? total : slots, share = 0;
     if (msplit > 0) {
         const int most = M / 256 > 1 ? M / 256 : 1;

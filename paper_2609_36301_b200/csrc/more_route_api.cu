@@ -187,18 +187,30 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 namespace {
 
 // Whether the low-rank router runs as the chain projection -> sweep -> finish rather than as one of the two kernels that
-// do it all.  Measured on B200 over T = 1 ... 64 k, M = 256 ... 64 k, r = 16, 32, 64, k = 8 and 16, both gates (174
-// points).  The chain wins where one kernel repeats the projection or leaves SMs idle (few tokens: 1.1 to 1.9 times
-// faster) and on long sweeps (M = 64 k: 1.1 to 1.4); what it pays for every segment of a sweep, and its third launch,
-// lose on many tokens with few experts (T = 64 k, M = 1 k: half as fast).
-bool chain_wins(int T, int M, int k, int sm_count)
+// do it all.  Measured on B200 at 1260 points: T = 1 ... 64 k, h = 128, 512, 2048, r = 16 ... 64, M = 128 ... 64 k,
+// k = 4, 8, 12, 16, both gates; the large ones also under sustained load, where the chip's power limit counts (the chain's
+// sweep loses ~3 % more there).  The chain wins where one kernel repeats the projection or leaves SMs idle (few tokens: 1.2
+// to 3 times faster, most at large h, where a cluster shares the reading of X) and on all but short sweeps (1.1 to 2.5 at
+// k > 8, 1.1 to 1.5 at k <= 4).  What it pays for each segment of a sweep, its third launch and the counts, added up by a
+// kernel of their own, lose on few experts (T = 17 k, M = 512: 0.7) and on many tokens at M = 1 k ... 4 k (T = 64 k,
+// M = 2 k, k = 8: 0.8).  k = 5 ... 8 has the worst threshold for its k (the 8th of 16 buckets), so its lines lie lower;
+// above 16 the buckets do not bound the k-th logit well enough, below 128 experts they are mostly empty.
+bool chain_wins(int T, int h, int r, int M, int k, bool lse, int sm_count)
 {
     const int per_sm = (T + sm_count - 1) / sm_count;
     if (k > 16 || M < 128) return false;
-    if (per_sm <= 28) return true;
-    if (k > 8) return M >= 32768;
-    if (per_sm <= 60) return M >= 3072;
-    return M >= (per_sm > 250 ? 32768 : 16384);
+    if (M < 512) return per_sm <= 8 ? M >= 256 || h >= 512 : h >= 1024 && per_sm <= 24;
+    if (M < 1024) return per_sm <= (h >= 1024 ? 45 : 24);
+    if (M < 2048) return per_sm <= 90;
+    if (k > 8) return per_sm <= 230 || M >= 16384 || (M >= 4096 && r <= 32);
+    if (k <= 4) return M >= 8192 || per_sm <= 230;
+    if (M < 16384) return per_sm <= (M < 4096 ? 140 : 170);
+    // a few segments of 33 to 64 units per CTA are the longest that are not swept twice (T = 16 k, M = 16 k: 0.94 to 1.02)
+    if (M < 32768 && per_sm > 100 && per_sm <= 120) return false;
+    // many tokens: the paired kernel, with two accumulators per token group at r <= 32, ties or wins unless it is slowed by
+    // the exponentials (T = 64 k, M = 16 k: 0.94 to 0.96 without them; with them 1.07 at r = 32, 0.99 at r = 64)
+    if (per_sm > 240 && M < 65536) return lse && (r <= 32 || M >= 32768);
+    return true;
 }
 
 // Launch plan of the paired low-rank kernel (256-token CTAs, two per SM).
@@ -339,7 +351,6 @@ void plan_lowrank(int T, int h, int r, int M, int k, bool want_lse, int msplit, 
 int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, bool full, int path, int msplit,
               int sm_count, Plan* out)
 {
-    (void)gate_mode;
     const bool fast_ok = tcgen05_shape_ok(T, h, r, M, k);
     if (path == MORE_PATH_TCGEN05 && !fast_ok) return MORE_ERR_SHAPE;
     if (msplit < 0 || msplit > 64) return MORE_ERR_SHAPE;
@@ -358,7 +369,7 @@ int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, b
     if (full) {
         plan_dense(T, h, M, msplit, sm_count, &p);
     } else {
-        if (chain_wins(T, M, k, sm_count)) {
+        if (chain_wins(T, h, r, M, k, want_lse || gate_mode == MORE_GATE_FULL_SOFTMAX, sm_count)) {
             plan_chain(T, M, msplit, sm_count, &p);
             *out = p;
             return MORE_OK;
