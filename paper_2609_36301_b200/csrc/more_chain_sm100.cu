@@ -14,6 +14,7 @@
 #include "sm100_common.cuh"
 
 #include <cuda_bf16.h>
+#include <float.h>
 
 #include <type_traits>
 
@@ -227,14 +228,14 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 // Selection.  A thread keeps the maxima of NB disjoint sets of its columns ("buckets": runs of 8 or 4 columns, by their
 // position in the units) and a threshold.  The k-th largest of a token's 4 NB bucket maxima is reached by
 // at least k of its logits, so nothing strictly below it can be selected; its expected rank is ~11 for k = 8 of 16
-// buckets, ~22 for k = 16 of 32.  Every group of four whose maximum beats the threshold is appended, values and first
+// buckets, ~22 for k = 16 of 32.  Every group of four whose maximum reaches the threshold is appended, values and first
 // column, to the thread's list in global scratch (which stays in L2): two predicated stores and an add, and nothing
 // waits for them.  A sweep starts with a threshold: the bucket maxima of its first eighth (of its first two units, if
 // that is no more) are formed before anything is selected; this costs an eighth more MMAs, and saves the appends of the
 // start, when nearly everything beats what has been seen.  After 1/8 of the sweep, and whenever half as much again is done, the buckets are published
 // in shared memory, one of the four warps of a lane quarter computes new thresholds from them, and the others pick these
 // up when they see them (all values are monotone lower bounds, so no synchronisation is needed).  At the end of a
-// segment a thread goes once through its list and keeps what beats the final threshold (~11 logits per token).
+// segment a thread goes once through its list and keeps what reaches the final threshold (~11 logits per token).
 constexpr int kSThreads = 576;
 constexpr int kEpi = 512;
 constexpr int W = 128;                             // experts of a unit
@@ -319,7 +320,7 @@ __device__ __forceinline__ void bitonic_down(float (&s)[N])
         for (int i = 0; i < N; ++i)
             if ((i & d) == 0) cx(s[i], s[i + d]);
 }
-// Append the groups of four (maxima t, values v, first column col + 4 i) that beat thr to a list that ends at `end`.  The
+// Append the groups of four (maxima t, values v, first column col + 4 i) that reach thr to a list that ends at `end`.  The
 // four tests come first: only the adds to the list's end depend on each other.  `one` is 1, unknown to the compiler: a
 // predicated 64-bit multiply-add is one instruction, a predicated 64-bit add is four.
 __device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t, const float* v, int col, uint32_t one)
@@ -329,7 +330,7 @@ __device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t
     "@" P " mad.wide.u32 %0, %24, %22, %0;\n\t"
     asm volatile(
         "{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 c1, c2, c3;\n\t"
-        "setp.gt.f32 p0, %2, %1;\n\tsetp.gt.f32 p1, %3, %1;\n\tsetp.gt.f32 p2, %4, %1;\n\tsetp.gt.f32 p3, %5, %1;\n\t"
+        "setp.ge.f32 p0, %2, %1;\n\tsetp.ge.f32 p1, %3, %1;\n\tsetp.ge.f32 p2, %4, %1;\n\tsetp.ge.f32 p3, %5, %1;\n\t"
         "add.u32 c1, %23, 4;\n\tadd.u32 c2, %23, 8;\n\tadd.u32 c3, %23, 12;\n\t"
         MORE_APPEND("p0", "%23", "%6", "%7", "%8", "%9") MORE_APPEND("p1", "c1", "%10", "%11", "%12", "%13")
         MORE_APPEND("p2", "c2", "%14", "%15", "%16", "%17") MORE_APPEND("p3", "c3", "%18", "%19", "%20", "%21") "}"
@@ -340,8 +341,13 @@ __device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t
         : "memory");
 #undef MORE_APPEND
 }
-// strictly below x, by a hair: a logit equal to x still beats it
-__device__ __forceinline__ float just_below(float x) { return fmaf(-fabsf(x), 2.4e-7f, x) - 1e-37f; }
+// the next float above x
+__device__ __forceinline__ float just_above(float x)
+{
+    const int b = x == 0.f ? 0 : __float_as_int(x);
+    const int key = (b ^ ((b >> 31) & 0x7fffffff)) + 1;      // ordered as the floats are
+    return __int_as_float(key ^ ((key >> 31) & 0x7fffffff));
+}
 
 __device__ __forceinline__ bool elect_one()
 {
@@ -555,7 +561,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
 #pragma unroll
                 for (int i = 1; i < 2 * NB; ++i) kth = (i < p.k) ? a[i] : kth;
             }
-            return just_below(kth);
+            return kth;
         };
         // k-th largest logit of this thread's own list and how many equal to it are wanted (all of them in a short list)
         auto own_kth = [&](int& equal) {
@@ -586,7 +592,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 float mine = b[0];
 #pragma unroll
                 for (int i = 1; i < NB; ++i) mine = fminf(mine, b[i]);
-                thr = fmaxf(thr, just_below(mine));
+                thr = fmaxf(thr, mine);
             }
             auto keep = [&](float low, int equal) {
                 uint64_t wr = first;
@@ -602,17 +608,18 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 }
                 ptr = wr;
             };
-            keep(just_below(thr), 0);
+            keep(thr, INT_MAX);
             if (ptr > warn) {
                 int equal;
                 const float kth = own_kth(equal);
                 keep(kth, equal);
-                thr = fmaxf(thr, kth);
+                thr = fmaxf(thr, just_above(kth));
             }
             __syncwarp();
         };
-        // candidates of the list that beat `low` (or are among the first `equal` that equal it) -> scratch
-        auto emit = [&](uint2* dst, float low, int equal) {
+        // Candidates of the list that beat `low` -> scratch, and of those that equal it the first `equal`; with `every`, only
+        // while fewer than `equal` have been passed on at all: where k of this thread are not below `low`, later equals lose.
+        auto emit = [&](uint2* dst, float low, int equal, bool every) {
             constexpr int U = 4;                             // (independent loads: one round trip for four entries)
             for (uint64_t o = first; o < ptr; o += U * kEntry) {
                 float4 e[U];
@@ -630,7 +637,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     for (int j = 0; j < 4; ++j) {
                         const bool eq = x[j] == low && equal > 0;
                         if (x[j] > low || eq) {
-                            equal -= eq ? 1 : 0;
+                            equal -= eq || every ? 1 : 0;
                             int at;
                             asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(at) : "r"(s_cnt) : "memory");
                             if (at < p.cap) dst[at] = make_uint2(__float_as_uint(x[j]), (uint32_t)(c + j));
@@ -652,12 +659,21 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             const bool row_live = row < live;
 #pragma unroll
             for (int i = 0; i < NB; ++i) b[i] = -INFINITY;
-            thr = row_live ? -INFINITY : INFINITY;
+            thr = row_live ? -FLT_MAX : INFINITY;
             m2 = -INFINITY;
             zsum = 0.f;
             ptr = first;
             const int lead = lead_of(steps, KCAP > 8), again = lead > 2 ? lead : 0;      // units ahead, and how many of them come again
             int next = lead + (lead + 1) / 2, turn = 0;
+            // Where the threshold is final from the start, a thread with k groups that reach it wants no more that only equal
+            // it: looked at once, when some thread of the warp first has that many (a token whose logits are all equal, as of
+            // padding, would overflow its list again and again: T = 4096, M = 16384 450 us against 42).
+            uint64_t limit = lead == steps ? first + max(p.k, 8) * kEntry : warn;
+            auto full = [&]() {
+                if (limit < warn && ptr > limit) thr = fmaxf(thr, just_above(lds(s_thr)));
+                if (__any_sync(kFull, ptr > warn)) compact();
+                limit = warn;
+            };
             // maxima of 16 columns' groups of four; what lies beyond M is nothing (M is a multiple of 8)
             auto group_max = [&](auto masked, const float (&v)[16], int col, float (&t)[4]) {
 #pragma unroll
@@ -747,13 +763,13 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                         }
                         zsum += (a0 + a1) + (a2 + a3);
                     }
-                    if (__any_sync(kFull, m > thr)) {
-                        // (a bucket matters only once it beats the threshold, so it need not be kept up elsewhere)
+                    if (__any_sync(kFull, m >= thr)) {
+                        // (a bucket matters only once it reaches the threshold, so it need not be kept up elsewhere)
                         bucket(h, t);
                         append4(ptr, thr, t, v, col, one);
                     }
                 }
-                if (__any_sync(kFull, ptr > warn)) compact();
+                if (__builtin_expect(__any_sync(kFull, ptr > limit), 0)) full();
                 ++n;
             };
             if (!warp_live) {
@@ -779,7 +795,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 }
                 if (whole < steps) unit(std::true_type{}, steps - 1);
             }
-            // ---- end of the segment: what still beats the threshold goes to scratch
+            // ---- end of the segment: what still reaches the threshold goes to scratch
             if (warp_live) {
                 const bool final = lead == steps;                    // (the threshold is that of all units already)
                 if (!final) publish();
@@ -787,14 +803,14 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 if (LSE && sub > 0)
                     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(s_mz + (sub - 1) * (kRows * 8)), "f"(m2), "f"(zsum) : "memory");
                 quarter_sync(q);
-                if (!final) thr = fmaxf(thr, compute_thr());
+                const float low = fmaxf(final ? lds(s_thr) : compute_thr(), -FLT_MAX);
                 const int seg = (int)blockIdx.x - owner_of((long long)blk * nsteps, p.total, g);
                 const size_t slot = (size_t)blk * p.maxseg + seg;
                 uint2* dst = p.ent + (slot * kRows + row) * p.cap;
-                if (row_live) emit(dst, just_below(thr), 0);
+                if (row_live) emit(dst, low, p.k, true);
                 quarter_sync(q);
                 int total = __float_as_int(lds(s_cnt));
-                if (__any_sync(kFull, total > p.cap)) {              // (the same in all four warps)
+                if (__builtin_expect(__any_sync(kFull, total > p.cap), 0)) {              // (the same in all four warps)
                     // more than the scratch holds: the threads of such a token pass on their own k best each
                     quarter_sync(q);
                     if (sub == 0 && total > p.cap) sts(s_cnt, 0.f);
@@ -802,7 +818,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     if (row_live && total > p.cap) {
                         int equal;
                         const float low = own_kth(equal);
-                        emit(dst, low, equal);
+                        emit(dst, low, equal, false);
                     }
                     quarter_sync(q);
                     total = __float_as_int(lds(s_cnt));
@@ -1107,7 +1123,7 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     __shared__ float2 smz[kWarps];
     __shared__ Cand keep[kKeep];
     __shared__ Cand buf[64];
-    __shared__ int s_count, s_nseg;
+    __shared__ int s_count, s_nseg, s_last;
     __shared__ float s_thr;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tok = blockIdx.x;
     const int blk = tok / kRows, row = tok % kRows;
@@ -1190,7 +1206,47 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
         }
     }
     __syncthreads();
-    const int n = s_count;
+    int n = s_count;
+    if (__builtin_expect(n > kKeep, 0)) {
+        // More near the top than the buffer holds: many logits that equal the bound, of which those with the smallest ids
+        // count.  The k-th smallest of the 64 groups' smallest ids bounds the k-th smallest of them; collected again with it.
+        auto each = [&](auto what) {
+            const uint2* e = my_ent;
+#pragma unroll 1
+            for (int s = half; s < nseg; s += kManyThreads / 16, e += next_ent) {
+                const int count = p.cnt[slot0 + (size_t)s * kRows];
+#pragma unroll 1
+                for (int i = hl; i < count; i += 16) {
+                    const Cand x = load_cand(e + (i - hl));
+                    if (x.v >= thr && x.v > -INFINITY) what(x);
+                }
+            }
+        };
+        int least = INT_MAX;
+        each([&](Cand x) { if (x.v == thr) least = min(least, x.id); });
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) least = min(least, __shfl_xor_sync(kFull, least, o));
+        int* const ids = reinterpret_cast<int*>(maxima);
+        if ((lane & 7) == 0) ids[warp * 4 + (lane >> 3)] = least;
+        __syncthreads();                                      // (also: everyone has read s_count)
+        if (threadIdx.x == 0) s_count = 0;
+        if (threadIdx.x < 64) {
+            const int mine = ids[threadIdx.x];
+            int rank = 0;
+            for (int j = 0; j < 64; ++j) rank += (ids[j] < mine) | ((ids[j] == mine) & (j < (int)threadIdx.x));
+            if (rank == p.k - 1) s_last = mine;
+        }
+        __syncthreads();
+        const int last = s_last;
+        each([&](Cand x) {
+            if (x.v > thr || x.id <= last) {
+                const int at = atomicAdd(&s_count, 1);
+                if (at < kKeep) keep[at] = x;
+            }
+        });
+        __syncthreads();
+        n = s_count;
+    }
     if (n <= kKeep) {
         for (int i = threadIdx.x; i < n; i += kManyThreads) {
             const Cand e = keep[i];

@@ -56,8 +56,7 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
     }
     const float thr = __shfl_sync(kAll, warp_sort_down(m, lane), k - 1);
     int count = 0;
-    auto take = [&](Cand x) {
-        const bool in = x.v >= thr && x.v > -INFINITY;
+    auto take = [&](Cand x, bool in) {
         const unsigned who = __ballot_sync(kAll, in);
         const int at = count + __popc(who & ((1u << lane) - 1u));
         if (in && at < 64) buf[at] = x;
@@ -66,13 +65,32 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
     if (held) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-            if (32 * r < n) take(c[r]);
+            if (32 * r < n) take(c[r], c[r].v >= thr && c[r].v > -INFINITY);
     } else {
-        for (int f = lane; f - lane < n; f += 32) take(f < n ? get(f) : no_cand());
+        for (int f = lane; f - lane < n; f += 32) {
+            const Cand x = f < n ? get(f) : no_cand();
+            take(x, x.v >= thr && x.v > -INFINITY);
+        }
+    }
+    if (__builtin_expect(count > 64, 0)) {
+        // More than the buffer holds: many logits that equal thr, of which those with the smallest ids count.  The k-th
+        // smallest of the 32 lanes' smallest ids bounds the k-th smallest of them; collected again with that.
+        float least = -INFINITY;
+        for (int f = lane; f < n; f += 32) {
+            const Cand x = get(f);
+            if (x.v == thr) least = fmaxf(least, -(float)x.id);
+        }
+        const float last = -__shfl_sync(kAll, warp_sort_down(least, lane), k - 1);
+        __syncwarp();
+        count = 0;
+        for (int f = lane; f - lane < n; f += 32) {
+            const Cand x = f < n ? get(f) : no_cand();
+            take(x, x.v > thr || (x.v == thr && x.v > -INFINITY && (float)x.id <= last));
+        }
     }
     __syncwarp();
     Cand best = no_cand();
-    if (count <= 64) {
+    if (__builtin_expect(count <= 64, 1)) {
         // Ranks by the logits alone, and by the ids as well only if the ranks' sum shows that two logits were equal.
         Cand mine[2];
         int rank[2], sum = 0;
@@ -107,12 +125,12 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
         if (lane < k && lane < count) best = buf[lane];
     } else {
         // more near the top than the buffer holds (many equal logits): k rounds of a maximum
-        Cand last{INFINITY, -1};
+        Cand before{INFINITY, -1};
         for (int r = 0; r < k; ++r) {
             Cand top = no_cand();
             for (int f = lane; f < n; f += 32) {
                 const Cand x = get(f);
-                if (x.v > -INFINITY && ahead(last, x) && ahead(x, top)) top = x;
+                if (x.v > -INFINITY && ahead(before, x) && ahead(x, top)) top = x;
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -120,7 +138,7 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
                 if (ahead(x, top)) top = x;
             }
             if (lane == r) best = top;
-            last = top;
+            before = top;
         }
     }
     __syncwarp();

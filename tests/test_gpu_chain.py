@@ -91,3 +91,14 @@ def test_long_segments(k, gate_mode):
     """More than 32 units per segment: the leading units are computed twice, the threshold rises on the way."""
     case = inputs.gaussian_case(4800, 64, 16, 36008, k, gate_mode, seed=17)
     _route_and_check(case, np.concatenate([np.arange(40), np.arange(2400, 2440), np.arange(4760, 4800)]))
+
+
+@pytest.mark.parametrize("T,M,k", [(3, 256, 16), (40, 16384, 8), (300, 65536, 16), (3000, 4096, 8), (4100, 8192, 16), (4800, 36008, 8)])
+def test_tokens_of_zeros(T, M, k):
+    """Padding: every third token is zero, so all its logits are equal; the others are as ever."""
+    case = inputs.gaussian_case(T, 512, 16, M, k, 1, seed=19)
+    case.X[::3] = 0
+    _route_and_check(case, None if T < 1000 else np.arange(T - 64, T))
+    import torch
+    res = mr.route(*to_device(case), k, 1)
+    assert bool((res.idx[::3] == torch.arange(k, device="cuda", dtype=torch.int32)).all())
