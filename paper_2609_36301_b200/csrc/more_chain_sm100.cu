@@ -665,12 +665,25 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             ptr = first;
             const int lead = lead_of(steps, KCAP > 8), again = lead > 2 ? lead : 0;      // units ahead, and how many of them come again
             int next = lead + (lead + 1) / 2, turn = 0;
-            // Where the threshold is final from the start, a thread with k groups that reach it wants no more that only equal
-            // it: looked at once, when some thread of the warp first has that many (a token whose logits are all equal, as of
-            // padding, would overflow its list again and again: T = 4096, M = 16384 450 us against 42).
-            uint64_t limit = lead == steps ? first + max(p.k, 8) * kEntry : warn;
+            // A token whose logits are all equal (padding) would overflow its list again and again.  So, once, when some thread
+            // of the warp first has more than `limit` groups: where the threshold is final from the start, those k reach it
+            // and later ones that only equal it lose to them; elsewhere, if the first and the last group have the same
+            // maximum, the same holds for the smallest maximum in the list.  (All tokens zero: T = 4096, M = 16384 450 us
+            // -> 74, M = 65536 466 -> 135.)
+            uint64_t limit = first + (lead == steps ? max(p.k, 8) : max(p.k + 8, 16)) * kEntry;
             auto full = [&]() {
-                if (limit < warn && ptr > limit) thr = fmaxf(thr, just_above(lds(s_thr)));
+                if (limit < warn && ptr > limit) {
+                    if (lead == steps) {
+                        thr = fmaxf(thr, just_above(lds(s_thr)));
+                    } else {
+                        auto top = [&](uint64_t o) { const float4 e = ent4(o); return fmaxf(max3(e.x, e.y, e.z), e.w); };
+                        float least = top(first);
+                        if (least == top(ptr - kEntry)) {
+                            for (uint64_t o = first + kEntry; o < ptr; o += kEntry) least = fminf(least, top(o));
+                            thr = fmaxf(thr, just_above(least));
+                        }
+                    }
+                }
                 if (__any_sync(kFull, ptr > warn)) compact();
                 limit = warn;
             };
