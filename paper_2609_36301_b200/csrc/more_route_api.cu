@@ -204,7 +204,9 @@ bool chain_wins(int T, int h, int r, int M, int k, bool lse, int sm_count)
     if (M < 2048) return per_sm <= 90;
     if (k > 8) return per_sm <= 230 || M >= 16384 || (M >= 4096 && r <= 32);
     if (k <= 4) return M >= 8192 || per_sm <= 230;
-    if (M < 16384) return per_sm <= (M < 4096 ? 140 : 170);
+    if (M < 4096) return per_sm <= 140;
+    if (M < 8192) return per_sm <= (lse ? 170 : 230);
+    if (M < 16384) return per_sm <= 170;
     // a few segments of 33 to 64 units per CTA are the longest that are not swept twice (T = 16 k, M = 16 k: 0.94 to 1.02)
     if (M < 32768 && per_sm > 100 && per_sm <= 120) return false;
     // many tokens: the paired kernel, with two accumulators per token group at r <= 32, ties or wins unless it is slowed by
