@@ -679,6 +679,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                         auto top = [&](uint64_t o) { const float4 e = ent4(o); return fmaxf(max3(e.x, e.y, e.z), e.w); };
                         float least = top(first);
                         if (least == top(ptr - kEntry)) {
+#pragma unroll 1
                             for (uint64_t o = first + kEntry; o < ptr; o += kEntry) least = fminf(least, top(o));
                             thr = fmaxf(thr, just_above(least));
                         }
@@ -1129,9 +1130,56 @@ __global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
 constexpr int kManyThreads = 512;
 constexpr int kManyPer = 10;                       // segments per half warp
 constexpr int kManySegs = kManyPer * (kManyThreads / 16);
+// More near the top than `keep` holds: many logits that equal the bound, of which those with the smallest ids count.  The k-th
+// smallest of the 64 groups' smallest ids bounds the k-th smallest of them; collected again with it.  Returns how many.  (Not
+// inlined: in the kernel's way it costs every call 0.5 us of instruction fetches.)
+constexpr int kKeep = 512;
+__device__ __noinline__ int collect_equals(const int* cnt, const uint2* ent, size_t next_ent, int nseg, int k, float thr, int* ids,
+                                           Cand* keep, int* count, int* bound)
+{
+    const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
+    auto each = [&](auto what) {
+        const uint2* e = ent;
+        const int* c = cnt;
+#pragma unroll 1
+        for (int s = half; s < nseg; s += kManyThreads / 16, e += next_ent, c += kManyThreads / 16 * kRows) {
+            const int n = *c;
+#pragma unroll 1
+            for (int i = hl; i < n; i += 16) {
+                const Cand x = load_cand(e + (i - hl));
+                if (x.v >= thr && x.v > -INFINITY) what(x);
+            }
+        }
+    };
+    int least = INT_MAX;
+    each([&](Cand x) { if (x.v == thr) least = min(least, x.id); });
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) least = min(least, __shfl_xor_sync(kFull, least, o));
+    if ((threadIdx.x & 7) == 0) ids[threadIdx.x >> 3] = least;
+    __syncthreads();                                          // (also: everyone has read the count)
+    if (threadIdx.x == 0) *count = 0;
+    if (threadIdx.x < 64) {
+        const int mine = ids[threadIdx.x];
+        int rank = 0;
+#pragma unroll 1
+        for (int j = 0; j < 64; ++j) rank += (ids[j] < mine) | ((ids[j] == mine) & (j < (int)threadIdx.x));
+        if (rank == k - 1) *bound = mine;
+    }
+    __syncthreads();
+    const int last = *bound;
+    each([&](Cand x) {
+        if (x.v > thr || x.id <= last) {
+            const int at = atomicAdd(count, 1);
+            if (at < kKeep) keep[at] = x;
+        }
+    });
+    __syncthreads();
+    return *count;
+}
+
 __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishParams p)
 {
-    constexpr int kWarps = kManyThreads / 32, kKeep = 512;
+    constexpr int kWarps = kManyThreads / 32;
     __shared__ __align__(16) float maxima[64];
     __shared__ float2 smz[kWarps];
     __shared__ Cand keep[kKeep];
@@ -1221,44 +1269,8 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     __syncthreads();
     int n = s_count;
     if (__builtin_expect(n > kKeep, 0)) {
-        // More near the top than the buffer holds: many logits that equal the bound, of which those with the smallest ids
-        // count.  The k-th smallest of the 64 groups' smallest ids bounds the k-th smallest of them; collected again with it.
-        auto each = [&](auto what) {
-            const uint2* e = my_ent;
-#pragma unroll 1
-            for (int s = half; s < nseg; s += kManyThreads / 16, e += next_ent) {
-                const int count = p.cnt[slot0 + (size_t)s * kRows];
-#pragma unroll 1
-                for (int i = hl; i < count; i += 16) {
-                    const Cand x = load_cand(e + (i - hl));
-                    if (x.v >= thr && x.v > -INFINITY) what(x);
-                }
-            }
-        };
-        int least = INT_MAX;
-        each([&](Cand x) { if (x.v == thr) least = min(least, x.id); });
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) least = min(least, __shfl_xor_sync(kFull, least, o));
-        int* const ids = reinterpret_cast<int*>(maxima);
-        if ((lane & 7) == 0) ids[warp * 4 + (lane >> 3)] = least;
-        __syncthreads();                                      // (also: everyone has read s_count)
-        if (threadIdx.x == 0) s_count = 0;
-        if (threadIdx.x < 64) {
-            const int mine = ids[threadIdx.x];
-            int rank = 0;
-            for (int j = 0; j < 64; ++j) rank += (ids[j] < mine) | ((ids[j] == mine) & (j < (int)threadIdx.x));
-            if (rank == p.k - 1) s_last = mine;
-        }
-        __syncthreads();
-        const int last = s_last;
-        each([&](Cand x) {
-            if (x.v > thr || x.id <= last) {
-                const int at = atomicAdd(&s_count, 1);
-                if (at < kKeep) keep[at] = x;
-            }
-        });
-        __syncthreads();
-        n = s_count;
+        n = collect_equals(p.cnt + slot0 + (size_t)half * kRows, my_ent, next_ent, nseg, p.k, thr, reinterpret_cast<int*>(maxima), keep,
+                           &s_count, &s_last);
     }
     if (n <= kKeep) {
         for (int i = threadIdx.x; i < n; i += kManyThreads) {

@@ -76,6 +76,7 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
         // More than the buffer holds: many logits that equal thr, of which those with the smallest ids count.  The k-th
         // smallest of the 32 lanes' smallest ids bounds the k-th smallest of them; collected again with that.
         float least = -INFINITY;
+#pragma unroll 1
         for (int f = lane; f < n; f += 32) {
             const Cand x = get(f);
             if (x.v == thr) least = fmaxf(least, -(float)x.id);
@@ -83,6 +84,7 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
         const float last = -__shfl_sync(kAll, warp_sort_down(least, lane), k - 1);
         __syncwarp();
         count = 0;
+#pragma unroll 1
         for (int f = lane; f - lane < n; f += 32) {
             const Cand x = f < n ? get(f) : no_cand();
             take(x, x.v > thr || (x.v == thr && x.v > -INFINITY && (float)x.id <= last));
@@ -126,8 +128,10 @@ __device__ __forceinline__ Cand warp_topk(int n, int k, Get get, Cand* buf, int 
     } else {
         // more near the top than the buffer holds (many equal logits): k rounds of a maximum
         Cand before{INFINITY, -1};
+#pragma unroll 1
         for (int r = 0; r < k; ++r) {
             Cand top = no_cand();
+#pragma unroll 1
             for (int f = lane; f < n; f += 32) {
                 const Cand x = get(f);
                 if (x.v > -INFINITY && ahead(before, x) && ahead(x, top)) top = x;
