@@ -71,6 +71,8 @@ def lib() -> ctypes.CDLL:
         L.more_debug_expire_wait.restype = i32
         L.more_debug_scratch_guard.argtypes = [vp]
         L.more_debug_scratch_guard.restype = i32
+        L.more_debug_scratch_bytes.argtypes = [i32] * 9
+        L.more_debug_scratch_bytes.restype = ctypes.c_longlong
         L.more_strerror.argtypes = [i32]
         L.more_strerror.restype = ctypes.c_char_p
         L.more_version.argtypes = []
@@ -247,6 +249,14 @@ def debug_expire_wait(budget_cycles: int, stream=None) -> int:
 def debug_scratch_guard(stream=None) -> int:
     """Diagnostic: 1 if the guard region behind the library's scratch allocation is intact, 0 if it was written to."""
     return int(lib().more_debug_scratch_guard(_stream(stream)))
+
+
+def debug_scratch_bytes(T, h, r, M, k, gate_mode=0, want_lse=False, path=PATH_AUTO, msplit=0) -> int:
+    """Diagnostic: bytes of device memory that a routing call of this shape makes the library's scratch hold."""
+    n = int(lib().more_debug_scratch_bytes(T, h, r, M, k, gate_mode, int(want_lse), path, msplit))
+    if n < 0:
+        raise MoreRouteError(n, "more_debug_scratch_bytes")
+    return n
 
 
 @dataclass

@@ -242,7 +242,7 @@ constexpr int W = 128;                             // experts of a unit
 constexpr int kCols = W / 4;                       // columns of a thread
 constexpr int kMaxStages = 8;
 constexpr int kListCap = 64;                       // entries of a thread's list
-constexpr uint32_t kEntry = kEpi * 32;             // bytes between its entries (32 bytes each: four logits, the first one's column)
+constexpr uint32_t kEntry = kRows * 32;            // bytes between its entries (32 bytes each: four logits, the first one's column)
 
 // Units whose bucket maxima are formed ahead of a segment of `steps` units.  All of a short one: its threshold is then the
 // final one before the first candidate is kept, and a thread keeps one or two groups instead of the ten that a rising
@@ -264,7 +264,8 @@ struct SweepParams {
     int maxseg, cap;                               // candidate lists per token block in scratch, entries per list and token
     int nst, st_bytes, zbufs, z_bytes;
     int off_r2, off_pub, off_ctl;
-    uint8_t* list;                                 // [CTA][kListCap][512] x 32 bytes
+    int list_quarters, list_cap;
+    uint8_t* list;                                 // [CTA][list_quarters][list_cap][128 = column quarter x lane] x 32 bytes
     uint2* ent;                                    // [block][seg][128][cap] (logit bits, expert id)
     int* cnt;                                      // [block][seg][128]
     float2* mz;                                    // [block][seg][128] (max in log2 units, sum); LSE only
@@ -498,7 +499,10 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         const int M = p.M, nsteps = p.nsteps;
         const uint32_t t_col = tmem_base + ((uint32_t)(q * 32) << 16) + sub * kCols;
         // the thread's list; a unit adds at most 8 entries between two looks at its length
-        const uint64_t first = reinterpret_cast<uint64_t>(p.list) + (uint64_t)blockIdx.x * (kListCap * kEntry) + (threadIdx.x - 64) * 32;
+        // (a list shorter than kListCap is one that so few units cannot fill; quarters without tokens have none, and their
+        // warps touch none)
+        const uint64_t first = reinterpret_cast<uint64_t>(p.list) +
+                               (uint64_t)(blockIdx.x * p.list_quarters + q) * (uint32_t)(p.list_cap * kEntry) + (sub * 32 + lane) * 32;
         const uint64_t warn = first + (kListCap - kCols / 4) * kEntry;
         // shared memory: published buckets [sub][128][NB], thresholds [128], counters [128], (m, Z) [sub - 1][128]
         const uint32_t pub0 = base + p.off_pub + row * (NB * 4);
@@ -1363,23 +1367,25 @@ cudaError_t launch(void (*kern)(Args...), int grid, int block, int smem, cudaStr
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 constexpr int kChunkTokens = 131072;               // tokens per pass: bounds the scratch, whatever T is
+long long resident_ctas(int sm_count) { return 2 * sm_count < kManySegs - 2 ? 2 * sm_count : kManySegs - 2; }
 
 struct Layout {
     size_t z, list, ent, cnt, mz, total;
 };
 
+// The largest there is (T >= 131072, k = 16, r > 32): 32 MiB of z, 296 MiB of lists, 130 MiB of candidates and counts.
 Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
 {
     Layout L{};
     const size_t tokens = (size_t)(a.T < kChunkTokens ? a.T : kChunkTokens);
-    const size_t blocks = (tokens + kRows - 1) / kRows;
+    const size_t blocks = (tokens + kRows - 1) / kRows, lists = (size_t)p.sweep_blocks * p.maxseg;
     size_t off = 0;
     L.z = off; off += align_up(blocks * kRows * (a.r <= 32 ? 128 : 256), 1024);
-    L.list = off; off += (size_t)p.parts * kListCap * kEntry;
-    L.ent = off; off += align_up(blocks * p.maxseg * (size_t)(4 * a.k) * kRows * 8, 1024);
-    L.cnt = off; off += align_up(blocks * p.maxseg * kRows * 4, 1024);
+    L.list = off; off += (size_t)p.parts * p.list_quarters * p.list_cap * kEntry;
+    L.ent = off; off += align_up(lists * (size_t)(4 * a.k) * kRows * 8, 1024);
+    L.cnt = off; off += align_up(lists * kRows * 4, 1024);
     L.mz = off;
-    if (lse) off += align_up(blocks * p.maxseg * kRows * 8, 1024);
+    if (lse) off += align_up(lists * kRows * 8, 1024);
     L.total = off;
     return L;
 }
@@ -1390,14 +1396,15 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
 // either equal ones wherever these begin (stretches of several token blocks are then cut into segments), or an equal share
 // of one block each.  The second leaves some SMs idle but every CTA with one segment; what a segment costs on its own (its
 // first MMAs, the threshold to start with, the pass through the lists at its end) is worth about eight units.  A forced
-// split of s CTAs per token block is the second with that s.
+// split of s CTAs per token block is the second with that s, in as many launches as it takes for no launch to have more
+// CTAs than are resident at once: each has lists of its own, up to 1 MiB (T = 131072, s = 64 in one launch: 64 GiB).
 void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
 {
     const long long blocks = ((T < kChunkTokens ? T : kChunkTokens) + kRows - 1) / kRows;
     const long long nsteps = (M + W - 1) / W, total = blocks * nsteps;
-    const long long slots = 2 * sm_count < kManySegs - 2 ? 2 * sm_count : kManySegs - 2;
+    const long long slots = resident_ctas(sm_count);
     const double kSegment = 8.0;
-    long long g = total < slots ? total : slots, share = 0;
+    long long g = total < slots ? total : slots, share = 0, sweep_blocks = blocks;
     if (msplit > 0) {
         const int most = M / 256 > 1 ? M / 256 : 1;
         share = msplit < most ? msplit : most;
@@ -1408,14 +1415,20 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
         if (blocks == 1 || whole <= cut) share = s;
     }
     if (share > 0) {
-        g = blocks * share;
+        if (blocks * share > slots) sweep_blocks = slots / share > 1 ? slots / share : 1;
+        g = sweep_blocks * share;
         p->maxseg = (int)share;
     } else {
         p->maxseg = (int)(g / blocks) + 2;
     }
     p->parts = (int)g;
+    p->sweep_blocks = (int)sweep_blocks;
+    p->list_quarters = T < kRows ? (T + 31) / 32 : kRows / 32;
+    // a unit adds at most kCols / 4 entries to a list (a later, shorter chunk may have longer segments)
+    const long long units = share > 0 ? (nsteps + share - 1) / share : (total + g - 1) / g;
+    p->list_cap = T <= kChunkTokens && units < kListCap / (kCols / 4) ? (int)units * (kCols / 4) : kListCap;
     // reported: CTAs; where a token block is split, the two CTAs of an SM count as one
-    p->ctas = (int)(blocks < sm_count && g > sm_count && msplit <= 0 ? sm_count : g);
+    p->ctas = (int)(share > 0 && msplit > 0 ? blocks * share : (blocks < sm_count && g > sm_count ? sm_count : g));
     p->msplit = msplit > 0 ? (int)share : (int)(p->ctas / blocks > 1 ? p->ctas / blocks : 1);
     p->share = (int)share;
     p->chain = true;
@@ -1454,6 +1467,7 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
     sp.off_ctl = sp.off_pub + pub;
     const int smem = sp.off_ctl + ctl + 1024;
     sp.list = reinterpret_cast<uint8_t*>(base + L.list);
+    sp.list_quarters = plan.list_quarters; sp.list_cap = plan.list_cap;
     sp.ent = reinterpret_cast<uint2*>(base + L.ent);
     sp.cnt = reinterpret_cast<int*>(base + L.cnt);
     sp.mz = lse ? reinterpret_cast<float2*>(base + L.mz) : nullptr;
@@ -1489,41 +1503,45 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
         const int psmem = psmem_max - (pp.cs == 1 ? kPExchange : 0);
         if (launch(project_kernel, blocks * pp.cs, kPThreads, psmem, a.stream, true, pp.cs, mx, mr1, pp) != cudaSuccess)
             return MORE_ERR_CUDA;
+        count_launch(1);
 
-        sp.T = T;
-        sp.total = (long long)blocks * nsteps;
-        int g = plan.parts;
-        if (a.T > kChunkTokens) {                            // (the last chunk of a long call may be shorter)
-            if (plan.share > 0) {
-                g = blocks * plan.share;
-            } else {
-                const long long most = (long long)(plan.maxseg - 1) * blocks - 1;      // floor(g / blocks) + 2 <= maxseg
+        const int step = plan.share > 0 && plan.sweep_blocks < blocks ? plan.sweep_blocks : blocks;      // blocks per sweep
+        for (int b0 = 0; b0 < blocks; b0 += step) {
+            const int nblk = blocks - b0 < step ? blocks - b0 : step, first = t0 + b0 * kRows;
+            const int tokens = T - b0 * kRows < nblk * kRows ? T - b0 * kRows : nblk * kRows;
+            if (b0 > 0) rc = get_tensor_map(base + L.z + (size_t)b0 * kRows * zc * 2, nblk * kRows, zc, kRows, 64, &mz);
+            if (rc != MORE_OK) return rc;
+            sp.T = tokens;
+            sp.total = (long long)nblk * nsteps;
+            int g = plan.share > 0 ? nblk * plan.share : plan.parts;
+            if (plan.share == 0 && a.T > kChunkTokens) {     // (the last chunk of a long call may be shorter)
+                const long long most = (long long)(plan.maxseg - 1) * blocks - 1;  // floor(g / blocks) + 2 <= maxseg
                 if (g > sp.total) g = (int)sp.total;
                 if (g > most) g = (int)(most > 1 ? most : 1);
             }
-        }
-        if (launch(sweep, g, kSThreads, smem, a.stream, true, 1, mz, mr2, sp) != cudaSuccess) return MORE_ERR_CUDA;
+            if (launch(sweep, g, kSThreads, smem, a.stream, true, 1, mz, mr2, sp) != cudaSuccess) return MORE_ERR_CUDA;
 
-        FinishParams fp{};
-        fp.T = T; fp.M = a.M; fp.k = a.k; fp.gate_mode = a.gate_mode;
-        fp.nsteps = nsteps; fp.g = g; fp.share = plan.share; fp.maxseg = plan.maxseg; fp.cap = sp.cap; fp.total = sp.total;
-        fp.ent = sp.ent; fp.cnt = sp.cnt; fp.mz = sp.mz;
-        const size_t ro = (size_t)t0 * a.k;
-        fp.out_idx = a.out_idx + ro; fp.out_gate = a.out_gate + ro; fp.out_counts = a.out_counts;
-        fp.out_topval = a.out_topval ? a.out_topval + ro : nullptr;
-        fp.out_lse = a.out_lse ? a.out_lse + t0 : nullptr;
-        cudaError_t e;
-        // Eight threads per token rank up to two short lists by counting everything against everything; where there is
-        // more, the threshold of a warp's selection saves more than its 32 lanes per token cost (k = 16: T = 17000,
-        // M = 8192 121 -> 88 us, T = 32768, M = 4096 174 -> 114; k = 8 with two lists each, T = 17000, M = 4096 54 -> 51).
-        if (a.k <= 8 && plan.maxseg <= (plan.share > 0 ? 1 : kFewSegs))
-            e = launch(finish_few_kernel, (T + 31) / 32, 256, 0, a.stream, true, 1, fp);
-        else if (plan.maxseg <= kWarpSegs)
-            e = launch(finish_warp_kernel, (T + 7) / 8, 256, 0, a.stream, true, 1, fp);
-        else
-            e = launch(finish_many_kernel, T, kManyThreads, 0, a.stream, true, 1, fp);
-        if (e != cudaSuccess) return MORE_ERR_CUDA;
-        count_launch(3);
+            FinishParams fp{};
+            fp.T = tokens; fp.M = a.M; fp.k = a.k; fp.gate_mode = a.gate_mode;
+            fp.nsteps = nsteps; fp.g = g; fp.share = plan.share; fp.maxseg = plan.maxseg; fp.cap = sp.cap; fp.total = sp.total;
+            fp.ent = sp.ent; fp.cnt = sp.cnt; fp.mz = sp.mz;
+            const size_t ro = (size_t)first * a.k;
+            fp.out_idx = a.out_idx + ro; fp.out_gate = a.out_gate + ro; fp.out_counts = a.out_counts;
+            fp.out_topval = a.out_topval ? a.out_topval + ro : nullptr;
+            fp.out_lse = a.out_lse ? a.out_lse + first : nullptr;
+            cudaError_t e;
+            // Eight threads per token rank up to two short lists by counting everything against everything; where there is
+            // more, the threshold of a warp's selection saves more than its 32 lanes per token cost (k = 16: T = 17000,
+            // M = 8192 121 -> 88 us, T = 32768, M = 4096 174 -> 114; k = 8 with two lists each, T = 17000, M = 4096 54 -> 51).
+            if (a.k <= 8 && plan.maxseg <= (plan.share > 0 ? 1 : kFewSegs))
+                e = launch(finish_few_kernel, (tokens + 31) / 32, 256, 0, a.stream, true, 1, fp);
+            else if (plan.maxseg <= kWarpSegs)
+                e = launch(finish_warp_kernel, (tokens + 7) / 8, 256, 0, a.stream, true, 1, fp);
+            else
+                e = launch(finish_many_kernel, tokens, kManyThreads, 0, a.stream, true, 1, fp);
+            if (e != cudaSuccess) return MORE_ERR_CUDA;
+            count_launch(2);
+        }
     }
     return MORE_OK;
 }

@@ -32,6 +32,12 @@ int more_debug_expire_wait(long long budget_cycles, void* stream);
  */
 int more_debug_scratch_guard(void* stream);
 
+/*
+ * more_debug_scratch_bytes -- device memory, in bytes, that more_route_ex with these arguments makes the library's cached
+ * scratch allocation hold (the plan for 148 SMs), or a negative MORE_ERR_* code.  Host-only; needs no device.
+ */
+long long more_debug_scratch_bytes(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int path, int msplit);
+
 #ifdef __cplusplus
 }
 #endif

@@ -57,7 +57,10 @@ struct Plan {
     bool chain = false;    // low-rank router: projection, sweep and finish as three kernels
     int parts = 1;         // ... CTAs of its sweep,
     int share = 0;         // ... how many of them share one token block each, or 0 where their parts begin anywhere,
-    int maxseg = 1;        // ... and the most that can share one
+    int maxseg = 1;        // ... and the most that can share one;
+    int sweep_blocks = 1;  // ... token blocks per launch of the sweep;
+    int list_quarters = 4; // ... lists of a CTA: 32-token quarters of its blocks that hold tokens,
+    int list_cap = 1;      // ... and entries per thread
 };
 
 bool tcgen05_shape_ok(int T, int h, int r, int M, int k);

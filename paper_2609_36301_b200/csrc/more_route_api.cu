@@ -105,6 +105,14 @@ int check_shape(int T, int h, int r, int M, int k, int gate_mode, int path)
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
+size_t scratch_bytes(const RouteArgs& a, const Plan& plan)
+{
+    if (plan.path != MORE_PATH_TCGEN05) return generic_scratch_bytes(a);
+    if (a.full) return full_scratch_bytes(a, plan);
+    if (plan.chain) return chain_scratch_bytes(a, plan);
+    return plan.paired ? paired_scratch_bytes(a, plan) : lowrank_scratch_bytes(a, plan);
+}
+
 // The body of every routing entry point.  The caller holds g_mutex.
 int route_device_locked(const RouteArgs& a, int path, int msplit)
 {
@@ -156,12 +164,7 @@ int route_device_locked(const RouteArgs& a, int path, int msplit)
             if (used < kPlanCache) ++used;
         }
     }
-    const size_t need = plan.path != MORE_PATH_TCGEN05
-                            ? generic_scratch_bytes(a)
-                            : (a.full ? full_scratch_bytes(a, plan)
-                                      : (plan.chain ? chain_scratch_bytes(a, plan)
-                                                    : (plan.paired ? paired_scratch_bytes(a, plan) : lowrank_scratch_bytes(a, plan))));
-    rc = ensure_scratch(ctx, need, a.stream);
+    rc = ensure_scratch(ctx, scratch_bytes(a, plan), a.stream);
     if (rc != MORE_OK) return rc;
     if (a.T == 0 || plan.path != MORE_PATH_TCGEN05) {
         // (the tensor-core launchers clear out_counts themselves, after their last step that can fail)
@@ -645,6 +648,19 @@ int more_debug_scratch_guard(void* stream)
     for (size_t i = 0; i < kGuardBytes; ++i)
         if (host[i] != kGuardPattern) return 0;
     return 1;
+}
+
+long long more_debug_scratch_bytes(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int path, int msplit)
+{
+    int rc = check_shape(T, h, r, M, k, gate_mode, path);
+    if (rc != MORE_OK) return rc;
+    RouteArgs a{};
+    float lse;                                               // (only whether it is asked for counts)
+    a.T = T; a.h = h; a.r = r; a.M = M; a.k = k; a.gate_mode = gate_mode;
+    a.out_lse = want_lse ? &lse : nullptr;
+    Plan p;
+    rc = make_plan(T, h, r, M, k, gate_mode, want_lse != 0 || gate_mode == MORE_GATE_FULL_SOFTMAX, false, path, msplit, 148, &p);
+    return rc == MORE_OK ? (long long)scratch_bytes(a, p) : rc;
 }
 
 const char* more_strerror(int code)

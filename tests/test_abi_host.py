@@ -95,3 +95,25 @@ def test_shared_memory_plan_of_the_grouped_kernel_fits():
                     p = PX(T, 512, r, M - M % 8 if M >= 8 else 8, k)
                     assert p.path == mr.PATH_TCGEN05 and p.ctas >= 1
                     assert p.block_tokens % 32 == 0 and 32 <= p.block_tokens <= 512
+
+
+def test_device_memory_of_a_routing_call_is_bounded():
+    """The sweep's lists are sized for the CTAs that run at once (two per SM, 1 MiB each at most), whatever split of the
+    experts is forced, and for the tokens and experts that a CTA has: T tokens of z, lists, candidates."""
+    B = mr.debug_scratch_bytes
+    MiB = 1 << 20
+
+    def bound(T, r, M, k):
+        blocks = -(-min(T, 131072) // 128)
+        z = blocks * 128 * (128 if r <= 32 else 256)
+        segments = 2 * 148 + 2 * blocks
+        return z + 2 * 148 * MiB + segments * 128 * (4 * k * 8 + 12) + MiB
+
+    for T, M, k in ((131072, 16384, 4), (65536, 65536, 4), (65536, 16384, 16), (4096, 131072, 16), (300000, 32768, 8), (300, 65536, 8)):
+        for msplit in (0, 1, 2, 7, 64):
+            assert B(T, 512, 64, M, k, 1, msplit=msplit) <= bound(T, 64, M, k), (T, M, k, msplit)
+    # largest there is without a forced split
+    assert B(131072, 512, 64, 131072, 16, 1) <= 512 * MiB
+    # few tokens: only the rows that are there, and no longer lists than a CTA's experts can fill
+    assert B(1, 2048, 64, 16384, 8) <= 9 * MiB
+    assert B(64, 4096, 64, 131072, 16) <= 96 * MiB

@@ -86,6 +86,34 @@ def test_more_tokens_than_one_chunk():
     _route_and_check(case, rows, launches=6)
 
 
+@pytest.mark.parametrize("T,M,k,msplit,sweeps", [
+    (9000, 4096, 8, 16, 4),           # 71 token blocks, 18 per sweep
+    (5000, 16384, 12, 64, 10),        # 40 token blocks, 4 per sweep
+    (40000, 8192, 4, 1, 2),           # one CTA per token block, 296 of 313 blocks in the first sweep
+    (131072 + 130, 8192, 4, 3, 12),   # two chunks: 98 token blocks per sweep, then two blocks
+])
+def test_a_forced_split_in_several_sweeps(T, M, k, msplit, sweeps):
+    """More CTAs than are resident at once: as many sweeps as that takes, the same results as without a split."""
+    import torch
+    case = inputs.gaussian_case(T, 64, 8, M, k, 1, seed=T)
+    X, R1, R2 = to_device(case)
+    whole = mr.route(X, R1, R2, k, 1, want_topval=True, want_lse=True)
+    before = mr.launches()
+    res = mr.route(X, R1, R2, k, 1, want_topval=True, want_lse=True, msplit=msplit)
+    assert mr.launches() - before == (2 if T > 131072 else 1) + 2 * sweeps
+    torch.cuda.synchronize()
+    assert mr.more_route_status() == 0 and mr.debug_scratch_guard() == 1
+    for a, b in ((res.idx, whole.idx), (res.topval, whole.topval), (res.counts, whole.counts)):
+        assert torch.equal(a, b)
+    # (the sums of exponentials are added segment by segment: fp32 rounding of a few additions)
+    assert float((res.lse - whole.lse).abs().max()) <= 1e-5
+    np.testing.assert_allclose(res.gate.cpu().numpy(), whole.gate.cpu().numpy(), rtol=2e-5)
+    rows = np.unique(np.concatenate([np.arange(32), np.arange(T // 2, T // 2 + 32), np.arange(T - 32, T)]))
+    sel = torch.from_numpy(rows).cuda()
+    check_rows(case, rows, res.idx[sel].cpu().numpy(), res.gate[sel].cpu().numpy(), res.topval[sel].cpu().numpy(),
+               res.lse[sel].cpu().numpy(), gate_mode=1, k=k)
+
+
 @pytest.mark.parametrize("k,gate_mode", [(8, 1), (12, 0)])
 def test_long_segments(k, gate_mode):
     """More than 32 units per segment: the leading units are computed twice, the threshold rises on the way."""
