@@ -240,14 +240,11 @@ def time_router(mr, torch, bufs, k, gate_mode, steps, warmup, stream):
     return ev0.elapsed_time(ev1) * 1e-3
 
 
-def kernel_of(mr, plan, bufs, k, gate_mode, stream):
-    """Which kernels serve a shape: the chain launches three per call, the others are one kernel each."""
-    X, R1, R2, idx, gate, counts = bufs[0]
-    l0 = mr.launches()
-    mr.more_route(X, R1, R2, k, gate_mode, idx, gate, counts, stream)
+def kernel_of(plan):
+    """Which kernels serve a shape, by its launch plan."""
     if plan.path != 2:
         return "generic_route_tokens"
-    if mr.launches() - l0 > 1:
+    if plan.chain:
         return "project_kernel + sweep_kernel + finish"
     return "route_tcgen05_kernel" if plan.paired else "route_lowrank_kernel"
 
@@ -500,7 +497,7 @@ def main():
     cnt = counters.get(f"{name}/mode{gate_mode}", {})
     plan = mr.more_route_plan_ex(case.T, case.h, case.r, case.M, k, gate_mode)
     roof = roofline(case.T, case.h, case.r, case.M, k, secs / args.steps, peaks, cnt.get("dram_bytes"))
-    roof["kernel"] = kernel_of(mr, plan, bufs, k, gate_mode, stream)
+    roof["kernel"] = kernel_of(plan)
     roof.update(diagnostic_bounds(case.T, case.M, gate_mode, cnt.get("warp_instr_per_chunk"), clocks.get("sm_mhz")))
     roof["traffic_source"] = cnt.get("source")
     line = dict(metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
@@ -521,7 +518,7 @@ def main():
 
     if not args.no_context:
         extra_entry_points(mr, torch, bufs, case, k, gate_mode, stream, peaks, line)
-        # decode-sized batches: 64 tokens, the expert range cut over the SMs and merged by the last CTA to finish
+        # decode-sized batches: 64 tokens, the expert range cut over the SMs
         dec = {}
         for (dh, dr, dM, dk) in ((2048, 64, 16384, 8), (4096, 64, 131072, 16)):
             dcase = inputs.gaussian_case(64, dh, dr, dM, dk, gate_mode, seed=3)
@@ -530,7 +527,7 @@ def main():
             dplan = mr.more_route_plan_ex(64, dh, dr, dM, dk, gate_mode)
             r = roofline(64, dh, dr, dM, dk, dsecs, peaks)
             dec[f"T=64 h={dh} r={dr} M={dM} k={dk}"] = dict(us=dsecs * 1e6, ctas=dplan.ctas, msplit=dplan.msplit,
-                                                            expert_ranges=dplan.expert_ranges, bound=r["bound"],
+                                                            expert_ranges=dplan.expert_ranges, kernel=kernel_of(dplan), bound=r["bound"],
                                                             roofline_frac=r["frac"])
             del dbufs
         line["decode"] = dec
@@ -571,7 +568,7 @@ def main():
                                                     bound=r["bound"], roofline_frac=r["frac"], msplit=oplan.msplit,
                                                     ctas=oplan.ctas, block_tokens=oplan.block_tokens,
                                                     expert_ranges=oplan.expert_ranges,
-                                                    kernel=kernel_of(mr, oplan, obufs, ocase.k, gm, stream),
+                                                    kernel=kernel_of(oplan),
                                                     host_us_per_call=host_us_per_call(mr, torch, obufs, ocase.k, gm, stream, 100),
                                                     **diagnostic_bounds(ocase.T, ocase.M, gm, ocnt.get("warp_instr_per_chunk"),
                                                                         clocks.get("sm_mhz")))

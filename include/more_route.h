@@ -19,10 +19,10 @@
  * Every function returns MORE_OK (0) or a negative MORE_ERR_* code.  On an error detected before launch
  * nothing is launched and no output is touched.  Calls are asynchronous on the given stream unless stated.
  * Buffers are owned by the caller; the library keeps, per device, one cached scratch allocation (grown on
- * demand by cudaMalloc, which may synchronise the device the first time a larger problem is seen) and a
- * small cache of TMA descriptors.  Calls on different host threads are serialised internally; two calls
- * whose kernels may overlap on the GPU (different streams) must not be issued for the same device, because
- * they share that scratch.
+ * demand by cudaMalloc, which may synchronise the device the first time a larger problem is seen; at most 0.5 GB
+ * for the low-rank router's tensor-core path, unless a split of the experts is forced) and a small cache of TMA
+ * descriptors.  Calls on different host threads are serialised internally; two calls whose kernels may overlap
+ * on the GPU (different streams) must not be issued for the same device, because they share that scratch.
  */
 #ifndef MORE_ROUTE_H_
 #define MORE_ROUTE_H_
@@ -92,7 +92,8 @@ int more_route(const void* X, const void* R1, const void* R2,
  *               gate mode when requested (it forces the full-softmax sweep).
  *   path        MORE_PATH_*; a forced path that cannot run the shape gives MORE_ERR_SHAPE.
  *   msplit      tensor-core path only: number of CTAs (at most 64) that share one token block by splitting the expert
- *               range (partial top-k lists and (m, Z) pairs are merged by the last CTA to finish);
+ *               range (partial top-k lists and (m, Z) pairs are merged by the last CTA to finish, or by the finishing
+ *               kernel of the chain); fewer where there are not that many 64- or 128-expert steps;
  *               0 = chosen by the library.  Results do not depend on it.
  */
 int more_route_ex(const void* X, const void* R1, const void* R2,
@@ -224,7 +225,7 @@ int more_dispatch(const int32_t* idx, const int32_t* counts, int T, int k, int M
  * more_route_plan -- report, without launching, what more_route_ex would do for a shape:
  *   *path_out   MORE_PATH_GENERIC or MORE_PATH_TCGEN05
  *   *msplit_out CTAs per token block (1 on the generic path)
- *   *ctas_out   total CTAs of the main kernel
+ *   *ctas_out   total CTAs of the main kernel (the sweep, where the router runs as a chain of kernels)
  * Any of the three may be NULL.  Host-only; needs no device.
  */
 int more_route_plan(int T, int h, int r, int M, int k, int gate_mode, int path, int msplit,
@@ -236,8 +237,12 @@ int more_route_plan(int T, int h, int r, int M, int k, int gate_mode, int path, 
  *   out8[0] path   out8[1] CTAs per token block   out8[2] total CTAs   out8[3] tokens per CTA
  *   out8[4] 128-token groups per CTA   out8[5] expert ranges swept side by side inside a CTA
  *   out8[6] reserved (0)
- *   out8[7] which of the two kernels: 1 = 256-token CTAs, two per SM, 64-expert steps (many tokens per SM);
- *           0 = one CTA per SM holding up to four token groups / expert ranges (few tokens per SM)
+ *   out8[7] which kernels of the tensor-core path: 2 = a chain of three, projection, sweep and finish (most shapes with
+ *           k <= 16); 1 = one kernel of 256-token CTAs, two per SM, 64-expert steps (many tokens per SM);
+ *           0 = one kernel of one CTA per SM holding up to four token groups / expert ranges (few tokens per SM)
+ * For the chain, the numbers are those of the sweep: two CTAs per SM take equal parts of the token blocks' experts, and
+ * where these parts do not end with a token block, out8[1] is out8[2] divided by the token blocks, rounded down but at
+ * least 1.  (A call is swept in passes of at most 131072 tokens: the numbers are those of the first.)
  * Host-only; needs no device.
  */
 int more_route_plan_ex(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int path, int msplit,

@@ -126,6 +126,7 @@ class RoutePlan:
     expert_ranges: int = 1
     filter: bool = False
     paired: bool = False
+    chain: bool = False
 
 
 def more_route_plan(T, h, r, M, k, gate_mode=0, path=PATH_AUTO, msplit=0) -> RoutePlan:
@@ -141,7 +142,7 @@ def more_route_plan_ex(T, h, r, M, k, gate_mode=0, want_lse=False, path=PATH_AUT
     rc = lib().more_route_plan_ex(T, h, r, M, k, gate_mode, int(want_lse), path, msplit, o)
     if rc != 0:
         raise MoreRouteError(rc, "more_route_plan_ex")
-    return RoutePlan(o[0], o[1], o[2], o[3], o[4], o[5], bool(o[6]), bool(o[7]))
+    return RoutePlan(o[0], o[1], o[2], o[3], o[4], o[5], bool(o[6]), o[7] == 1, o[7] == 2)
 
 
 def _ptr(t):

@@ -1406,8 +1406,7 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
     const double kSegment = 8.0;
     long long g = total < slots ? total : slots, share = 0, sweep_blocks = blocks;
     if (msplit > 0) {
-        const int most = M / 256 > 1 ? M / 256 : 1;
-        share = msplit < most ? msplit : most;
+        share = msplit < nsteps ? msplit : nsteps;
     } else if (blocks <= slots) {
         const long long s = slots / blocks < nsteps ? slots / blocks : nsteps;
         const double whole = (double)((nsteps + s - 1) / s) + kSegment;
@@ -1427,14 +1426,12 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
     // a unit adds at most kCols / 4 entries to a list (a later, shorter chunk may have longer segments)
     const long long units = share > 0 ? (nsteps + share - 1) / share : (total + g - 1) / g;
     p->list_cap = T <= kChunkTokens && units < kListCap / (kCols / 4) ? (int)units * (kCols / 4) : kListCap;
-    // reported: CTAs; where a token block is split, the two CTAs of an SM count as one
-    p->ctas = (int)(share > 0 && msplit > 0 ? blocks * share : (blocks < sm_count && g > sm_count ? sm_count : g));
-    p->msplit = msplit > 0 ? (int)share : (int)(p->ctas / blocks > 1 ? p->ctas / blocks : 1);
+    p->ctas = (int)(share > 0 ? blocks * share : g);
+    p->msplit = (int)(p->ctas / blocks > 1 ? p->ctas / blocks : 1);      // (whole ones; a part that begins anywhere can reach into two blocks)
     p->share = (int)share;
     p->chain = true;
     p->block_tokens = kRows;
-    p->tg = 1;
-    p->es = 4;
+    p->tg = p->es = 1;
 }
 
 size_t chain_scratch_bytes(const RouteArgs& a, const Plan& p)

@@ -576,7 +576,7 @@ int more_route_plan_ex(int T, int h, int r, int M, int k, int gate_mode, int wan
                    148, &p);
     if (rc != MORE_OK) return rc;
     out8[0] = p.path; out8[1] = p.msplit; out8[2] = p.ctas; out8[3] = p.block_tokens;
-    out8[4] = p.tg; out8[5] = p.es; out8[6] = p.filter ? 1 : 0; out8[7] = p.paired ? 1 : 0;
+    out8[4] = p.tg; out8[5] = p.es; out8[6] = p.filter ? 1 : 0; out8[7] = p.chain ? 2 : (p.paired ? 1 : 0);
     return MORE_OK;
 }
 

@@ -67,7 +67,7 @@ def test_plan_picks_paths_and_splits():
     PX = mr.more_route_plan_ex
     # few token blocks, many experts: the experts are split, inside a CTA and over CTAs, and one wave is not exceeded
     p = PX(8192, 4096, 64, 131072, 16, gate_mode=1)
-    assert p.ctas % p.msplit == 0 and p.ctas <= 148
+    assert p.ctas % p.msplit == 0 and p.ctas <= (296 if p.chain else 148)
     assert p.msplit * p.expert_ranges >= 4 and p.token_groups * p.expert_ranges <= 4
     # many tokens: the kernel with 256-token CTAs, two per SM, in one wave
     p = PX(65536, 2048, 64, 16384, 8)
@@ -80,6 +80,26 @@ def test_plan_picks_paths_and_splits():
     assert P(300, 256, 32, 4096, 8, msplit=5).msplit == 5
     # asking for the log-sum-exp changes the kernel variant but is always accepted
     assert PX(32768, 512, 32, 16384, 8, want_lse=True).path == mr.PATH_TCGEN05
+
+
+def test_plan_names_the_kernel_and_its_real_numbers():
+    """The chain's plan is its sweep's: two CTAs per SM, 128 tokens each, one expert range per CTA."""
+    PX = mr.more_route_plan_ex
+    p = PX(8192, 4096, 64, 131072, 16, gate_mode=1)              # parts that begin anywhere: 296 of them for 64 token blocks
+    assert p.chain and not p.paired
+    assert (p.ctas, p.msplit, p.block_tokens, p.token_groups, p.expert_ranges) == (296, 4, 128, 1, 1)
+    p = PX(1, 2048, 64, 16384, 8)                                # one CTA per unit of 128 experts
+    assert p.chain and (p.ctas, p.msplit) == (128, 128)
+    p = PX(300, 256, 32, 4096, 8, msplit=5)                      # forced
+    assert p.chain and (p.ctas, p.msplit) == (15, 5)
+    p = PX(9000, 64, 8, 4096, 8, msplit=64)                      # no more CTAs than the 32 units of 128 experts
+    assert p.chain and (p.ctas, p.msplit) == (71 * 32, 32)
+    p = PX(65536, 2048, 64, 16384, 8)
+    assert p.paired and not p.chain
+    p = PX(32768, 512, 32, 1024, 8)
+    assert not p.paired and not p.chain and p.token_groups * p.expert_ranges <= 4 and p.ctas <= 148
+    assert not PX(64, 2048, 64, 16384, 32).chain                 # more than 16: the chain does not take it
+    assert not PX(100, 20, 5, 33, 3).chain
 
 
 def test_shared_memory_plan_of_the_grouped_kernel_fits():

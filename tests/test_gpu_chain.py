@@ -49,6 +49,18 @@ def test_edges(T, h, r, M, k, gate_mode):
     _route_and_check(inputs.gaussian_case(T, h, r, M, k, gate_mode, seed=T + M))
 
 
+@pytest.mark.parametrize("T,h,r,M,k", [(300, 128, 32, 4096, 8), (64, 128, 64, 16384, 20), (20000, 64, 16, 512, 8), (45000, 64, 16, 512, 4)])
+def test_the_plan_names_the_kernels_that_run(T, h, r, M, k):
+    import torch
+    plan = mr.more_route_plan_ex(T, h, r, M, k)
+    X, R1, R2 = to_device(inputs.gaussian_case(T, h, r, M, k, 0, seed=2))
+    before = mr.launches()
+    mr.route(X, R1, R2, k, 0)
+    torch.cuda.synchronize()
+    assert mr.more_route_status() == 0
+    assert mr.launches() - before == (3 if plan.chain else 1)
+
+
 @pytest.mark.parametrize("k", [1, 8, 16])
 @pytest.mark.parametrize("descending", [False, True])
 def test_logits_that_rise_or_fall_with_the_expert_id(k, descending):
