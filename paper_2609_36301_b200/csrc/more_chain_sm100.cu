@@ -242,7 +242,7 @@ constexpr int W = 128;                             // experts of a unit
 constexpr int kCols = W / 4;                       // columns of a thread
 constexpr int kMaxStages = 8;
 constexpr int kListCap = 64;                       // entries of a thread's list
-constexpr uint32_t kEntry = kRows * 32;            // bytes between its entries (32 bytes each: four logits, the first one's column)
+constexpr uint32_t kEntry = kEpi * 32;             // bytes between its entries (32 bytes each: four logits, the first one's column)
 
 // Units whose bucket maxima are formed ahead of a segment of `steps` units.  All of a short one: its threshold is then the
 // final one before the first candidate is kept, and a thread keeps one or two groups instead of the ten that a rising
@@ -264,8 +264,8 @@ struct SweepParams {
     int maxseg, cap;                               // candidate lists per token block in scratch, entries per list and token
     int nst, st_bytes, zbufs, z_bytes;
     int off_r2, off_pub, off_ctl;
-    int list_quarters, list_cap;
-    uint8_t* list;                                 // [CTA][list_quarters][list_cap][128 = column quarter x lane] x 32 bytes
+    int list_cap, list_shift;                      // entries of a list; log2 of the CTAs whose lists lie side by side (0, 1, 2)
+    uint8_t* list;                                 // [CTA >> shift][list_cap][512 = (CTA, 32-token quarter), column quarter, lane] x 32 bytes
     uint2* ent;                                    // [block][seg][128][cap] (logit bits, expert id)
     int* cnt;                                      // [block][seg][128]
     float2* mz;                                    // [block][seg][128] (max in log2 units, sum); LSE only
@@ -499,10 +499,11 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         const int M = p.M, nsteps = p.nsteps;
         const uint32_t t_col = tmem_base + ((uint32_t)(q * 32) << 16) + sub * kCols;
         // the thread's list; a unit adds at most 8 entries between two looks at its length
-        // (a list shorter than kListCap is one that so few units cannot fill; quarters without tokens have none, and their
-        // warps touch none)
-        const uint64_t first = reinterpret_cast<uint64_t>(p.list) +
-                               (uint64_t)(blockIdx.x * p.list_quarters + q) * (uint32_t)(p.list_cap * kEntry) + (sub * 32 + lane) * 32;
+        // (A list shorter than kListCap is one that so few units cannot fill.  Where only one or two quarters of the block hold
+        // tokens, four or two CTAs share an area: the other quarters' warps touch no lists.)
+        const uint32_t side = ((blockIdx.x & ((1u << p.list_shift) - 1)) << (2 - p.list_shift)) + q;
+        const uint64_t first = reinterpret_cast<uint64_t>(p.list) + (uint64_t)(blockIdx.x >> p.list_shift) * (p.list_cap * kEntry) +
+                               (side * (kEpi / 4) + sub * 32 + lane) * 32;
         const uint64_t warn = first + (kListCap - kCols / 4) * kEntry;
         // shared memory: published buckets [sub][128][NB], thresholds [128], counters [128], (m, Z) [sub - 1][128]
         const uint32_t pub0 = base + p.off_pub + row * (NB * 4);
@@ -1381,7 +1382,7 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
     const size_t blocks = (tokens + kRows - 1) / kRows, lists = (size_t)p.sweep_blocks * p.maxseg;
     size_t off = 0;
     L.z = off; off += align_up(blocks * kRows * (a.r <= 32 ? 128 : 256), 1024);
-    L.list = off; off += (size_t)p.parts * p.list_quarters * p.list_cap * kEntry;
+    L.list = off; off += (size_t)((p.parts - 1 >> p.list_shift) + 1) * p.list_cap * kEntry;
     L.ent = off; off += align_up(lists * (size_t)(4 * a.k) * kRows * 8, 1024);
     L.cnt = off; off += align_up(lists * kRows * 4, 1024);
     L.mz = off;
@@ -1422,7 +1423,7 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
     }
     p->parts = (int)g;
     p->sweep_blocks = (int)sweep_blocks;
-    p->list_quarters = T < kRows ? (T + 31) / 32 : kRows / 32;
+    p->list_shift = T <= 32 ? 2 : (T <= 64 ? 1 : 0);
     // a unit adds at most kCols / 4 entries to a list (a later, shorter chunk may have longer segments)
     const long long units = share > 0 ? (nsteps + share - 1) / share : (total + g - 1) / g;
     p->list_cap = T <= kChunkTokens && units < kListCap / (kCols / 4) ? (int)units * (kCols / 4) : kListCap;
@@ -1464,7 +1465,7 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
     sp.off_ctl = sp.off_pub + pub;
     const int smem = sp.off_ctl + ctl + 1024;
     sp.list = reinterpret_cast<uint8_t*>(base + L.list);
-    sp.list_quarters = plan.list_quarters; sp.list_cap = plan.list_cap;
+    sp.list_cap = plan.list_cap; sp.list_shift = plan.list_shift;
     sp.ent = reinterpret_cast<uint2*>(base + L.ent);
     sp.cnt = reinterpret_cast<int*>(base + L.cnt);
     sp.mz = lse ? reinterpret_cast<float2*>(base + L.mz) : nullptr;

@@ -59,8 +59,8 @@ struct Plan {
     int share = 0;         // ... how many of them share one token block each, or 0 where their parts begin anywhere,
     int maxseg = 1;        // ... and the most that can share one;
     int sweep_blocks = 1;  // ... token blocks per launch of the sweep;
-    int list_quarters = 4; // ... lists of a CTA: 32-token quarters of its blocks that hold tokens,
-    int list_cap = 1;      // ... and entries per thread
+    int list_cap = 1;      // ... entries of a thread's list,
+    int list_shift = 0;    // ... and log2 of the CTAs whose lists lie side by side in one area
 };
 
 bool tcgen05_shape_ok(int T, int h, int r, int M, int k);
