@@ -91,6 +91,9 @@ def _fast():
         L = lib()
         if not os.path.exists(_build.BINDING_PATH):
             raise FileNotFoundError(f"{_build.BINDING_PATH} is missing: build it with `python -m paper_2609_36301_b200.build`")
+        if not _build.binding_fits():
+            raise ImportError(f"{_build.BINDING_PATH} was not built for {_build.binding_built_for()}: "
+                              "build it again with `python -m paper_2609_36301_b200.build`")
         import importlib.machinery
         import importlib.util
 

@@ -25,11 +25,30 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
-def build_binding(force: bool = False) -> str:
-    """Compile the extension module if it is missing or older than its sources; return its path."""
+def binding_built_for() -> str:
+    """What the extension module depends on besides its sources: it is compiled against torch's C++ headers and Python's."""
+    import sys
+    import torch
+    return f"torch {torch.__version__}, {sys.implementation.cache_tag}"
+
+
+def binding_fits() -> bool:
+    """Whether the extension module that is there was built for this torch and this Python (it holds both as text: loading
+    one that was not could crash)."""
+    with open(BINDING_PATH, "rb") as f:
+        return f"built for {binding_built_for()};".encode() in f.read()
+
+
+def binding_is_current() -> bool:
+    """Whether the extension module exists, is as new as its sources, and fits."""
     header = os.path.join(os.path.dirname(_HERE), "include", "more_route.h")
     newest = max(os.path.getmtime(BINDING_SOURCE), os.path.getmtime(header))
-    if not force and os.path.exists(BINDING_PATH) and os.path.getmtime(BINDING_PATH) >= newest:
+    return os.path.exists(BINDING_PATH) and os.path.getmtime(BINDING_PATH) >= newest and binding_fits()
+
+
+def build_binding(force: bool = False) -> str:
+    """Compile the extension module unless the one that is there is current; return its path."""
+    if not force and binding_is_current():
         return BINDING_PATH
     import sysconfig
     import torch
@@ -37,7 +56,8 @@ def build_binding(force: bool = False) -> str:
     includes = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                 sysconfig.get_paths()["include"], os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + i for i in includes] + \
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DMORE_BUILT_FOR="{binding_built_for()}"'] + ["-I" + i for i in includes] + \
           ["-o", BINDING_PATH, BINDING_SOURCE, "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
            "-Wl,-rpath," + os.path.join(root, "lib")]
     subprocess.run(cmd, check=True)

@@ -254,7 +254,8 @@ PyObject* py_merge(PyObject*, PyObject* const* a, Py_ssize_t n)
 PyMethodDef methods[] = {
     MORE_FAST("bind", py_bind), MORE_FAST("route", py_route), MORE_FAST("route_ex", py_route_ex), MORE_FAST("psum", py_psum),
     MORE_FAST("dispatch", py_dispatch), MORE_FAST("full", py_full), MORE_FAST("merge", py_merge), {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module = {PyModuleDef_HEAD_INIT, "_more_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+// (the text by which build.py tells whether the module fits the torch and the Python that are installed)
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_more_binding", "built for " MORE_BUILT_FOR ";", -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 

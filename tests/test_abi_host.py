@@ -137,3 +137,15 @@ def test_device_memory_of_a_routing_call_is_bounded():
     # few tokens: only the rows that are there, and no longer lists than a CTA's experts can fill
     assert B(1, 2048, 64, 16384, 8) <= 9 * MiB
     assert B(64, 4096, 64, 131072, 16) <= 96 * MiB
+
+
+def test_extension_module_of_another_torch_is_not_used(monkeypatch):
+    """The module is compiled against torch's C++ headers: after an upgrade it is built again, and until then refused."""
+    import torch
+    mr_build.build_binding()
+    assert mr_build.binding_is_current()
+    monkeypatch.setattr(torch, "__version__", "0.0.1+other")
+    assert not mr_build.binding_is_current()
+    monkeypatch.setattr(mr, "_fast_module", None)
+    with pytest.raises(ImportError, match="was not built for torch 0.0.1"):
+        mr._fast()
