@@ -89,9 +89,10 @@ constexpr int kMaxStages1 = 8;                     // k-tiles of the projection 
 constexpr int kFallbackSlots = 16;                 // tokens re-routed per round of the fallback (one per epilogue warp)
 constexpr float kLog2e = 1.4426950408889634f;
 
-// (the ...Fan modes are the exact modes with the fanned-out merge of parked lists compiled in for lists longer than 8
-// entries: launched only when a token block is split over 8 or more CTAs, because that code costs the sweep of such
-// kernels ~3 %; lists of up to 8 entries always have it)
+// (The ...Fan modes are the exact modes with the fanned-out merge of parked lists compiled in, launched when a token block
+// is split over 8 or more CTAs; in the other kernels that code would cost the sweep ~3 %.  Only for lists of 32 entries: for
+// shorter ones the chain takes the shapes whose plan splits so far.  k = 32, without and with it: T = 64, M = 16384 200 and
+// 147 us, T = 256 with the softmax sweep 231 and 133; T = 64, M = 131072 265 and 287, a long sweep for so few lists.)
 enum { kModeExact = 0, kModeExactLse = 1, kModeFilter = 2, kModeExactFan = 3, kModeExactLseFan = 4 };
 
 struct RouteParams {
@@ -208,8 +209,7 @@ __device__ __forceinline__ void merge_parked_lists(const RouteParams& p, int blk
     // With few tokens and many splits (decode shapes) one thread per token would walk all lists one
     // L2 round trip after the other; instead `fan` threads per token merge a contiguous share of the
     // ranges each, park their result in the idle ring, and the token's own thread merges those.
-    // (FAN: always for lists of up to 8 entries; for longer ones this code raises the register needs of the whole kernel,
-    // which costs the sweep of the large k = 16 configurations ~3 %, so it is compiled into instantiations of their own
+    // (FAN: this code raises the register needs of the whole kernel, so it is compiled into instantiations of its own
     // that are launched only when a token block is split over 8 or more CTAs.)
     int fan = 1;
     if constexpr (FAN)
@@ -225,7 +225,7 @@ __device__ __forceinline__ void merge_parked_lists(const RouteParams& p, int blk
         // in log2(fan) levels.
         const int bt = p.block_tokens;
         constexpr int kPerList = KCAP * 8 + 8;
-    constexpr int kInFlight = KCAP <= 8 ? 4 : 2;          // loads per array and thread in flight during the copy
+        constexpr int kInFlight = 2;                        // loads per array and thread in flight during the copy
         float* sv = reinterpret_cast<float*>(ring_ptr);                  // [fan][KCAP][bt]
         int* si = reinterpret_cast<int*>(sv + fan * KCAP * bt);         // [fan][KCAP][bt]
         float2* smz = reinterpret_cast<float2*>(si + fan * KCAP * bt);  // [fan][bt]
@@ -340,7 +340,7 @@ route_lowrank_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
 {
     constexpr bool FILTER = MODE == kModeFilter;
     constexpr bool LSE = MODE == kModeExactLse || MODE == kModeExactLseFan;
-    constexpr bool FAN = KCAP <= 8 || MODE == kModeExactFan || MODE == kModeExactLseFan;
+    constexpr bool FAN = MODE == kModeExactFan || MODE == kModeExactLseFan;
     constexpr int kKSteps = RPAD / 16;                               // UMMA K = 16
     constexpr int kMmasPerBuf = FILTER ? kKSteps : 2 * kKSteps;      // exact modes: hi then lo into one accumulator
     constexpr int kZopCols = FILTER ? RPAD / 2 : RPAD;               // A operand: two bf16 per 32-bit column
@@ -1137,11 +1137,11 @@ KernelFn kernel_mode(int mode)
         case kModeExact: return kernel_ready<RPAD, KCAP, kModeExact>();
         case kModeExactLse: return kernel_ready<RPAD, KCAP, kModeExactLse>();
         case kModeExactFan:
-            if constexpr (KCAP > 8) return kernel_ready<RPAD, KCAP, kModeExactFan>();
-            return kernel_ready<RPAD, KCAP, kModeExact>();
+            if constexpr (KCAP > 16) return kernel_ready<RPAD, KCAP, kModeExactFan>();
+            return nullptr;
         case kModeExactLseFan:
-            if constexpr (KCAP > 8) return kernel_ready<RPAD, KCAP, kModeExactLseFan>();
-            return kernel_ready<RPAD, KCAP, kModeExactLse>();
+            if constexpr (KCAP > 16) return kernel_ready<RPAD, KCAP, kModeExactLseFan>();
+            return nullptr;
         default:
 #ifdef MORE_WITH_FILTER
             if constexpr (KCAP <= 16) return kernel_ready<RPAD, KCAP, kModeFilter>();
@@ -1265,7 +1265,7 @@ int launch_lowrank(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scra
     }
     const bool lse = (a.gate_mode == MORE_GATE_FULL_SOFTMAX) || (a.out_lse != nullptr);
     int mode = lse ? kModeExactLse : kModeExact;
-    if (p.msplit >= 8) mode = lse ? kModeExactLseFan : kModeExactFan;
+    if (p.msplit >= 8 && a.k > 16) mode = lse ? kModeExactLseFan : kModeExactFan;
     if (p.filter) {
         if (lse || a.k > 16) return MORE_ERR_SHAPE;
         mode = kModeFilter;
