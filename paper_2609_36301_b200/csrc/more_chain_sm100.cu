@@ -229,13 +229,15 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 // position in the units) and a threshold.  The k-th largest of a token's 4 NB bucket maxima is reached by
 // at least k of its logits, so nothing strictly below it can be selected; its expected rank is ~11 for k = 8 of 16
 // buckets, ~22 for k = 16 of 32.  Every group of four whose maximum reaches the threshold is appended, values and first
-// column, to the thread's list in global scratch (which stays in L2): two predicated stores and an add, and nothing
-// waits for them.  A sweep starts with a threshold: the bucket maxima of its first eighth (of its first two units, if
-// that is no more) are formed before anything is selected; this costs an eighth more MMAs, and saves the appends of the
-// start, when nearly everything beats what has been seen.  After 1/8 of the sweep, and whenever half as much again is done, the buckets are published
-// in shared memory, one of the four warps of a lane quarter computes new thresholds from them, and the others pick these
-// up when they see them (all values are monotone lower bounds, so no synchronisation is needed).  At the end of a
-// segment a thread goes once through its list and keeps what reaches the final threshold (~11 logits per token).
+// column, to the thread's list in global scratch: two predicated stores and an add, and nothing waits for them.  (Most of
+// a list stays in L2.  What leaves it, 115 MB of a call with k = 16 of 131072 experts for 8192 tokens, is 18 us of DRAM
+// time in a sweep of 510.)  A sweep starts with a threshold: the bucket maxima of its first units (lead_of: all of a short
+// segment, an eighth of a long one) are formed before anything is selected; this costs their MMAs and the reading of their
+// accumulators again, and saves the appends of the start, when nearly everything beats what has been seen.  Whenever half
+// as much again of a long segment is done, the buckets are published in shared memory, one of the four warps of a lane
+// quarter computes new thresholds from them, and the others pick these up when they see them (all values are monotone
+// lower bounds, so no synchronisation is needed).  At the end of a segment a thread goes once through its list and passes
+// on what reaches the final threshold (~11 logits per token for k = 8).
 constexpr int kSThreads = 576;
 constexpr int kEpi = 512;
 constexpr int W = 128;                             // experts of a unit
@@ -322,13 +324,13 @@ __device__ __forceinline__ void bitonic_down(float (&s)[N])
             if ((i & d) == 0) cx(s[i], s[i + d]);
 }
 // Append the groups of four (maxima t, values v, first column col + 4 i) that reach thr to a list that ends at `end`.  The
-// four tests come first: only the adds to the list's end depend on each other.  `one` is 1, unknown to the compiler: a
-// predicated 64-bit multiply-add is one instruction, a predicated 64-bit add is four.
-__device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t, const float* v, int col, uint32_t one)
+// four tests come first: only the adds to the list's end depend on each other.  (These as multiply-adds by a register that
+// holds 1 take the same time: T = 32768, M = 65536 425 us; T = 8192, M = 131072, k = 16 507 +- 4; T = 16384, M = 4096 63.1.)
+__device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t, const float* v, int col)
 {
 #define MORE_APPEND(P, COL, A, B, C, D)                                                                     \
     "@" P " st.global.v4.f32 [%0], {" A ", " B ", " C ", " D "};\n\t@" P " st.global.b32 [%0+16], " COL ";\n\t" \
-    "@" P " mad.wide.u32 %0, %24, %22, %0;\n\t"
+    "@" P " add.u64 %0, %0, %22;\n\t"
     asm volatile(
         "{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 c1, c2, c3;\n\t"
         "setp.ge.f32 p0, %2, %1;\n\tsetp.ge.f32 p1, %3, %1;\n\tsetp.ge.f32 p2, %4, %1;\n\tsetp.ge.f32 p3, %5, %1;\n\t"
@@ -338,7 +340,7 @@ __device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t
         : "+l"(end)
         : "f"(thr), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]),
           "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]),
-          "f"(v[15]), "n"(kEntry), "r"(col), "r"(one)
+          "f"(v[15]), "n"(kEntry), "r"(col)
         : "memory");
 #undef MORE_APPEND
 }
@@ -510,8 +512,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         const uint32_t s_thr = base + p.off_pub + 4 * kRows * NB * 4 + row * 4;
         const uint32_t s_cnt = s_thr + kRows * 4;
         const uint32_t s_mz = base + p.off_pub + 4 * kRows * NB * 4 + kRows * 8 + row * 8;
-        uint32_t n = 0, one;
-        asm volatile("mov.u32 %0, 1;" : "=r"(one));
+        uint32_t n = 0;
         float b[NB];
         float thr, m2, zsum;
         uint64_t ptr;                                        // where the next entry goes
@@ -785,7 +786,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     if (__any_sync(kFull, m >= thr)) {
                         // (a bucket matters only once it reaches the threshold, so it need not be kept up elsewhere)
                         bucket(h, t);
-                        append4(ptr, thr, t, v, col, one);
+                        append4(ptr, thr, t, v, col);
                     }
                 }
                 if (__builtin_expect(__any_sync(kFull, ptr > limit), 0)) full();
