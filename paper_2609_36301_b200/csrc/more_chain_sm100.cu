@@ -569,9 +569,10 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             }
             return kth;
         };
-        // k-th largest logit of this thread's own list and how many equal to it are wanted (all of them in a short list)
+        // k-th largest logit of this thread's own list and how many equal to it are wanted (all of them in a short list).
+        // (Starting from NaN, which nothing reaches: an infinite logit, of finite inputs that overflow, is one like any other.)
         auto own_kth = [&](int& equal) {
-            float cur = INFINITY;
+            float cur = __int_as_float(0x7fffffff);
             int need = p.k;
             for (;;) {
                 float m = -INFINITY;
@@ -581,7 +582,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     const float x[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        if (x[j] < cur) {
+                        if (!(x[j] >= cur)) {
                             if (x[j] > m) { m = x[j]; c = 1; }
                             else if (x[j] == m) ++c;
                         }
@@ -844,7 +845,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     total = __float_as_int(lds(s_cnt));
                 }
                 if (sub == 0 && row_live) {
-                    p.cnt[slot * kRows + row] = total;
+                    p.cnt[slot * kRows + row] = min(total, p.cap);
                     if (LSE) {
                         float m = m2, z = zsum;
 #pragma unroll

@@ -142,3 +142,39 @@ def test_tokens_of_zeros(T, M, k):
     import torch
     res = mr.route(*to_device(case), k, 1)
     assert bool((res.idx[::3] == torch.arange(k, device="cuda", dtype=torch.int32)).all())
+
+
+@pytest.mark.parametrize("gate_mode", [0, 1])
+@pytest.mark.parametrize("T,M,k", [
+    (300, 16384, 8),       # one or two units per segment
+    (8000, 16384, 2),      # 27 units, the threshold final from the start
+    (4800, 36008, 16),     # long segments of lists longer than 8
+    (4800, 36008, 8),
+    (40, 65536, 8),        # hundreds of segments per token
+    (8500, 3072, 8),       # the finishing kernel with eight threads per token
+])
+def test_infinite_logits(T, M, k, gate_mode):
+    """Finite inputs whose logits overflow: tokens for which every second expert's logit is +inf.  They are logits like any
+    other (the lists must not grow past their end), other tokens are unaffected."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(T + M + k)
+    X = torch.randn((T, 64), generator=gen, device="cuda").to(torch.bfloat16)
+    R1 = (torch.randn((64, 8), generator=gen, device="cuda") / 8).to(torch.bfloat16)
+    R2 = torch.randn((8, M), generator=gen, device="cuda").to(torch.bfloat16)
+    R1[0] = 0
+    R1[0, 0] = 1
+    R2[0, ::2], R2[0, 1::2] = 4, 1
+    half = torch.arange(5, T, 97, device="cuda")
+    X[half] = 0
+    clean = mr.route(X, R1, R2, k, gate_mode, want_topval=True)
+    X[half, 0] = 2e38
+    res = mr.route(X, R1, R2, k, gate_mode, want_topval=True)
+    assert mr.more_route_plan_ex(T, 64, 8, M, k, gate_mode).chain
+    torch.cuda.synchronize()
+    assert mr.more_route_status() == 0 and mr.debug_scratch_guard() == 1
+    assert bool((res.idx[half] == 2 * torch.arange(k, device="cuda", dtype=torch.int32)).all())
+    assert bool(torch.isinf(res.topval[half]).all())
+    others = torch.ones(T, dtype=torch.bool, device="cuda")
+    others[half] = False
+    assert torch.equal(res.idx[others], clean.idx[others]) and torch.equal(res.gate[others], clean.gate[others])
+    check_counts(res.idx.cpu().numpy(), res.counts.cpu().numpy(), M)
