@@ -517,6 +517,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         float thr, m2, zsum;
         uint64_t ptr;                                        // where the next entry goes
 
+        auto lds = [&](uint32_t a) { float v; asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory"); return v; };
+        auto sts = [&](uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); };
         auto ent4 = [&](uint64_t o) { return *reinterpret_cast<const float4*>(o); };
         auto ent_col = [&](uint64_t o) { return *reinterpret_cast<const int*>(o + 16); };
         auto put = [&](uint64_t o, float4 e, int c) {
@@ -592,15 +594,18 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 cur = m;
             }
         };
-        // make room in the lists of a warp: drop what has fallen below the threshold, first raising it by what the thread
-        // knows itself; a list that stays long is cut to its k best (later equals then lose to those: larger ids)
+        // Make room in the lists of a warp: drop what is below a bound that k logits are known to reach, and cut a list that
+        // stays long to its k best (later equals then lose to those: larger ids).  The bound is not thr, which may lie just
+        // above logits that the list has to keep: it was raised when enough of their equals were in.
         auto compact = [&]() {
+            float known = lds(s_thr);
             if (p.k <= NB) {
                 float mine = b[0];
 #pragma unroll
                 for (int i = 1; i < NB; ++i) mine = fminf(mine, b[i]);
-                thr = fmaxf(thr, mine);
+                known = fmaxf(known, mine);
             }
+            thr = fmaxf(thr, known);
             auto keep = [&](float low, int equal) {
                 uint64_t wr = first;
                 for (uint64_t rd = first; rd < ptr; rd += kEntry) {
@@ -615,7 +620,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 }
                 ptr = wr;
             };
-            keep(thr, INT_MAX);
+            keep(known, INT_MAX);
             if (ptr > warn) {
                 int equal;
                 const float kth = own_kth(equal);
@@ -653,8 +658,6 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 }
             }
         };
-        auto lds = [&](uint32_t a) { float v; asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory"); return v; };
-        auto sts = [&](uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); };
 
         // (units of this CTA as a block, a step in it and a count: 32-bit loop state)
         int blk = (int)(lo / nsteps), s0 = (int)(lo - (long long)blk * nsteps);

@@ -154,27 +154,61 @@ def test_tokens_of_zeros(T, M, k):
     (8500, 3072, 8),       # the finishing kernel with eight threads per token
 ])
 def test_infinite_logits(T, M, k, gate_mode):
-    """Finite inputs whose logits overflow: tokens for which every second expert's logit is +inf.  They are logits like any
-    other (the lists must not grow past their end), other tokens are unaffected."""
+    """Finite inputs whose logits overflow: a token for which every second expert's logit is +inf, one with three such experts
+    among equals.  They are logits like any other (the lists must not grow past their end), other tokens are unaffected."""
     import torch
     gen = torch.Generator(device="cuda").manual_seed(T + M + k)
     X = torch.randn((T, 64), generator=gen, device="cuda").to(torch.bfloat16)
     R1 = (torch.randn((64, 8), generator=gen, device="cuda") / 8).to(torch.bfloat16)
     R2 = torch.randn((8, M), generator=gen, device="cuda").to(torch.bfloat16)
-    R1[0] = 0
-    R1[0, 0] = 1
+    R1[0], R1[1] = 0, 0
+    R1[0, 0] = R1[1, 1] = 1
     R2[0, ::2], R2[0, 1::2] = 4, 1
-    half = torch.arange(5, T, 97, device="cuda")
-    X[half] = 0
+    R2[1], few = 0, torch.tensor([M // 3, M // 2, M - 1], device="cuda")
+    R2[1, few] = 4
+    half, three = torch.arange(5, T, 97, device="cuda"), torch.arange(6, T, 97, device="cuda")
+    X[half], X[three] = 0, 0
     clean = mr.route(X, R1, R2, k, gate_mode, want_topval=True)
-    X[half, 0] = 2e38
+    X[half, 0], X[three, 1] = 2e38, 2e38
     res = mr.route(X, R1, R2, k, gate_mode, want_topval=True)
     assert mr.more_route_plan_ex(T, 64, 8, M, k, gate_mode).chain
     torch.cuda.synchronize()
     assert mr.more_route_status() == 0 and mr.debug_scratch_guard() == 1
     assert bool((res.idx[half] == 2 * torch.arange(k, device="cuda", dtype=torch.int32)).all())
     assert bool(torch.isinf(res.topval[half]).all())
+    want = torch.cat([few.int(), torch.arange(k, device="cuda", dtype=torch.int32)])[:k]
+    assert bool((res.idx[three] == want).all())
     others = torch.ones(T, dtype=torch.bool, device="cuda")
-    others[half] = False
+    others[half], others[three] = False, False
     assert torch.equal(res.idx[others], clean.idx[others]) and torch.equal(res.gate[others], clean.gate[others])
+    check_counts(res.idx.cpu().numpy(), res.counts.cpu().numpy(), M)
+
+
+@pytest.mark.parametrize("equals", [False, True])
+@pytest.mark.parametrize("T,M,k", [(4800, 36008, 16), (4800, 36008, 8), (4800, 36008, 3), (2000, 131072, 8), (8000, 16384, 12)])
+def test_lists_that_overflow_at_different_times(T, M, k, equals):
+    """A warp makes room in all its lists when one overflows.  Eight kinds of tokens side by side, whose logits rise with the
+    expert id up to an eighth, two eighths, ... of the experts and are low from there on, so that lists overflow in turn;
+    with `equals`, tokens of zeros but for three experts stand between them."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(M + k)
+    e = torch.arange(M, device="cuda")
+    X = torch.zeros((T, 64), device="cuda")
+    kind = torch.arange(T, device="cuda") % 8
+    X[torch.arange(T, device="cuda"), kind] = 1 + torch.rand(T, generator=gen, device="cuda")
+    R1 = torch.eye(64, device="cuda")[:, :8]
+    R2 = torch.stack([torch.where(e < M * (j + 1) // 8, torch.exp2(20.0 * e / M), -1.0) for j in range(8)])
+    if equals:
+        R2[1::2] = 0
+        R2[1::2, torch.tensor([M // 5, M // 3, M - 1], device="cuda")] = 3
+    X, R1, R2 = X.to(torch.bfloat16), R1.to(torch.bfloat16).contiguous(), R2.to(torch.bfloat16)
+    assert mr.more_route_plan_ex(T, 64, 8, M, k, 0).chain
+    res = mr.route(X, R1, R2, k, 0, want_topval=True)
+    torch.cuda.synchronize()
+    assert mr.more_route_status() == 0 and mr.debug_scratch_guard() == 1
+    # (z has one element that is not zero, and it is a bf16: the logits are exact in fp32)
+    rows = torch.cat([torch.arange(i, i + 64, device="cuda") for i in range(0, T - 63, max(64, T // 12))])
+    val, idx = (X[rows, :8].float() @ R2.float()).sort(dim=1, descending=True, stable=True)
+    assert torch.equal(res.topval[rows], val[:, :k])
+    assert torch.equal(res.idx[rows], idx[:, :k].int())
     check_counts(res.idx.cpu().numpy(), res.counts.cpu().numpy(), M)
