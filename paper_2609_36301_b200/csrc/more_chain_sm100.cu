@@ -161,7 +161,7 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     zr[lo_off + 2 * c + 1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
                 }
             }
-        } else if (ok && row - lane < live) {      // (rows past the last token are not exchanged: nothing reads them)
+        } else if (ok && row - lane < live) {      // (rows past the last token are not exchanged)
             const int share = kRows / cs, dst = row / share;
             const uint32_t a = smem_u32(exch) + (uint32_t)((rank * share + row % share) * 64) * 4u;
             uint32_t remote;
@@ -184,11 +184,14 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         cluster_sync();
         if (warp >= 2) {
             const int share = kRows / cs, q4_bits = p.zc == 64 ? 3 : 4, q4 = 1 << q4_bits;        // float4s of one row of z
-            const int mine = min(share, live - rank * share);
-            for (int i = threadIdx.x - 64; i < mine * q4; i += kRows) {
+            // Rows past the last token, up to the 32 that a warp of the sweep looks at, are zero.  (What an earlier call left
+            // there would be swept as tokens whose logits can be infinite, reach any threshold and fill their lists again
+            // and again: T = 7284, M = 16384 2330 us instead of 83.)
+            const int mine = live - rank * share, rows = min(share, ((live + 31) & ~31) - rank * share);
+            for (int i = threadIdx.x - 64; i < rows * q4; i += kRows) {
                 const int rr = i >> q4_bits, c4 = i & (q4 - 1);
                 float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (c4 * 4 < p.n) {
+                if (c4 * 4 < p.n && rr < mine) {
                     const float* e = exch + rr * 64 + c4 * 4;
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {

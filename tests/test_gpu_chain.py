@@ -212,3 +212,38 @@ def test_lists_that_overflow_at_different_times(T, M, k, equals):
     assert torch.equal(res.topval[rows], val[:, :k])
     assert torch.equal(res.idx[rows], idx[:, :k].int())
     check_counts(res.idx.cpu().numpy(), res.counts.cpu().numpy(), M)
+
+
+def test_what_an_earlier_call_left_behind_the_last_token_is_not_swept():
+    """Rows of z behind the last token are not written.  An earlier call leaves large values there, with which the weights of
+    this one overflow to infinity: such rows must not be taken for tokens that beat every threshold (their lists would
+    overflow all the time; the call took 20 times as long)."""
+    import torch
+    T, h, r, M, k = 57 * 128 - 12, 256, 8, 16384, 2              # two CTAs share a block's projection, and 25 units per sweep
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    X, R1, R2 = (torch.randn(s, generator=gen, device="cuda").to(torch.bfloat16) for s in ((T, h), (h, r), (r, M)))
+    R1 /= 16
+    R2[0] = 8 + R2[0].abs()
+
+    def timed(leftover):
+        X0 = torch.zeros((T + 12, h), dtype=torch.bfloat16, device="cuda")
+        R10 = torch.zeros((h, r), dtype=torch.bfloat16, device="cuda")
+        X0[:, 0], R10[0, 0] = 1.0, leftover
+        mr.route(X0, R10, torch.zeros_like(R2), k, 0)
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            res = mr.route(X, R1, R2, k, 0, want_topval=True)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        assert mr.more_route_status() == 0
+        return best, res
+
+    assert mr.more_route_plan_ex(T, h, r, M, k).chain
+    clean, res = timed(0.0)
+    left, res2 = timed(1e38)
+    assert torch.equal(res.idx, res2.idx) and torch.equal(res.topval, res2.topval)
+    assert left < 2 * clean, f"{clean * 1e3:.0f} us with zeros behind the last token, {left * 1e3:.0f} us with large values"
