@@ -190,32 +190,25 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 namespace {
 
 // Whether the low-rank router runs as the chain projection -> sweep -> finish rather than as one of the two kernels that
-// do it all.  Measured on B200 at 1260 points: T = 1 ... 64 k, h = 128, 512, 2048, r = 16 ... 64, M = 128 ... 64 k,
-// k = 4, 8, 12, 16, both gates; the large ones also under sustained load, where the chip's power limit counts (the chain's
-// sweep loses ~3 % more there).  The chain wins where one kernel repeats the projection or leaves SMs idle (few tokens: 1.2
-// to 3 times faster, most at large h, where a cluster shares the reading of X) and on all but short sweeps (1.1 to 2.5 at
-// k > 8, 1.1 to 1.5 at k <= 4).  What it pays for each segment of a sweep, its third launch and the counts, added up by a
-// kernel of their own, lose on few experts (T = 17 k, M = 512: 0.7) and on many tokens at M = 1 k ... 4 k (T = 64 k,
-// M = 2 k, k = 8: 0.8).  k = 5 ... 8 has the worst threshold for its k (the 8th of 16 buckets), so its lines lie lower;
-// above 16 the buckets do not bound the k-th logit well enough, below 128 experts they are mostly empty.
-bool chain_wins(int T, int h, int r, int M, int k, bool lse, int sm_count)
+// do it all: by experts against tokens per SM.  What the chain pays on top (a threshold, the reading back of a list and the
+// finishing kernel's ranking and counting, per token and segment) grows with the tokens and not with the experts, what it
+// gains (a projection that is not repeated, an even cut of the units, cheaper selection) with both; a larger h favours it,
+// as a cluster shares the reading of X.  So the lines are straight: M >= c x (tokens per SM), c by how tight the bound on
+// the k-th logit is for the number of buckets (k <= 4 of 16, k <= 8 of 16, k <= 16 of 32; above that it is too loose), and
+// with fewer than 1024 experts, eight units or less per token block, about twice that.  From 340 tokens per SM on, the paired
+// kernel's two CTAs per SM fill up, and for k = 5 ... 8 it wins up to c = 40 (20 where the exponentials slow it down).
+// Measured on B200 at 14300 shapes drawn from T = 1 ... 64 k, M = 128 ... 128 k, h = 128, 512, 2048, r = 16, 32, 64,
+// k = 2 ... 16, both gates, one call after the other, and at large ones with each side running for 0.1 s at a time, where the
+// chip's power limit counts.  profiles/kernel_choice.csv holds 2891 more, to which nothing was fitted: there the choice costs
+// 0.4 % on average against the better side of each shape and more than 5 % at 2.8 % of them (1.32 at most); always the chain
+// would cost 7 %, never 33 %.
+bool chain_wins(int T, int h, int M, int k, bool lse, int sm_count)
 {
-    const int per_sm = (T + sm_count - 1) / sm_count;
+    const int per_sm = (T + sm_count - 1) / sm_count, wide = h < 4096 ? h : 4096;
     if (k > 16 || M < 128) return false;
-    if (M < 512) return per_sm <= 8 ? M >= 256 || h >= 512 : h >= 1024 && per_sm <= 24;
-    if (M < 1024) return per_sm <= (h >= 1024 ? 45 : 24);
-    if (M < 2048) return per_sm <= 90;
-    if (k > 8) return per_sm <= 230 || M >= 16384 || (M >= 4096 && r <= 32);
-    if (k <= 4) return M >= 8192 || per_sm <= 230;
-    if (M < 4096) return per_sm <= 140;
-    if (M < 8192) return per_sm <= (lse ? 170 : 230);
-    if (M < 16384) return per_sm <= 170;
-    // a few segments of 33 to 64 units per CTA are the longest that are not swept twice (T = 16 k, M = 16 k: 0.94 to 1.02)
-    if (M < 32768 && per_sm > 100 && per_sm <= 120) return false;
-    // many tokens: the paired kernel, with two accumulators per token group at r <= 32, ties or wins unless it is slowed by
-    // the exponentials (T = 64 k, M = 16 k: 0.94 to 0.96 without them; with them 1.07 at r = 32, 0.99 at r = 64)
-    if (per_sm > 240 && M < 65536) return lse && (r <= 32 || M >= 32768);
-    return true;
+    if (M < 1024) return M + wide / 4 - 128 >= (k <= 4 ? 8 : 18) * per_sm;
+    const double c = k <= 4 ? 4.5 : (k > 8 ? 7 : (per_sm <= 340 ? 12 : (lse ? 20 : 40)));
+    return M + wide / 8 >= c * per_sm;
 }
 
 // Launch plan of the paired low-rank kernel (256-token CTAs, two per SM).
@@ -374,7 +367,7 @@ int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, b
     if (full) {
         plan_dense(T, h, M, msplit, sm_count, &p);
     } else {
-        if (chain_wins(T, h, r, M, k, want_lse || gate_mode == MORE_GATE_FULL_SOFTMAX, sm_count)) {
+        if (chain_wins(T, h, M, k, want_lse || gate_mode == MORE_GATE_FULL_SOFTMAX, sm_count)) {
             plan_chain(T, M, msplit, sm_count, &p);
             *out = p;
             return MORE_OK;

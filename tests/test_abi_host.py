@@ -102,6 +102,26 @@ def test_plan_names_the_kernel_and_its_real_numbers():
     assert not PX(100, 20, 5, 33, 3).chain
 
 
+def test_choice_of_the_chain_has_no_holes():
+    """More experts or fewer tokens never take a shape off the chain, nor does a smaller k within a class of buckets."""
+    def chain(T, M, k, h, gate):
+        return mr.more_route_plan_ex(T, h, 32, M, k, gate).chain
+
+    Ts = [1, 1000, 3000, 5000, 8000, 11000, 14000, 16000, 18000, 25000, 34000, 36000, 45000, 50400, 55000, 65536, 200000]
+    Ms = [64, 120, 128, 256, 512, 1016, 1024, 1536, 2048, 3072, 4096, 8192, 12000, 16384, 20000, 24576, 32768, 65536, 131072]
+    for h in (128, 1024, 4096, 16384):
+        for gate in (0, 1):
+            for k in (1, 4, 5, 8, 9, 16):
+                grid = [[chain(T, M, k, h, gate) for M in Ms] for T in Ts]
+                for row in grid:
+                    assert row == sorted(row), (h, gate, k)
+                for column in zip(*grid):
+                    assert list(column) == sorted(column, reverse=True), (h, gate, k)
+                assert all(grid[0][2:]) or h < 512, "a single token is always served by the chain"
+    for T, M in ((1, 128), (16000, 16384), (16000, 24576), (30000, 4096), (40000, 65536)):
+        assert chain(T, M, 4, 2048, 0) == chain(T, M, 1, 2048, 0) and chain(T, M, 8, 2048, 0) == chain(T, M, 5, 2048, 0)
+
+
 def test_shared_memory_plan_of_the_grouped_kernel_fits():
     """Every (rank, token groups, expert ranges) the planner may pick leaves room for at least two R2 stages and one
     phase-1 stage in the 208 KB ring (checked through the plans of shapes that exercise them)."""
@@ -129,7 +149,7 @@ def test_device_memory_of_a_routing_call_is_bounded():
         segments = 2 * 148 + 2 * blocks
         return z + 2 * 148 * MiB + segments * 128 * (4 * k * 8 + 12) + MiB
 
-    for T, M, k in ((131072, 16384, 4), (65536, 65536, 4), (65536, 16384, 16), (4096, 131072, 16), (300000, 32768, 8), (300, 65536, 8)):
+    for T, M, k in ((131072, 16384, 4), (65536, 65536, 4), (65536, 16384, 16), (4096, 131072, 16), (300000, 32768, 4), (300, 65536, 8)):
         for msplit in (0, 1, 2, 7, 64):
             assert B(T, 512, 64, M, k, 1, msplit=msplit) <= bound(T, 64, M, k), (T, M, k, msplit)
     # largest there is without a forced split
