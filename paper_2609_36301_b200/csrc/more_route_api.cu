@@ -262,10 +262,12 @@ void plan_dense(int T, int h, int M, int msplit, int sm_count, Plan* p)
             const long long ctas = (long long)blocks * s;
             const double waves = (double)((ctas + sm_count - 1) / sm_count);
             const double steps = (double)((tiles + s - 1) / s);
-            // microseconds, fitted to B200 measurements: 1.2 per k-tile of a step (the L2 -> SM traffic of the
-            // stages), 2.1 for its epilogue, 8 per CTA for start and pipeline fill, 25 more when the lists are
-            // parked and merged
-            double cost = waves * (steps * (1.2 * ktiles + 2.1) + 8.0 + (s > 1 ? 25.0 : 0.0));
+            // Microseconds, fitted to 990 shapes on B200 at forced splits of 1 to 16 (T = 64 ... 20000, h = 128 ... 4096,
+            // M = 256 ... 16384): 0.6 per k-tile of a step (its eight MMAs of 128 x 256 x 16 take 0.58), 4.7 for its epilogue,
+            // 21 per CTA for start, pipeline fill and output, 6 more when the lists are parked and merged.  The split chosen
+            // costs 0.3 % on average against the best of them, 2 % with the figures of the four MMAs of N = 64 (1.2, 2.1, 8,
+            // 25), which split too little: T = 500, h = 256, M = 1000 55 us against 40.
+            double cost = waves * (steps * (0.6 * ktiles + 4.7) + 21.0 + (s > 1 ? 6.0 : 0.0));
             cost *= 1.0 + 0.02 * (kBlockTokens - bt) / 32.0;          // prefer full blocks on a tie
             if (cost < best * 0.999) { best = cost; best_bt = bt; best_s = s; }
         }
