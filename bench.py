@@ -68,13 +68,19 @@ def roofline(T, h, r, M, k, seconds, peaks, traffic=None):
 
 def load_counters():
     """Per-workload hardware counters of the router kernel, written when the ncu captures are refreshed: DRAM bytes per
-    launch (dram__bytes_read.sum + dram__bytes_write.sum) and warp instructions per 16-column x 32-token chunk.  A
+    call (dram__bytes_read.sum + dram__bytes_write.sum) and warp instructions per 16-column x 32-token chunk.  A
     workload that was not captured has no entry."""
     path = os.path.join(ROOT, "profiles", "counters.json")
     try:
         return json.load(open(path))
     except (OSError, ValueError):
         return {}
+
+
+def counters_of(counters, name, gate_mode, plan):
+    """The counters of a workload, unless they were captured on another kernel than the one that serves it now."""
+    entry = counters.get(f"{name}/mode{gate_mode}", {})
+    return entry if entry and entry["kernel"].split("<")[0] in kernel_of(plan) else {}
 
 
 SM_COUNT = 148
@@ -494,8 +500,8 @@ def main():
         return
 
     counters = load_counters()
-    cnt = counters.get(f"{name}/mode{gate_mode}", {})
     plan = mr.more_route_plan_ex(case.T, case.h, case.r, case.M, k, gate_mode)
+    cnt = counters_of(counters, name, gate_mode, plan)
     roof = roofline(case.T, case.h, case.r, case.M, k, secs / args.steps, peaks, cnt.get("dram_bytes"))
     roof["kernel"] = kernel_of(plan)
     roof.update(diagnostic_bounds(case.T, case.M, gate_mode, cnt.get("warp_instr_per_chunk"), clocks.get("sm_mhz")))
@@ -563,7 +569,7 @@ def main():
                 owarm = time_router(mr, torch, obufs[:1], ocase.k, gm, 200, 5, stream) / 200
                 r = roofline(ocase.T, ocase.h, ocase.r, ocase.M, ocase.k, osecs, peaks)
                 oplan = mr.more_route_plan_ex(ocase.T, ocase.h, ocase.r, ocase.M, ocase.k, gm)
-                ocnt = counters.get(f"{oname}/mode{gm}", {})
+                ocnt = counters_of(counters, oname, gm, oplan)
                 others[f"{oname}/mode{gm}"] = dict(us=osecs * 1e6, us_warm=owarm * 1e6, tokens_per_s=ocase.T / osecs,
                                                     bound=r["bound"], roofline_frac=r["frac"], msplit=oplan.msplit,
                                                     ctas=oplan.ctas, block_tokens=oplan.block_tokens,

@@ -169,3 +169,22 @@ def test_extension_module_of_another_torch_is_not_used(monkeypatch):
     monkeypatch.setattr(mr, "_fast_module", None)
     with pytest.raises(ImportError, match="was not built for torch 0.0.1"):
         mr._fast()
+
+
+def test_committed_counters_are_of_the_kernels_that_run():
+    """Every entry of profiles/counters.json was captured on a kernel of the plan that serves its workload, and bench.py
+    would not attach it otherwise."""
+    import json
+
+    import bench
+    from paper_2609_36301_b200 import inputs
+    counters = json.load(open(os.path.join(ROOT, "profiles", "counters.json")))
+    assert counters
+    for key, entry in counters.items():
+        name, gate_mode = key.split("/mode")
+        c = inputs.CONFIGS[name]
+        plan = mr.more_route_plan_ex(c["T"], c["h"], c["r"], c["M"], c["k"], int(gate_mode))
+        assert bench.counters_of(counters, name, int(gate_mode), plan) == entry, f"{key} was captured on {entry['kernel']}"
+        assert os.path.exists(os.path.join(ROOT, re.search(r"profiles/\S+\.md", entry["source"]).group()))
+        other = mr.more_route_plan_ex(2000, 64, 16, 64, 2)                 # too few experts for the chain, too few tokens for pairs
+        assert bench.counters_of(counters, name, int(gate_mode), other) == {}
