@@ -248,8 +248,14 @@ void plan_paired(int T, int h, int M, int msplit, int sm_count, Plan* p)
 // Launch plan of the fused standard router: one CTA per SM, 256-expert steps that each run over all h/64 k-tiles.  A
 // step costs the same whatever the block's fill (the MMAs are 128 tokens tall regardless), so what counts is waves x
 // steps per CTA; splitting the experts over a few CTAs per token block evens out the last wave.
-void plan_dense(int T, int h, int M, int msplit, int sm_count, Plan* p)
+void plan_dense(int T, int h, int M, int k, int msplit, int sm_count, Plan* p)
 {
+    // Microseconds on B200: 0.6 per k-tile of a step (its eight MMAs of 128 x 256 x 16 take 0.58), and by the length of the
+    // lists what a step's epilogue, a CTA (start, pipeline fill, first candidates, output) and the merge of parked lists cost
+    // on top.  Fitted to 3300 shapes (T = 1 ... 20000, h = 128 ... 4096, M = 280 ... 16384, k = 1 ... 32, both gates) at forced
+    // splits of 1 to 16: the split chosen costs 0.5 % on average against the best of them, 2 % with one set for all k from
+    // before a K-slice was one MMA of N = 256 (T = 500, h = 256, M = 1000, k = 8 55 us against 40).
+    const double epilogue = k <= 8 ? 2.0 : 7.0, start = k <= 8 ? 21.0 : (k <= 16 ? 40.0 : 60.0), merge = k <= 8 ? 7.0 : (k <= 16 ? 25.0 : 35.0);
     const int tiles = (M + 255) / 256;
     const double ktiles = (h + 63) / 64;
     double best = 1e300;
@@ -262,12 +268,7 @@ void plan_dense(int T, int h, int M, int msplit, int sm_count, Plan* p)
             const long long ctas = (long long)blocks * s;
             const double waves = (double)((ctas + sm_count - 1) / sm_count);
             const double steps = (double)((tiles + s - 1) / s);
-            // Microseconds, fitted to 990 shapes on B200 at forced splits of 1 to 16 (T = 64 ... 20000, h = 128 ... 4096,
-            // M = 256 ... 16384): 0.6 per k-tile of a step (its eight MMAs of 128 x 256 x 16 take 0.58), 4.7 for its epilogue,
-            // 21 per CTA for start, pipeline fill and output, 6 more when the lists are parked and merged.  The split chosen
-            // costs 0.3 % on average against the best of them, 2 % with the figures of the four MMAs of N = 64 (1.2, 2.1, 8,
-            // 25), which split too little: T = 500, h = 256, M = 1000 55 us against 40.
-            double cost = waves * (steps * (0.6 * ktiles + 4.7) + 21.0 + (s > 1 ? 6.0 : 0.0));
+            double cost = waves * (steps * (0.6 * ktiles + epilogue) + start + (s > 1 ? merge : 0.0));
             cost *= 1.0 + 0.02 * (kBlockTokens - bt) / 32.0;          // prefer full blocks on a tie
             if (cost < best * 0.999) { best = cost; best_bt = bt; best_s = s; }
         }
@@ -367,7 +368,7 @@ int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, b
     p.path = MORE_PATH_TCGEN05;
     if (sm_count <= 0) sm_count = 148;
     if (full) {
-        plan_dense(T, h, M, msplit, sm_count, &p);
+        plan_dense(T, h, M, k, msplit, sm_count, &p);
     } else {
         if (chain_wins(T, h, M, k, want_lse || gate_mode == MORE_GATE_FULL_SOFTMAX, sm_count)) {
             plan_chain(T, M, msplit, sm_count, &p);
