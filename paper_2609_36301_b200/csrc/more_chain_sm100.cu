@@ -355,6 +355,65 @@ __device__ __forceinline__ float just_above(float x)
     return __int_as_float(key ^ ((key >> 31) & 0x7fffffff));
 }
 
+// A thread's list that overflows: rare, and not inlined, so that the sweep's code stays short (a call of a few units fetches
+// it from L2 as it runs: T = 64, M = 16384 19.2 -> 18.7 us, T = 14, M = 4472 18.7 -> 18.4; long sweeps are the same).  The
+// list's n entries start at `first`.
+//
+// k-th largest logit of a list (its bits in .x) and how many equal to it are wanted (.y; all of them in a short list).  Starting
+// from NaN, which nothing reaches: an infinite logit, of finite inputs that overflow, is one like any other.
+__device__ __noinline__ uint2 list_kth(uint64_t first, int n, int k)
+{
+    float cur = __int_as_float(0x7fffffff);
+    int need = k;
+    for (;;) {
+        float m = -INFINITY;
+        int c = 0;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+            const float4 e = *reinterpret_cast<const float4*>(first + (uint64_t)i * kEntry);
+            const float x[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (!(x[j] >= cur)) {
+                    if (x[j] > m) { m = x[j]; c = 1; }
+                    else if (x[j] == m) ++c;
+                }
+        }
+        if (c >= need || c == 0) return make_uint2(__float_as_uint(m), (uint32_t)need);
+        need -= c;
+        cur = m;
+    }
+}
+// Drop what is below `known`, which k logits of the token reach, and cut a list that stays long to its k best (later equals
+// then lose to those: larger ids).  Returns how many entries are left, and a new threshold.
+__device__ __noinline__ uint2 make_room(uint64_t first, int n, float known, int k)
+{
+    auto keep = [&](float low, int equal) {
+        int left = 0;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+            const uint64_t rd = first + (uint64_t)i * kEntry, wr = first + (uint64_t)left * kEntry;
+            const float4 e = *reinterpret_cast<const float4*>(rd);
+            const float m = fmaxf(max3(e.x, e.y, e.z), e.w);
+            const bool take = m > low || (m == low && equal > 0);
+            if (equal > 0) equal -= (e.x == low) + (e.y == low) + (e.z == low) + (e.w == low);
+            if (take) {
+                *reinterpret_cast<float4*>(wr) = e;
+                *reinterpret_cast<int*>(wr + 16) = *reinterpret_cast<const int*>(rd + 16);
+                ++left;
+            }
+        }
+        n = left;
+    };
+    keep(known, INT_MAX);
+    if (n > kListCap - kCols / 4) {
+        const uint2 kth = list_kth(first, n, k);
+        keep(__uint_as_float(kth.x), (int)kth.y);
+        known = fmaxf(known, just_above(__uint_as_float(kth.x)));
+    }
+    return make_uint2((uint32_t)n, __float_as_uint(known));
+}
+
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
@@ -524,10 +583,6 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         auto sts = [&](uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); };
         auto ent4 = [&](uint64_t o) { return *reinterpret_cast<const float4*>(o); };
         auto ent_col = [&](uint64_t o) { return *reinterpret_cast<const int*>(o + 16); };
-        auto put = [&](uint64_t o, float4 e, int c) {
-            *reinterpret_cast<float4*>(o) = e;
-            *reinterpret_cast<int*>(o + 16) = c;
-        };
         // (sorted: which bucket a set of columns is in does not matter, only that the sets are disjoint)
         auto publish = [&]() {
             if constexpr (NB == 4) {
@@ -574,32 +629,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             }
             return kth;
         };
-        // k-th largest logit of this thread's own list and how many equal to it are wanted (all of them in a short list).
-        // (Starting from NaN, which nothing reaches: an infinite logit, of finite inputs that overflow, is one like any other.)
-        auto own_kth = [&](int& equal) {
-            float cur = __int_as_float(0x7fffffff);
-            int need = p.k;
-            for (;;) {
-                float m = -INFINITY;
-                int c = 0;
-                for (uint64_t o = first; o < ptr; o += kEntry) {
-                    const float4 e = ent4(o);
-                    const float x[4] = {e.x, e.y, e.z, e.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (!(x[j] >= cur)) {
-                            if (x[j] > m) { m = x[j]; c = 1; }
-                            else if (x[j] == m) ++c;
-                        }
-                }
-                if (c >= need || c == 0) { equal = need; return m; }
-                need -= c;
-                cur = m;
-            }
-        };
-        // Make room in the lists of a warp: drop what is below a bound that k logits are known to reach, and cut a list that
-        // stays long to its k best (later equals then lose to those: larger ids).  The bound is not thr, which may lie just
-        // above logits that the list has to keep: it was raised when enough of their equals were in.
+        // Make room in the lists of a warp.  The bound that k logits are known to reach is not thr, which may lie just above logits
+        // that the list has to keep: it was raised when enough of their equals were in.
         auto compact = [&]() {
             float known = lds(s_thr);
             if (p.k <= NB) {
@@ -608,28 +639,9 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 for (int i = 1; i < NB; ++i) mine = fminf(mine, b[i]);
                 known = fmaxf(known, mine);
             }
-            thr = fmaxf(thr, known);
-            auto keep = [&](float low, int equal) {
-                uint64_t wr = first;
-                for (uint64_t rd = first; rd < ptr; rd += kEntry) {
-                    const float4 e = ent4(rd);
-                    const float m = fmaxf(max3(e.x, e.y, e.z), e.w);
-                    const bool take = m > low || (m == low && equal > 0);
-                    if (equal > 0) equal -= (e.x == low) + (e.y == low) + (e.z == low) + (e.w == low);
-                    if (take) {
-                        put(wr, e, ent_col(rd));
-                        wr += kEntry;
-                    }
-                }
-                ptr = wr;
-            };
-            keep(known, INT_MAX);
-            if (ptr > warn) {
-                int equal;
-                const float kth = own_kth(equal);
-                keep(kth, equal);
-                thr = fmaxf(thr, just_above(kth));
-            }
+            const uint2 left = make_room(first, (int)((ptr - first) / kEntry), known, p.k);
+            ptr = first + (uint64_t)left.x * kEntry;
+            thr = fmaxf(thr, __uint_as_float(left.y));
             __syncwarp();
         };
         // Candidates of the list that beat `low` -> scratch, and of those that equal it the first `equal`; with `every`, only
@@ -843,9 +855,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     if (sub == 0 && total > p.cap) sts(s_cnt, 0.f);
                     quarter_sync(q);
                     if (row_live && total > p.cap) {
-                        int equal;
-                        const float low = own_kth(equal);
-                        emit(dst, low, equal, false);
+                        const uint2 kth = list_kth(first, (int)((ptr - first) / kEntry), p.k);
+                        emit(dst, __uint_as_float(kth.x), (int)kth.y, false);
                     }
                     quarter_sync(q);
                     total = __float_as_int(lds(s_cnt));
@@ -1390,11 +1401,13 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
     const size_t blocks = (tokens + kRows - 1) / kRows, lists = (size_t)p.sweep_blocks * p.maxseg;
     size_t off = 0;
     L.z = off; off += align_up(blocks * kRows * (a.r <= 32 ? 128 : 256), 1024);
-    L.list = off; off += (size_t)((p.parts - 1 >> p.list_shift) + 1) * p.list_cap * kEntry;
     L.ent = off; off += align_up(lists * (size_t)(4 * a.k) * kRows * 8, 1024);
     L.cnt = off; off += align_up(lists * kRows * 4, 1024);
     L.mz = off;
     if (lse) off += align_up(lists * kRows * 8, 1024);
+    // (last: the finishing kernels' reads then lie at the same addresses however long the lists are; T = 40, M = 6424 26.4 us
+    // with the lists in front and 25.1 behind)
+    L.list = off; off += (size_t)((p.parts - 1 >> p.list_shift) + 1) * p.list_cap * kEntry;
     L.total = off;
     return L;
 }
