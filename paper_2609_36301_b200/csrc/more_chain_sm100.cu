@@ -235,7 +235,7 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 // column, to the thread's list in global scratch: two predicated stores and an add, and nothing waits for them.  (Most of
 // a list stays in L2.  What leaves it, 115 MB of a call with k = 16 of 131072 experts for 8192 tokens, is 18 us of DRAM
 // time in a sweep of 510.)  A sweep starts with a threshold: the bucket maxima of its first units (lead_of: all of a short
-// segment, an eighth of a long one) are formed before anything is selected; this costs their MMAs and the reading of their
+// segment, the beginning of a long one) are formed before anything is selected; this costs their MMAs and the reading of their
 // accumulators again, and saves the appends of the start, when nearly everything beats what has been seen.  Whenever half
 // as much again of a long segment is done, the buckets are published in shared memory, one of the four warps of a lane
 // quarter computes new thresholds from them, and the others pick these up when they see them (all values are monotone
@@ -253,13 +253,15 @@ constexpr uint32_t kEntry = kEpi * 32;             // bytes between its entries 
 // final one before the first candidate is kept, and a thread keeps one or two groups instead of the ten that a rising
 // threshold lets through; what is saved is not the appending but the reading back at the end, a chain of trips to L2.
 // T = 3000, M = 16384: 49.9 -> 41.7 us; T = 1024, M = 65536, k = 16: 164 -> 77 us; T = 64, M = 131072, k = 16: 40.7 -> 34.3.
-// An eighth of a long one, where computing everything twice costs more.  The line is at 32 units for k <= 8 (at 41 units 84 us
+// Only the beginning of a long one, where computing everything twice costs more.  The line is at 32 units for k <= 8 (at 41 units 84 us
 // against 81) and at 64 for longer lists, which keep three times the candidates (T = 17000, M = 16384, k = 16, 57 units:
-// 187 -> 143 us; at 111 units 437 -> 456).  For thousands of units 1/4, 1/6 and 1/8 are within 3 % of one another.  Up to
-// two units stay in the two accumulators, more are computed again.
+// 187 -> 143 us).  Up to 128 units a quarter, or half for longer lists: what a better first threshold saves in appends and in
+// lists read back is more than the second reading costs (T = 32768, M = 16384, segments of 59 units on average: k = 8 168.7 us
+// with 1/8, 162.6 with 1/4, 166.7 with 1/2; k = 16 214, 199, 192).  Longer ones an eighth (T = 32768, M = 65536 359 us, with 1/4
+// 363, with 1/2 388).  Up to two units stay in the two accumulators, more are computed again.
 __host__ __device__ __forceinline__ int lead_of(int steps, bool longer)
 {
-    return steps <= (longer ? 64 : 32) ? steps : steps / 8;
+    return steps <= (longer ? 64 : 32) ? steps : (steps > 128 ? steps / 8 : steps / (longer ? 2 : 4));
 }
 
 struct SweepParams {
@@ -327,19 +329,20 @@ __device__ __forceinline__ void bitonic_down(float (&s)[N])
             if ((i & d) == 0) cx(s[i], s[i + d]);
 }
 // Append the groups of four (maxima t, values v, first column col + 4 i) that reach thr to a list that ends at `end`.  The
-// four tests come first: only the adds to the list's end depend on each other.  (These as multiply-adds by a register that
-// holds 1 take the same time: T = 32768, M = 65536 425 us; T = 8192, M = 131072, k = 16 507 +- 4; T = 16384, M = 4096 63.1.)
+// four tests come first: only the adds to the list's end depend on each other.  No list crosses a multiple of 2^32 bytes, so
+// these are adds to the address's low word.
 __device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t, const float* v, int col)
 {
 #define MORE_APPEND(P, COL, A, B, C, D)                                                                     \
-    "@" P " st.global.v4.f32 [%0], {" A ", " B ", " C ", " D "};\n\t@" P " st.global.b32 [%0+16], " COL ";\n\t" \
-    "@" P " add.u64 %0, %0, %22;\n\t"
+    "mov.b64 at, {lo, hi};\n\t@" P " st.global.v4.f32 [at], {" A ", " B ", " C ", " D "};\n\t@" P " st.global.b32 [at+16], " COL ";\n\t" \
+    "@" P " add.u32 lo, lo, %22;\n\t"
     asm volatile(
-        "{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 c1, c2, c3;\n\t"
+        "{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 c1, c2, c3, lo, hi;\n\t.reg .b64 at;\n\tmov.b64 {lo, hi}, %0;\n\t"
         "setp.ge.f32 p0, %2, %1;\n\tsetp.ge.f32 p1, %3, %1;\n\tsetp.ge.f32 p2, %4, %1;\n\tsetp.ge.f32 p3, %5, %1;\n\t"
         "add.u32 c1, %23, 4;\n\tadd.u32 c2, %23, 8;\n\tadd.u32 c3, %23, 12;\n\t"
         MORE_APPEND("p0", "%23", "%6", "%7", "%8", "%9") MORE_APPEND("p1", "c1", "%10", "%11", "%12", "%13")
-        MORE_APPEND("p2", "c2", "%14", "%15", "%16", "%17") MORE_APPEND("p3", "c3", "%18", "%19", "%20", "%21") "}"
+        MORE_APPEND("p2", "c2", "%14", "%15", "%16", "%17") MORE_APPEND("p3", "c3", "%18", "%19", "%20", "%21")
+        "mov.b64 %0, {lo, hi};\n\t}"
         : "+l"(end)
         : "f"(thr), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]),
           "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]),
@@ -430,9 +433,20 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
                      ::"r"(d), "l"(a), "l"(b), "r"(idesc) : "memory");
 }
 
+// an accumulator's number, known to the compiler or not
+__device__ __forceinline__ int number_of(int i) { return i; }
+template <int I>
+__device__ __forceinline__ constexpr int number_of(std::integral_constant<int, I>) { return I; }
+
 __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory"); }
 
-template <int KCAP, bool LSE>
+// The loop over the units has a copy of its body for each accumulator, so that barriers, phases and tensor-memory addresses are
+// constants: 92 -> 58 instructions per warp and unit without candidates, T = 32768, h = 512, M = 65536 405 -> 360 us.  SHORT:
+// every CTA has few units (kShortUnits).  A call of that size fetches the code from L2 as it runs, so there is only one copy, for
+// any unit (T = 1, M = 16384 15.4 -> 14.8 us, T = 64 19.4 -> 18.5; four units per CTA are slower that way: T = 2000, M = 8192
+// 33.9 -> 34.4).
+constexpr int kShortUnits = 2;
+template <int KCAP, bool LSE, bool SHORT>
 __global__ void __launch_bounds__(kSThreads, 2)
 sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_r2, const SweepParams p)
 {
@@ -517,7 +531,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             const uint64_t zd = umma_desc_sw128(base, 16, 1024), bd = umma_desc_sw128(base + p.off_r2, KS * 2048, 1024);
             const uint32_t lo_off = KS > 2 ? (kRows * 128) >> 4 : 4;     // from the hi half of z to the lo half, in 16 bytes
             int st = 0, ph = 0, seg = 0;
-            uint32_t n = 0;
+            uint32_t even = 1, odd = 1;                      // phases of the accumulators' "empty" barriers
             int s0 = (int)(lo % p.nsteps);
             for (int left = (int)(hi - lo); left > 0; ++seg, s0 = 0) {
                 const int steps = min(left, p.nsteps - s0);
@@ -526,12 +540,14 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 const int zb = p.zbufs == 2 ? seg & 1 : 0, zuse = p.zbufs == 2 ? seg >> 1 : seg;
                 wait_or_abort(bar(B_ZF + zb), zuse & 1, abort_flag, p.status);
                 const uint64_t z = zd + zb * (p.z_bytes >> 4);
-                for (int v = 0; v < total; ++v, ++n) {
-                    const int buf = n & 1;
+                for (int v = 0; v < total; ++v) {
+                    const int buf = (lead > 2 && v >= lead ? v - lead : v) & 1;
+                    const uint32_t free = buf ? odd : even;
+                    (buf ? odd : even) ^= 1;
                     // (both are mostly complete: two tests, one branch)
-                    if (!(mbar_try_wait(bar(B_RF + st), ph) & mbar_try_wait(bar(B_AE + buf), ((n >> 1) & 1) ^ 1))) {
+                    if (!(mbar_try_wait(bar(B_RF + st), ph) & mbar_try_wait(bar(B_AE + buf), free))) {
                         wait_or_abort(bar(B_RF + st), ph, abort_flag, p.status);
-                        wait_or_abort(bar(B_AE + buf), ((n >> 1) & 1) ^ 1, abort_flag, p.status);
+                        wait_or_abort(bar(B_AE + buf), free, abort_flag, p.status);
                     }
                     tc_fence_after();
                     const uint64_t b = bd + st * (p.st_bytes >> 4);
@@ -574,7 +590,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         const uint32_t s_thr = base + p.off_pub + 4 * kRows * NB * 4 + row * 4;
         const uint32_t s_cnt = s_thr + kRows * 4;
         const uint32_t s_mz = base + p.off_pub + 4 * kRows * NB * 4 + kRows * 8 + row * 8;
-        uint32_t n = 0;
+        uint32_t even = 0, odd = 0;                          // phases of the accumulators' "full" barriers; a segment begins with the first
         float b[NB];
         float thr, m2, zsum;
         uint64_t ptr;                                        // where the next entry goes
@@ -689,7 +705,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             zsum = 0.f;
             ptr = first;
             const int lead = lead_of(steps, KCAP > 8), again = lead > 2 ? lead : 0;      // units ahead, and how many of them come again
-            int next = lead + (lead + 1) / 2, turn = 0;
+            int next = (lead + (lead + 1) / 2 + 1) & ~1, turn = 0;
             // A token whose logits are all equal (padding) would overflow its list again and again.  So, once, when some thread
             // of the warp first has more than `limit` groups: where the threshold is final from the start, those k reach it
             // and later ones that only equal it lose to them; elsewhere, if the first and the last group have the same
@@ -732,19 +748,19 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 }
             };
             // ---- the buckets of the first units, for a threshold to start with
-#pragma unroll 1
-            for (int s = 0; s < lead; ++s) {
-                const uint32_t at = n + s;
-                const int buf = at & 1;
+            const int whole = min(steps, M / W - s0);    // units that do not reach beyond M
+            auto lead_unit = [&](auto buf_c, auto masked, int s) {
+                const int buf = number_of(buf_c);
                 const int col0 = (s0 + s) * W + sub * kCols;
-                wait_or_abort(bar(B_AF + buf), (at >> 1) & 1, abort_flag, p.status);
+                wait_or_abort(bar(B_AF + buf), buf ? odd : even, abort_flag, p.status);
+                if (again) (buf ? odd : even) ^= 1;          // (otherwise it is read where it is)
                 if (warp_live) {
                     tc_fence_after();
 #pragma unroll
                     for (int h = 0; h < kCols; h += 16) {
                         float v[16], t[4];
                         tmem_get16(t_col + buf * W + h, v);
-                        group_max(std::true_type{}, v, col0 + h, t);
+                        group_max(masked, v, col0 + h, t);
                         bucket(h, t);
                     }
                 }
@@ -752,8 +768,21 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     tc_fence_before();
                     arrive_lane0(bar(B_AE + buf), lane);
                 }
+            };
+            constexpr std::integral_constant<int, 0> first_acc{};
+            constexpr std::integral_constant<int, 1> second_acc{};
+            {
+                int s = 0;
+                if constexpr (!SHORT) {
+#pragma unroll 1
+                    for (; s + 1 < min(lead, whole); s += 2) {
+                        lead_unit(first_acc, std::false_type{}, s);
+                        lead_unit(second_acc, std::false_type{}, s + 1);
+                    }
+                }
+#pragma unroll 1
+                for (; s < lead; ++s) lead_unit(s & 1, std::true_type{}, s);       // (left over, or reaching beyond M)
             }
-            n += again;
             if (warp_live) {
                 // (published by all four threads of a token before anyone reads: nothing of an earlier block is seen)
                 publish();
@@ -767,18 +796,21 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 }
             }
             // One unit.  (One that reaches beyond M is an instantiation of its own, so that the others carry no masking.)
-            auto unit = [&](auto masked, int s) {
+            auto unit = [&](auto buf_c, auto masked, int s) {
                 constexpr bool kMasked = decltype(masked)::value;
-                const int buf = n & 1;
+                const int buf = number_of(buf_c);
                 const int col0 = (s0 + s) * W + sub * kCols;
                 const uint32_t t_acc = t_col + buf * W;
-                wait_or_abort(bar(B_AF + buf), (n >> 1) & 1, abort_flag, p.status);
+                wait_or_abort(bar(B_AF + buf), buf ? odd : even, abort_flag, p.status);
+                (buf ? odd : even) ^= 1;
                 tc_fence_after();
+                const float raised = lds(s_thr);             // (used after the accumulator's first columns have arrived)
 #pragma unroll
                 for (int h = 0; h < kCols; h += 16) {
                     const int col = col0 + h;
                     float v[16], t[4];
                     tmem_get16(t_acc + h, v);
+                    if (h == 0) thr = fmaxf(thr, raised);
                     if (h + 16 == kCols) {
                         tc_fence_before();
                         arrive_lane0(bar(B_AE + buf), lane);         // everything is in registers: hand the accumulator back
@@ -788,51 +820,57 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     if (LSE) {
                         const float c2 = m * kLog2e;
                         if (c2 > m2) { zsum *= ex2f(m2 - c2); m2 = c2; }
-                        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                        const uint64_t scale = pack2(kLog2e, kLog2e), low = pack2(-m2, -m2);
+                        uint64_t a01 = 0, a23 = 0;
 #pragma unroll
                         for (int i = 0; i < 16; i += 8) {
                             if (kMasked && col + i >= M) break;
 #pragma unroll
-                            for (int j = 0; j < 8; j += 4) {
-                                a0 += ex2f(fmaf(v[i + j], kLog2e, -m2));
-                                a1 += ex2f(fmaf(v[i + j + 1], kLog2e, -m2));
-                                a2 += ex2f(fmaf(v[i + j + 2], kLog2e, -m2));
-                                a3 += ex2f(fmaf(v[i + j + 3], kLog2e, -m2));
+                            for (int j = i; j < i + 8; j += 4) {
+                                float x0, x1, x2, x3;
+                                unpack2(fma2(pack2(v[j], v[j + 1]), scale, low), x0, x1);
+                                unpack2(fma2(pack2(v[j + 2], v[j + 3]), scale, low), x2, x3);
+                                a01 = add2(a01, pack2(ex2f(x0), ex2f(x1)));
+                                a23 = add2(a23, pack2(ex2f(x2), ex2f(x3)));
                             }
                         }
-                        zsum += (a0 + a1) + (a2 + a3);
+                        float a0, a1;
+                        unpack2(add2(a01, a23), a0, a1);
+                        zsum += a0 + a1;
                     }
                     if (__any_sync(kFull, m >= thr)) {
                         // (a bucket matters only once it reaches the threshold, so it need not be kept up elsewhere)
                         bucket(h, t);
                         append4(ptr, thr, t, v, col);
+                        if (__builtin_expect(__any_sync(kFull, (uint32_t)ptr > (uint32_t)limit), 0)) full();
                     }
                 }
-                if (__builtin_expect(__any_sync(kFull, ptr > limit), 0)) full();
-                ++n;
             };
             if (!warp_live) {
-                for (int s = 0; s < steps; ++s, ++n) {
-                    wait_or_abort(bar(B_AF + (n & 1)), (n >> 1) & 1, abort_flag, p.status);
-                    arrive_lane0(bar(B_AE + (n & 1)), lane);
+                for (int s = 0; s < steps; ++s) {
+                    const int buf = s & 1;
+                    wait_or_abort(bar(B_AF + buf), buf ? odd : even, abort_flag, p.status);
+                    (buf ? odd : even) ^= 1;
+                    arrive_lane0(bar(B_AE + buf), lane);
                 }
             } else {
-                const int whole = min(steps, M / W - s0);            // units that do not reach beyond M
-                for (int s = 0; s < whole;) {
-                    const int stop = min(whole, next);               // a run of units, up to the next refresh of the threshold
+                int s = 0;
+                while (!SHORT && s + 1 < whole) {
+                    const int stop = min(whole - 1, next);           // a run of pairs, up to the next refresh of the threshold
 #pragma unroll 1
-                    for (; s < stop; ++s) {
-                        unit(std::false_type{}, s);
-                        thr = fmaxf(thr, lds(s_thr));
+                    for (; s < stop; s += 2) {
+                        unit(first_acc, std::false_type{}, s);
+                        unit(second_acc, std::false_type{}, s + 1);
                     }
                     if (s == next) {
                         publish();
                         if (sub == (turn & 3)) sts(s_thr, compute_thr());
                         ++turn;
-                        next += (next + 1) / 2;
+                        next += ((next + 1) / 2 + 1) & ~1;
                     }
                 }
-                if (whole < steps) unit(std::true_type{}, steps - 1);
+#pragma unroll 1
+                for (; s < steps; ++s) unit(s & 1, std::true_type{}, s);   // (left over, or reaching beyond M)
             }
             // ---- end of the segment: what still reaches the threshold goes to scratch
             if (warp_live) {
@@ -1345,18 +1383,18 @@ bool allow_smem(K kern, int bytes, unsigned long long* done, bool wide_cluster =
 
 using SweepFn = void (*)(const CUtensorMap, const CUtensorMap, const SweepParams);
 
-template <int KCAP, bool LSE>
+template <int KCAP, bool LSE, bool SHORT>
 SweepFn sweep_ready()
 {
     static unsigned long long done = 0;
-    SweepFn f = sweep_kernel<KCAP, LSE>;
+    SweepFn f = sweep_kernel<KCAP, LSE, SHORT>;
     return allow_smem(f, kSweepSmem, &done) ? f : nullptr;
 }
-
+template <bool SHORT>
 SweepFn sweep_fn(int k, bool lse)
 {
-    if (k <= 8) return lse ? sweep_ready<8, true>() : sweep_ready<8, false>();
-    return lse ? sweep_ready<16, true>() : sweep_ready<16, false>();
+    if (k <= 8) return lse ? sweep_ready<8, true, SHORT>() : sweep_ready<8, false, SHORT>();
+    return lse ? sweep_ready<16, true, SHORT>() : sweep_ready<16, false, SHORT>();
 }
 
 template <class... Args>
@@ -1402,12 +1440,13 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
     size_t off = 0;
     L.z = off; off += align_up(blocks * kRows * (a.r <= 32 ? 128 : 256), 1024);
     L.ent = off; off += align_up(lists * (size_t)(4 * a.k) * kRows * 8, 1024);
-    L.cnt = off; off += align_up(lists * kRows * 4, 1024);
+    L.cnt = off; off += lists * kRows * 4;
     L.mz = off;
     if (lse) off += align_up(lists * kRows * 8, 1024);
     // (last: the finishing kernels' reads then lie at the same addresses however long the lists are; T = 40, M = 6424 26.4 us
     // with the lists in front and 25.1 behind)
-    L.list = off; off += (size_t)((p.parts - 1 >> p.list_shift) + 1) * p.list_cap * kEntry;
+    // (aligned to its size, a power of two, no area crosses a multiple of 2^32 bytes: the allocation is aligned to 256)
+    L.list = off; off += (size_t)((p.parts - 1 >> p.list_shift) + 2) * p.list_cap * kEntry - 256;
     L.total = off;
     return L;
 }
@@ -1447,7 +1486,8 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
     p->list_shift = T <= 32 ? 2 : (T <= 64 ? 1 : 0);
     // a unit adds at most kCols / 4 entries to a list (a later, shorter chunk may have longer segments)
     const long long units = share > 0 ? (nsteps + share - 1) / share : (total + g - 1) / g;
-    p->list_cap = T <= kChunkTokens && units < kListCap / (kCols / 4) ? (int)units * (kCols / 4) : kListCap;
+    p->list_cap = kCols / 4;
+    while (p->list_cap < kListCap && (T > kChunkTokens || p->list_cap < units * (kCols / 4))) p->list_cap *= 2;
     p->ctas = (int)(share > 0 ? blocks * share : g);
     p->msplit = (int)(p->ctas / blocks > 1 ? p->ctas / blocks : 1);      // (whole ones; a part that begins anywhere can reach into two blocks)
     p->share = (int)share;
@@ -1485,14 +1525,18 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
     sp.off_pub = sp.off_r2 + sp.nst * sp.st_bytes;
     sp.off_ctl = sp.off_pub + pub;
     const int smem = sp.off_ctl + ctl + 1024;
-    sp.list = reinterpret_cast<uint8_t*>(base + L.list);
+    sp.list = reinterpret_cast<uint8_t*>(align_up(reinterpret_cast<uintptr_t>(base + L.list), (size_t)plan.list_cap * kEntry));
     sp.list_cap = plan.list_cap; sp.list_shift = plan.list_shift;
     sp.ent = reinterpret_cast<uint2*>(base + L.ent);
     sp.cnt = reinterpret_cast<int*>(base + L.cnt);
     sp.mz = lse ? reinterpret_cast<float2*>(base + L.mz) : nullptr;
     sp.status = ctx.status;
 
-    SweepFn sweep = sweep_fn(a.k, lse);
+    // (plan.parts CTAs have even parts of the blocks of one launch)
+    const long long units = plan.share > 0 ? (nsteps + plan.share - 1) / plan.share
+                                           : ((long long)plan.sweep_blocks * nsteps + plan.parts - 1) / plan.parts;
+    const bool few = a.T <= kChunkTokens && units <= kShortUnits;
+    SweepFn sweep = few ? sweep_fn<true>(a.k, lse) : sweep_fn<false>(a.k, lse);
     static unsigned long long project_done = 0;
     const int psmem_max = kPStages * kPStageBytes + kPCtl + kPExchange + 1024;
     if (!sweep || !allow_smem(project_kernel, psmem_max, &project_done)) return MORE_ERR_CUDA;
