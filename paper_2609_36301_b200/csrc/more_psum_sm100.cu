@@ -20,6 +20,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 namespace more {
 
 namespace {
@@ -42,6 +44,7 @@ __device__ __forceinline__ void tmem_get16(uint32_t taddr, float (&v)[16])
 
 struct PsumParams {
     int T, h, r, M, msplit, tiles_total;
+    int block;           // tokens of a block: a multiple of 32, 160 ... 256 (what a CTA computes z for beyond them is not used)
     const float* lse;    // [T] natural-log log-sum-exp of every token's logits
     float* psum;         // [M], zeroed before the launch
     int* status;
@@ -77,7 +80,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int blk = blockIdx.x / p.msplit, split = blockIdx.x % p.msplit;
-    const int tok0 = blk * kBlockTokens;
+    const int tok0 = blk * p.block;
     const int tile_lo = (int)(((long long)p.tiles_total * split) / p.msplit);
     const int tile_hi = (int)(((long long)p.tiles_total * (split + 1)) / p.msplit);
     const int ntiles = tile_hi - tile_lo;
@@ -163,6 +166,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         if (ok) tc_commit_elect(bar(B_ZACC));
         ok = __all_sync(kFull, ok && mbar_wait(bar(B_ZOP), 0, abort_flag, p.status));
         tc_fence_after();
+        const uint32_t idesc_tail = (idesc2 & ~(0x3fu << 17)) | ((uint32_t)((p.block - 128) >> 3) << 17);    // the second half's tokens
         const uint64_t ad0 = umma_desc_sw128(r2ring, RPAD * 128, 1024), zd0 = umma_desc_sw128(zop, 16, 1024);
         const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32), z_lo0 = (uint32_t)zd0, z_hi = (uint32_t)(zd0 >> 32);
         for (int it = 0; it < ntiles && ok; ++it) {
@@ -179,8 +183,8 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 for (int j = 0; j < 2 * kKSteps; ++j) {
                     const uint32_t zbyte = j * 32;                                       // K offset in [hi | lo]
                     tc_mma_bf16_ss_elect(tmem_base + a * 128, a_lo + (j % kKSteps) * (2048 >> 4), a_hi,
-                                         z_lo0 + ((a * kZopOne + (zbyte >> 7) * 16384 + (zbyte & 127)) >> 4), z_hi, idesc2,
-                                         j != 0);
+                                         z_lo0 + ((a * kZopOne + (zbyte >> 7) * 16384 + (zbyte & 127)) >> 4), z_hi,
+                                         a == 0 ? idesc2 : idesc_tail, j != 0);
                 }
                 tc_commit_elect(bar(B_ACCF + a));
             }
@@ -191,7 +195,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         // ========================================================================================= epilogue
         const int q = warp & 3;                              // TMEM lane group: token rows (phase 1), experts (phase 2)
         const int half = ((warp - 2) >> 2) & 1;              // which 128-token half
-        const int part = (warp - 2) >> 3;                    // which 64 of its columns
+        const int part = (warp - 2) >> 3;                    // which half of its columns
         const int row_in_half = q * 32 + lane;
         const int row_in_blk = half * 128 + row_in_half;
         const int64_t row = (int64_t)tok0 + row_in_blk;
@@ -201,7 +205,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             tc_fence_after();
             // (the phase-1 ring is free now) minus the log2-scaled log-sum-exp of my token; -inf for rows past T, whose
             // zero-filled logits then contribute exp(-inf) = 0
-            lse2[row_in_blk] = (row < p.T) ? -p.lse[row] * kLog2e : -INFINITY;
+            lse2[row_in_blk] = (row < p.T && row_in_blk < p.block) ? -p.lse[row] * kLog2e : -INFINITY;
             uint8_t* zrow = ring_ptr + half * kZopOne + row_in_half * 128;
 #pragma unroll
             for (int c = 0; c < RPAD / 16; ++c) {
@@ -234,39 +238,48 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         asm volatile("bar.sync 1, 512;" ::: "memory");
 
         ok = __all_sync(0xffffffffu, ok);
-        const ulonglong2* lse4 = reinterpret_cast<const ulonglong2*>(lse2 + half * 128 + part * 64);
-        const uint64_t scale = pack2(kLog2e, kLog2e);
-        for (int it = 0; it < ntiles && ok; ++it) {
-            const int expert = (tile_lo + it) * kTileExperts + q * 32 + lane;     // my lane's expert in this tile
-            ok = __all_sync(0xffffffffu, mbar_wait(bar(B_ACCF + half), it & 1, abort_flag, p.status));
-            if (!ok) break;
-            tc_fence_after();
-            uint64_t acc01 = 0, acc23 = 0;
+        // The sweep, for a number of 16-column chunks that the compiler knows.
+        auto sweep = [&](auto chunks_c) {
+            constexpr int kChunks = decltype(chunks_c)::value;
+            const ulonglong2* lse4 = reinterpret_cast<const ulonglong2*>(lse2 + half * 128 + part * kChunks * 16);
+            const uint64_t scale = pack2(kLog2e, kLog2e);
+            for (int it = 0; it < ntiles && ok; ++it) {
+                const int expert = (tile_lo + it) * kTileExperts + q * 32 + lane;     // my lane's expert in this tile
+                ok = __all_sync(0xffffffffu, mbar_wait(bar(B_ACCF + half), it & 1, abort_flag, p.status));
+                if (!ok) break;
+                tc_fence_after();
+                uint64_t acc01 = 0, acc23 = 0;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float v[16];
-                tmem_get16(t_lane + part * 64 + c * 16, v);
-                if (c == 3) {                                    // all columns are in registers: hand the accumulator back
-                    tc_fence_before();
-                    warp_arrive(bar(B_ACCE + half), lane);
-                }
+                for (int c = 0; c < kChunks; ++c) {
+                    float v[16];
+                    tmem_get16(t_lane + (part * kChunks + c) * 16, v);
+                    if (c + 1 == kChunks) {                      // all columns are in registers: hand the accumulator back
+                        tc_fence_before();
+                        warp_arrive(bar(B_ACCE + half), lane);
+                    }
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const ulonglong2 l = lse4[c * 4 + g];        // same address in every lane: a broadcast
-                    float x0, x1, x2, x3;
-                    unpack2(fma2(pack2(v[4 * g], v[4 * g + 1]), scale, l.x), x0, x1);
-                    unpack2(fma2(pack2(v[4 * g + 2], v[4 * g + 3]), scale, l.y), x2, x3);
-                    // (one exponential in four on the FMA pipe: the special-function unit's 16 results per clock per SM
-                    // are this loop's narrowest resource)
-                    acc01 = add2(acc01, pack2(ex2f(x0), ex2f(x1)));
-                    acc23 = add2(acc23, pack2(ex2f(x2), ex2_poly(x3)));
+                    for (int g = 0; g < 4; ++g) {
+                        const ulonglong2 l = lse4[c * 4 + g];    // same address in every lane: a broadcast
+                        float x0, x1, x2, x3;
+                        unpack2(fma2(pack2(v[4 * g], v[4 * g + 1]), scale, l.x), x0, x1);
+                        unpack2(fma2(pack2(v[4 * g + 2], v[4 * g + 3]), scale, l.y), x2, x3);
+                        // (one exponential in four on the FMA pipe: the special-function unit's 16 results per clock per SM
+                        // are this loop's narrowest resource)
+                        acc01 = add2(acc01, pack2(ex2f(x0), ex2f(x1)));
+                        acc23 = add2(acc23, pack2(ex2f(x2), ex2_poly(x3)));
+                    }
                 }
+                float a0, a1, a2, a3;
+                unpack2(acc01, a0, a1);
+                unpack2(acc23, a2, a3);
+                if (expert < p.M) atomicAdd(p.psum + expert, (a0 + a1) + (a2 + a3));
             }
-            float a0, a1, a2, a3;
-            unpack2(acc01, a0, a1);
-            unpack2(acc23, a2, a3);
-            if (expert < p.M) atomicAdd(p.psum + expert, (a0 + a1) + (a2 + a3));
-        }
+        };
+        const int chunks = half == 0 ? 4 : (p.block - 128) / 32;
+        if (chunks == 4) sweep(std::integral_constant<int, 4>{});
+        else if (chunks == 3) sweep(std::integral_constant<int, 3>{});
+        else if (chunks == 2) sweep(std::integral_constant<int, 2>{});
+        else sweep(std::integral_constant<int, 1>{});
     }
 
     tc_fence_before();
@@ -314,12 +327,26 @@ int launch_psum_tcgen05(const __nv_bfloat16* X, const __nv_bfloat16* R1, const _
     pp.T = T; pp.h = h; pp.r = r; pp.M = M;
     pp.tiles_total = (M + kTileExperts - 1) / kTileExperts;
     pp.lse = lse; pp.psum = psum; pp.status = ctx.status;
-    const int blocks = (T + kBlockTokens - 1) / kBlockTokens;
+    // Tokens of a block, and CTAs per block: what fills the waves of resident CTAs (two per SM) best.  A CTA's time is that of
+    // its 16-token chunks x tiles, and what every one pays at its start (256 rows of X per k-tile, narrowing) is worth about
+    // 300 + 4 h / 64 of those; each keeps four expert tiles or more.  T = 65536, h = 512, M = 8192: 256 blocks of 256 tokens
+    // give 108 SMs two CTAs and 40 one, 293 of 224 give all of them two: 171 -> 160 us; T = 40000, h = 4096, M = 4096 157 blocks
+    // or 250 of 160: 149 -> 128; T = 512, M = 1024 (192 tokens) 14.3 -> 12.8; T = 3001, M = 5000 27.1 with 256 and 27.8 with 224.
     const int slots = 2 * (ctx.sm_count > 0 ? ctx.sm_count : 148);
-    int s = slots / blocks;                       // fill one wave of resident CTAs; each keeps >= 4 expert tiles
-    if (s > pp.tiles_total / 4) s = pp.tiles_total / 4;
-    if (s < 1) s = 1;
-    if (s > 64) s = 64;
+    double best = 1e300;
+    int blocks = 0, s = 1;
+    for (int block = kBlockTokens; block >= 160; block -= 32) {
+        const int n = (T + block - 1) / block;
+        int split = slots / n;
+        if (split > pp.tiles_total / 4) split = pp.tiles_total / 4;
+        if (split < 1) split = 1;
+        if (split > 64) split = 64;
+        const long long ctas = (long long)n * split, waves = (ctas + slots - 1) / slots;
+        // the last wave's CTAs have an SM each if there are no more of them
+        const double last = 2 * (ctas - (waves - 1) * slots) <= slots ? 0.6 : 1.0;
+        const double cost = ((double)waves - 1.0 + last) * (block / 16.0 * ((pp.tiles_total + split - 1) / split) + 300.0 + 4.0 * (h / 64));
+        if (cost < best * 0.97) { best = cost; blocks = n; s = split; pp.block = block; }
+    }
     pp.msplit = s;
     switch (rpad) {
         case 16: return launch_psum_rpad<16>(mx, m1, m2, pp, blocks * s, stream);
