@@ -44,7 +44,7 @@ constexpr int kPExchange = kRows * 64 * 4;         // [rank][row share][64] fp32
 constexpr int kPCtl = 1024;
 
 struct ProjectParams {
-    int T, h, cs, n, zc;                           // n: columns of z computed (16, 32, 48, 64); zc: bf16 per row of z
+    int T, h, cs, cs_bits, n, zc;                           // n: columns of z computed (16, 32, 48, 64); zc: bf16 per row of z
     uint32_t* z;                                   // [blocks * 128][zc / 2]
     int32_t* counts;                               // cleared here: [M] (null for the later chunks of one call)
     int M;
@@ -75,9 +75,9 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cs = p.cs, rank = blockIdx.x % cs, blk = blockIdx.x / cs;
+    const int cs = p.cs, rank = blockIdx.x & (cs - 1), blk = blockIdx.x >> p.cs_bits;
     const int nkt = (p.h + 63) / 64;
-    const int kt_lo = nkt * rank / cs, kt_hi = nkt * (rank + 1) / cs;
+    const int kt_lo = nkt * rank >> p.cs_bits, kt_hi = nkt * (rank + 1) >> p.cs_bits;
     const int live = min(kRows, p.T - blk * kRows);
 
     if (threadIdx.x == 0) {
@@ -162,8 +162,8 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 }
             }
         } else if (ok && row - lane < live) {      // (rows past the last token are not exchanged)
-            const int share = kRows / cs, dst = row / share;
-            const uint32_t a = smem_u32(exch) + (uint32_t)((rank * share + row % share) * 64) * 4u;
+            const int share = kRows >> p.cs_bits, dst = row >> (7 - p.cs_bits);
+            const uint32_t a = smem_u32(exch) + (uint32_t)((rank * share + (row & (share - 1))) * 64) * 4u;
             uint32_t remote;
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(a), "r"(dst));
             for (int c = 0; c * 16 < p.n; ++c) {
@@ -183,7 +183,7 @@ project_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if (cs > 1) {
         cluster_sync();
         if (warp >= 2) {
-            const int share = kRows / cs, q4_bits = p.zc == 64 ? 3 : 4, q4 = 1 << q4_bits;        // float4s of one row of z
+            const int share = kRows >> p.cs_bits, q4_bits = p.zc == 64 ? 3 : 4, q4 = 1 << q4_bits;        // float4s of one row of z
             // Rows past the last token, up to the 32 that a warp of the sweep looks at, are zero.  (What an earlier call left
             // there would be swept as tokens whose logits can be infinite, reach any threshold and fill their lists again
             // and again: T = 7284, M = 16384 2330 us instead of 83.)
@@ -264,10 +264,29 @@ __host__ __device__ __forceinline__ int lead_of(int steps, bool longer)
     return steps <= (longer ? 64 : 32) ? steps : (steps > 128 ? steps / 8 : steps / (longer ? 2 : 4));
 }
 
+// The line of units and the CTAs that share it.  Every warp of a CTA starts by dividing, in code that is fetched as it runs: by
+// multiplication with inverses from the host where total g fits 32 bits (inv_total = 0 where it does not).  With four 64-bit
+// divisions T = 64, h = 4096, M = 131072, k = 16 took 36.3 us, with these 33.9, T = 1, M = 16384 14.6 and 13.8.
+struct Cut {
+    long long total;                               // units
+    int nsteps, g;                                 // units per token block; CTAs
+    uint32_t inv_total, inv_nsteps, inv_g;
+};
+Cut make_cut(long long total, int nsteps, int g)
+{
+    Cut t{total, nsteps, g, 0, 0, 0};
+    if (total < (1ll << 32) / g) {                 // (then total g < 2^32)
+        t.inv_total = 0xffffffffu / (uint32_t)total;
+        t.inv_nsteps = 0xffffffffu / (uint32_t)nsteps;
+        t.inv_g = 0xffffffffu / (uint32_t)g;
+    }
+    return t;
+}
+
 struct SweepParams {
     int T, M, k;
-    int nsteps, ks, rk, wide;                      // steps per token block; K-steps per half; rows of an R2 box; r > 32
-    long long total;                               // units
+    Cut cut;
+    int ks, rk, wide;                              // K-steps per half; rows of an R2 box; r > 32
     int maxseg, cap;                               // candidate lists per token block in scratch, entries per list and token
     int nst, st_bytes, zbufs, z_bytes;
     int off_r2, off_pub, off_ctl;
@@ -279,8 +298,35 @@ struct SweepParams {
     int* status;
 };
 
-// CTA that owns unit u when `total` units are cut into g parts, part c = [total c / g, total (c + 1) / g)
-__host__ __device__ __forceinline__ int owner_of(long long u, long long total, int g) { return (int)(((u + 1) * g - 1) / total); }
+__device__ __forceinline__ uint32_t divide(uint32_t x, uint32_t d, uint32_t inv)        // x / d, inv = (2^32 - 1) / d
+{
+    const uint32_t q = __umulhi(x, inv);           // x / d or one less
+    return x - q * d >= d ? q + 1 : q;
+}
+// CTA that owns unit u; the part of CTA c, [total c / g, total (c + 1) / g), as a block, a step in it and a count; which segment
+// of that block its first one is.
+__device__ __noinline__ int wide_owner(long long total, int g, long long u) { return (int)(((u + 1) * g - 1) / total); }
+__device__ __forceinline__ int owner_of(const Cut& t, long long u)
+{
+    return t.inv_total ? (int)divide((uint32_t)(u + 1) * (uint32_t)t.g - 1u, (uint32_t)t.total, t.inv_total) : wide_owner(t.total, t.g, u);
+}
+struct Part {
+    int blk, s0, units, seg;
+};
+__device__ __noinline__ Part wide_part(long long total, int g, int nsteps, int c)
+{
+    const long long lo = total * c / g, hi = total * (c + 1) / g;
+    const int blk = (int)(lo / nsteps), s0 = (int)(lo - (long long)blk * nsteps);
+    return Part{blk, s0, (int)(hi - lo), s0 == 0 ? 0 : c - wide_owner(total, g, lo - s0)};
+}
+__device__ __forceinline__ Part part_of(const Cut& t, int c)
+{
+    if (!t.inv_total) return wide_part(t.total, t.g, t.nsteps, c);
+    const uint32_t total = (uint32_t)t.total, g = (uint32_t)t.g, n = (uint32_t)t.nsteps;
+    const uint32_t lo = divide(total * (uint32_t)c, g, t.inv_g), hi = divide(total * (uint32_t)(c + 1), g, t.inv_g);
+    const uint32_t blk = divide(lo, n, t.inv_nsteps), s0 = lo - blk * n;
+    return Part{(int)blk, (int)s0, (int)(hi - lo), s0 == 0 ? 0 : c - owner_of(t, blk * n)};
+}
 
 // 16 consecutive fp32 columns of this thread's tensor-memory lane, complete on return.  (Load and wait in one statement:
 // with the destination registers tied to a separate wait the compiler copies them.)
@@ -464,8 +510,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
     const int warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // (the compiler sees a uniform value)
-    const int g = (int)gridDim.x;
-    const long long lo = p.total * blockIdx.x / g, hi = p.total * (blockIdx.x + 1) / g;
+    const Part part = part_of(p.cut, (int)blockIdx.x);
+    const int nsteps = p.cut.nsteps;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < B_AE; ++i) mbar_init(bar(i), 1);
@@ -499,9 +545,9 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     tma_load_2d(r2 + st * p.st_bytes + j * p.rk * 128, &map_r2, bar(B_RF + st), step * W + j * 64, 0);
                 if (++st == p.nst) { st = 0; ph ^= 1; }
             };
-            int blk = (int)(lo / p.nsteps), s0 = (int)(lo - (long long)blk * p.nsteps), seg = 0;
-            for (int left = (int)(hi - lo); left > 0 && ok; ++blk, ++seg, s0 = 0) {
-                const int steps = min(left, p.nsteps - s0);
+            int blk = part.blk, s0 = part.s0, seg = 0;
+            for (int left = part.units; left > 0 && ok; ++blk, ++seg, s0 = 0) {
+                const int steps = min(left, nsteps - s0);
                 left -= steps;
                 const int lead = lead_of(steps, KCAP > 8), total = steps + (lead > 2 ? lead : 0);
                 auto step_of = [&](int v) { return s0 + (v >= lead && lead > 2 ? v - lead : v); };
@@ -532,9 +578,9 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             const uint32_t lo_off = KS > 2 ? (kRows * 128) >> 4 : 4;     // from the hi half of z to the lo half, in 16 bytes
             int st = 0, ph = 0, seg = 0;
             uint32_t even = 1, odd = 1;                      // phases of the accumulators' "empty" barriers
-            int s0 = (int)(lo % p.nsteps);
-            for (int left = (int)(hi - lo); left > 0; ++seg, s0 = 0) {
-                const int steps = min(left, p.nsteps - s0);
+            int s0 = part.s0;
+            for (int left = part.units; left > 0; ++seg, s0 = 0) {
+                const int steps = min(left, nsteps - s0);
                 left -= steps;
                 const int lead = lead_of(steps, KCAP > 8), total = steps + (lead > 2 ? lead : 0);
                 const int zb = p.zbufs == 2 ? seg & 1 : 0, zuse = p.zbufs == 2 ? seg >> 1 : seg;
@@ -576,7 +622,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         const int q = warp & 3;                              // tensor-memory lane quarter
         const int sub = (warp - 2) >> 2;                     // column quarter
         const int row = q * 32 + lane;                       // token of the block
-        const int M = p.M, nsteps = p.nsteps;
+        const int M = p.M;
         const uint32_t t_col = tmem_base + ((uint32_t)(q * 32) << 16) + sub * kCols;
         // the thread's list; a unit adds at most 8 entries between two looks at its length
         // (A list shorter than kListCap is one that so few units cannot fill.  Where only one or two quarters of the block hold
@@ -663,18 +709,20 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         // Candidates of the list that beat `low` -> scratch, and of those that equal it the first `equal`; with `every`, only
         // while fewer than `equal` have been passed on at all: where k of this thread are not below `low`, later equals lose.
         auto emit = [&](uint2* dst, float low, int equal, bool every) {
-            constexpr int U = 4;                             // (independent loads: one round trip for four entries)
+            constexpr int U = 4;                             // (independent loads: one round trip for four entries, columns and all;
+                                                             // a trip for each column cost 2 % of most sweeps)
             for (uint64_t o = first; o < ptr; o += U * kEntry) {
                 float4 e[U];
+                int c[U];
 #pragma unroll
                 for (int i = 0; i < U; ++i) {
                     e[i] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                    if (o + i * kEntry < ptr) e[i] = ent4(o + i * kEntry);
+                    c[i] = 0;
+                    if (o + i * kEntry < ptr) { e[i] = ent4(o + i * kEntry); c[i] = ent_col(o + i * kEntry); }
                 }
 #pragma unroll
                 for (int i = 0; i < U; ++i) {
                     if (!(fmaxf(max3(e[i].x, e[i].y, e[i].z), e[i].w) >= low) || o + i * kEntry >= ptr) continue;
-                    const int c = ent_col(o + i * kEntry);
                     const float x[4] = {e[i].x, e[i].y, e[i].z, e[i].w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -683,7 +731,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                             equal -= eq || every ? 1 : 0;
                             int at;
                             asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(at) : "r"(s_cnt) : "memory");
-                            if (at < p.cap) dst[at] = make_uint2(__float_as_uint(x[j]), (uint32_t)(c + j));
+                            if (at < p.cap) dst[at] = make_uint2(__float_as_uint(x[j]), (uint32_t)(c[i] + j));
                         }
                     }
                 }
@@ -691,8 +739,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         };
 
         // (units of this CTA as a block, a step in it and a count: 32-bit loop state)
-        int blk = (int)(lo / nsteps), s0 = (int)(lo - (long long)blk * nsteps);
-        for (int left = (int)(hi - lo); left > 0; ++blk, s0 = 0) {
+        int blk = part.blk, s0 = part.s0;
+        for (int left = part.units; left > 0; ++blk, s0 = 0) {
             const int steps = min(left, nsteps - s0);
             left -= steps;
             const int live = min(kRows, p.T - blk * kRows);
@@ -881,7 +929,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(s_mz + (sub - 1) * (kRows * 8)), "f"(m2), "f"(zsum) : "memory");
                 quarter_sync(q);
                 const float low = fmaxf(final ? lds(s_thr) : compute_thr(), -FLT_MAX);
-                const int seg = (int)blockIdx.x - owner_of((long long)blk * nsteps, p.total, g);
+                const int seg = blk == part.blk ? part.seg : 0;
                 const size_t slot = (size_t)blk * p.maxseg + seg;
                 uint2* dst = p.ent + (slot * kRows + row) * p.cap;
                 if (row_live) emit(dst, low, p.k, true);
@@ -935,8 +983,8 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
 // ================================================================================================= finish
 struct FinishParams {
     int T, M, k, gate_mode;
-    int nsteps, g, share, maxseg, cap;
-    long long total;
+    int share, maxseg, cap;
+    Cut cut;
     const uint2* ent;
     const int* cnt;
     const float2* mz;
@@ -959,8 +1007,8 @@ __device__ __forceinline__ void join_mz(float& m, float& z, float om, float oz)
 __device__ __forceinline__ int segments_of(const FinishParams& p, int blk)
 {
     if (p.share > 0) return p.share;
-    const long long u0 = (long long)blk * p.nsteps;
-    return owner_of(u0 + p.nsteps - 1, p.total, p.g) - owner_of(u0, p.total, p.g) + 1;
+    const long long u0 = (long long)blk * p.cut.nsteps;
+    return owner_of(p.cut, u0 + p.cut.nsteps - 1) - owner_of(p.cut, u0) + 1;
 }
 __device__ __forceinline__ Cand load_cand(const uint2* at)
 {
@@ -1510,7 +1558,7 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
 
     SweepParams sp{};
     const int nsteps = (a.M + W - 1) / W;
-    sp.M = a.M; sp.k = a.k; sp.nsteps = nsteps; sp.ks = n16 / 16; sp.rk = n16; sp.wide = a.r > 32;
+    sp.M = a.M; sp.k = a.k; sp.ks = n16 / 16; sp.rk = n16; sp.wide = a.r > 32;
     sp.maxseg = plan.maxseg; sp.cap = 4 * a.k;
     sp.st_bytes = W * n16 * 2;
     sp.z_bytes = kRows * zc * 2;
@@ -1562,7 +1610,7 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
         pp.status = ctx.status;
         pp.cs = 1;
         const int nkt = (a.h + 63) / 64;
-        while (pp.cs < 8 && 2 * pp.cs * blocks <= sms && nkt >= 4 * pp.cs) pp.cs *= 2;
+        while (pp.cs < 8 && 2 * pp.cs * blocks <= sms && nkt >= 4 * pp.cs) { pp.cs *= 2; ++pp.cs_bits; }
         const int psmem = psmem_max - (pp.cs == 1 ? kPExchange : 0);
         if (launch(project_kernel, blocks * pp.cs, kPThreads, psmem, a.stream, true, pp.cs, mx, mr1, pp) != cudaSuccess)
             return MORE_ERR_CUDA;
@@ -1575,18 +1623,19 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
             if (b0 > 0) rc = get_tensor_map(base + L.z + (size_t)b0 * kRows * zc * 2, nblk * kRows, zc, kRows, 64, &mz);
             if (rc != MORE_OK) return rc;
             sp.T = tokens;
-            sp.total = (long long)nblk * nsteps;
+            const long long total = (long long)nblk * nsteps;
             int g = plan.share > 0 ? nblk * plan.share : plan.parts;
             if (plan.share == 0 && a.T > kChunkTokens) {     // (the last chunk of a long call may be shorter)
                 const long long most = (long long)(plan.maxseg - 1) * blocks - 1;  // floor(g / blocks) + 2 <= maxseg
-                if (g > sp.total) g = (int)sp.total;
+                if (g > total) g = (int)total;
                 if (g > most) g = (int)(most > 1 ? most : 1);
             }
+            sp.cut = make_cut(total, nsteps, g);
             if (launch(sweep, g, kSThreads, smem, a.stream, true, 1, mz, mr2, sp) != cudaSuccess) return MORE_ERR_CUDA;
 
             FinishParams fp{};
             fp.T = tokens; fp.M = a.M; fp.k = a.k; fp.gate_mode = a.gate_mode;
-            fp.nsteps = nsteps; fp.g = g; fp.share = plan.share; fp.maxseg = plan.maxseg; fp.cap = sp.cap; fp.total = sp.total;
+            fp.share = plan.share; fp.maxseg = plan.maxseg; fp.cap = sp.cap; fp.cut = sp.cut;
             fp.ent = sp.ent; fp.cnt = sp.cnt; fp.mz = sp.mz;
             const size_t ro = (size_t)first * a.k;
             fp.out_idx = a.out_idx + ro; fp.out_gate = a.out_gate + ro; fp.out_counts = a.out_counts;
