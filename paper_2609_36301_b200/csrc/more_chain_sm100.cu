@@ -802,7 +802,23 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
                 const int col0 = (s0 + s) * W + sub * kCols;
                 wait_or_abort(bar(B_AF + buf), buf ? odd : even, abort_flag, p.status);
                 if (again) (buf ? odd : even) ^= 1;          // (otherwise it is read where it is)
-                if (warp_live) {
+                const int valid = M - (s0 + s) * W;
+                if (warp_live && NB == 4 && decltype(masked)::value && valid <= W / 2 && lead == steps) {
+                    // Half a unit or less: in groups of four columns that go round the token's threads they fill up to all 16 of
+                    // its buckets.  (Eight columns to a bucket gave 40 columns five: no threshold for k > 5, every logit a
+                    // candidate and the scratch's share of them exceeded.  T = 256, h = 704, r = 40, M = 5800, one unit per CTA:
+                    // k = 8 50.4 -> 26.1 us, k = 4 22.9 -> 19.7; T = 1, M = 16424 26.0 -> 14.0.)
+                    tc_fence_after();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int c = 4 * (sub + 4 * i);
+                        uint32_t x[4];
+                        tmem_ld4(t_col - sub * kCols + buf * W + c, x);
+                        tmem_ld_wait4(x);
+                        const float m = fmaxf(max3(__uint_as_float(x[0]), __uint_as_float(x[1]), __uint_as_float(x[2])), __uint_as_float(x[3]));
+                        if (c < valid) b[i] = fmaxf(b[i], m);
+                    }
+                } else if (warp_live) {
                     tc_fence_after();
 #pragma unroll
                     for (int h = 0; h < kCols; h += 16) {

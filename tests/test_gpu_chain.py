@@ -49,6 +49,14 @@ def test_edges(T, h, r, M, k, gate_mode):
     _route_and_check(inputs.gaussian_case(T, h, r, M, k, gate_mode, seed=T + M))
 
 
+@pytest.mark.parametrize("k", [1, 3, 5, 8, 16])
+@pytest.mark.parametrize("tail", [8, 24, 32, 40, 56, 64, 72, 120])
+@pytest.mark.parametrize("T", [1, 130])
+def test_a_part_of_few_experts(T, tail, k):
+    """One unit per CTA, the last of fewer than 128 experts: the threshold of its tokens comes from those alone."""
+    _route_and_check(inputs.gaussian_case(T, 128, 40, 1024 + tail, k, k & 1, seed=tail + k))
+
+
 @pytest.mark.parametrize("T,h,r,M,k", [(300, 128, 32, 4096, 8), (64, 128, 64, 16384, 20), (20000, 64, 16, 512, 8), (45000, 64, 16, 512, 4)])
 def test_the_plan_names_the_kernels_that_run(T, h, r, M, k):
     import torch
