@@ -1203,8 +1203,12 @@ __device__ __forceinline__ void put_token(const FinishParams& p, int tok, Cand c
     if (lane == 0 && p.out_lse) p.out_lse[tok] = (m2 + log2f(z)) * kLn2;
 }
 
-// Up to kWarpSegs segments per token, or long lists: a warp per token.
+// Up to kWarpSegs segments per token: a warp per token.
 constexpr int kWarpSegs = 64;
+// LONG: with up to 512 candidates held in registers, whose loads then are one trip to L2, and not one for each 128 of them, twice
+// (T = 600, M = 1024, k = 16 20.7 -> 18.7 us); short code otherwise, as it is fetched as it runs.
+constexpr int kLongSure = 64;                      // candidates that are sure; there are 1.4 times as many, in places for up to three
+template <bool LONG>
 __global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
 {
     __shared__ Cand buf[8][64];
@@ -1244,7 +1248,11 @@ __global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
         const int s = inv ? (int)__umulhi((uint32_t)f, inv) : f, i = f - s * most;
         return i < counts[warp][s] ? load_cand(p.ent + (slot0 + (size_t)s * kRows) * p.cap + i) : no_cand();
     };
-    const Cand c = warp_topk<4>(nseg * most, p.k, get, buf[warp], lane);
+    const int n = nseg * most;
+    Cand c;
+    if (!LONG || n <= 128 || n > 512) c = warp_topk<4>(n, p.k, get, buf[warp], lane);
+    else if (n <= 256) c = warp_topk<8>(n, p.k, get, buf[warp], lane);
+    else c = warp_topk<16>(n, p.k, get, buf[warp], lane);
     put_token(p, tok, c, m2, z, lane);
 }
 
@@ -1254,12 +1262,15 @@ __global__ void __launch_bounds__(256) finish_warp_kernel(const FinishParams p)
 // ranked by counting.  Code that runs once is fetched from L2 as it runs, so it is kept short (entries held in registers and
 // 20 unrolled tests took 2.5 us where reading them again takes 1).
 constexpr int kManyThreads = 512;
+constexpr int kSomeThreads = 128;                  // where there are more tokens and fewer segments
 constexpr int kManyPer = 10;                       // segments per half warp
 constexpr int kManySegs = kManyPer * (kManyThreads / 16);
+static_assert(kWarpSegs <= kManyPer * (kSomeThreads / 16), "the smaller CTAs take what a warp takes");
 // More near the top than `keep` holds: many logits that equal the bound, of which those with the smallest ids count.  The k-th
 // smallest of the 64 groups' smallest ids bounds the k-th smallest of them; collected again with it.  Returns how many.  (Not
 // inlined: in the kernel's way it costs every call 0.5 us of instruction fetches.)
 constexpr int kKeep = 512;
+template <int THREADS>
 __device__ __noinline__ int collect_equals(const int* cnt, const uint2* ent, size_t next_ent, int nseg, int k, float thr, int* ids,
                                            Cand* keep, int* count, int* bound)
 {
@@ -1268,7 +1279,7 @@ __device__ __noinline__ int collect_equals(const int* cnt, const uint2* ent, siz
         const uint2* e = ent;
         const int* c = cnt;
 #pragma unroll 1
-        for (int s = half; s < nseg; s += kManyThreads / 16, e += next_ent, c += kManyThreads / 16 * kRows) {
+        for (int s = half; s < nseg; s += THREADS / 16, e += next_ent, c += THREADS / 16 * kRows) {
             const int n = *c;
 #pragma unroll 1
             for (int i = hl; i < n; i += 16) {
@@ -1280,8 +1291,8 @@ __device__ __noinline__ int collect_equals(const int* cnt, const uint2* ent, siz
     int least = INT_MAX;
     each([&](Cand x) { if (x.v == thr) least = min(least, x.id); });
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) least = min(least, __shfl_xor_sync(kFull, least, o));
-    if ((threadIdx.x & 7) == 0) ids[threadIdx.x >> 3] = least;
+    for (int o = 1; o < THREADS / 64; o <<= 1) least = min(least, __shfl_xor_sync(kFull, least, o));
+    if (threadIdx.x % (THREADS / 64) == 0) ids[threadIdx.x / (THREADS / 64)] = least;
     __syncthreads();                                          // (also: everyone has read the count)
     if (threadIdx.x == 0) *count = 0;
     if (threadIdx.x < 64) {
@@ -1303,9 +1314,10 @@ __device__ __noinline__ int collect_equals(const int* cnt, const uint2* ent, siz
     return *count;
 }
 
-__global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishParams p)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) finish_many_kernel(const FinishParams p)
 {
-    constexpr int kWarps = kManyThreads / 32;
+    constexpr int kWarps = THREADS / 32, kGroup = THREADS / 64;
     __shared__ __align__(16) float maxima[64];
     __shared__ float2 smz[kWarps];
     __shared__ Cand keep[kKeep];
@@ -1322,15 +1334,15 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
     const int* const my_cnt = p.cnt + slot0 + (size_t)half * kRows;
     const uint2* const my_ent = p.ent + (slot0 + (size_t)half * kRows) * p.cap + hl;
-    const size_t next_ent = (size_t)(kManyThreads / 16) * kRows * p.cap;
+    const size_t next_ent = (size_t)(THREADS / 16) * kRows * p.cap;
     pdl_wait();
     int c[kManyPer];
 #pragma unroll
     for (int u = 0; u < kManyPer; ++u)
-        c[u] = half + u * (kManyThreads / 16) < nseg ? my_cnt[u * (kManyThreads / 16) * kRows] : 0;
+        c[u] = half + u * (THREADS / 16) < nseg ? my_cnt[u * (THREADS / 16) * kRows] : 0;
     float m2 = -INFINITY, z = 0.f;
     if (p.mz) {
-        for (int s = threadIdx.x; s < nseg; s += kManyThreads) {
+        for (int s = threadIdx.x; s < nseg; s += THREADS) {
             const float2 o = p.mz[slot0 + (size_t)s * kRows];
             join_mz(m2, z, o.x, o.y);
         }
@@ -1352,8 +1364,8 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
         }
     }
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));          // eight threads' maximum: 64 of them
-    if ((lane & 7) == 0) maxima[warp * 4 + (lane >> 3)] = m;
+    for (int o = 1; o < kGroup; o <<= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));     // a group of threads' maximum: 64 of them
+    if (lane % kGroup == 0) maxima[threadIdx.x / kGroup] = m;
     if (p.mz) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -1380,7 +1392,7 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     if (m >= thr && m > -INFINITY) {                          // (few threads: their entries are read again, from L1)
         const uint2* e = my_ent;
 #pragma unroll 1
-        for (int s = half; s < nseg; s += kManyThreads / 16, e += next_ent) {
+        for (int s = half; s < nseg; s += THREADS / 16, e += next_ent) {
             const int count = p.cnt[slot0 + (size_t)s * kRows];
 #pragma unroll 1
             for (int i = hl; i < count; i += 16) {
@@ -1395,11 +1407,11 @@ __global__ void __launch_bounds__(kManyThreads) finish_many_kernel(const FinishP
     __syncthreads();
     int n = s_count;
     if (__builtin_expect(n > kKeep, 0)) {
-        n = collect_equals(p.cnt + slot0 + (size_t)half * kRows, my_ent, next_ent, nseg, p.k, thr, reinterpret_cast<int*>(maxima), keep,
+        n = collect_equals<THREADS>(p.cnt + slot0 + (size_t)half * kRows, my_ent, next_ent, nseg, p.k, thr, reinterpret_cast<int*>(maxima), keep,
                            &s_count, &s_last);
     }
     if (n <= kKeep) {
-        for (int i = threadIdx.x; i < n; i += kManyThreads) {
+        for (int i = threadIdx.x; i < n; i += THREADS) {
             const Cand e = keep[i];
             int rank = 0;
             for (int j = 0; j < n; ++j) {
@@ -1661,12 +1673,22 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
             // Eight threads per token rank up to two short lists by counting everything against everything; where there is
             // more, the threshold of a warp's selection saves more than its 32 lanes per token cost (k = 16: T = 17000,
             // M = 8192 121 -> 88 us, T = 32768, M = 4096 174 -> 114; k = 8 with two lists each, T = 17000, M = 4096 54 -> 51).
+            // A warp goes through many lists one after the other: from about 128 candidates on that are sure, a CTA per token
+            // is quicker, of 512 threads while all of them fit on the chip in about one go, of 128 for up to five times as many tokens
+            // as there are candidates.  (h = 512, r = 32; warp, 128, 512 threads: T = 256, M = 8192, k = 8 26.6, 19.3, 17.4 us,
+            // k = 16 33.6, 23.3, 20.5; T = 512, M = 4096, k = 8 20.7, 18.0, 20.7; T = 1024, M = 8192, k = 16 39.3, 32.4, 40.3,
+            // k = 4 21.2, 21.9, 30.1; T = 2048, M = 8192, k = 8 28.3, 31.9.)
+            const int sure = plan.maxseg * a.k;
             if (a.k <= 8 && plan.maxseg <= (plan.share > 0 ? 1 : kFewSegs))
                 e = launch(finish_few_kernel, (tokens + 31) / 32, 256, 0, a.stream, true, 1, fp);
-            else if (plan.maxseg <= kWarpSegs)
-                e = launch(finish_warp_kernel, (tokens + 7) / 8, 256, 0, a.stream, true, 1, fp);
+            else if (plan.maxseg > kWarpSegs || (tokens <= 2 * sms && plan.maxseg >= 16 && sure >= 128))
+                e = launch(finish_many_kernel<kManyThreads>, tokens, kManyThreads, 0, a.stream, true, 1, fp);
+            else if (sure >= 128 && tokens <= 5 * sure)
+                e = launch(finish_many_kernel<kSomeThreads>, tokens, kSomeThreads, 0, a.stream, true, 1, fp);
+            else if (sure >= kLongSure)
+                e = launch(finish_warp_kernel<true>, (tokens + 7) / 8, 256, 0, a.stream, true, 1, fp);
             else
-                e = launch(finish_many_kernel, tokens, kManyThreads, 0, a.stream, true, 1, fp);
+                e = launch(finish_warp_kernel<false>, (tokens + 7) / 8, 256, 0, a.stream, true, 1, fp);
             if (e != cudaSuccess) return MORE_ERR_CUDA;
             count_launch(2);
         }

@@ -152,6 +152,24 @@ def test_tokens_of_zeros(T, M, k):
     assert bool((res.idx[::3] == torch.arange(k, device="cuda", dtype=torch.int32)).all())
 
 
+@pytest.mark.parametrize("zeros", [False, True])
+@pytest.mark.parametrize("T,M,k", [
+    (290, 2048, 8),        # 16 segments per token: CTAs of 512 threads
+    (296, 2048, 16),       # the most tokens that they take
+    (297, 2048, 16),       # 16 segments: CTAs of 128 threads
+    (310, 4096, 8),
+    (700, 8200, 16),       # 49 segments, the last of 8 experts
+    (600, 1024, 16),       # 8 segments: a warp per token, candidates in registers
+    (1300, 4096, 4),       # 26 segments
+    (1300, 512, 4),        # four segments: the short code
+])
+def test_finishing_by_the_number_of_segments(T, M, k, zeros):
+    case = inputs.gaussian_case(T, 64, 16, M, k, 1, seed=23)
+    if zeros:
+        case.X[::5] = 0
+    _route_and_check(case)
+
+
 @pytest.mark.parametrize("gate_mode", [0, 1])
 @pytest.mark.parametrize("T,M,k", [
     (300, 16384, 8),       # one or two units per segment
