@@ -1498,6 +1498,25 @@ cudaError_t launch(void (*kern)(Args...), int grid, int block, int smem, cudaStr
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Eight threads per token rank up to two short lists by counting everything against everything; where there is
+// more, the threshold of a warp's selection saves more than its 32 lanes per token cost (k = 16: T = 17000,
+// M = 8192 121 -> 88 us, T = 32768, M = 4096 174 -> 114; k = 8 with two lists each, T = 17000, M = 4096 54 -> 51).
+// A warp goes through many lists one after the other: from about 128 candidates on that are sure, a CTA per token
+// is quicker, of 512 threads while all of them fit on the chip in about one go, of 128 for up to five times as many tokens
+// as there are candidates.  (h = 512, r = 32; warp, 128, 512 threads: T = 256, M = 8192, k = 8 26.6, 19.3, 17.4 us,
+// k = 16 33.6, 23.3, 20.5; T = 512, M = 4096, k = 8 20.7, 18.0, 20.7; T = 1024, M = 8192, k = 16 39.3, 32.4, 40.3,
+// k = 4 21.2, 21.9, 30.1; T = 2048, M = 8192, k = 8 28.3, 31.9.)
+cudaError_t finish(const FinishParams& fp, int tokens, int maxseg, bool few, int sms, cudaStream_t st)
+{
+    const int sure = maxseg * fp.k;
+    if (few) return launch(finish_few_kernel, (tokens + 31) / 32, 256, 0, st, true, 1, fp);
+    if (maxseg > kWarpSegs || (tokens <= 2 * sms && maxseg >= 16 && sure >= 128))
+        return launch(finish_many_kernel<kManyThreads>, tokens, kManyThreads, 0, st, true, 1, fp);
+    if (sure >= 128 && tokens <= 5 * sure) return launch(finish_many_kernel<kSomeThreads>, tokens, kSomeThreads, 0, st, true, 1, fp);
+    if (sure >= kLongSure) return launch(finish_warp_kernel<true>, (tokens + 7) / 8, 256, 0, st, true, 1, fp);
+    return launch(finish_warp_kernel<false>, (tokens + 7) / 8, 256, 0, st, true, 1, fp);
+}
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 constexpr int kChunkTokens = 131072;               // tokens per pass: bounds the scratch, whatever T is
@@ -1575,6 +1594,20 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
 size_t chain_scratch_bytes(const RouteArgs& a, const Plan& p)
 {
     return layout_of(a, p, a.gate_mode == MORE_GATE_FULL_SOFTMAX || a.out_lse != nullptr).total;
+}
+
+int launch_finish(const RouteArgs& a, DeviceCtx& ctx, int segments, int cap, const uint2* ent, const int* cnt, const float2* mz)
+{
+    static_assert(kFinishTokens == kRows && kFinishMaxSegments <= kManySegs, "what the header promises");
+    FinishParams fp{};
+    fp.T = a.T; fp.M = a.M; fp.k = a.k; fp.gate_mode = a.gate_mode;
+    fp.share = fp.maxseg = segments; fp.cap = cap;
+    fp.ent = ent; fp.cnt = cnt; fp.mz = mz;
+    fp.out_idx = a.out_idx; fp.out_gate = a.out_gate; fp.out_counts = a.out_counts;
+    fp.out_topval = a.out_topval; fp.out_lse = a.out_lse;
+    if (finish(fp, a.T, segments, false, ctx.sm_count, a.stream) != cudaSuccess) return MORE_ERR_CUDA;
+    count_launch(1);
+    return MORE_OK;
 }
 
 int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scratch)
@@ -1669,27 +1702,8 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
             fp.out_idx = a.out_idx + ro; fp.out_gate = a.out_gate + ro; fp.out_counts = a.out_counts;
             fp.out_topval = a.out_topval ? a.out_topval + ro : nullptr;
             fp.out_lse = a.out_lse ? a.out_lse + first : nullptr;
-            cudaError_t e;
-            // Eight threads per token rank up to two short lists by counting everything against everything; where there is
-            // more, the threshold of a warp's selection saves more than its 32 lanes per token cost (k = 16: T = 17000,
-            // M = 8192 121 -> 88 us, T = 32768, M = 4096 174 -> 114; k = 8 with two lists each, T = 17000, M = 4096 54 -> 51).
-            // A warp goes through many lists one after the other: from about 128 candidates on that are sure, a CTA per token
-            // is quicker, of 512 threads while all of them fit on the chip in about one go, of 128 for up to five times as many tokens
-            // as there are candidates.  (h = 512, r = 32; warp, 128, 512 threads: T = 256, M = 8192, k = 8 26.6, 19.3, 17.4 us,
-            // k = 16 33.6, 23.3, 20.5; T = 512, M = 4096, k = 8 20.7, 18.0, 20.7; T = 1024, M = 8192, k = 16 39.3, 32.4, 40.3,
-            // k = 4 21.2, 21.9, 30.1; T = 2048, M = 8192, k = 8 28.3, 31.9.)
-            const int sure = plan.maxseg * a.k;
-            if (a.k <= 8 && plan.maxseg <= (plan.share > 0 ? 1 : kFewSegs))
-                e = launch(finish_few_kernel, (tokens + 31) / 32, 256, 0, a.stream, true, 1, fp);
-            else if (plan.maxseg > kWarpSegs || (tokens <= 2 * sms && plan.maxseg >= 16 && sure >= 128))
-                e = launch(finish_many_kernel<kManyThreads>, tokens, kManyThreads, 0, a.stream, true, 1, fp);
-            else if (sure >= 128 && tokens <= 5 * sure)
-                e = launch(finish_many_kernel<kSomeThreads>, tokens, kSomeThreads, 0, a.stream, true, 1, fp);
-            else if (sure >= kLongSure)
-                e = launch(finish_warp_kernel<true>, (tokens + 7) / 8, 256, 0, a.stream, true, 1, fp);
-            else
-                e = launch(finish_warp_kernel<false>, (tokens + 7) / 8, 256, 0, a.stream, true, 1, fp);
-            if (e != cudaSuccess) return MORE_ERR_CUDA;
+            if (finish(fp, tokens, plan.maxseg, a.k <= 8 && plan.maxseg <= (plan.share > 0 ? 1 : kFewSegs), sms, a.stream) != cudaSuccess)
+                return MORE_ERR_CUDA;
             count_launch(2);
         }
     }

@@ -83,6 +83,11 @@ size_t paired_scratch_bytes(const RouteArgs& a, const Plan& p);
 // Launchers: enqueue on a.stream, return MORE_OK / MORE_ERR_*.  `scratch` is at least *_scratch_bytes().
 int launch_generic(const RouteArgs& a, DeviceCtx& ctx, void* scratch);
 int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
+// The chain's finishing kernels for candidate lists of another sweep, `segments` per token, token t's list s at
+// slot = ((t / 128) segments + s) 128 + t % 128: cnt[slot] entries (logit bits, expert id) from ent[slot cap] on, and where
+// the log-sum-exp counts mz[slot] = (max in log2 units, sum).  out_counts is clear when the work on the stream before is done.
+constexpr int kFinishTokens = 128, kFinishMaxSegments = 256;
+int launch_finish(const RouteArgs& a, DeviceCtx& ctx, int segments, int cap, const uint2* ent, const int* cnt, const float2* mz);
 // All tensor-core launchers clear out_counts on the stream themselves, after every host-side step that can fail.
 int launch_lowrank(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
 int launch_full(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);

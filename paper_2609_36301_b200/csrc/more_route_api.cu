@@ -255,7 +255,10 @@ void plan_dense(int T, int h, int M, int k, int msplit, int sm_count, Plan* p)
     // on top.  Fitted to 3300 shapes (T = 1 ... 20000, h = 128 ... 4096, M = 280 ... 16384, k = 1 ... 32, both gates) at forced
     // splits of 1 to 16: the split chosen costs 0.5 % on average against the best of them, 2 % with one set for all k from
     // before a K-slice was one MMA of N = 256 (T = 500, h = 256, M = 1000, k = 8 55 us against 40).
-    const double epilogue = k <= 8 ? 2.0 : 7.0, start = k <= 8 ? 21.0 : (k <= 16 ? 40.0 : 60.0), merge = k <= 8 ? 7.0 : (k <= 16 ? 25.0 : 35.0);
+    // (Since the parked lists have finishing kernels of their own they cost 1 more than a CTA that writes its results itself (T = 173,
+    // h = 552, M = 440 43.2 us by one CTA, 32.4 by two), whatever their length, and as many CTAs may share a
+    // block as there are SMs: T = 10, h = 1448, M = 20920 158 -> 50 us, T = 500, h = 4096, M = 65536 789 -> 238.)
+    const double epilogue = k <= 8 ? 2.0 : 7.0, start = k <= 8 ? 21.0 : (k <= 16 ? 40.0 : 60.0), merge = 1.0;
     const int tiles = (M + 255) / 256;
     const double ktiles = (h + 63) / 64;
     double best = 1e300;
@@ -263,7 +266,8 @@ void plan_dense(int T, int h, int M, int k, int msplit, int sm_count, Plan* p)
     for (int bt = kBlockTokens; bt >= 128; bt -= 32) {
         const int blocks = (T + bt - 1) / bt;
         const int s_lo = msplit > 0 ? (msplit < tiles ? msplit : tiles) : 1;
-        const int s_hi = msplit > 0 ? s_lo : (tiles < 16 ? tiles : 16);
+        const int s_max = sm_count / blocks > 16 ? (sm_count / blocks < kFinishMaxSegments ? sm_count / blocks : kFinishMaxSegments) : 16;
+        const int s_hi = msplit > 0 ? s_lo : (tiles < s_max ? tiles : s_max);
         for (int s = s_lo; s <= s_hi; ++s) {
             const long long ctas = (long long)blocks * s;
             const double waves = (double)((ctas + sm_count - 1) / sm_count);

@@ -76,6 +76,10 @@ struct KernelParams {
     float* part_val;
     int* part_id;
     float2* part_mz;
+    // standard router: lists for the finishing kernels instead
+    uint2* ent;
+    int* cnt;
+    float2* mz;
     // filter mode: transposed copy of R2 ([M][RPAD] bf16, ranks >= r zero); colnorm[0] = largest column norm of R2,
     // colnorm[1] = largest column norm of the error of its fp16 copy; R2 itself for the fallback sweep; the low halves
     // of z, [CTA][rank / 8][256 threads] x 16 B
@@ -751,11 +755,25 @@ route_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
             }
         };
         if (*abort_flag == 0) {
-            if (p.msplit == 1) {
+            if (FULL && p.msplit > 1) {
+                if (row_live) {
+                    const size_t slot = ((size_t)(row / kFinishTokens) * p.msplit + split) * kFinishTokens + (size_t)(row % kFinishTokens);
+                    int n = 0;
+#pragma unroll
+                    for (int s = 0; s < KCAP; ++s) {
+                        if (s < p.k && L.v[s] > -INFINITY) {
+                            p.ent[slot * p.k + s] = make_uint2(__float_as_uint(L.v[s]), (uint32_t)L.id[s]);
+                            n = s + 1;
+                        }
+                    }
+                    p.cnt[slot] = n;
+                    if (LSE) p.mz[slot] = make_float2(m2, zsum);
+                }
+            } else if (p.msplit == 1) {
                 hist_clear();
                 if (row_live) write_token<KCAP>(p, row, L, m2, zsum, hist);
                 hist_flush();
-            } else {
+            } else if constexpr (!FULL) {
                 // park the partial list; the CTA that arrives last for this token block merges all of them
                 const int64_t slot = ((int64_t)blk * kBlockTokens + row_in_blk) * p.msplit + split;
 #pragma unroll
@@ -950,14 +968,25 @@ int kcap_of(int k) { return k <= 8 ? 8 : (k <= 16 ? 16 : 32); }
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct PairedScratch {
-    size_t counters, part_val, part_id, part_mz, r2t, r2h, partial, zlo, total;
+    size_t counters, part_val, part_id, part_mz, ent, cnt, mz, r2t, r2h, partial, zlo, total;
 };
+
+// The partial lists of a standard router go to the finishing kernels, a CTA or a warp per token.  (Merged by whichever CTA of a
+// block was last, a thread per token, each list took 0.8 us, and no more than 16 CTAs per block were worth it: T = 64, h = 2048,
+// M = 16384 142 us, with 64 CTAs 46; T = 1, h = 4096, M = 131072, k = 16 1400 and 336; T = 5000, h = 512, M = 2048, k = 16 in four
+// 108 and 76.)
+bool lists_apart(const RouteArgs& a, const Plan& p) { return a.full && p.msplit > 1; }
 
 PairedScratch paired_layout(const RouteArgs& a, const Plan& p)
 {
     PairedScratch L{};
     size_t off = 0;
-    if (p.msplit > 1) {
+    if (lists_apart(a, p)) {
+        const size_t slots = align_up((size_t)a.T, kFinishTokens) * (size_t)p.msplit;
+        L.ent = off; off += align_up(slots * (size_t)a.k * 8, 256);
+        L.cnt = off; off += align_up(slots * 4, 256);
+        L.mz = off; off += align_up(slots * 8, 256);
+    } else if (p.msplit > 1) {
         const size_t blocks = (size_t)(a.T + p.block_tokens - 1) / p.block_tokens;
         const size_t slots = blocks * kBlockTokens * (size_t)p.msplit;
         const size_t kc = (size_t)kcap_of(a.k);
@@ -1014,7 +1043,12 @@ int launch_paired(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scrat
     kp.status = ctx.status;
     kp.stats = ctx.stats;
     kp.R2 = a.R2;
-    if (p.msplit > 1) {
+    const bool apart = lists_apart(a, p);
+    if (apart) {
+        kp.ent = reinterpret_cast<uint2*>(base + L.ent);
+        kp.cnt = reinterpret_cast<int*>(base + L.cnt);
+        kp.mz = reinterpret_cast<float2*>(base + L.mz);
+    } else if (p.msplit > 1) {
         kp.counters = reinterpret_cast<unsigned*>(base + L.counters);
         kp.part_val = reinterpret_cast<float*>(base + L.part_val);
         kp.part_id = reinterpret_cast<int*>(base + L.part_id);
@@ -1035,7 +1069,10 @@ int launch_paired(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scrat
         if (rc != MORE_OK) return rc;
     }
     const bool clear = !p.filter;
-    if (a.full) return launch_kcap<64, true>(a.k, mode, mx, m1, m2, kp, p.ctas, a.stream, clear);
+    if (a.full) {
+        rc = launch_kcap<64, true>(a.k, mode, mx, m1, m2, kp, p.ctas, a.stream, clear);
+        return rc == MORE_OK && apart ? launch_finish(a, ctx, p.msplit, a.k, kp.ent, kp.cnt, lse ? kp.mz : nullptr) : rc;
+    }
     switch (rpad) {
         case 16: return launch_kcap<16, false>(a.k, mode, mx, m1, m2, kp, p.ctas, a.stream, clear);
         case 32: return launch_kcap<32, false>(a.k, mode, mx, m1, m2, kp, p.ctas, a.stream, clear);

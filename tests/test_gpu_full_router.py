@@ -56,6 +56,20 @@ def test_full_router_with_expert_split(msplit):
     _run(case, msplit=msplit)
 
 
+@pytest.mark.parametrize("gate_mode", [0, 1])
+@pytest.mark.parametrize("T,h,M,k", [
+    (1, 72, 37896, 1),            # one token, 148 CTAs of one tile of 256 experts, the last of eight experts
+    (1, 512, 40000, 32),          # the longest lists
+    (10, 1448, 5000, 3),          # 20 CTAs
+    (130, 64, 9000, 17),          # two runs of 128 tokens in one block
+    (300, 136, 20008, 16),        # two blocks, ragged
+    (600, 64, 520, 8),            # two or three tiles: the fewest lists
+])
+def test_full_router_with_few_tokens(T, h, M, k, gate_mode):
+    """Many CTAs per token block, whose lists the finishing kernels join."""
+    _run(inputs.full_rank_case(T, h, M, k, gate_mode, seed=T + M))
+
+
 def test_full_router_agrees_with_low_rank_router_on_the_identity():
     """Same inputs through ``more_route_ex`` with R1 = I (r = h = 64, the largest the low-rank tensor path takes):
     the two GPU paths must pick the same experts."""
