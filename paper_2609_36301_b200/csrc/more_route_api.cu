@@ -195,19 +195,19 @@ namespace {
 // gains (a projection that is not repeated, an even cut of the units, cheaper selection) with both; a larger h favours it,
 // as a cluster shares the reading of X.  So the lines are straight: M >= c x (tokens per SM), c by how tight the bound on
 // the k-th logit is for the number of buckets (k <= 4 of 16, k <= 8 of 16, k <= 16 of 32; above that it is too loose), and
-// with fewer than 1024 experts, eight units or less per token block, about twice that.  From 340 tokens per SM on, the paired
-// kernel's two CTAs per SM fill up, and for k = 5 ... 8 it wins up to c = 40 (20 where the exponentials slow it down).
-// Measured on B200 at 14300 shapes drawn from T = 1 ... 64 k, M = 128 ... 128 k, h = 128, 512, 2048, r = 16, 32, 64,
-// k = 2 ... 16, both gates, one call after the other, and at large ones with each side running for 0.1 s at a time, where the
-// chip's power limit counts.  profiles/kernel_choice.csv holds 2891 more, to which nothing was fitted: there the choice costs
-// 0.4 % on average against the better side of each shape and more than 5 % at 2.8 % of them (1.32 at most); always the chain
-// would cost 7 %, never 33 %.
+// with fewer than 1024 experts, eight units or less per token block, somewhat more.  From 340 tokens per SM on, the paired
+// kernel's two CTAs per SM fill up, and for k = 5 ... 8 it keeps what lies below c = 40 (20 where the exponentials slow it down):
+// a single call is quicker on the chain (T = 65536, h = 2048, r = 64, M = 16384: 343 us against 366), but under sustained load,
+// where the chip's power limit counts, it is not (400 against 390).  Measured on B200, one call after the other: the lines are
+// fitted to 1000 shapes of T = 6 k ... 64 k, M = 192 ... 12 k, h = 128 ... 2048, r = 16, 32, 64, k = 1 ... 16, both gates;
+// profiles/kernel_choice.csv holds others, to which nothing was fitted, where the choice costs 2 % on average against the better side of
+// each shape (3 % with fewer than 1024 experts, 1 % with more; always the chain would cost 15 %, never the chain 23 %).
 bool chain_wins(int T, int h, int M, int k, bool lse, int sm_count)
 {
     const int per_sm = (T + sm_count - 1) / sm_count, wide = h < 4096 ? h : 4096;
     if (k > 16 || M < 128) return false;
-    if (M < 1024) return M + wide / 4 - 128 >= (k <= 4 ? 8 : 18) * per_sm;
-    const double c = k <= 4 ? 4.5 : (k > 8 ? 7 : (per_sm <= 340 ? 12 : (lse ? 20 : 40)));
+    if (M < 1024) return M + wide / 4 - 128 >= (k <= 4 ? 5 : 14) * per_sm;
+    const int c = k <= 4 ? 4 : (k > 8 ? 6 : (per_sm <= 340 ? 9 : (lse ? 20 : 40)));
     return M + wide / 8 >= c * per_sm;
 }
 
