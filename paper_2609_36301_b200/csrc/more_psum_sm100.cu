@@ -28,6 +28,10 @@ namespace {
 
 constexpr int kPsumEpi = 512;
 constexpr int kPsumThreads = 64 + kPsumEpi;
+// Up to 128 tokens: the second half does nothing, X tiles are half as tall, and four stages of them fit where otherwise two do (the
+// first contraction is a chain of trips to memory then: T = 4, h = 2152, r = 32, M = 1584 25.0 -> 16.7 us, T = 24, h = 3360, r = 56, M = 20224 36.8 -> 20.7).
+constexpr int kFewTokens = 128, kFewStages = 4, kFewXBytes = kXTileBytes / 2, kFewStageBytes = kFewXBytes + 64 * 128;
+static_assert(kFewStages * kFewStageBytes <= kRingBytes, "phase-1 stages do not fit");
 
 // 16 consecutive fp32 columns of this thread's tensor-memory lane, complete on return.  (Load and wait in one statement:
 // with the destination registers tied to a separate wait the compiler copies them.)
@@ -44,7 +48,7 @@ __device__ __forceinline__ void tmem_get16(uint32_t taddr, float (&v)[16])
 
 struct PsumParams {
     int T, h, r, M, msplit, tiles_total;
-    int block;           // tokens of a block: a multiple of 32, 160 ... 256 (what a CTA computes z for beyond them is not used)
+    int block;           // tokens of a block: a multiple of 32, 128 or 160 ... 256 (what a CTA computes z for beyond them is not used)
     const float* lse;    // [T] natural-log log-sum-exp of every token's logits
     float* psum;         // [M], zeroed before the launch
     int* status;
@@ -70,7 +74,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     uint8_t* ring_ptr = smem_raw + (ring - raw);
     uint8_t* ctl = ring_ptr + kRingBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(ctl);
-    constexpr int B_FULL1 = 0, B_EMPTY1 = B_FULL1 + kStagesP1, B_ZACC = B_EMPTY1 + kStagesP1, B_ZOP = B_ZACC + 1,
+    constexpr int B_FULL1 = 0, B_EMPTY1 = B_FULL1 + kFewStages, B_ZACC = B_EMPTY1 + kFewStages, B_ZOP = B_ZACC + 1,
                   B_FULL2 = B_ZOP + 1, B_EMPTY2 = B_FULL2 + 8, B_ACCF = B_EMPTY2 + 8, B_ACCE = B_ACCF + 2,
                   B_COUNT = B_ACCE + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ctl + B_COUNT * 8);
@@ -85,9 +89,11 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     const int tile_hi = (int)(((long long)p.tiles_total * (split + 1)) / p.msplit);
     const int ntiles = tile_hi - tile_lo;
     const int ktiles1 = (p.h + 63) / 64;
+    const bool few = p.block <= kFewTokens;
+    const int stages1 = few ? kFewStages : kStagesP1, x_bytes = few ? kFewXBytes : kXTileBytes, st1_bytes = few ? kFewStageBytes : kP1StageBytes;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kStagesP1; ++i) { mbar_init(bar(B_FULL1 + i), 1); mbar_init(bar(B_EMPTY1 + i), 1); }
+        for (int i = 0; i < kFewStages; ++i) { mbar_init(bar(B_FULL1 + i), 1); mbar_init(bar(B_EMPTY1 + i), 1); }
         mbar_init(bar(B_ZACC), 1);
         mbar_init(bar(B_ZOP), kEpilogueThreads);
         for (int i = 0; i < 8; ++i) { mbar_init(bar(B_FULL2 + i), 1); mbar_init(bar(B_EMPTY2 + i), 1); }
@@ -113,14 +119,14 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         // ===================================================================================== TMA producer
         if (lane == 0) {
             bool ok = true;
-            for (int kt = 0; kt < ktiles1 && ok; ++kt) {
-                const int s = kt % kStagesP1;
-                if (kt >= kStagesP1) ok = mbar_wait(bar(B_EMPTY1 + s), ((kt / kStagesP1) - 1) & 1, abort_flag, p.status);
+            for (int kt = 0, s = 0, ph = 1; kt < ktiles1 && ok; ++kt) {
+                ok = mbar_wait(bar(B_EMPTY1 + s), ph, abort_flag, p.status);
                 if (!ok) break;
-                const uint32_t dst = ring + s * kP1StageBytes;
-                mbar_expect_tx(bar(B_FULL1 + s), kP1StageBytes);
+                const uint32_t dst = ring + s * st1_bytes;
+                mbar_expect_tx(bar(B_FULL1 + s), st1_bytes);
                 tma_load_2d(dst, &map_x, bar(B_FULL1 + s), kt * 64, tok0);
-                tma_load_2d(dst + kXTileBytes, &map_r1, bar(B_FULL1 + s), 0, kt * 64);
+                tma_load_2d(dst + x_bytes, &map_r1, bar(B_FULL1 + s), 0, kt * 64);
+                if (++s == stages1) { s = 0; ph ^= 1; }
             }
             ok = ok && mbar_wait(bar(B_ZACC), 0, abort_flag, p.status);
             for (int it = 0; it < ntiles && ok; ++it) {
@@ -145,22 +151,23 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         constexpr uint32_t idesc2 = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (0u << 16) |
                                     ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         {
-            const uint64_t xd = umma_desc_sw128(ring, 16, 1024), rd = umma_desc_sw128(ring + kXTileBytes, 8192, 1024);
+            const uint64_t xd = umma_desc_sw128(ring, 16, 1024), rd = umma_desc_sw128(ring + x_bytes, 8192, 1024);
             const uint32_t x_lo0 = (uint32_t)xd, x_hi = (uint32_t)(xd >> 32), r_lo0 = (uint32_t)rd, r_hi = (uint32_t)(rd >> 32);
-            for (int kt = 0; kt < ktiles1 && ok; ++kt) {
-                const int s = kt % kStagesP1;
-                ok = __all_sync(kFull, mbar_wait(bar(B_FULL1 + s), (kt / kStagesP1) & 1, abort_flag, p.status));
+            for (int kt = 0, s = 0, ph = 0; kt < ktiles1 && ok; ++kt) {
+                ok = __all_sync(kFull, mbar_wait(bar(B_FULL1 + s), ph, abort_flag, p.status));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t x_lo = x_lo0 + s * (kP1StageBytes >> 4), r_lo = r_lo0 + s * (kP1StageBytes >> 4);
+                const uint32_t x_lo = x_lo0 + s * (st1_bytes >> 4), r_lo = r_lo0 + s * (st1_bytes >> 4);
 #pragma unroll
                 for (int a = 0; a < 2; ++a) {
+                    if (a == 1 && few) break;
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
                         tc_mma_bf16_ss_elect(tmem_base + a * kTileExperts, x_lo + a * (16384 >> 4) + kk * 2, x_hi,
                                              r_lo + kk * (2048 >> 4), r_hi, idesc1, (kt | kk) != 0);
                 }
                 tc_commit_elect(bar(B_EMPTY1 + s));
+                if (++s == stages1) { s = 0; ph ^= 1; }
             }
         }
         if (ok) tc_commit_elect(bar(B_ZACC));
@@ -176,6 +183,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             const uint32_t a_lo = a_lo0 + s * (kR2StageBytes >> 4);
 #pragma unroll
             for (int a = 0; a < 2; ++a) {            // token half a -> TMEM columns a*128 ..
+                if (a == 1 && few) break;
                 ok = __all_sync(kFull, ok && mbar_wait(bar(B_ACCE + a), (it & 1) ^ 1, abort_flag, p.status));
                 if (!ok) break;
                 tc_fence_after();
@@ -201,7 +209,9 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         const int64_t row = (int64_t)tok0 + row_in_blk;
         const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16) + half * 128;
         bool ok = mbar_wait(bar(B_ZACC), 0, abort_flag, p.status);
-        if (ok && part == 0) {
+        if (ok && part == 0 && half == 1 && few) {
+            mbar_arrive(bar(B_ZOP));
+        } else if (ok && part == 0) {
             tc_fence_after();
             // (the phase-1 ring is free now) minus the log2-scaled log-sum-exp of my token; -inf for rows past T, whose
             // zero-filled logits then contribute exp(-inf) = 0
@@ -279,7 +289,7 @@ psum_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         if (chunks == 4) sweep(std::integral_constant<int, 4>{});
         else if (chunks == 3) sweep(std::integral_constant<int, 3>{});
         else if (chunks == 2) sweep(std::integral_constant<int, 2>{});
-        else sweep(std::integral_constant<int, 1>{});
+        else if (chunks == 1) sweep(std::integral_constant<int, 1>{});
     }
 
     tc_fence_before();
@@ -318,8 +328,9 @@ int launch_psum_tcgen05(const __nv_bfloat16* X, const __nv_bfloat16* R1, const _
                         int M, const float* lse, float* psum, DeviceCtx& ctx, cudaStream_t stream)
 {
     CUtensorMap mx, m1, m2;
+    const bool few = T <= kFewTokens;
     const int rpad = (r <= 16) ? 16 : (r <= 32 ? 32 : 64);
-    int rc = get_tensor_map(X, T, h, kBlockTokens, 64, &mx);
+    int rc = get_tensor_map(X, T, h, few ? kFewTokens : kBlockTokens, 64, &mx);
     if (rc == MORE_OK) rc = get_tensor_map(R1, h, r, 64, 64, &m1);
     if (rc == MORE_OK) rc = get_tensor_map(R2, r, M, rpad, 64, &m2);
     if (rc != MORE_OK) return rc;
@@ -346,6 +357,12 @@ int launch_psum_tcgen05(const __nv_bfloat16* X, const __nv_bfloat16* R1, const _
         const double last = 2 * (ctas - (waves - 1) * slots) <= slots ? 0.6 : 1.0;
         const double cost = ((double)waves - 1.0 + last) * (block / 16.0 * ((pp.tiles_total + split - 1) / split) + 300.0 + 4.0 * (h / 64));
         if (cost < best * 0.97) { best = cost; blocks = n; s = split; pp.block = block; }
+    }
+    if (few) {                                     // a CTA per SM at most, two tiles or more
+        pp.block = kFewTokens;
+        blocks = 1;
+        s = pp.tiles_total / 2 < slots / 2 ? pp.tiles_total / 2 : slots / 2;
+        if (s < 1) s = 1;
     }
     pp.msplit = s;
     switch (rpad) {

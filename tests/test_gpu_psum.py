@@ -37,10 +37,10 @@ def test_psum_tensor_core_path(T, h, r, M):
     np.testing.assert_allclose(got.sum(), T, rtol=1e-4)                          # rows of P sum to one
 
 
-@pytest.mark.parametrize("T,h,r,M", [(160, 64, 8, 65536), (161, 64, 8, 65536), (192, 256, 32, 1024), (193, 256, 32, 1024),
+@pytest.mark.parametrize("T,h,r,M", [(1, 2152, 32, 1584), (127, 72, 64, 40000), (128, 320, 16, 520), (129, 320, 16, 520), (160, 64, 8, 65536), (161, 64, 8, 65536), (192, 256, 32, 1024), (193, 256, 32, 1024),
                                       (577, 256, 64, 1000), (16301, 72, 16, 4096)])
 def test_psum_blocks_of_fewer_than_256_tokens(T, h, r, M):
-    """Blocks of 160, 192 and 224 tokens: their last token and the one after it, ragged last blocks and tiles."""
+    """Blocks of 128, 160, 192 and 224 tokens: their last token and the one after it, ragged last blocks and tiles."""
     case = inputs.gaussian_case(T, h, r, M, 4, 1, seed=63)
     got, _ = run_psum(case, mr.PATH_TCGEN05)
     want, _ = oracle.psum(case.X, case.R1, case.R2)
