@@ -73,6 +73,8 @@ def lib() -> ctypes.CDLL:
         L.more_debug_scratch_guard.restype = i32
         L.more_debug_scratch_bytes.argtypes = [i32] * 9
         L.more_debug_scratch_bytes.restype = ctypes.c_longlong
+        L.more_debug_chain_lists.argtypes = [i32] * 8 + [ctypes.c_ulonglong, ctypes.POINTER(ctypes.c_ulonglong)]
+        L.more_debug_chain_lists.restype = i32
         L.more_strerror.argtypes = [i32]
         L.more_strerror.restype = ctypes.c_char_p
         L.more_version.argtypes = []
@@ -261,6 +263,16 @@ def debug_scratch_bytes(T, h, r, M, k, gate_mode=0, want_lse=False, path=PATH_AU
     if n < 0:
         raise MoreRouteError(n, "more_debug_scratch_bytes")
     return n
+
+
+def debug_chain_lists(T, h, r, M, k, gate_mode=0, want_lse=False, msplit=0, scratch=0):
+    """Diagnostic: where the sweep's lists lie in a scratch allocation at address ``scratch``: address of the first area, number
+    of areas, places of a list, bytes from one place to the next."""
+    out = (ctypes.c_ulonglong * 4)()
+    rc = int(lib().more_debug_chain_lists(T, h, r, M, k, gate_mode, int(want_lse), msplit, scratch, out))
+    if rc != 0:
+        raise MoreRouteError(rc, "more_debug_chain_lists")
+    return tuple(out)
 
 
 @dataclass

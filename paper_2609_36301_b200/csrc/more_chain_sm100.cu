@@ -246,7 +246,7 @@ constexpr int kEpi = 512;
 constexpr int W = 128;                             // experts of a unit
 constexpr int kCols = W / 4;                       // columns of a thread
 constexpr int kMaxStages = 8;
-constexpr int kListCap = 64;                       // entries of a thread's list
+constexpr int kListCap = 64;                       // places of a thread's list (fewer where so few units cannot fill them)
 constexpr uint32_t kEntry = kEpi * 32;             // bytes between its entries (32 bytes each: four logits, the first one's column)
 
 // Units whose bucket maxima are formed ahead of a segment of `steps` units.  All of a short one: its threshold is then the
@@ -290,7 +290,7 @@ struct SweepParams {
     int maxseg, cap;                               // candidate lists per token block in scratch, entries per list and token
     int nst, st_bytes, zbufs, z_bytes;
     int off_r2, off_pub, off_ctl;
-    int list_cap, list_shift;                      // entries of a list; log2 of the CTAs whose lists lie side by side (0, 1, 2)
+    int list_cap, list_shift;                      // places of a list; log2 of the CTAs whose lists lie side by side (0, 1, 2)
     uint8_t* list;                                 // [CTA >> shift][list_cap][512 = (CTA, 32-token quarter), column quarter, lane] x 32 bytes
     uint2* ent;                                    // [block][seg][128][cap] (logit bits, expert id)
     int* cnt;                                      // [block][seg][128]
@@ -375,8 +375,8 @@ __device__ __forceinline__ void bitonic_down(float (&s)[N])
             if ((i & d) == 0) cx(s[i], s[i + d]);
 }
 // Append the groups of four (maxima t, values v, first column col + 4 i) that reach thr to a list that ends at `end`.  The
-// four tests come first: only the adds to the list's end depend on each other.  No list crosses a multiple of 2^32 bytes, so
-// these are adds to the address's low word.
+// four tests come first: only the adds to the list's end depend on each other.  No list's places lie on both sides of a multiple
+// of 2^32 bytes (lists_at), and its end is one of them (the last place is never filled), so these are adds to the address's low word.
 __device__ __forceinline__ void append4(uint64_t& end, float thr, const float* t, const float* v, int col)
 {
 #define MORE_APPEND(P, COL, A, B, C, D)                                                                     \
@@ -625,12 +625,14 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
         const int M = p.M;
         const uint32_t t_col = tmem_base + ((uint32_t)(q * 32) << 16) + sub * kCols;
         // the thread's list; a unit adds at most 8 entries between two looks at its length
-        // (A list shorter than kListCap is one that so few units cannot fill.  Where only one or two quarters of the block hold
-        // tokens, four or two CTAs share an area: the other quarters' warps touch no lists.)
+        // (A list of fewer than kListCap places is one whose last place so few units cannot reach; `warn` is then that place, and
+        // nothing comes behind it.  Where only one or two quarters of the block hold tokens, four or two CTAs share an area: the
+        // other quarters' warps touch no lists.)
         const uint32_t side = ((blockIdx.x & ((1u << p.list_shift) - 1)) << (2 - p.list_shift)) + q;
         const uint64_t first = reinterpret_cast<uint64_t>(p.list) + (uint64_t)(blockIdx.x >> p.list_shift) * (p.list_cap * kEntry) +
                                (side * (kEpi / 4) + sub * 32 + lane) * 32;
-        const uint64_t warn = first + (kListCap - kCols / 4) * kEntry;
+        const int warn_at = min(kListCap - kCols / 4, p.list_cap - 1);
+        const uint64_t warn = first + warn_at * kEntry;
         // shared memory: published buckets [sub][128][NB], thresholds [128], counters [128], (m, Z) [sub - 1][128]
         const uint32_t pub0 = base + p.off_pub + row * (NB * 4);
         const uint32_t s_thr = base + p.off_pub + 4 * kRows * NB * 4 + row * 4;
@@ -759,7 +761,7 @@ sweep_kernel(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ 
             // and later ones that only equal it lose to them; elsewhere, if the first and the last group have the same
             // maximum, the same holds for the smallest maximum in the list.  (All tokens zero: T = 4096, M = 16384 450 us
             // -> 74, M = 65536 466 -> 135.)
-            uint64_t limit = first + (lead == steps ? max(p.k, 8) : max(p.k + 8, 16)) * kEntry;
+            uint64_t limit = first + min(lead == steps ? max(p.k, 8) : max(p.k + 8, 16), warn_at) * kEntry;
             auto full = [&]() {
                 if (limit < warn && ptr > limit) {
                     if (lead == steps) {
@@ -1525,8 +1527,9 @@ long long resident_ctas(int sm_count) { return 2 * sm_count < kManySegs - 2 ? 2 
 struct Layout {
     size_t z, list, ent, cnt, mz, total;
 };
+int list_areas(const Plan& p) { return (p.parts - 1 >> p.list_shift) + 1; }
 
-// The largest there is (T >= 131072, k = 16, r > 32): 32 MiB of z, 296 MiB of lists, 130 MiB of candidates and counts.
+// The largest there is (T >= 131072, k = 16, r > 32): 32 MiB of z, 297 MiB of lists, 130 MiB of candidates and counts.
 Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
 {
     Layout L{};
@@ -1540,10 +1543,19 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
     if (lse) off += align_up(lists * kRows * 8, 1024);
     // (last: the finishing kernels' reads then lie at the same addresses however long the lists are; T = 40, M = 6424 26.4 us
     // with the lists in front and 25.1 behind)
-    // (aligned to its size, a power of two, no area crosses a multiple of 2^32 bytes: the allocation is aligned to 256)
-    L.list = off; off += (size_t)((p.parts - 1 >> p.list_shift) + 2) * p.list_cap * kEntry - 256;
+    // (one area more than there are: lists_at)
+    L.list = off; off += (size_t)(list_areas(p) + 1) * p.list_cap * kEntry;
     L.total = off;
     return L;
+}
+
+// Where the lists of a scratch at `base` begin.  An area that would have a multiple of 2^32 bytes between its first and its last
+// byte begins there instead, and all the others move with it: a list's end is advanced by adds to its low word.
+uint64_t lists_at(uint64_t base, const Layout& L, const Plan& p)
+{
+    const uint64_t area = (uint64_t)p.list_cap * kEntry, first = base + L.list, end = first + list_areas(p) * area;
+    const uint64_t multiple = ((first >> 32) + 1) << 32;
+    return multiple < end ? first + (multiple - first) % area : first;
 }
 
 }  // namespace
@@ -1579,10 +1591,10 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
     p->parts = (int)g;
     p->sweep_blocks = (int)sweep_blocks;
     p->list_shift = T <= 32 ? 2 : (T <= 64 ? 1 : 0);
-    // a unit adds at most kCols / 4 entries to a list (a later, shorter chunk may have longer segments)
-    const long long units = share > 0 ? (nsteps + share - 1) / share : (total + g - 1) / g;
-    p->list_cap = kCols / 4;
-    while (p->list_cap < kListCap && (T > kChunkTokens || p->list_cap < units * (kCols / 4))) p->list_cap *= 2;
+    // A unit adds at most kCols / 4 entries to a list (a later, shorter chunk may have longer segments).  One place more than
+    // those, so that the end of a full list is still a place of it (append4).
+    const long long units = share > 0 ? (nsteps + share - 1) / share : (total + g - 1) / g, most = units * (kCols / 4);
+    p->list_cap = T <= kChunkTokens && most < kListCap ? (int)most + 1 : kListCap;
     p->ctas = (int)(share > 0 ? blocks * share : g);
     p->msplit = (int)(p->ctas / blocks > 1 ? p->ctas / blocks : 1);      // (whole ones; a part that begins anywhere can reach into two blocks)
     p->share = (int)share;
@@ -1594,6 +1606,15 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p)
 size_t chain_scratch_bytes(const RouteArgs& a, const Plan& p)
 {
     return layout_of(a, p, a.gate_mode == MORE_GATE_FULL_SOFTMAX || a.out_lse != nullptr).total;
+}
+
+void chain_lists(const RouteArgs& a, const Plan& p, unsigned long long scratch, unsigned long long* out4)
+{
+    const Layout L = layout_of(a, p, a.gate_mode == MORE_GATE_FULL_SOFTMAX || a.out_lse != nullptr);
+    out4[0] = lists_at(scratch, L, p);
+    out4[1] = (unsigned long long)list_areas(p);
+    out4[2] = (unsigned long long)p.list_cap;
+    out4[3] = kEntry;
 }
 
 int launch_finish(const RouteArgs& a, DeviceCtx& ctx, int segments, int cap, const uint2* ent, const int* cnt, const float2* mz)
@@ -1634,7 +1655,7 @@ int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& plan, void* scr
     sp.off_pub = sp.off_r2 + sp.nst * sp.st_bytes;
     sp.off_ctl = sp.off_pub + pub;
     const int smem = sp.off_ctl + ctl + 1024;
-    sp.list = reinterpret_cast<uint8_t*>(align_up(reinterpret_cast<uintptr_t>(base + L.list), (size_t)plan.list_cap * kEntry));
+    sp.list = reinterpret_cast<uint8_t*>(lists_at(reinterpret_cast<uint64_t>(base), L, plan));
     sp.list_cap = plan.list_cap; sp.list_shift = plan.list_shift;
     sp.ent = reinterpret_cast<uint2*>(base + L.ent);
     sp.cnt = reinterpret_cast<int*>(base + L.cnt);

@@ -38,6 +38,14 @@ int more_debug_scratch_guard(void* stream);
  */
 long long more_debug_scratch_bytes(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int path, int msplit);
 
+/*
+ * more_debug_chain_lists -- where the sweep's lists of such a call lie if the scratch allocation is at address `scratch` (the
+ * plan for 148 SMs): out4 = address of the first area, number of areas, places of a list, bytes from one place to the next; an
+ * area is places x bytes long.  MORE_ERR_SHAPE if the chain does not serve the call.  Host-only; needs no device.
+ */
+int more_debug_chain_lists(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int msplit, unsigned long long scratch,
+                           unsigned long long* out4);
+
 #ifdef __cplusplus
 }
 #endif

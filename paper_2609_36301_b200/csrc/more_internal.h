@@ -59,7 +59,7 @@ struct Plan {
     int share = 0;         // ... how many of them share one token block each, or 0 where their parts begin anywhere,
     int maxseg = 1;        // ... and the most that can share one;
     int sweep_blocks = 1;  // ... token blocks per launch of the sweep;
-    int list_cap = 1;      // ... entries of a thread's list,
+    int list_cap = 1;      // ... places of a thread's list,
     int list_shift = 0;    // ... and log2 of the CTAs whose lists lie side by side in one area
 };
 
@@ -75,6 +75,8 @@ void plan_chain(int T, int M, int msplit, int sm_count, Plan* p);
 
 // Scratch bytes each path needs for a problem.
 size_t chain_scratch_bytes(const RouteArgs& a, const Plan& p);
+// The chain's lists in a scratch at that address: where they begin, areas of them, places of a list, bytes between its places.
+void chain_lists(const RouteArgs& a, const Plan& p, unsigned long long scratch, unsigned long long* out4);
 size_t generic_scratch_bytes(const RouteArgs& a);
 size_t lowrank_scratch_bytes(const RouteArgs& a, const Plan& p);
 size_t full_scratch_bytes(const RouteArgs& a, const Plan& p);

@@ -663,6 +663,24 @@ long long more_debug_scratch_bytes(int T, int h, int r, int M, int k, int gate_m
     return rc == MORE_OK ? (long long)scratch_bytes(a, p) : rc;
 }
 
+int more_debug_chain_lists(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int msplit, unsigned long long scratch,
+                           unsigned long long* out4)
+{
+    int rc = check_shape(T, h, r, M, k, gate_mode, MORE_PATH_AUTO);
+    if (rc != MORE_OK) return rc;
+    if (!out4) return MORE_ERR_NULL;
+    RouteArgs a{};
+    float lse;                                               // (only whether it is asked for counts)
+    a.T = T; a.h = h; a.r = r; a.M = M; a.k = k; a.gate_mode = gate_mode;
+    a.out_lse = want_lse ? &lse : nullptr;
+    Plan p;
+    rc = make_plan(T, h, r, M, k, gate_mode, want_lse != 0 || gate_mode == MORE_GATE_FULL_SOFTMAX, false, MORE_PATH_AUTO, msplit, 148, &p);
+    if (rc != MORE_OK) return rc;
+    if (!p.chain) return MORE_ERR_SHAPE;
+    chain_lists(a, p, scratch, out4);
+    return MORE_OK;
+}
+
 const char* more_strerror(int code)
 {
     switch (code) {

@@ -159,6 +159,45 @@ def test_device_memory_of_a_routing_call_is_bounded():
     assert B(64, 4096, 64, 131072, 16) <= 96 * MiB
 
 
+def test_a_full_list_ends_inside_its_area():
+    """The sweep advances the end of a list by adds to the low word of its address.  So whatever the scratch's address, no place of
+    a list may lie behind a multiple of 2^32 bytes that the first one lies before, and the place behind the last entry that a
+    CTA's units can add (eight each) has to be one of them.  (Lists of 64 places are cut at 56 and end at 60 at most.)"""
+    shapes = [(T, M, k) for T in (1, 40, 128, 300, 1000, 2000, 4800) for M in (128, 1024, 5800, 16384, 40000, 131072) for k in (1, 8, 16)]
+    shapes += [(131072, 8192, 4), (131072 + 130, 32768, 4), (20000, 16384, 16)]
+    checked = set()
+    for T, M, k in shapes:
+        for msplit in (0, 1, 3, 16, 64):
+            if not mr.more_route_plan_ex(T, 512, 64, M, k, msplit=msplit).chain:
+                continue
+            size = mr.debug_scratch_bytes(T, 512, 64, M, k, msplit=msplit)
+            at, areas, places, step = mr.debug_chain_lists(T, 512, 64, M, k, msplit=msplit, scratch=1 << 40)
+            # the largest part of the units: equal parts of all blocks, or of one block each
+            blocks, units = -(-min(T, 131072) // 128), -(-M // 128)
+            if T <= 131072:
+                ctas = mr.more_route_plan_ex(T, 512, 64, M, k, msplit=msplit).ctas
+                most = -(-blocks * units // ctas) if not msplit else -(-units // min(msplit, units))
+            else:
+                most = 64
+            assert 8 * most < places or places == 64, (T, M, k, msplit)
+            checked.add(places)
+            area = places * step
+            for where in (0, 256, area // 2, area - 256, area, area + 256, 2 * area - 16384, (areas - 1) * area + 512, areas * area - 256,
+                          areas * area, (areas + 1) * area - 256, (areas + 1) * area):
+                scratch = (9 << 32) - (at - (1 << 40)) - where // 256 * 256
+                first = mr.debug_chain_lists(T, 512, 64, M, k, msplit=msplit, scratch=scratch)[0]
+                assert first % 256 == 0 and scratch <= first and first + areas * area <= scratch + size
+                for a in (first + i * area for i in range(areas)):
+                    assert a >> 32 == a + area - 1 >> 32, (T, M, k, msplit, where)
+                # as the kernel does it: the last thread's list, filled to its last entry
+                for a in (first + i * area for i in range(areas)):
+                    begin = a + step - 32
+                    n = min(8 * most, 60)
+                    end = begin & ~0xffffffff | begin + n * step & 0xffffffff
+                    assert (end - begin) // step == n
+    assert {9, 17, 33, 64} <= checked
+
+
 def test_extension_module_of_another_torch_is_not_used(monkeypatch):
     """The module is compiled against torch's C++ headers: after an upgrade it is built again, and until then refused."""
     import torch
