@@ -75,6 +75,8 @@ def lib() -> ctypes.CDLL:
         L.more_debug_scratch_bytes.restype = ctypes.c_longlong
         L.more_debug_chain_lists.argtypes = [i32] * 8 + [ctypes.c_ulonglong, ctypes.POINTER(ctypes.c_ulonglong)]
         L.more_debug_chain_lists.restype = i32
+        L.more_debug_join_lists.argtypes = [i32] * 5 + [vp] * 10
+        L.more_debug_join_lists.restype = i32
         L.more_strerror.argtypes = [i32]
         L.more_strerror.restype = ctypes.c_char_p
         L.more_version.argtypes = []
@@ -273,6 +275,16 @@ def debug_chain_lists(T, h, r, M, k, gate_mode=0, want_lse=False, msplit=0, scra
     if rc != 0:
         raise MoreRouteError(rc, "more_debug_chain_lists")
     return tuple(out)
+
+
+def debug_join_lists(val, idx, mz, swept, M, gate_mode, out_idx, out_gate, out_counts, out_topval=None, out_lse=None, stream=None):
+    """Diagnostic: the second half of a split standard router, on lists of the caller's: ``val``, ``idx`` [T, parts, k] in descending
+    order, ``mz`` [T, parts, 2], and ``swept`` [T, parts] uint8, 0 where the part's CTA gave up."""
+    T, parts, k = val.shape
+    rc = lib().more_debug_join_lists(T, M, k, gate_mode, parts, _ptr(val), _ptr(idx), _ptr(mz), _ptr(swept), _ptr(out_idx),
+                                     _ptr(out_gate), _ptr(out_counts), _ptr(out_topval), _ptr(out_lse), _stream(stream))
+    if rc != 0:
+        raise MoreRouteError(rc, "more_debug_join_lists")
 
 
 @dataclass

@@ -46,6 +46,16 @@ long long more_debug_scratch_bytes(int T, int h, int r, int M, int k, int gate_m
 int more_debug_chain_lists(int T, int h, int r, int M, int k, int gate_mode, int want_lse, int msplit, unsigned long long scratch,
                            unsigned long long* out4);
 
+/*
+ * more_debug_join_lists -- the second half of a standard router whose experts are split into `parts` (2 ... 256): every part's
+ * list of a token, val and id [T][parts][k] (descending, -inf where it is shorter) and mz [T][parts] = (largest logit x log2 e,
+ * sum), is left in the library's scratch as the part's CTA leaves it, over a pattern, and joined by the finishing kernels.
+ * Where swept [T][parts] is 0 it is left as by a CTA whose wait gave up.  Device pointers; asynchronous on `stream`.
+ */
+int more_debug_join_lists(int T, int M, int k, int gate_mode, int parts, const float* val, const int32_t* id, const void* mz,
+                          const unsigned char* swept, int32_t* out_idx, float* out_gate, int32_t* out_counts, float* out_topval,
+                          float* out_lse, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

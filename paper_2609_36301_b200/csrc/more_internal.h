@@ -87,13 +87,18 @@ int launch_generic(const RouteArgs& a, DeviceCtx& ctx, void* scratch);
 int launch_chain(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
 // The chain's finishing kernels for candidate lists of another sweep, `segments` per token, token t's list s at
 // slot = ((t / 128) segments + s) 128 + t % 128: cnt[slot] entries (logit bits, expert id) from ent[slot cap] on, and where
-// the log-sum-exp counts mz[slot] = (max in log2 units, sum).  out_counts is clear when the work on the stream before is done.
+// the log-sum-exp counts mz[slot] = (max in log2 units, sum).  Every count has to be in 0 ... cap, also where the other sweep gave
+// up.  out_counts is clear when the work on the stream before is done.
 constexpr int kFinishTokens = 128, kFinishMaxSegments = 256;
 int launch_finish(const RouteArgs& a, DeviceCtx& ctx, int segments, int cap, const uint2* ent, const int* cnt, const float2* mz);
 // All tensor-core launchers clear out_counts on the stream themselves, after every host-side step that can fail.
 int launch_lowrank(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
 int launch_full(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
 int launch_paired(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch);
+// The second half of a split standard router (p.msplit parts) alone: lists val, id [T][part][k] in descending order, mz [T][part]
+// as above, parked as the parts' CTAs do, where swept [T][part] is 0 as one that gave up, and joined.
+int launch_park_and_join(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, const float* val, const int* id, const float2* mz,
+                         const unsigned char* swept, void* scratch);
 // Filter mode's preparation: fp16 copy and transposed copy of R2, column-norm maxima, out_counts cleared.
 int launch_route_prepare(const RouteArgs& a, int rpad, void* r2h, void* r2t, void* partial, DeviceCtx& ctx);
 

@@ -681,6 +681,30 @@ int more_debug_chain_lists(int T, int h, int r, int M, int k, int gate_mode, int
     return MORE_OK;
 }
 
+int more_debug_join_lists(int T, int M, int k, int gate_mode, int parts, const float* val, const int32_t* id, const void* mz,
+                          const unsigned char* swept, int32_t* out_idx, float* out_gate, int32_t* out_counts, float* out_topval,
+                          float* out_lse, void* stream)
+{
+    if (T < 1 || M < 1 || k < 1 || k > 32 || parts < 2 || parts > kFinishMaxSegments) return MORE_ERR_SHAPE;
+    if (!val || !id || !mz || !swept || !out_idx || !out_gate || !out_counts) return MORE_ERR_NULL;
+    std::lock_guard<std::mutex> lock(g_mutex);
+    DeviceCtx* ctx = nullptr;
+    int rc = get_ctx(&ctx);
+    if (rc != MORE_OK) return rc;
+    RouteArgs a{};
+    a.T = T; a.M = M; a.k = k; a.gate_mode = gate_mode; a.full = true;
+    a.out_idx = out_idx; a.out_gate = out_gate; a.out_counts = out_counts; a.out_topval = out_topval; a.out_lse = out_lse;
+    a.stream = static_cast<cudaStream_t>(stream);
+    Plan p{};
+    p.msplit = parts;
+    const size_t need = full_scratch_bytes(a, p);
+    rc = ensure_scratch(ctx, need, a.stream);
+    if (rc != MORE_OK) return rc;
+    if (cudaMemsetAsync(ctx->scratch, 0x7f, need, a.stream) != cudaSuccess) return MORE_ERR_CUDA;
+    if (cudaMemsetAsync(out_counts, 0, (size_t)M * sizeof(int32_t), a.stream) != cudaSuccess) return MORE_ERR_CUDA;
+    return launch_park_and_join(a, *ctx, p, val, id, static_cast<const float2*>(mz), swept, ctx->scratch);
+}
+
 const char* more_strerror(int code)
 {
     switch (code) {

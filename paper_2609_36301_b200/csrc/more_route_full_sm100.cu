@@ -119,6 +119,37 @@ __device__ __forceinline__ void write_token(const KernelParams& p, int64_t row, 
     if (p.out_lse) p.out_lse[row] = (m2 + log2f(zsum)) * kLn2;
 }
 
+// A part's list of one token for the finishing kernels.  These come in any case, so where the sweep gave up it is empty.
+template <int KCAP, bool LSE>
+__device__ __forceinline__ void park_list(const KernelParams& p, int64_t row, int part, const TopList<KCAP>& L, float m2, float zsum,
+                                          bool swept)
+{
+    const size_t slot = ((size_t)(row / kFinishTokens) * p.msplit + part) * kFinishTokens + (size_t)(row % kFinishTokens);
+    int n = 0;
+#pragma unroll
+    for (int s = 0; s < KCAP; ++s) {
+        if (s < p.k && swept && L.v[s] > -INFINITY) {
+            p.ent[slot * p.k + s] = make_uint2(__float_as_uint(L.v[s]), (uint32_t)L.id[s]);
+            n = s + 1;
+        }
+    }
+    p.cnt[slot] = n;
+    if (LSE) p.mz[slot] = swept ? make_float2(m2, zsum) : make_float2(-INFINITY, 0.f);
+}
+
+// (diagnostics: lists of the caller's, parked as the sweep does)
+__global__ void park_lists_kernel(const KernelParams p, const float* val, const int* id, const float2* mz, const unsigned char* swept)
+{
+    const int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (at >= (int64_t)p.T * p.msplit) return;
+    TopList<32> L;
+    L.init();
+#pragma unroll
+    for (int s = 0; s < 32; ++s)
+        if (s < p.k) { L.v[s] = val[at * p.k + s]; L.id[s] = id[at * p.k + s]; }
+    park_list<32, true>(p, at / p.msplit, (int)(at % p.msplit), L, mz[at].x, mz[at].y, swept[at] != 0);
+}
+
 // ------------------------------------------------------------------------------------------------- the kernel
 // FULL = true is the fused STANDARD router (logits = X W with W [h][M], no low-rank bottleneck: Alg. 1 without z, the
 // contraction running over K = h): there is no phase 1; every step accumulates 256 experts over all h/64 k-tiles of X
@@ -754,22 +785,10 @@ route_tcgen05_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_con
                 }
             }
         };
-        if (*abort_flag == 0) {
-            if (FULL && p.msplit > 1) {
-                if (row_live) {
-                    const size_t slot = ((size_t)(row / kFinishTokens) * p.msplit + split) * kFinishTokens + (size_t)(row % kFinishTokens);
-                    int n = 0;
-#pragma unroll
-                    for (int s = 0; s < KCAP; ++s) {
-                        if (s < p.k && L.v[s] > -INFINITY) {
-                            p.ent[slot * p.k + s] = make_uint2(__float_as_uint(L.v[s]), (uint32_t)L.id[s]);
-                            n = s + 1;
-                        }
-                    }
-                    p.cnt[slot] = n;
-                    if (LSE) p.mz[slot] = make_float2(m2, zsum);
-                }
-            } else if (p.msplit == 1) {
+        if (FULL && p.msplit > 1) {
+            if (row_live) park_list<KCAP, LSE>(p, row, split, L, m2, zsum, *abort_flag == 0);
+        } else if (*abort_flag == 0) {
+            if (p.msplit == 1) {
                 hist_clear();
                 if (row_live) write_token<KCAP>(p, row, L, m2, zsum, hist);
                 hist_flush();
@@ -1006,6 +1025,13 @@ PairedScratch paired_layout(const RouteArgs& a, const Plan& p)
     return L;
 }
 
+void set_lists(KernelParams& kp, const PairedScratch& L, char* base)
+{
+    kp.ent = reinterpret_cast<uint2*>(base + L.ent);
+    kp.cnt = reinterpret_cast<int*>(base + L.cnt);
+    kp.mz = reinterpret_cast<float2*>(base + L.mz);
+}
+
 }  // namespace
 
 size_t full_scratch_bytes(const RouteArgs& a, const Plan& p) { return paired_layout(a, p).total; }
@@ -1045,9 +1071,7 @@ int launch_paired(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scrat
     kp.R2 = a.R2;
     const bool apart = lists_apart(a, p);
     if (apart) {
-        kp.ent = reinterpret_cast<uint2*>(base + L.ent);
-        kp.cnt = reinterpret_cast<int*>(base + L.cnt);
-        kp.mz = reinterpret_cast<float2*>(base + L.mz);
+        set_lists(kp, L, base);
     } else if (p.msplit > 1) {
         kp.counters = reinterpret_cast<unsigned*>(base + L.counters);
         kp.part_val = reinterpret_cast<float*>(base + L.part_val);
@@ -1078,6 +1102,19 @@ int launch_paired(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scrat
         case 32: return launch_kcap<32, false>(a.k, mode, mx, m1, m2, kp, p.ctas, a.stream, clear);
         default: return launch_kcap<64, false>(a.k, mode, mx, m1, m2, kp, p.ctas, a.stream, clear);
     }
+}
+
+int launch_park_and_join(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, const float* val, const int* id, const float2* mz,
+                         const unsigned char* swept, void* scratch)
+{
+    const PairedScratch L = paired_layout(a, p);
+    KernelParams kp{};
+    kp.T = a.T; kp.k = a.k; kp.msplit = p.msplit;
+    set_lists(kp, L, static_cast<char*>(scratch));
+    const long long lists = (long long)a.T * p.msplit;
+    park_lists_kernel<<<(unsigned)((lists + 255) / 256), 256, 0, a.stream>>>(kp, val, id, mz, swept);
+    if (cudaGetLastError() != cudaSuccess) return MORE_ERR_CUDA;
+    return launch_finish(a, ctx, p.msplit, a.k, kp.ent, kp.cnt, kp.mz);
 }
 
 int launch_full(const RouteArgs& a, DeviceCtx& ctx, const Plan& p, void* scratch) { return launch_paired(a, ctx, p, scratch); }

@@ -70,6 +70,67 @@ def test_full_router_with_few_tokens(T, h, M, k, gate_mode):
     _run(inputs.full_rank_case(T, h, M, k, gate_mode, seed=T + M))
 
 
+@pytest.mark.parametrize("values", ["plain", "equal", "infinite", "gave up"])
+@pytest.mark.parametrize("T,k,parts", [
+    (3, 16, 100),             # more than 64 lists: a CTA of 512 threads per token
+    (2, 32, 256),             # the most and the longest lists
+    (200, 8, 16),             # 512 threads
+    (600, 8, 20),             # 128 threads
+    (700, 16, 8),             # a warp per token, up to 512 entries in registers
+    (900, 8, 8),              # ... up to 256
+    (300, 3, 4),              # a warp per token, the short code
+])
+def test_joining_lists(T, k, parts, values):
+    """The split router's second half alone.  Lists of 0 to k entries, some tokens without any; logits that are all equal or
+    infinite; and parts whose CTA gave up waiting, which must count as empty whatever the scratch held before."""
+    import torch
+    rng = np.random.default_rng(T + k)
+    M = 3 * parts * k
+    val = -np.sort(-rng.standard_normal((T, parts, k)).astype(np.float32), axis=-1)
+    if values == "equal":
+        val[:] = 1.5
+    if values == "infinite":
+        val = -np.sort(-np.where(rng.random(val.shape) < 0.3, np.float32(np.inf), val), axis=-1)
+    length = rng.integers(0, k + 1, (T, parts))
+    length[1::50] = 0                                                        # tokens without a candidate
+    val[np.arange(k) >= length[..., None]] = -np.inf
+    ids = np.argsort(rng.random((T, M)), axis=-1)[:, :parts * k].reshape(T, parts, k).astype(np.int32)
+    mz = np.stack([rng.standard_normal((T, parts)) + 3, rng.random((T, parts)) + 1], axis=-1).astype(np.float32)
+    swept = np.ones((T, parts), dtype=np.uint8)
+    if values == "gave up":
+        swept = (rng.random((T, parts)) < 0.6).astype(np.uint8)
+        swept[0], swept[-1, 0] = 0, 1
+
+    there = (swept != 0)[..., None] & (val > -np.inf)
+    v = np.where(there, val, -np.inf).reshape(T, -1)
+    i = np.where(there, ids, 2**31 - 1).reshape(T, -1)
+    order = np.lexsort((i, -v), axis=-1)[:, :k]
+    want_val, want_idx = np.take_along_axis(v, order, -1), np.take_along_axis(i, order, -1)
+    some = swept.any(axis=1)
+    m = np.where(swept != 0, mz[..., 0].astype(np.float64), -np.inf)
+    top = np.where(some, m.max(axis=1), 0.0)
+    with np.errstate(divide="ignore"):
+        want_lse = (top + np.log2((mz[..., 1] * np.exp2(m - top[:, None])).sum(axis=1))) * np.log(2.0)
+
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    lists = dev(val), dev(ids), dev(mz), dev(swept)
+    for gate_mode in (0, 1):
+        idx = torch.full((T, k), -3, dtype=torch.int32, device="cuda")
+        gate, topval = torch.empty((T, k), device="cuda"), torch.empty((T, k), device="cuda")
+        lse, counts = torch.empty((T,), device="cuda"), torch.full((M,), 77, dtype=torch.int32, device="cuda")
+        mr.debug_join_lists(*lists, M, gate_mode, idx, gate, counts, topval, lse)
+        torch.cuda.synchronize()
+        assert mr.debug_scratch_guard() == 1
+        assert np.array_equal(idx.cpu().numpy(), want_idx) and np.array_equal(topval.cpu().numpy(), want_val)
+        assert np.array_equal(counts.cpu().numpy(), np.bincount(want_idx[want_idx < M], minlength=M))
+        # a few hundred fp32 additions and exponentials good to 2^-22
+        np.testing.assert_allclose(lse.cpu().numpy()[some], want_lse[some], atol=2e-5)
+        sure = np.isfinite(want_val).all(axis=1)
+        e = np.exp(want_val[sure].astype(np.float64) - (want_lse[sure, None] if gate_mode else want_val[sure, :1]))
+        want_gate = e if gate_mode else e / e.sum(-1, keepdims=True)
+        np.testing.assert_allclose(gate.cpu().numpy()[sure], want_gate, rtol=5e-5)
+
+
 def test_full_router_agrees_with_low_rank_router_on_the_identity():
     """Same inputs through ``more_route_ex`` with R1 = I (r = h = 64, the largest the low-rank tensor path takes):
     the two GPU paths must pick the same experts."""
