@@ -1543,19 +1543,20 @@ Layout layout_of(const RouteArgs& a, const Plan& p, bool lse)
     if (lse) off += align_up(lists * kRows * 8, 1024);
     // (last: the finishing kernels' reads then lie at the same addresses however long the lists are; T = 40, M = 6424 26.4 us
     // with the lists in front and 25.1 behind)
-    // (one area more than there are: lists_at)
+    // (one area more than there are, mostly in front of them: lists_at)
     L.list = off; off += (size_t)(list_areas(p) + 1) * p.list_cap * kEntry;
     L.total = off;
     return L;
 }
 
-// Where the lists of a scratch at `base` begin.  An area that would have a multiple of 2^32 bytes between its first and its last
-// byte begins there instead, and all the others move with it: a list's end is advanced by adds to its low word.
+// Where the lists of a scratch at `base` begin.  They end where the scratch does, so that whatever is written behind them meets the
+// guard there.  Only where an area would have a multiple of 2^32 bytes between its first and its last byte does it end there
+// instead, and all the others move with it: a list's end is advanced by adds to its low word.
 uint64_t lists_at(uint64_t base, const Layout& L, const Plan& p)
 {
-    const uint64_t area = (uint64_t)p.list_cap * kEntry, first = base + L.list, end = first + list_areas(p) * area;
+    const uint64_t area = (uint64_t)p.list_cap * kEntry, end = base + L.total, first = end - list_areas(p) * area;
     const uint64_t multiple = ((first >> 32) + 1) << 32;
-    return multiple < end ? first + (multiple - first) % area : first;
+    return multiple < end ? first - (area - (multiple - first) % area) % area : first;
 }
 
 }  // namespace

@@ -198,6 +198,21 @@ def test_a_full_list_ends_inside_its_area():
     assert {9, 17, 33, 64} <= checked
 
 
+def test_the_guard_begins_where_the_lists_end():
+    """The sweep's lists are the last of the scratch, and what is written behind them is caught only in the guard behind it.  Only
+    lists that move because of a multiple of 2^32 bytes may leave room there, less than an area."""
+    for T, M, k in ((1, 1024, 8), (1, 131072, 16), (40, 1024, 3), (300, 5800, 8), (2000, 8192, 16), (20000, 16384, 16), (131202, 32768, 4)):
+        size = mr.debug_scratch_bytes(T, 512, 64, M, k)
+        at, areas, places, step = mr.debug_chain_lists(T, 512, 64, M, k, scratch=1 << 40)
+        end = at + areas * places * step
+        assert end == (1 << 40) + size and size % 256 == 0
+        for before in (0, 256, 16384, places * step, areas * places * step - 256):      # the multiple, so far in front of the end
+            scratch = (9 << 32) + before - size
+            at = mr.debug_chain_lists(T, 512, 64, M, k, scratch=scratch)[0]
+            slack = scratch + size - (at + areas * places * step)
+            assert 0 <= slack < places * step and (slack == 0 or before % (places * step))
+
+
 def test_extension_module_of_another_torch_is_not_used(monkeypatch):
     """The module is compiled against torch's C++ headers: after an upgrade it is built again, and until then refused."""
     import torch
