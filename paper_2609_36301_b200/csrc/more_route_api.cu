@@ -193,22 +193,29 @@ namespace {
 // do it all: by experts against tokens per SM.  What the chain pays on top (a threshold, the reading back of a list and the
 // finishing kernel's ranking and counting, per token and segment) grows with the tokens and not with the experts, what it
 // gains (a projection that is not repeated, an even cut of the units, cheaper selection) with both; a larger h favours it,
-// as a cluster shares the reading of X.  So the lines are straight: M >= c x (tokens per SM), c by how tight the bound on
-// the k-th logit is for the number of buckets (k <= 4 of 16, k <= 8 of 16, k <= 16 of 32; above that it is too loose), and
-// with fewer than 1024 experts, eight units or less per token block, somewhat more.  From 340 tokens per SM on, the paired
-// kernel's two CTAs per SM fill up, and for k = 5 ... 8 it keeps what lies below c = 40 (20 where the exponentials slow it down):
-// a single call is quicker on the chain (T = 65536, h = 2048, r = 64, M = 16384: 343 us against 366), but under sustained load,
-// where the chip's power limit counts, it is not (400 against 390).  Measured on B200, one call after the other: the lines are
-// fitted to 1000 shapes of T = 6 k ... 64 k, M = 192 ... 12 k, h = 128 ... 2048, r = 16, 32, 64, k = 1 ... 16, both gates;
-// profiles/kernel_choice.csv holds others, to which nothing was fitted, where the choice costs 2 % on average against the better side of
-// each shape (3 % with fewer than 1024 experts, 1 % with more; always the chain would cost 15 %, never the chain 23 %).
-bool chain_wins(int T, int h, int M, int k, bool lse, int sm_count)
+// as a cluster shares the reading of X.  So the lines are straight: M + h / 16 >= c x (tokens per SM), c by k (ranking and the
+// bound on the k-th logit: 16 buckets for k <= 8, 32 for k <= 16; above that it is too loose), and larger with fewer than
+// 1024 experts, eight units or less per token block, most of all where k is near half the buckets.
+// Beyond 340 tokens per SM the paired kernel's two CTAs per SM fill up, and for k = 5 ... 8 c is 10.  With k = 7, 8 and r > 48 a
+// call that is alone and calls under sustained load, where the chip's power limit counts, differ there, and it stays 40 (20 with
+// the softmax sweep).  h = 2048, r = 64, M = 16384, k = 8, T = 65536: chain 340 us, paired kernel 380, under load 388 and 384;
+// M = 8192: 241 and 257, under load 267 and 249; T = 53000: 275 and 341, 315 and 351.
+// Measured on B200, one call after the other: fitted to 4300 shapes of T = 1 ... 64 k, h = 128 ... 4096, r = 8 ... 64, M = 128 ... 16 k,
+// k = 1 ... 16, both gates, most of them near the lines.  profiles/kernel_choice.csv holds 1250 others, to which nothing was
+// fitted: there the choice costs 0.8 % on average against the better side and more than 5 % at 4 % of them, 1.46 at most (0.6 %
+// and 3 % up to 64 k tokens; beyond, where nothing was fitted, 1.9 % and 13 %, 1.30 at most); always the chain would cost 14 %,
+// never the chain 56 %.
+bool chain_wins(int T, int h, int r, int M, int k, bool lse, int sm_count)
 {
     const int per_sm = (T + sm_count - 1) / sm_count, wide = h < 4096 ? h : 4096;
     if (k > 16 || M < 128) return false;
-    if (M < 1024) return M + wide / 4 - 128 >= (k <= 4 ? 5 : 14) * per_sm;
-    const int c = k <= 4 ? 4 : (k > 8 ? 6 : (per_sm <= 340 ? 9 : (lse ? 20 : 40)));
-    return M + wide / 8 >= c * per_sm;
+    if (M < 1024) {
+        if ((k > 6 && k <= 8) || k > 12) return M + wide / 4 >= (k <= 8 ? 18 : 20) * per_sm;
+        return M + wide / 16 >= (k == 1 ? 2 : (k == 2 ? 4 : (k <= 4 ? 5 : (k <= 6 ? 9 : 10)))) * per_sm;
+    }
+    double c = k == 1 ? 2 : (k == 2 ? 3 : (k <= 4 ? 3.5 : (k <= 6 ? 7 : (k <= 8 ? 8 : 5))));
+    if (per_sm > 340 && k > 4 && k <= 8) c = r > 48 && k > 6 ? (lse ? 20 : 40) : 10;
+    return M + wide / 16 >= c * per_sm;
 }
 
 // Launch plan of the paired low-rank kernel (256-token CTAs, two per SM).
@@ -374,7 +381,7 @@ int make_plan(int T, int h, int r, int M, int k, int gate_mode, bool want_lse, b
     if (full) {
         plan_dense(T, h, M, k, msplit, sm_count, &p);
     } else {
-        if (chain_wins(T, h, M, k, want_lse || gate_mode == MORE_GATE_FULL_SOFTMAX, sm_count)) {
+        if (chain_wins(T, h, r, M, k, want_lse || gate_mode == MORE_GATE_FULL_SOFTMAX, sm_count)) {
             plan_chain(T, M, msplit, sm_count, &p);
             *out = p;
             return MORE_OK;

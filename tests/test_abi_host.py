@@ -122,6 +122,17 @@ def test_choice_of_the_chain_has_no_holes():
         assert chain(T, M, 4, 2048, 0) == chain(T, M, 1, 2048, 0) and chain(T, M, 8, 2048, 0) == chain(T, M, 5, 2048, 0)
 
 
+@pytest.mark.parametrize("T,h,r,M,k,gate,us_chain,us_one", [
+    (15019, 2048, 64, 208, 4, 0, 48.8, 32.9), (16652, 2680, 16, 168, 3, 1, 54.2, 34.8), (25521, 3608, 48, 440, 4, 1, 82.7, 72.7),
+    (9947, 3728, 40, 304, 15, 1, 84.7, 64.9), (14350, 1728, 40, 240, 3, 0, 38.2, 32.8), (1651, 136, 24, 144, 2, 1, 14.2, 23.4),
+    (6229, 128, 16, 304, 2, 0, 14.2, 20.8), (23020, 512, 16, 504, 1, 0, 25.9, 39.2), (50540, 1024, 48, 6784, 6, 0, 148.0, 182.0),
+    (45337, 584, 48, 8056, 5, 0, 125.9, 193.8), (54277, 136, 48, 9704, 7, 0, 161.7, 217.8), (36910, 2048, 64, 728, 12, 0, 120.4, 95.4),
+])
+def test_choice_of_the_quicker_kernel(T, h, r, M, k, gate, us_chain, us_one):
+    """Shapes near the lines of the choice whose two sides were measured far apart (microseconds on B200)."""
+    assert mr.more_route_plan_ex(T, h, r, M, k, gate).chain == (us_chain < us_one)
+
+
 def test_shared_memory_plan_of_the_grouped_kernel_fits():
     """Every (rank, token groups, expert ranges) the planner may pick leaves room for at least two R2 stages and one
     phase-1 stage in the 208 KB ring (checked through the plans of shapes that exercise them)."""
