@@ -77,6 +77,8 @@ def lib() -> ctypes.CDLL:
         L.more_debug_chain_lists.restype = i32
         L.more_debug_join_lists.argtypes = [i32] * 5 + [vp] * 10
         L.more_debug_join_lists.restype = i32
+        L.more_debug_psum_plan.argtypes = [i32] * 3 + [ctypes.POINTER(i32)]
+        L.more_debug_psum_plan.restype = i32
         L.more_strerror.argtypes = [i32]
         L.more_strerror.restype = ctypes.c_char_p
         L.more_version.argtypes = []
@@ -274,6 +276,15 @@ def debug_chain_lists(T, h, r, M, k, gate_mode=0, want_lse=False, msplit=0, scra
     rc = int(lib().more_debug_chain_lists(T, h, r, M, k, gate_mode, int(want_lse), msplit, scratch, out))
     if rc != 0:
         raise MoreRouteError(rc, "more_debug_chain_lists")
+    return tuple(out)
+
+
+def debug_psum_plan(T, h, M):
+    """Diagnostic: how ``more_route_psum`` cuts a call: tokens of a block, CTAs per block."""
+    out = (ctypes.c_int32 * 2)()
+    rc = int(lib().more_debug_psum_plan(T, h, M, out))
+    if rc != 0:
+        raise MoreRouteError(rc, "more_debug_psum_plan")
     return tuple(out)
 
 

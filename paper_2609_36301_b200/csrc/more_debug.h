@@ -56,6 +56,12 @@ int more_debug_join_lists(int T, int M, int k, int gate_mode, int parts, const f
                           const unsigned char* swept, int32_t* out_idx, float* out_gate, int32_t* out_counts, float* out_topval,
                           float* out_lse, void* stream);
 
+/*
+ * more_debug_psum_plan -- how more_route_psum cuts a call on its tensor-core path (148 SMs): out2 = tokens of a block, CTAs per
+ * block.  Host-only; needs no device.
+ */
+int more_debug_psum_plan(int T, int h, int M, int* out2);
+
 #ifdef __cplusplus
 }
 #endif

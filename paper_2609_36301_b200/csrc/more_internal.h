@@ -104,6 +104,8 @@ int launch_route_prepare(const RouteArgs& a, int rpad, void* r2h, void* r2t, voi
 
 int launch_generic_psum(const __nv_bfloat16* X, const __nv_bfloat16* R1, const __nv_bfloat16* R2, int T, int h, int r,
                         int M, const float* lse, float* psum, void* scratch, cudaStream_t stream);
+// How a call of the column sums is cut on its tensor-core path: tokens of a block, CTAs per block.
+void plan_psum(int T, int h, int M, int sm_count, int* block, int* split);
 int launch_psum_tcgen05(const __nv_bfloat16* X, const __nv_bfloat16* R1, const __nv_bfloat16* R2, int T, int h, int r,
                         int M, const float* lse, float* psum, DeviceCtx& ctx, cudaStream_t stream);
 

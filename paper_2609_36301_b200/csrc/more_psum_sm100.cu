@@ -322,7 +322,49 @@ int launch_psum_rpad(const CUtensorMap& mx, const CUtensorMap& m1, const CUtenso
     return cudaGetLastError() == cudaSuccess ? MORE_OK : MORE_ERR_CUDA;
 }
 
+// Tokens of a block, and CTAs per block, by a model of the time.  CTAs that have an SM each take less than half of what two on an
+// SM do where the projection counts, as 256 rows of X per k-tile, whatever the block, are bound by the SM's share of L2, and all
+// of them together slow each other down (T = 2737, h = 3800, M = 7136: 77 CTAs 51 us, 220 of them 82; T = 18993, h = 744, M = 184:
+// 75 CTAs 18.9 us, 119 22.7).  Microseconds, fitted to 300 shapes (T = 129 ... 64 k, h = 128 ... 4096, r = 8 ... 64, M = 128 ... 128 k)
+// at up to 35 pairs of block and split each.  On 200 others what is chosen takes 1.01 of the best pair's time on average and 1.12
+// at most; blocks of 256 and two CTAs per SM wherever there are four tiles for each take 1.14, and stay only where no other pair
+// should be 3 % better.
+void choose_blocks(int T, int h, int tiles, int slots, int* block_out, int* split_out)
+{
+    const double ktiles = (h + 63) / 64;
+    double best = 1e300;
+    auto consider = [&](int block, int split, double handicap) {
+        const int per = (tiles + split - 1) / split, s = (tiles + per - 1) / per;
+        const long long ctas = (long long)((T + block - 1) / block) * s, waves = (ctas + slots - 1) / slots;
+        const double chunks = block / 16.0;
+        const double alone = 0.88 + 0.234 * ktiles + per * (0.623 + 0.0545 * chunks);
+        const double shared = 2.14 + 0.537 * ktiles + per * (0.80 + 0.117 * chunks);
+        const double last = 2 * (ctas - (waves - 1) * slots) <= slots ? alone : shared;      // the last wave
+        const double us = (5.5 + (waves - 1) * shared + last + 0.0021 * ctas * ktiles) * handicap;
+        if (us < best) { best = us; *block_out = block; *split_out = s; }
+    };
+    const int n = (T + kBlockTokens - 1) / kBlockTokens, most = slots / n < tiles / 4 ? slots / n : tiles / 4;
+    consider(kBlockTokens, most < 1 ? 1 : (most < 64 ? most : 64), 0.97);
+    for (int block = kBlockTokens; block >= 160; block -= 32) {
+        const int blocks = (T + block - 1) / block;
+        for (int all = slots; all >= slots / 2; all -= slots / 2)
+            for (int part = 12; part >= 3; part -= 3) {
+                const int split = all / blocks * part / 12;
+                consider(block, split < 1 ? 1 : (split < tiles ? split : tiles), 1.0);
+            }
+    }
+}
+
 }  // namespace
+
+void plan_psum(int T, int h, int M, int sm_count, int* block, int* split)
+{
+    const int slots = 2 * (sm_count > 0 ? sm_count : 148), tiles = (M + kTileExperts - 1) / kTileExperts;
+    if (T > kFewTokens) return choose_blocks(T, h, tiles, slots, block, split);
+    *block = kFewTokens;                           // a CTA per SM at most, two tiles or more
+    *split = tiles / 2 < slots / 2 ? tiles / 2 : slots / 2;
+    if (*split < 1) *split = 1;
+}
 
 int launch_psum_tcgen05(const __nv_bfloat16* X, const __nv_bfloat16* R1, const __nv_bfloat16* R2, int T, int h, int r,
                         int M, const float* lse, float* psum, DeviceCtx& ctx, cudaStream_t stream)
@@ -338,33 +380,8 @@ int launch_psum_tcgen05(const __nv_bfloat16* X, const __nv_bfloat16* R1, const _
     pp.T = T; pp.h = h; pp.r = r; pp.M = M;
     pp.tiles_total = (M + kTileExperts - 1) / kTileExperts;
     pp.lse = lse; pp.psum = psum; pp.status = ctx.status;
-    // Tokens of a block, and CTAs per block: what fills the waves of resident CTAs (two per SM) best.  A CTA's time is that of
-    // its 16-token chunks x tiles, and what every one pays at its start (256 rows of X per k-tile, narrowing) is worth about
-    // 300 + 4 h / 64 of those; each keeps four expert tiles or more.  T = 65536, h = 512, M = 8192: 256 blocks of 256 tokens
-    // give 108 SMs two CTAs and 40 one, 293 of 224 give all of them two: 171 -> 160 us; T = 40000, h = 4096, M = 4096 157 blocks
-    // or 250 of 160: 149 -> 128; T = 512, M = 1024 (192 tokens) 14.3 -> 12.8; T = 3001, M = 5000 27.1 with 256 and 27.8 with 224.
-    const int slots = 2 * (ctx.sm_count > 0 ? ctx.sm_count : 148);
-    double best = 1e300;
-    int blocks = 0, s = 1;
-    for (int block = kBlockTokens; block >= 160; block -= 32) {
-        const int n = (T + block - 1) / block;
-        int split = slots / n;
-        if (split > pp.tiles_total / 4) split = pp.tiles_total / 4;
-        if (split < 1) split = 1;
-        if (split > 64) split = 64;
-        const long long ctas = (long long)n * split, waves = (ctas + slots - 1) / slots;
-        // the last wave's CTAs have an SM each if there are no more of them
-        const double last = 2 * (ctas - (waves - 1) * slots) <= slots ? 0.6 : 1.0;
-        const double cost = ((double)waves - 1.0 + last) * (block / 16.0 * ((pp.tiles_total + split - 1) / split) + 300.0 + 4.0 * (h / 64));
-        if (cost < best * 0.97) { best = cost; blocks = n; s = split; pp.block = block; }
-    }
-    if (few) {                                     // a CTA per SM at most, two tiles or more
-        pp.block = kFewTokens;
-        blocks = 1;
-        s = pp.tiles_total / 2 < slots / 2 ? pp.tiles_total / 2 : slots / 2;
-        if (s < 1) s = 1;
-    }
-    pp.msplit = s;
+    plan_psum(T, h, M, ctx.sm_count, &pp.block, &pp.msplit);
+    const int s = pp.msplit, blocks = (T + pp.block - 1) / pp.block;
     switch (rpad) {
         case 16: return launch_psum_rpad<16>(mx, m1, m2, pp, blocks * s, stream);
         case 32: return launch_psum_rpad<32>(mx, m1, m2, pp, blocks * s, stream);

@@ -712,6 +712,14 @@ int more_debug_join_lists(int T, int M, int k, int gate_mode, int parts, const f
     return launch_park_and_join(a, *ctx, p, val, id, static_cast<const float2*>(mz), swept, ctx->scratch);
 }
 
+int more_debug_psum_plan(int T, int h, int M, int* out2)
+{
+    if (T < 1 || h < 1 || M < 1) return MORE_ERR_SHAPE;
+    if (!out2) return MORE_ERR_NULL;
+    plan_psum(T, h, M, 148, &out2[0], &out2[1]);
+    return MORE_OK;
+}
+
 const char* more_strerror(int code)
 {
     switch (code) {

@@ -209,6 +209,27 @@ def test_a_full_list_ends_inside_its_area():
     assert {9, 17, 33, 64} <= checked
 
 
+@pytest.mark.parametrize("T,h,M,most,us,us_more", [
+    (2737, 3800, 7136, 148, 51.4, 82.2), (1218, 3520, 15256, 148, 38.0, 54.7), (46814, 1008, 312, 200, 27.4, 34.0),
+    (18993, 744, 184, 100, 18.9, 22.7), (1068, 2824, 29056, 148, 48.6, 73.0), (5902, 2872, 4304, 148, 41.4, 57.9),
+])
+def test_column_sums_take_no_more_ctas_than_pay(T, h, M, most, us, us_more):
+    """Shapes with a large projection and few tiles for each CTA, which up to `most` CTAs finish in `us` and more of them in
+    `us_more` (microseconds on B200)."""
+    block, split = mr.debug_psum_plan(T, h, M)
+    assert -(-T // block) * split <= most, (block, split, us, us_more)
+
+
+def test_cut_of_the_column_sums_is_sound():
+    for T in (1, 128, 129, 160, 161, 300, 1000, 5000, 40000, 47360, 47361, 65536, 1 << 20):
+        for h in (8, 512, 4096):
+            for M in (8, 128, 1000, 8192, 131072):
+                block, split = mr.debug_psum_plan(T, h, M)
+                tiles = -(-M // 128)
+                assert block == 128 if T <= 128 else block in (160, 192, 224, 256)
+                assert 1 <= split <= tiles and -(-T // block) * split <= max(296, -(-T // block))
+
+
 def test_the_guard_begins_where_the_lists_end():
     """The sweep's lists are the last of the scratch, and what is written behind them is caught only in the guard behind it.  Only
     lists that move because of a multiple of 2^32 bytes may leave room there, less than an area."""

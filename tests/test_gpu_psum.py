@@ -48,6 +48,19 @@ def test_psum_blocks_of_fewer_than_256_tokens(T, h, r, M):
     np.testing.assert_allclose(got.sum(), T, rtol=1e-4)
 
 
+@pytest.mark.parametrize("T,h,r,M,block", [(1793, 64, 64, 4096, 224), (3585, 64, 8, 1000, 224), (671, 72, 16, 4096, 224), (2881, 64, 32, 1000, 192),
+                                            (767, 128, 64, 4096, 192), (2049, 64, 16, 4096, 256), (2047, 128, 32, 4096, 256),
+                                            (129, 64, 16, 18944, 160)])
+def test_psum_edges_of_the_blocks_that_are_planned(T, h, r, M, block):
+    """A last block of one token and of one less than it holds, and a CTA for each of 148 tiles."""
+    assert mr.debug_psum_plan(T, h, M)[0] == block
+    case = inputs.gaussian_case(T, h, r, M, 4, 1, seed=64)
+    got, _ = run_psum(case, mr.PATH_TCGEN05)
+    want, _ = oracle.psum(case.X, case.R1, case.R2)
+    np.testing.assert_allclose(got, want, rtol=RTOL, atol=ATOL)
+    np.testing.assert_allclose(got.sum(), T, rtol=1e-4)
+
+
 @pytest.mark.parametrize("T,h,r,M", [(33, 40, 8, 130), (300, 100, 12, 1000), (64, 64, 96, 256)])
 def test_psum_generic_path(T, h, r, M):
     case = inputs.gaussian_case(T, h, r, M, 2, 1, seed=62)
