@@ -158,8 +158,10 @@ def test_tokens_of_zeros(T, M, k):
     (296, 2048, 16),       # the most tokens that they take
     (297, 2048, 16),       # 16 segments: CTAs of 128 threads
     (310, 4096, 8),
-    (700, 8200, 16),       # 49 segments, the last of 8 experts
-    (600, 1024, 16),       # 8 segments: a warp per token, candidates in registers
+    (700, 8200, 16),       # 49 segments of one or two units
+    (700, 6152, 16),       # 49 segments of one unit, the last of 8 experts
+    (600, 1024, 16),       # 8 segments
+    (700, 1024, 16),       # 8 segments: a warp per token, candidates in registers
     (1300, 4096, 4),       # 26 segments
     (1300, 512, 4),        # four segments: the short code
 ])

@@ -58,7 +58,8 @@ def test_full_router_with_expert_split(msplit):
 
 @pytest.mark.parametrize("gate_mode", [0, 1])
 @pytest.mark.parametrize("T,h,M,k", [
-    (1, 72, 37896, 1),            # one token, 148 CTAs of one tile of 256 experts, the last of eight experts
+    (1, 72, 37896, 1),            # one token, CTAs of one or two tiles of 256 experts, the last of eight experts
+    (1, 72, 37640, 1),            # 148 CTAs of one tile, the last of eight experts
     (1, 512, 40000, 32),          # the longest lists
     (10, 1448, 5000, 3),          # 20 CTAs
     (130, 64, 9000, 17),          # two runs of 128 tokens in one block
@@ -68,6 +69,46 @@ def test_full_router_with_expert_split(msplit):
 def test_full_router_with_few_tokens(T, h, M, k, gate_mode):
     """Many CTAs per token block, whose lists the finishing kernels join."""
     _run(inputs.full_rank_case(T, h, M, k, gate_mode, seed=T + M))
+
+
+@pytest.mark.parametrize("gate_mode", [0, 1])
+@pytest.mark.parametrize("T,M,k", [
+    (40, 37640, 32),              # 148 CTAs of one tile: more equals than the finishing kernel holds
+    (300, 20008, 16),
+    (600, 1032, 8),               # a warp per token
+])
+def test_full_router_with_extreme_logits_and_an_expert_split(T, M, k, gate_mode):
+    """Tokens with equal logits, with infinite ones (every second expert), and of NaN: the first two are sorted as any others,
+    and none of them changes the other tokens."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(T + M + k)
+    X = torch.randn((T, 72), generator=gen, device="cuda").to(torch.bfloat16)
+    W = (torch.randn((72, M), generator=gen, device="cuda") / 8).to(torch.bfloat16)
+    W[0, ::2], W[0, 1::2] = 4, 1
+    zero, half, nan = (torch.arange(i, T, 17, device="cuda") for i in (3, 4, 5))
+    X[zero], X[half], X[nan] = 0, 0, 0
+
+    def run():
+        idx = torch.full((T, k), -3, dtype=torch.int32, device="cuda")
+        gate, topval, lse = (torch.empty(s, device="cuda") for s in ((T, k), (T, k), (T,)))
+        counts = torch.full((M,), 77, dtype=torch.int32, device="cuda")
+        mr.more_route_full(X, W, k, gate_mode, idx, gate, counts, topval, lse)
+        torch.cuda.synchronize()
+        assert mr.more_route_status() == 0 and mr.debug_scratch_guard() == 1
+        valid = idx[(idx >= 0) & (idx < M)]
+        assert torch.equal(torch.bincount(valid.long(), minlength=M).int(), counts)
+        return idx, gate, topval
+
+    clean = run()
+    first = torch.arange(k, device="cuda", dtype=torch.int32)
+    assert bool((clean[0][zero] == first).all()) and bool((clean[0][nan] == first).all())
+    X[half, 0], X[nan, 1] = 2e38, float("nan")
+    idx, gate, topval = run()
+    assert bool((idx[zero] == first).all()) and bool((idx[half] == 2 * first).all()) and bool(torch.isinf(topval[half]).all())
+    others = torch.ones(T, dtype=torch.bool, device="cuda")
+    others[half], others[nan] = False, False
+    for a, b in zip(clean, (idx, gate, topval)):
+        assert torch.equal(a[others], b[others])
 
 
 @pytest.mark.parametrize("values", ["plain", "equal", "infinite", "gave up"])
