@@ -77,10 +77,22 @@ def load_counters():
         return {}
 
 
+def instantiation_of(c, gate_mode, plan):
+    """The main kernel of a workload's plan as the profiler names it, with its template arguments."""
+    kcap = 8 if c["k"] <= 8 else (16 if c["k"] <= 16 else 32)
+    if plan.chain:
+        units = -(-c["T"] // 128) * -(-c["M"] // 128)                        # of 128 tokens x 128 experts
+        return f"sweep_kernel<{kcap}, {gate_mode}, {int(c['T'] <= 131072 and -(-units // plan.ctas) <= 2)}>"
+    rpad = 16 if c["r"] <= 16 else (32 if c["r"] <= 32 else 64)
+    return f"route_tcgen05_kernel<{rpad}, {kcap}, {gate_mode}, 0, 0>" if plan.paired else kernel_of(plan)
+
+
 def counters_of(counters, name, gate_mode, plan):
-    """The counters of a workload, unless they were captured on another kernel than the one that serves it now."""
+    """The counters of a workload, unless they were captured on another kernel, or another instantiation of it, than the one
+    that serves it now."""
+    from paper_2609_36301_b200 import inputs
     entry = counters.get(f"{name}/mode{gate_mode}", {})
-    return entry if entry and entry["kernel"].split("<")[0] in kernel_of(plan) else {}
+    return entry if entry and entry["kernel"] == instantiation_of(inputs.CONFIGS[name], gate_mode, plan) else {}
 
 
 SM_COUNT = 148

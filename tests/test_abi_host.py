@@ -274,3 +274,17 @@ def test_committed_counters_are_of_the_kernels_that_run():
         assert os.path.exists(os.path.join(ROOT, re.search(r"profiles/\S+\.md", entry["source"]).group()))
         other = mr.more_route_plan_ex(2000, 64, 16, 64, 2)                 # too few experts for the chain, too few tokens for pairs
         assert bench.counters_of(counters, name, int(gate_mode), other) == {}
+
+
+@pytest.mark.parametrize("name,kernel,other", [("c2_M16384/mode0", "sweep_kernel<8, 0, 0>", "sweep_kernel<8, 0>"),
+                                               ("c3/mode1", "sweep_kernel<8, 1, 0>", "sweep_kernel<16, 1, 0>"),
+                                               ("c3/mode0", "route_tcgen05_kernel<64, 8, 0, 0, 0>", "route_tcgen05_kernel<32, 8, 0, 0, 0>")])
+def test_counters_of_another_instantiation_are_not_used(name, kernel, other):
+    import bench
+    from paper_2609_36301_b200 import inputs
+    config, gate_mode = name.split("/mode")
+    c = inputs.CONFIGS[config]
+    plan = mr.more_route_plan_ex(c["T"], c["h"], c["r"], c["M"], c["k"], int(gate_mode))
+    for k in (kernel, other):
+        entry = {"kernel": k, "dram_bytes": 1}
+        assert bench.counters_of({name: entry}, config, int(gate_mode), plan) == (entry if k == kernel else {})
