@@ -4,15 +4,16 @@
 // T x M probabilities never exist in memory.
 //
 // The first half of the kernel is the router's: TMA streams X and R1, tcgen05.mma accumulates z = X_blk R1 for a
-// block of 256 tokens in TMEM, the epilogue threads narrow it to bf16 hi + lo in shared memory.  The second
+// block of 128 or 160 ... 256 tokens in TMEM, the epilogue threads narrow it to bf16 hi + lo in shared memory.  The second
 // contraction is issued TRANSPOSED, D[expert][token] = R2[:, tile]^T z^T: the R2 tile is the (MN-major) A operand,
 // z the (K-major) B operand, so a TMEM lane is an expert and its columns are tokens.  Each epilogue thread then owns
-// one expert of the tile and adds exp(y - lse_token) over the 128 token columns of its half in registers -- a column
+// one expert of the tile and adds exp(y - lse_token) over its share of the block's token columns in registers -- a column
 // sum with no cross-lane traffic -- and finishes with one atomic add into psum.  (In the router the lanes are tokens,
 // because there the reduction runs along the expert axis.)
 //
 // Warp roles, shared-memory ring, barriers and the bounded waits are those of the router kernel, but for 16 epilogue warps:
-// four per lane quarter, two per 128-token half, which take 64 token columns each.  Bound by the exponentials: 12 of 16 go
+// four per lane quarter, two for the first 128 tokens, which take 64 token columns each, and two for what the block has beyond
+// them, 16 to 64 columns each (none up to 128 tokens).  Bound by the exponentials: 12 of 16 go
 // through the special-function unit (16 results per clock and SM), four through the FMA pipe, and with 32 epilogue warps
 // per SM the latencies around them are hidden (16 warps, which could each hold twice the registers: 53 % of the issue
 // slots used).

@@ -257,14 +257,12 @@ void plan_paired(int T, int h, int M, int msplit, int sm_count, Plan* p)
 // steps per CTA; splitting the experts over a few CTAs per token block evens out the last wave.
 void plan_dense(int T, int h, int M, int k, int msplit, int sm_count, Plan* p)
 {
-    // Microseconds on B200: 0.6 per k-tile of a step (its eight MMAs of 128 x 256 x 16 take 0.58), and by the length of the
-    // lists what a step's epilogue, a CTA (start, pipeline fill, first candidates, output) and the merge of parked lists cost
-    // on top.  Fitted to 3300 shapes (T = 1 ... 20000, h = 128 ... 4096, M = 280 ... 16384, k = 1 ... 32, both gates) at forced
-    // splits of 1 to 16: the split chosen costs 0.5 % on average against the best of them, 2 % with one set for all k from
-    // before a K-slice was one MMA of N = 256 (T = 500, h = 256, M = 1000, k = 8 55 us against 40).
-    // (Since the parked lists have finishing kernels of their own they cost 1 more than a CTA that writes its results itself (T = 173,
-    // h = 552, M = 440 43.2 us by one CTA, 32.4 by two), whatever their length, and as many CTAs may share a
-    // block as there are SMs: T = 10, h = 1448, M = 20920 158 -> 50 us, T = 500, h = 4096, M = 65536 789 -> 238.)
+    // Microseconds on B200: 0.6 per k-tile of a step (its eight MMAs of 128 x 256 x 16 take 0.58), by the length of the lists what
+    // a step's epilogue and a CTA (start, pipeline fill, first candidates, output) cost on top, and 1 for the finishing kernel
+    // that joins the lists of a split, whatever their length (T = 173, h = 552, M = 440 43.2 us by one CTA, 32.4 by two).  As many
+    // CTAs may share a block as there are SMs: T = 10, h = 1448, M = 20920 158 us by 16, 50 by 82; T = 500, h = 4096, M = 65536 789 and
+    // 238.  On 200 shapes drawn from T = 1 ... 16384, h = 128 ... 4096, M = 256 ... 128 k, k = 1 ... 32, both gates, the split chosen is at
+    // most 2 % behind the best of 14 forced ones from 1 to 64.
     const double epilogue = k <= 8 ? 2.0 : 7.0, start = k <= 8 ? 21.0 : (k <= 16 ? 40.0 : 60.0), merge = 1.0;
     const int tiles = (M + 255) / 256;
     const double ktiles = (h + 63) / 64;
